@@ -446,7 +446,7 @@ dbg_status dbg_autotune(dbg_ctx *ctx, uint64_t n, const char *cache_path, double
 
 /* ----------------------------------------------------------------------
  * Hybrid sort switch.  With it on (the default) the sorts of STEP-2 and
- * STEP-3 run the onesweep passes only over the high digits, which groups
+ * STEP-3 run global passes only over the high digits, which groups
  * keys with equal high bits, and finish each run of whole groups in shared
  * memory (for the edge keys fused with STEP-2's duplicate removal).  Runs
  * longer than shared memory holds (6144 keys for k <= 31, 3072 above; e.g.
@@ -472,30 +472,31 @@ dbg_status dbg_sort_count_first_set(dbg_ctx *ctx, int on);
 uint64_t dbg_sort_count_overflows(const dbg_ctx *ctx);
 
 /* ----------------------------------------------------------------------
- * Partition-first switch.  With it on (the default) the first global
- * radix pass over the edge keys (which carry no payload) is an unordered
- * partition by that digit: keys of one digit keep no particular order,
- * which no later step depends on (the later passes are stable and equal
- * keys are identical), and no tile waits for another.  Off, it is a
- * stable onesweep pass like the others.  The graph is the same either
- * way.  Node records, whose payload order matters, always sort stably.
+ * Partition switch.  With it on (the default) the hybrid sort's global
+ * passes are unordered partitions, most significant digit first: at most two,
+ * with digits of up to 12 bits, in which no tile waits for another.  Equal
+ * edge keys are identical, and the local pass puts node records with equal
+ * keys back into payload order (which needs the group-ranking switch below).
+ * Off, or where the key bits are too few for that, the global passes are
+ * stable onesweep passes, least significant digit first -- except, with the
+ * switch on, the first pass over keys without payload, whose input order
+ * does not matter.  The graph is the same either way.
  * -------------------------------------------------------------------- */
 dbg_status dbg_sort_partition_first_set(dbg_ctx *ctx, int on);
 
 /* ----------------------------------------------------------------------
- * Group-ranking switch for the local passes of the hybrid sort.  The
- * global passes leave keys with equal high bits (a group) contiguous; with
- * the switch on (the default) a local pass places each key at its group's
- * start plus the number of the group's keys that precede it (for the
- * count-first edge pass, the distinct keys below it; for 64-bit node
- * records, the records with smaller low bits or an equal key and an
- * earlier position, which keeps the sort stable).  Tiles holding a group
+ * Group-ranking switch for the local passes of the hybrid sort.  With the
+ * switch on (the default) a local pass spreads a tile's keys over small
+ * buckets by their high bits and places each at its bucket's start plus the
+ * number of the bucket's keys that precede it (for the count-first edge
+ * pass, the distinct keys below it; for node records, the records with a
+ * smaller key or an equal key and a smaller payload).  Tiles holding a bucket
  * too long for that (over 256 distinct edge keys or 512 records) take the
  * shared-memory digit passes, as every tile does with the switch off.
  * The graph is the same either way.
  * -------------------------------------------------------------------- */
 dbg_status dbg_sort_local_rank_set(dbg_ctx *ctx, int on);
-/* Tiles that met such a group, over the context's builds. */
+/* Tiles that met such a bucket, over the context's builds. */
 uint64_t dbg_sort_rank_fallbacks(const dbg_ctx *ctx);
 
 /* ----------------------------------------------------------------------

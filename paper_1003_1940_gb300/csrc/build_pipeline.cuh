@@ -8,6 +8,7 @@
 #include <type_traits>
 
 #include "k_build.cuh"
+#include "k_msd.cuh"
 #include "k_segsort.cuh"
 
 namespace dbg {
@@ -315,6 +316,65 @@ int hybrid_first_pass(uint64_t n, int bits) {
   return 0;
 }
 
+// ---------------------------------------------------------------------------
+// How a sort of n keys of `bits` bits goes: MSD (k_msd.cuh: up to two
+// partition passes, then the local pass), the least-significant-first hybrid
+// (first_pass > 0, or one local tile), or every digit globally.
+// ---------------------------------------------------------------------------
+// Mean group size the MSD passes aim at: a tile of TILE keys stretched to
+// group boundaries holds at most SegShape's capacity as long as groups stay
+// below TILE / 2, and a bucket's groups hold half to all of the mean.
+template <class K> constexpr uint32_t msd_mean() { return SegShape<K>::TILE / 4; }
+
+template <class K>
+struct SortPlan {
+  bool msd = false;
+  int first_pass = 0, adj = 0;  // least significant first
+  int bits = 0;                 // key bits
+  int need = 0;                 // MSD: bits that groups of the mean size take,
+  int w1 = 0, passes = 0;       // bits of the first digit, passes
+  int shift1() const { return bits - w1; }
+  DigitSpec digits() const {
+    DigitSpec d;
+    if (msd) {
+      d.first = shift1();
+      d.wide = w1;  // 0 (no pass): nothing is counted
+    } else {
+      d.first = first_pass;
+      d.passes = passes_for_bits(bits);
+      d.adj = adj;
+    }
+    return d;
+  }
+  bool local() const { return msd || first_pass > 0; }
+};
+
+// MSD where unordered passes are allowed (the partition switch) and leave
+// groups that end above the lowest bits: at most one key value per group in
+// four would be needed, so that the copies of one key alone seldom fill a
+// group.  Up to 2^10 groups in one pass; above, two digits of equal width
+// (the second then varies by bucket).
+template <class K>
+SortPlan<K> plan_sort(const dbg_ctx *ctx, uint64_t n, int bits, bool unordered) {
+  SortPlan<K> p;
+  p.bits = bits;
+  if (!ctx->hybrid_sort) return p;
+  if (unordered && n <= 0xffffffffull) {
+    int need = 0;
+    if (n > (uint64_t)SegShape<K>::TILE)
+      while (((uint64_t)msd_mean<K>() << need) < n) need++;
+    if (need + (need ? 2 : 0) <= bits && need <= 24) {
+      p.msd = true;
+      p.passes = need == 0 ? 0 : need <= 10 ? 1 : 2;
+      p.need = need;
+      p.w1 = p.passes == 2 ? need / 2 : need;
+      return p;
+    }
+  }
+  p.first_pass = hybrid_first_pass<K>(n, bits);
+  return p;
+}
+
 // ranking method of the local sort, by variant number (kinds 4 and 5)
 inline int local_rank_method(dbg_ctx *ctx, bool wide) {
   static const int methods[] = {RANK_MATCH, RANK_ATOMIC, RANK_BALLOT};
@@ -328,7 +388,7 @@ inline unsigned grid_for(uint64_t n, int per_block) {
 }
 
 // Exclusive scan of n u32 values into n + 1 u64 (the last is the total).
-inline dbg_status scan_u32(dbg_ctx *ctx, const uint32_t *in, uint64_t n, uint64_t *out, uint32_t *total, int stage) {
+inline dbg_status scan_u32_async(dbg_ctx *ctx, const uint32_t *in, uint64_t n, uint64_t *out, int stage) {
   cudaStream_t s = ctx->stream;
   const uint64_t tiles = (n + SCAN_TILE - 1) / SCAN_TILE;
   DBG_TRY(ensure_status(ctx, tiles));
@@ -339,6 +399,10 @@ inline dbg_status scan_u32(dbg_ctx *ctx, const uint32_t *in, uint64_t n, uint64_
              k_scan_excl<<<(unsigned)tiles, SCAN_BLOCK, 0, s>>>(in, n, out, ctx->d_status, ctx->d_counters, epoch,
                                                                 ctx->spin_limit, ctx->d_err, ctx->d_counters + 1));
   DBG_CUDA_TRY(cudaGetLastError());
+  return DBG_OK;
+}
+inline dbg_status scan_u32(dbg_ctx *ctx, const uint32_t *in, uint64_t n, uint64_t *out, uint32_t *total, int stage) {
+  DBG_TRY(scan_u32_async(ctx, in, n, out, stage));
   return read_small(ctx, ctx->d_counters + 1, sizeof(uint32_t), total);
 }
 
@@ -363,23 +427,163 @@ dbg_status run_length_reduce(dbg_ctx *ctx, const K *sorted, uint64_t n, K *uniq,
   return DBG_OK;
 }
 
-// Tile bounds of the local pass over n keys sorted by their bits from
-// low_bits up, and the oversize tiles (longer than the shared-memory
-// capacity) gathered into *gk / *gv and sorted over every digit.  Returns the
-// number of gathered keys in *G (0: none).
+// The groups that the global passes left: where each key's low bits start,
+// and, after MSD passes, the tables that say where each group lies.
+struct Groups {
+  LowBits lb;
+  DevBuf tables, goff;                  // MSD: bucket tables; the groups' places
+  DevBuf bound;                         // the local pass's tile bounds, once known
+  const uint32_t *ng_dev = nullptr;     // the groups' number (two passes), or
+  uint32_t ng = 0;                      // their number (one pass)
+  uint32_t ng_max = 0;                  // at most that many
+};
+
+// The local pass's tile bounds from the places of the groups, which are
+// copied to `cursor` (if given).
+template <class K>
+dbg_status msd_bounds(dbg_ctx *ctx, Groups &gr, uint64_t n, uint32_t *cursor, int stage) {
+  constexpr uint64_t T = SegShape<K>::TILE;
+  const uint64_t tiles = (n + T - 1) / T;
+  DBG_TRY(alloc_buf(ctx, gr.bound, (tiles + 1) * 8));
+  const uint64_t *places = gr.ng ? gr.tables.as<uint64_t>() : gr.goff.as<uint64_t>();
+  DBG_LAUNCH(ctx, stage, 0.0,
+             k_msd_bounds<<<std::min(grid_for(gr.ng_max, 256), 152u * 8), 256, 0, ctx->stream>>>(
+                 places, gr.ng_dev, gr.ng, n, T, tiles, gr.bound.as<uint64_t>(), cursor));
+  return DBG_OK;
+}
+
+// One partition pass (k_msd_part) in its shape for digits of up to max_bits.
+template <class K, bool HAS_VAL, bool WIDE>
+dbg_status launch_msd_part(dbg_ctx *ctx, const K *kin, K *kout, const uint32_t *vin, uint32_t *vout, uint64_t n, int shift,
+                     int bits, uint32_t W, const MsdTables &tb, bool two, uint32_t *cursor, int max_bits,
+                     uint64_t tiles) {
+  using Sh = MsdShape<K, HAS_VAL, WIDE>;
+  using S = MsdSmem<K, HAS_VAL, Sh::BLOCK, Sh::ITEMS>;
+  // the attribute is the kernel's, shared by every context: always the most
+  // that any launch of this shape asks for
+  constexpr size_t most = S::bytes(1 << (WIDE && !(HAS_VAL && sizeof(K) == 8) ? MSD_MAX_BITS : 11));
+  static_assert(Sh::MINB * (most + 1024) <= 228 * 1024, "MINB CTAs per SM");
+  auto kern = k_msd_part<K, HAS_VAL, Sh::BLOCK, Sh::ITEMS, Sh::MINB>;
+  const size_t smem = S::bytes(1 << max_bits);
+  if (smem > most) {
+    set_error("partition digit of %d bits", max_bits);
+    return DBG_EINTERNAL;
+  }
+  set_smem_attrs(kern, most);
+  const uint64_t slots = (uint64_t)Sh::MINB * (uint64_t)std::max(1, ctx->num_sms);
+  kern<<<(unsigned)std::min(tiles, slots), Sh::BLOCK, smem, ctx->stream>>>(
+      kin, kout, vin, vout, n, shift, bits, W, tb, two ? 1 : 0, cursor, 1u << max_bits, ctx->spin_limit, ctx->d_err);
+  return DBG_OK;
+}
+
+// The MSD passes of plan p over n keys (and payloads) whose first digit the
+// producer counted in d_hist.  On return the data is in *keys / *vals.  All
+// four arrays have MSD_PAD bytes behind their n entries.
 template <class K, bool HAS_VAL>
-dbg_status seg_prepare(dbg_ctx *ctx, const K *kin, const uint32_t *vin, uint64_t n, int low_bits, int key_bits,
-                       DevBuf &bound, DevBuf &osize, DevBuf &ooff, DevBuf &gk, DevBuf &gv, uint32_t *G, int stage) {
+dbg_status msd_sort(dbg_ctx *ctx, K **keys, K **alt_keys, uint32_t **vals, uint32_t **alt_vals, uint64_t n,
+                    const SortPlan<K> &p, const unsigned long long *d_hist, Groups &gr) {
+  cudaStream_t s = ctx->stream;
+  gr.lb.fixed = p.shift1();
+  if (p.passes == 0) return DBG_OK;
+  const uint32_t W = 1u << p.w1;
+  const bool two = p.passes == 2;
+  const bool wide1 = p.w1 >= 10, wide2 = p.need - p.w1 >= 10;
+  const uint32_t tile1 = wide1 ? MsdShape<K, HAS_VAL, true>::TILE : MsdShape<K, HAS_VAL, false>::TILE;
+  const uint32_t tile2 = wide2 ? MsdShape<K, HAS_VAL, true>::TILE : MsdShape<K, HAS_VAL, false>::TILE;
+  const uint64_t tiles1 = (n + tile1 - 1) / tile1;
+  const uint64_t tiles2 = n / tile2 + W;  // at most: every bucket's last tile may be partial
+  if (std::max(tiles1, tiles2) > 0x7fffffffull) return DBG_EOVERFLOW;
+  const int stage = HAS_VAL ? ST_SORT_NODES : ST_SORT_EDGES;
+  // the second digit of a bucket four times the average size, if it fits
+  const int max_w2 = std::min({HAS_VAL ? 11 : MSD_MAX_BITS, p.shift1(), p.need - p.w1 + 2});
+  // every bucket has at most max(1, 2 n_b / mean) groups
+  gr.ng_max = two ? (uint32_t)(2 * (n / msd_mean<K>()) + W) : W;
+  // [start: W + 1] u64, [cursor: W][gfirst: W + 1][tfirst: W + 1] u32, [tmap] u16, [w2][low] u8
+  const size_t bytes = (size_t)(W + 1) * 8 + (size_t)(3 * W + 2) * 4 + (two ? tiles2 * 2 : 0) + 2 * (size_t)W + 16;
+  DBG_TRY(alloc_buf(ctx, gr.tables, bytes));
+  MsdTables tb{};
+  tb.start = gr.tables.as<uint64_t>();
+  uint32_t *cursor = reinterpret_cast<uint32_t *>(tb.start + W + 1);
+  tb.gfirst = cursor + W;
+  tb.tfirst = tb.gfirst + W + 1;
+  tb.tmap = reinterpret_cast<uint16_t *>(tb.tfirst + W + 1);
+  tb.w2 = reinterpret_cast<uint8_t *>(tb.tmap + (two ? tiles2 : 0));
+  tb.low = tb.w2 + W;
+  DBG_LAUNCH(ctx, stage, 0.0,
+             k_msd_plan<<<1, 1024, 0, s>>>(d_hist, p.w1, p.shift1(), two ? 1 : 0, msd_mean<K>(), max_w2, tile2, tb,
+                                           cursor));
+  const double bytes_pass = 2.0 * (double)n * (double)(sizeof(K) + (HAS_VAL ? 4 : 0));
+  auto swap = [&]() {
+    std::swap(*keys, *alt_keys);
+    if (HAS_VAL) std::swap(*vals, *alt_vals);
+  };
+  const uint32_t *vi = HAS_VAL ? *vals : nullptr;
+  uint32_t *vt = HAS_VAL ? *alt_vals : nullptr;
+  DBG_LAUNCH(ctx, HAS_VAL ? ST_SORT_NODES : ST_PARTITION_EDGES, bytes_pass,
+             DBG_TRY((wide1 ? launch_msd_part<K, HAS_VAL, true>(ctx, *keys, *alt_keys, vi, vt, n, p.shift1(), p.w1, W,
+                                                                tb, false, cursor, p.w1, tiles1)
+                            : launch_msd_part<K, HAS_VAL, false>(ctx, *keys, *alt_keys, vi, vt, n, p.shift1(), p.w1,
+                                                                 W, tb, false, cursor, p.w1, tiles1))));
+  swap();
+  if (!two) {
+    gr.ng = W;
+    DBG_CUDA_TRY(cudaGetLastError());
+    return DBG_OK;
+  }
+  // the groups' sizes, their places, and the second pass
+  DevBuf gcount;
+  const uint64_t NG = gr.ng_max;
+  DBG_TRY(alloc_buf(ctx, gcount, NG * 4));
+  DBG_TRY(alloc_buf(ctx, gr.goff, (NG + 1) * 8));
+  DBG_CUDA_TRY(cudaMemsetAsync(gcount.p, 0, NG * 4, s));
+  DBG_LAUNCH(ctx, stage, (double)n * sizeof(K),
+             k_msd_count<K><<<(unsigned)std::min<uint64_t>(tiles2, 4ull * std::max(1, ctx->num_sms)), MSD_BLOCK,
+                              (size_t)4 << max_w2, s>>>(*keys, W, tile2, tb, gcount.as<uint32_t>()));
+  DBG_TRY(scan_u32_async(ctx, gcount.as<uint32_t>(), NG, gr.goff.as<uint64_t>(), stage));
+  gr.lb.low = tb.low;
+  gr.lb.shift1 = p.shift1();
+  gr.ng_dev = tb.gfirst + W;
+  // the counts' memory now takes the second pass's cursors (the places stay)
+  DBG_TRY(msd_bounds<K>(ctx, gr, n, gcount.as<uint32_t>(), stage));
+  vi = HAS_VAL ? *vals : nullptr;
+  vt = HAS_VAL ? *alt_vals : nullptr;
+  DBG_LAUNCH(ctx, stage, bytes_pass,
+             DBG_TRY((wide2 ? launch_msd_part<K, HAS_VAL, true>(ctx, *keys, *alt_keys, vi, vt, n, 0, 0, W, tb, true,
+                                                                gcount.as<uint32_t>(), max_w2, tiles2)
+                            : launch_msd_part<K, HAS_VAL, false>(ctx, *keys, *alt_keys, vi, vt, n, 0, 0, W, tb, true,
+                                                                 gcount.as<uint32_t>(), max_w2, tiles2))));
+  swap();
+  DBG_CUDA_TRY(cudaGetLastError());
+  return DBG_OK;
+}
+
+// The records' order by payload: *out = n words whose low halves list the
+// records by ascending payload << shift.  (64-bit keys' sort: build_u64.cu.)
+dbg_status order_by_payload(dbg_ctx *ctx, const uint32_t *v, uint64_t n, int shift, DevBuf &buf,
+                            const uint64_t **out);
+
+// Tile bounds of the local pass over n keys in the groups gr (sorted by
+// their bits from gr.lb up), and the oversize tiles (longer than the
+// shared-memory capacity) gathered into *gk / *gv and sorted over every
+// digit.  Returns the number of gathered keys in *G (0: none).
+template <class K, bool HAS_VAL>
+dbg_status seg_prepare(dbg_ctx *ctx, const K *kin, const uint32_t *vin, uint64_t n, Groups &gr, ValOrder vo,
+                       int key_bits, DevBuf &bound, DevBuf &osize, DevBuf &ooff, DevBuf &gk, DevBuf &gv, uint32_t *G, int stage) {
   using Sh = SegShape<K>;
   cudaStream_t s = ctx->stream;
   const uint64_t tiles = (n + Sh::TILE - 1) / Sh::TILE;
   if (tiles > 0x7fffffffull) return DBG_EOVERFLOW;
-  DBG_TRY(alloc_buf(ctx, bound, (tiles + 1) * 8));
   DBG_TRY(alloc_buf(ctx, osize, tiles * 4));
   DBG_TRY(alloc_buf(ctx, ooff, (tiles + 1) * 8));
-  DBG_LAUNCH(ctx, stage, 0.0,
-             k_seg_bounds<K><<<grid_for(tiles + 1, 256), 256, 0, s>>>(kin, n, low_bits, Sh::TILE, tiles,
-                                                                     bound.as<uint64_t>()));
+  if (gr.ng) DBG_TRY(msd_bounds<K>(ctx, gr, n, nullptr, stage));
+  if (gr.bound.p) {
+    bound = std::move(gr.bound);
+  } else {
+    DBG_TRY(alloc_buf(ctx, bound, (tiles + 1) * 8));
+    DBG_LAUNCH(ctx, stage, 0.0,
+               k_seg_bounds<K><<<grid_for(tiles + 1, 256), 256, 0, s>>>(kin, n, gr.lb.fixed, Sh::TILE, tiles,
+                                                                       bound.as<uint64_t>()));
+  }
   DBG_LAUNCH(ctx, stage, 0.0,
              k_seg_oversize<<<grid_for(tiles, 256), 256, 0, s>>>(bound.as<uint64_t>(), tiles,
                                                                  (uint32_t)(SEG_BLOCK * Sh::ITEMS),
@@ -390,11 +594,7 @@ dbg_status seg_prepare(dbg_ctx *ctx, const K *kin, const uint32_t *vin, uint64_t
   const uint64_t g = *G;
   DevBuf galt, gvalt, small;
   DBG_TRY(alloc_buf(ctx, gk, g * sizeof(K)));
-  DBG_TRY(alloc_buf(ctx, galt, g * sizeof(K)));
-  if (HAS_VAL) {
-    DBG_TRY(alloc_buf(ctx, gv, g * 4));
-    DBG_TRY(alloc_buf(ctx, gvalt, g * 4));
-  }
+  if (HAS_VAL) DBG_TRY(alloc_buf(ctx, gv, g * 4));
   DBG_TRY(alloc_buf(ctx, small, MAX_PASSES * RADIX * 16));
   unsigned long long *hist = small.as<unsigned long long>();
   uint64_t *dbase = reinterpret_cast<uint64_t *>(hist + MAX_PASSES * RADIX);
@@ -403,6 +603,19 @@ dbg_status seg_prepare(dbg_ctx *ctx, const K *kin, const uint32_t *vin, uint64_t
              k_seg_gather<K, HAS_VAL><<<(unsigned)std::min<uint64_t>(tiles, 152ull * 8), 256, 0, s>>>(
                  kin, vin, bound.as<uint64_t>(), osize.as<uint32_t>(), ooff.as<uint64_t>(), tiles, gk.as<K>(),
                  HAS_VAL ? gv.as<uint32_t>() : nullptr));
+  DevBuf order;  // for records in no order: the words that order them by payload
+  const uint64_t *words = nullptr;
+  if (HAS_VAL && vo.sort) DBG_TRY(order_by_payload(ctx, gv.as<uint32_t>(), g, vo.shift, order, &words));
+  DBG_TRY(alloc_buf(ctx, galt, g * sizeof(K)));
+  if (HAS_VAL) DBG_TRY(alloc_buf(ctx, gvalt, g * 4));
+  if (words) {
+    DBG_LAUNCH(ctx, stage, 2.0 * g * (sizeof(K) + 4),
+               k_permute<K><<<grid_for(g, 256 * 8), 256, 0, s>>>(words, g, gk.as<K>(), gv.as<uint32_t>(),
+                                                                 galt.as<K>(), gvalt.as<uint32_t>()));
+    std::swap(gk, galt);
+    std::swap(gv, gvalt);
+    order.release();
+  }
   DBG_CUDA_TRY(cudaMemsetAsync(hist, 0, MAX_PASSES * RADIX * 8, s));
   DBG_LAUNCH(ctx, stage, (double)g * sizeof(K),
              k_digit_hist<K><<<std::min(grid_for(g, 256 * 16), 152u * 8), 256, 0, s>>>(gk.as<K>(), g, 0, passes,
@@ -416,50 +629,48 @@ dbg_status seg_prepare(dbg_ctx *ctx, const K *kin, const uint32_t *vin, uint64_t
   return DBG_OK;
 }
 
-// The local pass over node records sorted by their bits from low_bits up:
-// k_seg_sort writes the fully sorted records to kout / vout.
+// The local pass over node records in the groups gr: the fully sorted
+// records (equal keys by payload, in the order vo) to kout / vout.
 template <class K>
 dbg_status seg_sort_records(dbg_ctx *ctx, const K *kin, const uint32_t *vin, K *kout, uint32_t *vout, uint64_t n,
-                            int low_bits, int key_bits) {
+                            Groups &gr, ValOrder vo, int key_bits) {
   using Sh = SegShape<K>;
   DevBuf bound, osize, ooff, gk, gv;
   uint32_t G = 0;
-  DBG_TRY((seg_prepare<K, true>(ctx, kin, vin, n, low_bits, key_bits, bound, osize, ooff, gk, gv, &G,
+  DBG_TRY((seg_prepare<K, true>(ctx, kin, vin, n, gr, vo, key_bits, bound, osize, ooff, gk, gv, &G,
                                 ST_LOCAL_SORT_NODES)));
   const int rank = local_rank_method(ctx, sizeof(K) == 16);
   const uint64_t tiles = (n + Sh::TILE - 1) / Sh::TILE;
-  {
-    if (ctx->seg_rank && (sizeof(K) == 16 || low_bits + 13 <= 64)) {
-      // ranking within groups; tiles with a long group are listed and
-      // sorted by the digit passes
-      static_assert(SegRankSmem<K>::CAP == SEG_BLOCK * Sh::ITEMS, "same tile capacity as the digit-pass kernel");
-      set_smem_attrs(k_seg_rank<K>, sizeof(SegRankSmem<K>));
-      DevBuf fb;
-      DBG_TRY(alloc_buf(ctx, fb, (tiles + 1) * 4));
-      uint32_t *fb_count = fb.as<uint32_t>(), *fb_list = fb_count + 1;
-      DBG_CUDA_TRY(cudaMemsetAsync(fb_count, 0, 4, ctx->stream));
-      DBG_LAUNCH(ctx, ST_LOCAL_SORT_NODES, 2.0 * (double)n * (sizeof(K) + 4),
-                 k_seg_rank<K><<<(unsigned)tiles, RANK_BLOCK, sizeof(SegRankSmem<K>), ctx->stream>>>(
-                     kin, vin, bound.as<uint64_t>(), osize.as<uint32_t>(), ooff.as<uint64_t>(), gk.as<K>(),
-                     gv.as<uint32_t>(), kout, vout, low_bits, fb_list, fb_count));
-      DBG_CUDA_TRY(cudaGetLastError());
-      uint32_t nfb = 0;
-      DBG_TRY(read_small(ctx, fb_count, sizeof(uint32_t), &nfb));
-      ctx->rank_fallback_tiles += nfb;
-      if (nfb == 0) return DBG_OK;
-      auto kern = rank == RANK_MATCH    ? k_seg_sort<K, Sh::ITEMS, RANK_MATCH>
-                  : rank == RANK_ATOMIC ? k_seg_sort<K, Sh::ITEMS, RANK_ATOMIC>
-                                        : k_seg_sort<K, Sh::ITEMS, RANK_BALLOT>;
-      constexpr size_t smem = sizeof(SegSortSmem<K, true, Sh::ITEMS>);
-      set_smem_attrs(kern, smem);
-      const unsigned grid = (unsigned)std::min<uint64_t>(nfb, 2ull * (uint64_t)std::max(1, ctx->num_sms));
-      DBG_LAUNCH(ctx, ST_LOCAL_SORT_NODES, 0.0,
-                 kern<<<grid, SEG_BLOCK, smem, ctx->stream>>>(
-                     kin, vin, bound.as<uint64_t>(), osize.as<uint32_t>(), ooff.as<uint64_t>(), gk.as<K>(),
-                     gv.as<uint32_t>(), kout, vout, low_bits, key_bits, fb_list, fb_count));
-      DBG_CUDA_TRY(cudaGetLastError());
-      return DBG_OK;
-    }
+  if (ctx->seg_rank) {
+    // ranking within buckets; tiles with a long bucket are listed and
+    // sorted by the digit passes
+    static_assert(SegRankSmem<K>::CAP == SEG_BLOCK * Sh::ITEMS, "same tile capacity as the digit-pass kernel");
+    set_smem_attrs(k_seg_rank<K>, sizeof(SegRankSmem<K>));
+    DevBuf fb;
+    DBG_TRY(alloc_buf(ctx, fb, (tiles + 1) * 4));
+    uint32_t *fb_count = fb.as<uint32_t>(), *fb_list = fb_count + 1;
+    DBG_CUDA_TRY(cudaMemsetAsync(fb_count, 0, 4, ctx->stream));
+    DBG_LAUNCH(ctx, ST_LOCAL_SORT_NODES, 2.0 * (double)n * (sizeof(K) + 4),
+               k_seg_rank<K><<<(unsigned)tiles, RANK_BLOCK, sizeof(SegRankSmem<K>), ctx->stream>>>(
+                   kin, vin, bound.as<uint64_t>(), osize.as<uint32_t>(), ooff.as<uint64_t>(), gk.as<K>(),
+                   gv.as<uint32_t>(), kout, vout, gr.lb, vo, fb_list, fb_count));
+    DBG_CUDA_TRY(cudaGetLastError());
+    uint32_t nfb = 0;
+    DBG_TRY(read_small(ctx, fb_count, sizeof(uint32_t), &nfb));
+    ctx->rank_fallback_tiles += nfb;
+    if (nfb == 0) return DBG_OK;
+    auto kern = rank == RANK_MATCH    ? k_seg_sort<K, Sh::ITEMS, RANK_MATCH>
+                : rank == RANK_ATOMIC ? k_seg_sort<K, Sh::ITEMS, RANK_ATOMIC>
+                                      : k_seg_sort<K, Sh::ITEMS, RANK_BALLOT>;
+    constexpr size_t smem = sizeof(SegSortSmem<K, true, Sh::ITEMS>);
+    set_smem_attrs(kern, smem);
+    const unsigned grid = (unsigned)std::min<uint64_t>(nfb, 2ull * (uint64_t)std::max(1, ctx->num_sms));
+    DBG_LAUNCH(ctx, ST_LOCAL_SORT_NODES, 0.0,
+               kern<<<grid, SEG_BLOCK, smem, ctx->stream>>>(
+                   kin, vin, bound.as<uint64_t>(), osize.as<uint32_t>(), ooff.as<uint64_t>(), gk.as<K>(),
+                   gv.as<uint32_t>(), kout, vout, gr.lb, vo, fb_list, fb_count));
+    DBG_CUDA_TRY(cudaGetLastError());
+    return DBG_OK;
   }
   const int v = ctx->sort_variant[sizeof(K) == 16 ? 5 : 4];
   if (v >= 3) {
@@ -474,7 +685,7 @@ dbg_status seg_sort_records(dbg_ctx *ctx, const K *kin, const uint32_t *vin, K *
     DBG_LAUNCH(ctx, ST_LOCAL_SORT_NODES, 2.0 * (double)n * (sizeof(K) + 4),
                kern<<<(unsigned)tiles, WB, smem, ctx->stream>>>(
                    kin, vin, bound.as<uint64_t>(), osize.as<uint32_t>(), ooff.as<uint64_t>(), gk.as<K>(),
-                   gv.as<uint32_t>(), kout, vout, low_bits, key_bits, nullptr, nullptr));
+                   gv.as<uint32_t>(), kout, vout, gr.lb, vo, nullptr, nullptr));
     DBG_CUDA_TRY(cudaGetLastError());
     return DBG_OK;
   }
@@ -486,22 +697,21 @@ dbg_status seg_sort_records(dbg_ctx *ctx, const K *kin, const uint32_t *vin, K *
   DBG_LAUNCH(ctx, ST_LOCAL_SORT_NODES, 2.0 * (double)n * (sizeof(K) + 4),
              kern<<<(unsigned)tiles, SEG_BLOCK, smem, ctx->stream>>>(
                  kin, vin, bound.as<uint64_t>(), osize.as<uint32_t>(), ooff.as<uint64_t>(), gk.as<K>(),
-                 gv.as<uint32_t>(), kout, vout, low_bits, key_bits, nullptr, nullptr));
+                 gv.as<uint32_t>(), kout, vout, gr.lb, vo, nullptr, nullptr));
   DBG_CUDA_TRY(cudaGetLastError());
   return DBG_OK;
 }
 
-// The local pass of STEP-2 over n edge keys sorted by their bits from
-// low_bits up.  Leaves the E distinct keys in kin[0, E) and their
+// The local pass of STEP-2 over n edge keys in the groups gr.  Leaves the E distinct keys in kin[0, E) and their
 // multiplicities in mult_out (allocated here); kstage (n keys) is scratch.
 template <class K>
-dbg_status seg_rle(dbg_ctx *ctx, K *kin, K *kstage, uint64_t n, int low_bits, int key_bits, DevBuf &mult_out,
+dbg_status seg_rle(dbg_ctx *ctx, K *kin, K *kstage, uint64_t n, Groups &gr, int key_bits, DevBuf &mult_out,
                    uint64_t *E) {
   using Sh = SegShape<K>;
   cudaStream_t s = ctx->stream;
   DevBuf bound, osize, ooff, gk, gv, gheads, guniq;
   uint32_t G = 0;
-  DBG_TRY((seg_prepare<K, false>(ctx, kin, nullptr, n, low_bits, key_bits, bound, osize, ooff, gk, gv, &G,
+  DBG_TRY((seg_prepare<K, false>(ctx, kin, nullptr, n, gr, ValOrder{}, key_bits, bound, osize, ooff, gk, gv, &G,
                                  ST_LOCAL_SORT_EDGES)));
   uint64_t H = 0;
   if (G > 0) {
@@ -540,7 +750,7 @@ dbg_status seg_rle(dbg_ctx *ctx, K *kin, K *kstage, uint64_t n, int low_bits, in
                  count<<<(unsigned)tiles, SEG_BLOCK, csmem, s>>>(
                      kin, bound.as<uint64_t>(), osize.as<uint32_t>(), ooff.as<uint64_t>(), guniq.as<K>(),
                      gheads.as<uint32_t>(), (uint32_t)H, kstage, mstage.as<uint32_t>(), tcount.as<uint32_t>(),
-                     over_list, over_count, low_bits, key_bits, ctx->seg_rank, rank_fb));
+                     over_list, over_count, gr.lb, ctx->seg_rank, rank_fb));
       DBG_CUDA_TRY(cudaGetLastError());
       uint32_t nover_fb[2] = {0, 0};
       DBG_TRY(read_small(ctx, over_count, 2 * sizeof(uint32_t), nover_fb));
@@ -552,7 +762,7 @@ dbg_status seg_rle(dbg_ctx *ctx, K *kin, K *kstage, uint64_t n, int low_bits, in
                    radix<<<nover, SEG_BLOCK, rsmem, s>>>(
                        kin, bound.as<uint64_t>(), osize.as<uint32_t>(), ooff.as<uint64_t>(), guniq.as<K>(),
                        gheads.as<uint32_t>(), (uint32_t)H, kstage, mstage.as<uint32_t>(), tcount.as<uint32_t>(),
-                       low_bits, key_bits, over_list));
+                       gr.lb, over_list));
       counted = true;
     }
   }
@@ -561,7 +771,7 @@ dbg_status seg_rle(dbg_ctx *ctx, K *kin, K *kstage, uint64_t n, int low_bits, in
                radix<<<(unsigned)tiles, SEG_BLOCK, rsmem, s>>>(
                    kin, bound.as<uint64_t>(), osize.as<uint32_t>(), ooff.as<uint64_t>(), guniq.as<K>(),
                    gheads.as<uint32_t>(), (uint32_t)H, kstage, mstage.as<uint32_t>(), tcount.as<uint32_t>(),
-                   low_bits, key_bits, nullptr));
+                   gr.lb, nullptr));
   DBG_CUDA_TRY(cudaGetLastError());
   uint32_t total = 0;
   DBG_TRY(scan_u32(ctx, tcount.as<uint32_t>(), tiles, toff.as<uint64_t>(), &total, ST_LOCAL_SORT_EDGES));
@@ -575,21 +785,63 @@ dbg_status seg_rle(dbg_ctx *ctx, K *kin, K *kstage, uint64_t n, int low_bits, in
   return DBG_OK;
 }
 
-// STEP-3's stable sort of R node records: hybrid (global passes from q0
-// up, then the local pass) when q0 > 0, else every digit globally.  The
-// producers accumulated the histograms of passes q0 and up only (with the
-// digit alignment adj, which needs q0 > 0).
+// STEP-2 over n edge keys by plan p (p.local()): the global passes, then the
+// local pass with the run-length reduce.  The E distinct keys end in *alt,
+// their multiplicities in mult.
 template <class K>
-dbg_status sort_records(dbg_ctx *ctx, K **rk, K **rk_alt, uint32_t **rv, uint32_t **rv_alt, uint64_t R, int nbits,
-                        int q0, unsigned long long *d_hist, uint64_t *d_digit_base, int adj = 0) {
-  if (q0 > 0 && R > 1) {
-    DBG_TRY((radix_sort<K, true>(ctx, rk, rk_alt, rv, rv_alt, R, nbits, d_hist, d_digit_base, q0, adj)));
-    DBG_TRY(seg_sort_records<K>(ctx, *rk, *rv, *rk_alt, *rv_alt, R, RADIX_BITS * q0 - adj, nbits));
-    std::swap(*rk, *rk_alt);
-    std::swap(*rv, *rv_alt);
-    return DBG_OK;
+dbg_status sort_count_keys(dbg_ctx *ctx, K **kp, K **alt, uint64_t n, const SortPlan<K> &p,
+                           const unsigned long long *d_hist, uint64_t *d_digit_base, DevBuf &mult, uint64_t *E) {
+  uint32_t *vn = nullptr, *van = nullptr;
+  Groups gr;
+  if (p.msd) {
+    DBG_TRY((msd_sort<K, false>(ctx, kp, alt, &vn, &van, n, p, d_hist, gr)));
+  } else {
+    DBG_TRY((radix_sort<K, false>(ctx, kp, alt, &vn, &van, n, p.bits, d_hist, d_digit_base, p.first_pass)));
+    gr.lb.fixed = RADIX_BITS * p.first_pass;
   }
-  return radix_sort<K, true>(ctx, rk, rk_alt, rv, rv_alt, R, nbits, d_hist, d_digit_base);
+  DBG_TRY(seg_rle<K>(ctx, *kp, *alt, n, gr, p.bits, mult, E));
+  std::swap(*kp, *alt);
+  return DBG_OK;
+}
+
+// STEP-3's sort of R records by key, equal keys by payload << vshift, by
+// plan p.  The records come in payload order, which the least-significant-
+// first passes keep and the local pass restores after the MSD passes.
+template <class K>
+dbg_status sort_records(dbg_ctx *ctx, K **rk, K **rk_alt, uint32_t **rv, uint32_t **rv_alt, uint64_t R,
+                        const SortPlan<K> &p, int vshift, unsigned long long *d_hist, uint64_t *d_digit_base) {
+  if (!p.local() || R <= 1) return radix_sort<K, true>(ctx, rk, rk_alt, rv, rv_alt, R, p.bits, d_hist, d_digit_base);
+  Groups gr;
+  ValOrder vo;
+  vo.shift = vshift;
+  if (p.msd) {
+    DBG_TRY((msd_sort<K, true>(ctx, rk, rk_alt, rv, rv_alt, R, p, d_hist, gr)));
+    vo.sort = p.passes > 0;
+  } else {
+    DBG_TRY((radix_sort<K, true>(ctx, rk, rk_alt, rv, rv_alt, R, p.bits, d_hist, d_digit_base, p.first_pass, p.adj)));
+    gr.lb.fixed = RADIX_BITS * p.first_pass - p.adj;
+  }
+  DBG_TRY(seg_sort_records<K>(ctx, *rk, *rv, *rk_alt, *rv_alt, R, gr, vo, p.bits));
+  std::swap(*rk, *rk_alt);
+  std::swap(*rv, *rv_alt);
+  return DBG_OK;
+}
+
+// The plan of a record sort.  Least significant first, with records ranked
+// within groups, the digits are aligned with the top of the key, so that the
+// global passes resolve 8 bits each of it and leave short groups.
+template <class K>
+SortPlan<K> plan_records(const dbg_ctx *ctx, uint64_t R, int bits, bool align) {
+  SortPlan<K> p = plan_sort<K>(ctx, R, bits, ctx->partition_first && ctx->seg_rank);
+  if (!p.msd && ctx->hybrid_sort && ctx->seg_rank && align) {
+    const int adj = (8 - bits % 8) % 8;
+    const int q0 = hybrid_first_pass<K>(R, bits + adj);
+    if (q0 > 0) {
+      p.first_pass = q0;
+      p.adj = adj;
+    }
+  }
+  return p;
 }
 
 // K6 by reduce-then-scan over R sorted node records; returns the node count
@@ -686,24 +938,22 @@ dbg_status count_node_kmers(dbg_ctx *ctx, const DevBuf &packed, const DevBuf &ba
   DBG_TRY(read_small(ctx, koff.as<uint64_t>() + n, sizeof(uint64_t), &M));
   if (M == 0) return DBG_OK;
   const int kbits = 2 * (int)k;
-  const int passes = passes_for_bits(kbits);
-  const int p0 = ctx->hybrid_sort ? hybrid_first_pass<K>(M, kbits) : 0;
+  const SortPlan<K> plan = plan_sort<K>(ctx, M, kbits, ctx->partition_first);
   DevBuf ka, kb, headpos;
-  DBG_TRY(alloc_buf(ctx, ka, M * sizeof(K)));
-  DBG_TRY(alloc_buf(ctx, kb, M * sizeof(K)));
+  DBG_TRY(alloc_buf(ctx, ka, M * sizeof(K) + MSD_PAD));
+  DBG_TRY(alloc_buf(ctx, kb, M * sizeof(K) + MSD_PAD));
   DBG_CUDA_TRY(cudaMemsetAsync(d_hist, 0, MAX_PASSES * RADIX * sizeof(unsigned long long), s));
   // emitting with k - 1 gives windows of k bases at the k-mer offsets
   DBG_LAUNCH(ctx, ST_NODE_MULT, 8.0 * n + (double)M * sizeof(K),
              k_emit<K><<<(unsigned)std::min<uint64_t>(grid_for(n, EMIT_BLOCK / 32), 152ull * 64), EMIT_BLOCK, 0, s>>>(
-                 packed.as<uint64_t>(), base_off.as<uint64_t>(), koff.as<uint64_t>(), n, k - 1, ka.as<K>(), p0,
-                 passes, d_hist, nullptr));
+                 packed.as<uint64_t>(), base_off.as<uint64_t>(), koff.as<uint64_t>(), n, k - 1, ka.as<K>(),
+                 plan.digits(), d_hist, nullptr));
   DBG_CUDA_TRY(cudaGetLastError());
   K *kp = ka.as<K>(), *alt = kb.as<K>();
   uint32_t *vn = nullptr, *van = nullptr;
   uint64_t D = 0;
-  if (p0 > 0) {
-    DBG_TRY((radix_sort<K, false>(ctx, &kp, &alt, &vn, &van, M, kbits, d_hist, d_digit_base, p0)));
-    DBG_TRY(seg_rle<K>(ctx, kp, alt, M, RADIX_BITS * p0, kbits, counts, &D));
+  if (plan.local()) {
+    DBG_TRY(sort_count_keys<K>(ctx, &kp, &alt, M, plan, d_hist, d_digit_base, counts, &D));
   } else {
     DBG_TRY(alloc_buf(ctx, headpos, (M + 1) * sizeof(uint32_t)));
     DBG_TRY((radix_sort<K, false>(ctx, &kp, &alt, &vn, &van, M, kbits, d_hist, d_digit_base)));
@@ -748,23 +998,23 @@ dbg_status count_node_reads(dbg_ctx *ctx, const DevBuf &packed, const DevBuf &ba
   if (M == 0) return DBG_OK;
   per.release();
   const int kbits = 2 * (int)k;
-  const int q0 = ctx->hybrid_sort ? hybrid_first_pass<K>(M, kbits) : 0;
+  const SortPlan<K> plan = plan_records<K>(ctx, M, kbits, false);
   DevBuf ka, kb, va, vb;
-  DBG_TRY(alloc_buf(ctx, ka, M * sizeof(K)));
-  DBG_TRY(alloc_buf(ctx, kb, M * sizeof(K)));
-  DBG_TRY(alloc_buf(ctx, va, M * sizeof(uint32_t)));
-  DBG_TRY(alloc_buf(ctx, vb, M * sizeof(uint32_t)));
+  DBG_TRY(alloc_buf(ctx, ka, M * sizeof(K) + MSD_PAD));
+  DBG_TRY(alloc_buf(ctx, kb, M * sizeof(K) + MSD_PAD));
+  DBG_TRY(alloc_buf(ctx, va, M * sizeof(uint32_t) + MSD_PAD));
+  DBG_TRY(alloc_buf(ctx, vb, M * sizeof(uint32_t) + MSD_PAD));
   DBG_CUDA_TRY(cudaMemsetAsync(d_hist, 0, MAX_PASSES * RADIX * sizeof(unsigned long long), s));
   // windows of k bases at the k-mer offsets, each with its read index
   DBG_LAUNCH(ctx, ST_NODE_MULT, 8.0 * n + (double)M * (sizeof(K) + 4),
              k_emit<K><<<(unsigned)std::min<uint64_t>(grid_for(n, EMIT_BLOCK / 32), 152ull * 64), EMIT_BLOCK, 0, s>>>(
-                 packed.as<uint64_t>(), base_off.as<uint64_t>(), koff.as<uint64_t>(), n, k - 1, ka.as<K>(), q0,
-                 passes_for_bits(kbits), d_hist, nullptr, va.as<uint32_t>()));
+                 packed.as<uint64_t>(), base_off.as<uint64_t>(), koff.as<uint64_t>(), n, k - 1, ka.as<K>(),
+                 plan.digits(), d_hist, nullptr, va.as<uint32_t>()));
   DBG_CUDA_TRY(cudaGetLastError());
   koff.release();
   K *kp = ka.as<K>(), *kalt = kb.as<K>();
   uint32_t *vp = va.as<uint32_t>(), *valt = vb.as<uint32_t>();
-  DBG_TRY((sort_records<K>(ctx, &kp, &kalt, &vp, &valt, M, kbits, q0, d_hist, d_digit_base)));
+  DBG_TRY(sort_records<K>(ctx, &kp, &kalt, &vp, &valt, M, plan, 0, d_hist, d_digit_base));
   // flags into the free payload buffer, their scan, the key runs
   DBG_LAUNCH(ctx, ST_NODE_MULT, (double)M * (2 * sizeof(K) + 12),
              k_read_change_flags<K><<<grid_for(M, 256 * 8), 256, 0, s>>>(kp, vp, M, valt));
@@ -831,15 +1081,12 @@ dbg_status build_graph_impl(dbg_ctx *ctx, const BuildInput &in, dbg_graph *g) {
   // ---- K2 set-up: key buffers and histograms come first, so that host
   // reads can be emitted chunk by chunk as they are packed ----
   const int kbits = 2 * ((int)k + 1);
-  const int kpasses = passes_for_bits(kbits);
   DevBuf keys_a, keys_b, headpos, mult_tmp, uniq;
   uint64_t E = 0;
-  K *sorted = nullptr;
-  // the hybrid sort needs the histograms of its global passes only
-  const int p0 = ctx->hybrid_sort ? hybrid_first_pass<K>(N, kbits) : 0;
+  const SortPlan<K> plan = plan_sort<K>(ctx, N, kbits, ctx->partition_first);
   if (N > 0) {
-    DBG_TRY(alloc_buf(ctx, keys_a, N * sizeof(K)));
-    DBG_TRY(alloc_buf(ctx, keys_b, N * sizeof(K)));
+    DBG_TRY(alloc_buf(ctx, keys_a, N * sizeof(K) + MSD_PAD));
+    DBG_TRY(alloc_buf(ctx, keys_b, N * sizeof(K) + MSD_PAD));
     DBG_CUDA_TRY(cudaMemsetAsync(d_hist, 0, MAX_PASSES * RADIX * sizeof(unsigned long long), s));
   }
   DevBuf packed;
@@ -849,7 +1096,7 @@ dbg_status build_graph_impl(dbg_ctx *ctx, const BuildInput &in, dbg_graph *g) {
     DBG_LAUNCH(ctx, ST_EMIT, bytes,
                k_emit<K><<<(unsigned)std::min<uint64_t>(grid_for(n, EMIT_BLOCK / 32), 152ull * 64), EMIT_BLOCK, 0,
                            s>>>(packed.as<uint64_t>(), base_off.as<uint64_t>(), edge_off.as<uint64_t>(), n, k,
-                                keys_a.as<K>(), p0, kpasses, d_hist, krange));
+                                keys_a.as<K>(), plan.digits(), d_hist, krange));
     DBG_CUDA_TRY(cudaGetLastError());
     return DBG_OK;
   };
@@ -906,12 +1153,10 @@ dbg_status build_graph_impl(dbg_ctx *ctx, const BuildInput &in, dbg_graph *g) {
     DBG_CUDA_TRY(cudaGetLastError());
     K *kp = keys_a.as<K>(), *alt = keys_b.as<K>();
     uint32_t *vn = nullptr, *van = nullptr;
-    if (p0 > 0) {
+    if (plan.local()) {
       // high digits globally, then the local sort with the run-length
       // reduce: distinct keys into alt, multiplicities into mult_tmp
-      DBG_TRY((radix_sort<K, false>(ctx, &kp, &alt, &vn, &van, N, kbits, d_hist, d_digit_base, p0)));
-      DBG_TRY(seg_rle<K>(ctx, kp, alt, N, RADIX_BITS * p0, kbits, mult_tmp, &E));
-      std::swap(kp, alt);  // the distinct keys are in the sort's buffer
+      DBG_TRY(sort_count_keys<K>(ctx, &kp, &alt, N, plan, d_hist, d_digit_base, mult_tmp, &E));
     } else {
       // every digit globally, then the run-length reduce
       DBG_TRY(alloc_buf(ctx, headpos, (N + 1) * sizeof(uint32_t)));
@@ -942,25 +1187,17 @@ dbg_status build_graph_impl(dbg_ctx *ctx, const BuildInput &in, dbg_graph *g) {
   // ---- K5 edge ends + records of reads of length k ----
   const uint64_t R = 2 * E + I;
   const int nbits = 2 * (int)k;
-  const int npasses = passes_for_bits(nbits);
   DBG_TRY(alloc_buf(ctx, g->edge_keys, std::max<uint64_t>(1, E) * sizeof(K)));
   DBG_TRY(alloc_buf(ctx, g->mult, std::max<uint64_t>(1, E) * sizeof(uint32_t)));
   DBG_TRY(alloc_buf(ctx, g->orient, std::max<uint64_t>(1, E)));
   DevBuf rk_a, rk_b, rv_a, rv_b;
-  DBG_TRY(alloc_buf(ctx, rk_a, std::max<uint64_t>(1, R) * sizeof(K)));
-  DBG_TRY(alloc_buf(ctx, rk_b, std::max<uint64_t>(1, R) * sizeof(K)));
-  DBG_TRY(alloc_buf(ctx, rv_a, std::max<uint64_t>(1, R) * sizeof(uint32_t)));
-  DBG_TRY(alloc_buf(ctx, rv_b, std::max<uint64_t>(1, R) * sizeof(uint32_t)));
+  DBG_TRY(alloc_buf(ctx, rk_a, R * sizeof(K) + MSD_PAD));
+  DBG_TRY(alloc_buf(ctx, rk_b, R * sizeof(K) + MSD_PAD));
+  DBG_TRY(alloc_buf(ctx, rv_a, R * sizeof(uint32_t) + MSD_PAD));
+  DBG_TRY(alloc_buf(ctx, rv_b, R * sizeof(uint32_t) + MSD_PAD));
   DBG_CUDA_TRY(cudaMemsetAsync(d_hist, 0, MAX_PASSES * RADIX * sizeof(unsigned long long), s));
-  // records ranked within groups: align the digits with the top of the
-  // 2k-bit key, so that the global passes resolve 8 bits each of it and
-  // leave short groups
-  int adj = ctx->seg_rank ? (8 - nbits % 8) % 8 : 0;
-  int q0 = ctx->hybrid_sort ? hybrid_first_pass<K>(R, nbits + adj) : 0;
-  if (q0 == 0) {
-    adj = 0;
-    q0 = ctx->hybrid_sort ? hybrid_first_pass<K>(R, nbits) : 0;
-  }
+  const SortPlan<K> rplan = plan_records<K>(ctx, R, nbits, true);
+  const DigitSpec nspec = rplan.digits();
   // below 2^29 edges the payloads carry both sides of each edge end, and
   // the node IDs pass stores them per adjacency slot (for the compaction)
   const bool sides = E > 0 && E < (1ull << 29);
@@ -969,15 +1206,15 @@ dbg_status build_graph_impl(dbg_ctx *ctx, const BuildInput &in, dbg_graph *g) {
                k_endpoints<K><<<grid_for(E, EMIT_TILE), EMIT_BLOCK, 0, s>>>(
         uniq.as<K>(), headpos.p ? headpos.as<uint32_t>() : nullptr, mult_tmp.as<uint32_t>(), E, k,
         g->edge_keys.as<K>(), g->mult.as<uint32_t>(),
-        g->orient.as<uint8_t>(), rk_a.as<K>(), rv_a.as<uint32_t>(), q0, npasses, d_hist, adj, sides));
+        g->orient.as<uint8_t>(), rk_a.as<K>(), rv_a.as<uint32_t>(), nspec, d_hist, sides));
   }
   if (I > 0) {
     DBG_CUDA_TRY(cudaMemsetAsync(ctx->d_counters + 2, 0, sizeof(uint32_t), s));
     DBG_LAUNCH(ctx, ST_ENDPOINTS, (double)n * 4 + (double)I * (sizeof(K) + 4),
                k_isolated<K><<<grid_for(n, 256), 256, 0, s>>>(packed.as<uint64_t>(), base_off.as<uint64_t>(),
                                                    in.d_lengths, n, k, rk_a.as<K>() + 2 * E,
-                                                   rv_a.as<uint32_t>() + 2 * E, ctx->d_counters + 2, q0, npasses,
-                                                   d_hist, adj));
+                                                   rv_a.as<uint32_t>() + 2 * E, ctx->d_counters + 2, nspec,
+                                                   d_hist));
   }
   DBG_CUDA_TRY(cudaGetLastError());
   uniq.release();
@@ -990,7 +1227,7 @@ dbg_status build_graph_impl(dbg_ctx *ctx, const BuildInput &in, dbg_graph *g) {
   // ---- STEP-3 sort of the node records (stable: payload order kept) ----
   K *rk = rk_a.as<K>(), *rk_alt = rk_b.as<K>();
   uint32_t *rv = rv_a.as<uint32_t>(), *rv_alt = rv_b.as<uint32_t>();
-  DBG_TRY((sort_records<K>(ctx, &rk, &rk_alt, &rv, &rv_alt, R, nbits, q0, d_hist, d_digit_base, adj)));
+  DBG_TRY(sort_records<K>(ctx, &rk, &rk_alt, &rv, &rv_alt, R, rplan, sides ? 2 : 0, d_hist, d_digit_base));
 
   // ---- K6 node IDs + adjacency rows, K7 neighbours ----
   DevBuf row_tmp;
@@ -1306,7 +1543,6 @@ dbg_status build_bucketed_impl(dbg_ctx *ctx, const BucketInput &in, uint64_t bud
   *n_edge_buckets = (uint32_t)ranges.size();
 
   const int kbits = 2 * m;
-  const int kpasses = passes_for_bits(kbits);
   std::vector<DevBuf> ck, cm, co;
   std::vector<uint64_t> ce;
   uint64_t E = 0;
@@ -1314,28 +1550,26 @@ dbg_status build_bucketed_impl(dbg_ctx *ctx, const BucketInput &in, uint64_t bud
     const uint64_t cnt = sizes[b];
     if (cnt == 0) continue;
     DevBuf ka, kb, headpos;
-    DBG_TRY(alloc_buf(ctx, ka, cnt * w));
-    DBG_TRY(alloc_buf(ctx, kb, cnt * w));
+    DBG_TRY(alloc_buf(ctx, ka, cnt * w + MSD_PAD));
+    DBG_TRY(alloc_buf(ctx, kb, cnt * w + MSD_PAD));
     DBG_TRY(alloc_buf(ctx, headpos, (cnt + 1) * 4));
     DBG_CUDA_TRY(cudaMemsetAsync(d_hist, 0, MAX_PASSES * RADIX * 8, s));
     DBG_CUDA_TRY(cudaMemsetAsync(ctx->d_counters + 8, 0, 4, s));
+    const SortPlan<K> plan = plan_sort<K>(ctx, cnt, kbits, ctx->partition_first);
     DBG_LAUNCH(ctx, ST_EMIT, 8.0 * nwords + 16.0 * n + (double)cnt * w,
                k_emit_range<K><<<emit_grid, EMIT_BLOCK, 0, s>>>(packed.as<uint64_t>(), base_off.as<uint64_t>(),
                                                                 edge_off.as<uint64_t>(), n, k, ranges[b].first,
                                                                 ranges[b].second, ka.as<K>(), ctx->d_counters + 8,
-                                                                kpasses, d_hist));
+                                                                plan.digits(), d_hist));
     DBG_CUDA_TRY(cudaGetLastError());
     K *kp = ka.as<K>(), *alt = kb.as<K>();
     uint32_t *vn = nullptr, *van = nullptr;
     uint64_t eb64 = 0;
-    const int p0 = ctx->hybrid_sort ? hybrid_first_pass<K>(cnt, kbits) : 0;
-    if (p0 > 0) {
+    if (plan.local()) {
       // multiplicities go where the run heads would (headpos is cnt + 1 long)
-      DBG_TRY((radix_sort<K, false>(ctx, &kp, &alt, &vn, &van, cnt, kbits, d_hist, d_digit_base, p0)));
       DevBuf mdense;
-      DBG_TRY(seg_rle<K>(ctx, kp, alt, cnt, RADIX_BITS * p0, kbits, mdense, &eb64));
+      DBG_TRY(sort_count_keys<K>(ctx, &kp, &alt, cnt, plan, d_hist, d_digit_base, mdense, &eb64));
       if (eb64) DBG_CUDA_TRY(cudaMemcpyAsync(headpos.p, mdense.p, eb64 * 4, cudaMemcpyDeviceToDevice, s));
-      std::swap(kp, alt);  // the distinct keys are in the sort's buffer
     } else {
       DBG_TRY((radix_sort<K, false>(ctx, &kp, &alt, &vn, &van, cnt, kbits, d_hist, d_digit_base)));
       DBG_TRY(run_length_reduce<K>(ctx, kp, cnt, alt, headpos.as<uint32_t>(), &eb64));
@@ -1348,7 +1582,7 @@ dbg_status build_bucketed_impl(dbg_ctx *ctx, const BucketInput &in, uint64_t bud
     DBG_TRY(alloc_buf(ctx, o1, std::max<uint64_t>(1, eb)));
     if (eb)
       DBG_LAUNCH(ctx, ST_ENDPOINTS, (double)eb * (2 * w + 9),
-                 k_edge_finish<K><<<grid_for(eb, 256), 256, 0, s>>>(alt, p0 > 0 ? nullptr : headpos.as<uint32_t>(),
+                 k_edge_finish<K><<<grid_for(eb, 256), 256, 0, s>>>(alt, plan.local() ? nullptr : headpos.as<uint32_t>(),
                                                                    headpos.as<uint32_t>(), eb, k, k1.as<K>(),
                                                                    m1.as<uint32_t>(), o1.as<uint8_t>()));
     ck.push_back(std::move(k1));
@@ -1396,7 +1630,6 @@ dbg_status build_bucketed_impl(dbg_ctx *ctx, const BucketInput &in, uint64_t bud
     DBG_TRY(alloc_buf(ctx, pos, (2 * E + 1) * 8));
   }
   const int nbits = 2 * (int)k;
-  const int npasses = passes_for_bits(nbits);
   std::vector<DevBuf> cnk, crp;
   std::vector<uint64_t> cv;
   uint64_t base_v = 0, base_slot = 0;
@@ -1412,17 +1645,20 @@ dbg_status build_bucketed_impl(dbg_ctx *ctx, const BucketInput &in, uint64_t bud
     const uint64_t cap = (uint64_t)Rc + I;
     if (cap == 0) continue;
     DevBuf ra, rb, va, vb, row_tmp;
-    DBG_TRY(alloc_buf(ctx, ra, cap * w));
-    DBG_TRY(alloc_buf(ctx, rb, cap * w));
-    DBG_TRY(alloc_buf(ctx, va, cap * 4));
-    DBG_TRY(alloc_buf(ctx, vb, cap * 4));
+    DBG_TRY(alloc_buf(ctx, ra, cap * w + MSD_PAD));
+    DBG_TRY(alloc_buf(ctx, rb, cap * w + MSD_PAD));
+    DBG_TRY(alloc_buf(ctx, va, cap * 4 + MSD_PAD));
+    DBG_TRY(alloc_buf(ctx, vb, cap * 4 + MSD_PAD));
+    // (planned for every record that the range may hold: isolated reads are
+    // counted by the range only)
+    const SortPlan<K> rplan = plan_records<K>(ctx, cap, nbits, false);
     DBG_CUDA_TRY(cudaMemsetAsync(d_hist, 0, MAX_PASSES * RADIX * 8, s));
     if (Rc > 0)
       DBG_LAUNCH(ctx, ST_ENDPOINTS, (double)E * (w + 8) + (double)Rc * (w + 4),
                  k_gather_ends<K><<<grid_for(E, 256 * 8), 256, 0, s>>>(g->edge_keys.as<K>(), E, k,
                                                                       flags.as<uint32_t>(), pos.as<uint64_t>(),
-                                                                      ra.as<K>(), va.as<uint32_t>(), npasses,
-                                                                      d_hist));
+                                                                      ra.as<K>(), va.as<uint32_t>(),
+                                                                      rplan.digits(), d_hist));
     uint64_t R = Rc;
     if (I > 0) {
       DBG_CUDA_TRY(cudaMemsetAsync(ctx->d_counters + 9, 0, 4, s));
@@ -1430,7 +1666,7 @@ dbg_status build_bucketed_impl(dbg_ctx *ctx, const BucketInput &in, uint64_t bud
                  k_isolated_range<K><<<grid_for(n, 256), 256, 0, s>>>(packed.as<uint64_t>(), base_off.as<uint64_t>(),
                                                                      in.d_lengths, n, k, lo, hi, ra.as<K>() + Rc,
                                                                      va.as<uint32_t>() + Rc, ctx->d_counters + 9,
-                                                                     npasses, d_hist));
+                                                                     rplan.digits(), d_hist));
       uint32_t iso = 0;
       DBG_TRY(read_small(ctx, ctx->d_counters + 9, 4, &iso));
       R += iso;
@@ -1438,8 +1674,7 @@ dbg_status build_bucketed_impl(dbg_ctx *ctx, const BucketInput &in, uint64_t bud
     if (R == 0) continue;
     K *rk = ra.as<K>(), *rk_alt = rb.as<K>();
     uint32_t *rv = va.as<uint32_t>(), *rv_alt = vb.as<uint32_t>();
-    const int q0 = ctx->hybrid_sort ? hybrid_first_pass<K>(R, nbits) : 0;
-    DBG_TRY((sort_records<K>(ctx, &rk, &rk_alt, &rv, &rv_alt, R, nbits, q0, d_hist, d_digit_base)));
+    DBG_TRY(sort_records<K>(ctx, &rk, &rk_alt, &rv, &rv_alt, R, rplan, 0, d_hist, d_digit_base));
     DBG_TRY(alloc_buf(ctx, row_tmp, (R + 1) * 8));
     uint64_t tot[2] = {0, 0};
     DBG_TRY(assign_node_ids<K>(ctx, rk, rv, R, rk_alt, row_tmp.as<uint64_t>(), g, (uint32_t)base_v, base_slot,

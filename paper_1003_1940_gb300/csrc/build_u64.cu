@@ -25,6 +25,25 @@ dbg_status build_bucketed_u64(dbg_ctx *ctx, const BucketInput &in, uint64_t budg
 }  // namespace dbg
 
 namespace dbg {
+dbg_status order_by_payload(dbg_ctx *ctx, const uint32_t *v, uint64_t n, int shift, DevBuf &buf,
+                            const uint64_t **out) {
+  cudaStream_t s = ctx->stream;
+  // two word buffers, the digit histograms and bases
+  DBG_TRY(alloc_buf(ctx, buf, 2 * n * 8 + MAX_PASSES * RADIX * 16));
+  uint64_t *a = buf.as<uint64_t>(), *b = a + n, *base = b + n;
+  unsigned long long *hist = reinterpret_cast<unsigned long long *>(base + MAX_PASSES * RADIX);
+  DBG_LAUNCH(ctx, ST_LOCAL_SORT_NODES, 12.0 * n, k_val_words<<<grid_for(n, 256 * 8), 256, 0, s>>>(v, n, shift, a));
+  DBG_CUDA_TRY(cudaMemsetAsync(hist, 0, MAX_PASSES * RADIX * 8, s));
+  DBG_LAUNCH(ctx, ST_LOCAL_SORT_NODES, 8.0 * n,
+             k_digit_hist<uint64_t><<<std::min(grid_for(n, 256 * 16), 152u * 8), 256, 0, s>>>(a, n, 4, 8, hist));
+  uint32_t *none = nullptr, *none2 = nullptr;
+  DBG_TRY((radix_sort<uint64_t, false>(ctx, &a, &b, &none, &none2, n, 64, hist, base, 4)));
+  *out = a;
+  return DBG_OK;
+}
+}  // namespace dbg
+
+namespace dbg {
 // flag[v] = 1 when node v's k-mer lies in at least t distinct reads
 static __global__ void k_roadmap_flags(const uint32_t *__restrict__ reads_per_node, uint64_t V, uint32_t t,
                                        uint32_t *__restrict__ flag) {

@@ -41,6 +41,10 @@ template <> struct KeyOps<uint64_t> {
   __device__ static uint64_t mask_low(uint64_t a, int nbits) {
     return nbits >= 64 ? a : (a & ((1ull << nbits) - 1ull));
   }
+  // a with its low `nbits` bits set
+  __device__ static uint64_t fill_low(uint64_t a, int nbits) {
+    return nbits >= 64 ? ~0ull : (a | ((1ull << nbits) - 1ull));
+  }
   __device__ static uint64_t low2(uint64_t a) { return a & 3ull; }
   __device__ static uint64_t words_hi(uint64_t) { return 0; }
   __device__ static uint64_t words_lo(uint64_t a) { return a; }
@@ -74,6 +78,10 @@ template <> struct KeyOps<Key128> {
     if (nbits >= 128) return a;
     if (nbits >= 64) return Key128{nbits == 64 ? 0 : (a.hi & ((1ull << (nbits - 64)) - 1ull)), a.lo};
     return Key128{0, a.lo & ((1ull << nbits) - 1ull)};
+  }
+  __device__ static Key128 fill_low(Key128 a, int nbits) {
+    if (nbits >= 64) return Key128{nbits >= 128 ? ~0ull : (a.hi | ((1ull << (nbits - 64)) - 1ull)), ~0ull};
+    return Key128{a.hi, a.lo | ((1ull << nbits) - 1ull)};
   }
   __device__ static uint64_t low2(Key128 a) { return a.lo & 3ull; }
   __device__ static uint64_t words_hi(Key128 a) { return a.hi; }

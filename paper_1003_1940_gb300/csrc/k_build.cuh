@@ -56,6 +56,34 @@ __device__ __forceinline__ uint32_t block_excl_scan_256(uint32_t v, uint32_t *tm
   return add + incl - v;
 }
 
+// The digits that the kernel producing a sort's keys counts on the way, in
+// shared memory and then in hist: the 8-bit digits of passes
+// [first, passes), pass p taking the bits from 8 p - adj up (hist[p * 256 +
+// digit]); or, with wide > 0, the one digit of `wide` bits from bit `first`
+// up (hist[digit]; at most 12 bits, MAX_PASSES * RADIX entries).
+struct DigitSpec {
+  int first = 0, passes = 0, adj = 0, wide = 0;
+  __host__ __device__ int entries() const { return wide ? 1 << wide : passes * RADIX; }
+  template <class K>
+  __device__ __forceinline__ void count(uint32_t *s_hist, const K &key) const {
+    if (wide) {
+      atomicAdd(&s_hist[KeyOps<K>::digit(key, first, wide)], 1u);
+    } else {
+      for (int ps = first; ps < passes; ps++)
+        atomicAdd(&s_hist[ps * RADIX + KeyOps<K>::digit(key, ps * RADIX_BITS - adj, RADIX_BITS)], 1u);
+    }
+  }
+  template <class K>
+  __device__ __forceinline__ void count_global(unsigned long long *hist, const K &key) const {
+    if (wide) {
+      atomicAdd(hist + KeyOps<K>::digit(key, first, wide), 1ull);
+    } else {
+      for (int ps = first; ps < passes; ps++)
+        atomicAdd(hist + ps * RADIX + KeyOps<K>::digit(key, ps * RADIX_BITS - adj, RADIX_BITS), 1ull);
+    }
+  }
+};
+
 // ---------------------------------------------------------------------------
 // read offsets: base_off[r] = sum of L before r, edge_off[r] = sum of
 // max(0, L - k) before r, plus the number of reads of length exactly k.
@@ -279,7 +307,7 @@ template <class K>
 __global__ __launch_bounds__(EMIT_BLOCK) void k_emit(const uint64_t *__restrict__ packed,
                                                      const uint64_t *__restrict__ base_off,
                                                      const uint64_t *__restrict__ edge_off, uint64_t n_reads,
-                                                     uint32_t k, K *__restrict__ keys, int first, int passes,
+                                                     uint32_t k, K *__restrict__ keys, DigitSpec ds,
                                                      unsigned long long *__restrict__ hist,
                                                      const uint64_t *__restrict__ krange,
                                                      uint32_t *__restrict__ read_of = nullptr) {
@@ -288,17 +316,16 @@ __global__ __launch_bounds__(EMIT_BLOCK) void k_emit(const uint64_t *__restrict_
   // krange is given), so lanes stay busy across read ends and every
   // warp-wide store writes 32 consecutive keys.  A lane follows the
   // read that holds its key: one binary search per warp, then a step to the
-  // next read when the key passes the current one's end.  The digit
-  // histograms of passes [first, passes) are accumulated on the way.
+  // next read when the key passes the current one's end.
   __shared__ uint32_t s_hist[MAX_PASSES * RADIX];
-  for (int i = threadIdx.x; i < passes * RADIX; i += EMIT_BLOCK) s_hist[i] = 0;
+  for (int i = threadIdx.x; i < ds.entries(); i += EMIT_BLOCK) s_hist[i] = 0;
   __syncthreads();
   const int lane = threadIdx.x & 31;
   const uint64_t warps = (uint64_t)gridDim.x * (EMIT_BLOCK / 32);
   const uint64_t wid = (uint64_t)blockIdx.x * (EMIT_BLOCK / 32) + (threadIdx.x >> 5);
   const int m = (int)k + 1;
-  const int G = passes - first;  // histogrammed passes
-  uint32_t *hbase = s_hist + first * RADIX;
+  const int G = ds.passes - ds.first;  // histogrammed passes
+  uint32_t *hbase = s_hist + ds.first * RADIX;
   const uint64_t lo = krange ? krange[0] : 0, hi = krange ? krange[1] : __ldg(edge_off + n_reads);
   const uint64_t per = ((hi - lo + warps - 1) / warps + 31) & ~31ull;
   const uint64_t a = lo + wid * per, b = min(a + per, hi);
@@ -318,20 +345,19 @@ __global__ __launch_bounds__(EMIT_BLOCK) void k_emit(const uint64_t *__restrict_
       const K key = kmin(z, revcomp(z, m));
       keys[i] = key;
       if (read_of) read_of[i] = (uint32_t)r;
-      if (G <= 4) {
+      if (!ds.wide && G <= 4) {
         // the histogrammed digits are the low bytes of one shifted word
-        const uint32_t w = (uint32_t)KeyOps<K>::words_lo(KeyOps<K>::shr(key, first * RADIX_BITS));
+        const uint32_t w = (uint32_t)KeyOps<K>::words_lo(KeyOps<K>::shr(key, ds.first * RADIX_BITS));
 #pragma unroll
         for (int g = 0; g < 4; g++)
           if (g < G) atomicAdd(hbase + g * RADIX + ((w >> (8 * g)) & 0xffu), 1u);
       } else {
-        for (int ps = first; ps < passes; ps++)
-          atomicAdd(&s_hist[ps * RADIX + KeyOps<K>::digit(key, ps * RADIX_BITS, RADIX_BITS)], 1u);
+        ds.count(s_hist, key);
       }
     }
   }
   __syncthreads();
-  for (int i = threadIdx.x; i < passes * RADIX; i += EMIT_BLOCK)
+  for (int i = threadIdx.x; i < ds.entries(); i += EMIT_BLOCK)
     if (s_hist[i]) atomicAdd(hist + i, (unsigned long long)s_hist[i]);
 }
 
@@ -1233,8 +1259,7 @@ static __global__ __launch_bounds__(SCAN_BLOCK) void k_scan_excl(const uint32_t 
 // negative strand, STEP-1's table gives (x^, y^, o1, o2) if x^ <= y^ and
 // (y^, x^, not o2, not o1) otherwise.  Writes orient, mult, a copy of the
 // key into the graph, and two node records per edge (payload e<<1 | role),
-// and accumulates the digit histograms of the node sort (pass ps takes the
-// 8 bits from 8 ps - adj up).  The multiplicity comes from the run heads
+// and accumulates the digit histograms of the node sort.  The multiplicity comes from the run heads
 // (headpos) or directly from mult_in.  With `sides` (E < 2^29), each payload
 // also carries the side of its own end (bit 30) and of the edge's other end
 // (bit 31), for k_write_nodes to store per adjacency slot.
@@ -1255,11 +1280,11 @@ __global__ __launch_bounds__(EMIT_BLOCK) void k_endpoints(const K *__restrict__ 
                                                           uint32_t k, K *__restrict__ edge_keys,
                                                           uint32_t *__restrict__ mult,
                                                           uint8_t *__restrict__ orient, K *__restrict__ rkeys,
-                                                          uint32_t *__restrict__ rvals, int first, int passes,
-                                                          unsigned long long *__restrict__ hist, int adj = 0,
+                                                          uint32_t *__restrict__ rvals, DigitSpec ds,
+                                                          unsigned long long *__restrict__ hist,
                                                           bool sides = false) {
   __shared__ uint32_t s_hist[MAX_PASSES * RADIX];
-  for (int i = threadIdx.x; i < passes * RADIX; i += EMIT_BLOCK) s_hist[i] = 0;
+  for (int i = threadIdx.x; i < ds.entries(); i += EMIT_BLOCK) s_hist[i] = 0;
   __syncthreads();
   const int kk = (int)k;
   for (uint64_t e = (uint64_t)blockIdx.x * EMIT_TILE + threadIdx.x; e < min(E, (uint64_t)(blockIdx.x + 1) * EMIT_TILE);
@@ -1283,13 +1308,11 @@ __global__ __launch_bounds__(EMIT_BLOCK) void k_endpoints(const K *__restrict__ 
     rvals[2 * e] = (uint32_t)(e << 1) | s0 << 30 | s1 << 31;
     rkeys[2 * e + 1] = d;
     rvals[2 * e + 1] = (uint32_t)(e << 1) | 1u | s1 << 30 | s0 << 31;
-    for (int ps = first; ps < passes; ps++) {
-      atomicAdd(&s_hist[ps * RADIX + KeyOps<K>::digit(s, ps * RADIX_BITS - adj, RADIX_BITS)], 1u);
-      atomicAdd(&s_hist[ps * RADIX + KeyOps<K>::digit(d, ps * RADIX_BITS - adj, RADIX_BITS)], 1u);
-    }
+    ds.count(s_hist, s);
+    ds.count(s_hist, d);
   }
   __syncthreads();
-  for (int i = threadIdx.x; i < passes * RADIX; i += EMIT_BLOCK)
+  for (int i = threadIdx.x; i < ds.entries(); i += EMIT_BLOCK)
     if (s_hist[i]) atomicAdd(hist + i, (unsigned long long)s_hist[i]);
 }
 
@@ -1299,8 +1322,8 @@ __global__ __launch_bounds__(EMIT_BLOCK) void k_endpoints(const K *__restrict__ 
 template <class K>
 __global__ void k_isolated(const uint64_t *__restrict__ packed, const uint64_t *__restrict__ base_off,
                            const uint32_t *__restrict__ len, uint64_t n, uint32_t k, K *__restrict__ rkeys,
-                           uint32_t *__restrict__ rvals, uint32_t *slot, int first, int passes,
-                           unsigned long long *__restrict__ hist, int adj = 0) {
+                           uint32_t *__restrict__ rvals, uint32_t *slot, DigitSpec ds,
+                           unsigned long long *__restrict__ hist) {
   for (uint64_t r = (uint64_t)blockIdx.x * blockDim.x + threadIdx.x; r < n; r += (uint64_t)gridDim.x * blockDim.x) {
     if (len[r] != k) continue;
     const K x = load_window<K>(packed, base_off[r], (int)k);
@@ -1308,8 +1331,7 @@ __global__ void k_isolated(const uint64_t *__restrict__ packed, const uint64_t *
     const uint32_t i = atomicAdd(slot, 1u);
     rkeys[i] = xh;
     rvals[i] = REC_NONE;
-    for (int ps = first; ps < passes; ps++)
-      atomicAdd(hist + ps * RADIX + KeyOps<K>::digit(xh, ps * RADIX_BITS - adj, RADIX_BITS), 1ull);
+    ds.count_global(hist, xh);
   }
 }
 
@@ -1393,10 +1415,10 @@ __global__ __launch_bounds__(EMIT_BLOCK) void k_emit_range(const uint64_t *__res
                                                            const uint64_t *__restrict__ base_off,
                                                            const uint64_t *__restrict__ edge_off, uint64_t n_reads,
                                                            uint32_t k, uint32_t lo, uint32_t hi,
-                                                           K *__restrict__ keys, uint32_t *count, int passes,
+                                                           K *__restrict__ keys, uint32_t *count, DigitSpec ds,
                                                            unsigned long long *__restrict__ hist) {
   __shared__ uint32_t s_hist[MAX_PASSES * RADIX];
-  for (int i = threadIdx.x; i < passes * RADIX; i += EMIT_BLOCK) s_hist[i] = 0;
+  for (int i = threadIdx.x; i < ds.entries(); i += EMIT_BLOCK) s_hist[i] = 0;
   __syncthreads();
   const int lane = threadIdx.x & 31, m = (int)k + 1;
   const uint64_t warps = (uint64_t)gridDim.x * (EMIT_BLOCK / 32);
@@ -1419,13 +1441,12 @@ __global__ __launch_bounds__(EMIT_BLOCK) void k_emit_range(const uint64_t *__res
       base = __shfl_sync(0xffffffffu, base, 0);
       if (in) {
         keys[base + __popc(b & ((1u << lane) - 1u))] = key;
-        for (int ps = 0; ps < passes; ps++)
-          atomicAdd(&s_hist[ps * RADIX + KeyOps<K>::digit(key, ps * RADIX_BITS, RADIX_BITS)], 1u);
+        ds.count(s_hist, key);
       }
     }
   }
   __syncthreads();
-  for (int i = threadIdx.x; i < passes * RADIX; i += EMIT_BLOCK)
+  for (int i = threadIdx.x; i < ds.entries(); i += EMIT_BLOCK)
     if (s_hist[i]) atomicAdd(hist + i, (unsigned long long)s_hist[i]);
 }
 
@@ -1500,10 +1521,10 @@ __global__ void k_flag_ends(const K *__restrict__ edge_keys, uint64_t E, uint32_
 template <class K>
 __global__ void k_gather_ends(const K *__restrict__ edge_keys, uint64_t E, uint32_t k,
                               const uint32_t *__restrict__ flags, const uint64_t *__restrict__ pos,
-                              K *__restrict__ rkeys, uint32_t *__restrict__ rvals, int passes,
+                              K *__restrict__ rkeys, uint32_t *__restrict__ rvals, DigitSpec ds,
                               unsigned long long *__restrict__ hist) {
   __shared__ uint32_t s_hist[MAX_PASSES * RADIX];
-  for (int i = threadIdx.x; i < passes * RADIX; i += blockDim.x) s_hist[i] = 0;
+  for (int i = threadIdx.x; i < ds.entries(); i += blockDim.x) s_hist[i] = 0;
   __syncthreads();
   for (uint64_t e = (uint64_t)blockIdx.x * blockDim.x + threadIdx.x; e < E; e += (uint64_t)gridDim.x * blockDim.x) {
     const uint32_t f0 = flags[2 * e], f1 = flags[2 * e + 1];
@@ -1517,12 +1538,11 @@ __global__ void k_gather_ends(const K *__restrict__ edge_keys, uint64_t E, uint3
       const uint64_t p = pos[2 * e + role];
       rkeys[p] = nk;
       rvals[p] = (uint32_t)(e << 1) | (uint32_t)role;
-      for (int ps = 0; ps < passes; ps++)
-        atomicAdd(&s_hist[ps * RADIX + KeyOps<K>::digit(nk, ps * RADIX_BITS, RADIX_BITS)], 1u);
+      ds.count(s_hist, nk);
     }
   }
   __syncthreads();
-  for (int i = threadIdx.x; i < passes * RADIX; i += blockDim.x)
+  for (int i = threadIdx.x; i < ds.entries(); i += blockDim.x)
     if (s_hist[i]) atomicAdd(hist + i, (unsigned long long)s_hist[i]);
 }
 
@@ -1531,7 +1551,7 @@ __global__ void k_gather_ends(const K *__restrict__ edge_keys, uint64_t E, uint3
 template <class K>
 __global__ void k_isolated_range(const uint64_t *__restrict__ packed, const uint64_t *__restrict__ base_off,
                                  const uint32_t *__restrict__ len, uint64_t n, uint32_t k, uint32_t lo, uint32_t hi,
-                                 K *__restrict__ rkeys, uint32_t *__restrict__ rvals, uint32_t *slot, int passes,
+                                 K *__restrict__ rkeys, uint32_t *__restrict__ rvals, uint32_t *slot, DigitSpec ds,
                                  unsigned long long *__restrict__ hist) {
   for (uint64_t r = (uint64_t)blockIdx.x * blockDim.x + threadIdx.x; r < n; r += (uint64_t)gridDim.x * blockDim.x) {
     if (len[r] != k) continue;
@@ -1542,8 +1562,7 @@ __global__ void k_isolated_range(const uint64_t *__restrict__ packed, const uint
     const uint32_t i = atomicAdd(slot, 1u);
     rkeys[i] = xh;
     rvals[i] = REC_NONE;
-    for (int ps = 0; ps < passes; ps++)
-      atomicAdd(hist + ps * RADIX + KeyOps<K>::digit(xh, ps * RADIX_BITS, RADIX_BITS), 1ull);
+    ds.count_global(hist, xh);
   }
 }
 

@@ -44,8 +44,30 @@ struct SegSortSmem {
   uint32_t hpos[HAS_VAL ? 1 : CAP + 1];  // run heads' positions by rank (run-length reduce)
   uint32_t tmp[8];
   uint64_t bound[2];
-  K base;
-  uint32_t tile, passes, excl, total, spread_bits;
+  K base, range;
+  uint32_t tile, passes, excl, total, span_bits;
+};
+
+// Where a key's group ends: the number of its bits below the group's shared
+// high bits, one for all keys (low == nullptr: fixed) or by bucket, the
+// key's bits from shift1 up (k_msd.cuh).
+struct LowBits {
+  int fixed = 0;
+  const uint8_t *low = nullptr;
+  int shift1 = 0;
+  template <class K>
+  __device__ __forceinline__ int of(const K &key) const {
+    return low ? low[(uint32_t)KeyOps<K>::words_lo(KeyOps<K>::shr(key, shift1))] : fixed;
+  }
+};
+
+// The order of records with equal keys: ascending payload << shift (the
+// shift drops the side bits that a node record's payload carries on top).
+// sort: they come in no particular order and payload digits take part in the
+// digit passes; otherwise they come in that order and stable passes keep it.
+struct ValOrder {
+  int shift = 0;
+  int sort = 0;
 };
 
 // bound[t] for t in [0, tiles]: the first index of the group holding
@@ -86,6 +108,23 @@ static __global__ void k_seg_oversize(const uint64_t *__restrict__ bound, uint64
   }
 }
 
+// Gathered records that come in no order are sorted by payload before the
+// stable sort by key: the words (payload << shift) << 32 | index are sorted by
+// their upper half, and the records follow.
+static __global__ void k_val_words(const uint32_t *__restrict__ v, uint64_t n, int shift, uint64_t *__restrict__ w) {
+  for (uint64_t i = (uint64_t)blockIdx.x * blockDim.x + threadIdx.x; i < n; i += (uint64_t)gridDim.x * blockDim.x)
+    w[i] = (uint64_t)(v[i] << shift) << 32 | (uint32_t)i;
+}
+template <class K>
+__global__ void k_permute(const uint64_t *__restrict__ w, uint64_t n, const K *__restrict__ kin,
+                          const uint32_t *__restrict__ vin, K *__restrict__ kout, uint32_t *__restrict__ vout) {
+  for (uint64_t i = (uint64_t)blockIdx.x * blockDim.x + threadIdx.x; i < n; i += (uint64_t)gridDim.x * blockDim.x) {
+    const uint32_t j = (uint32_t)w[i];
+    kout[i] = kin[j];
+    vout[i] = vin[j];
+  }
+}
+
 // Copies every oversize tile to gk[ooff[t] ...] (and its payloads), in tile
 // order, so that one sort of the gathered keys sorts each of them.
 template <class K, bool HAS_VAL>
@@ -104,23 +143,25 @@ __global__ void k_seg_gather(const K *__restrict__ kin, const uint32_t *__restri
   }
 }
 
-// The tile's range, its base (the first key with the low bits cleared) and
-// the number of local passes, into shared memory.  The caller checks that
-// the tile is not oversize.
+// The tile's range, its base (the first key with its group's low bits
+// cleared: no key of the tile is below it) and, from the last key with its
+// group's low bits set, the bits that key offsets span and the number of
+// local passes over them, into shared memory.  The caller checks that the
+// tile is not oversize.
 template <class K, class S>
 __device__ __forceinline__ void seg_setup(S &sm, const K *__restrict__ kin, const uint64_t *__restrict__ bound,
-                                          uint32_t tile, int low_bits, int key_bits) {
+                                          uint32_t tile, LowBits lb) {
   if (threadIdx.x == 0) {
     const uint64_t s = bound[tile], e = bound[tile + 1];
     sm.bound[0] = s;
     sm.bound[1] = e;
     if (e > s) {
       const K first = kin[s], last = kin[e - 1];
-      sm.base = KeyOps<K>::sub(first, KeyOps<K>::mask_low(first, low_bits));
-      const int spread_bits =
-          KeyOps<K>::bitlen(KeyOps<K>::sub(KeyOps<K>::shr(last, low_bits), KeyOps<K>::shr(first, low_bits)));
-      sm.passes = (uint32_t)((min(low_bits + spread_bits, key_bits) + RADIX_BITS - 1) / RADIX_BITS);
-      sm.spread_bits = (uint32_t)spread_bits;
+      sm.base = KeyOps<K>::sub(first, KeyOps<K>::mask_low(first, lb.of(first)));
+      const K range = KeyOps<K>::sub(KeyOps<K>::fill_low(last, lb.of(last)), sm.base);
+      sm.span_bits = (uint32_t)KeyOps<K>::bitlen(range);
+      sm.passes = (sm.span_bits + RADIX_BITS - 1) / RADIX_BITS;
+      sm.range = range;
     }
   }
   __syncthreads();
@@ -141,16 +182,16 @@ __device__ __forceinline__ uint32_t lower_bound_u32(const uint32_t *__restrict__
 // warp's equal digits so far, packed as (rank << 9) | digit, with digit
 // RADIX for invalid items.  Order: item, then lane.  An item is valid if its
 // index wofs + 32 i + lane is below lim.
-template <class K, int ITEMS, int RANK, class S>
-__device__ __forceinline__ void rank_items(S &sm, const K (&key)[ITEMS], uint32_t (&rank)[ITEMS], int nitems,
-                                           uint32_t wofs, uint32_t lim, int shift) {
+template <int ITEMS, int RANK, class S, class Digit>
+__device__ __forceinline__ void rank_digits(S &sm, uint32_t (&rank)[ITEMS], int nitems, uint32_t wofs, uint32_t lim,
+                                            Digit digit) {
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
   const unsigned lt_mask = (1u << lane) - 1u;
 #pragma unroll
   for (int i = 0; i < ITEMS; i++) {
     if (i >= nitems) break;  // warp-uniform
     const bool valid = wofs + i * 32 + lane < lim;
-    const uint32_t d = valid ? KeyOps<K>::digit(key[i], shift, RADIX_BITS) : (uint32_t)RADIX;
+    const uint32_t d = valid ? digit(i) : (uint32_t)RADIX;
     unsigned peers;
     if (RANK == RANK_MATCH) {
       peers = __match_any_sync(0xffffffffu, d);
@@ -179,6 +220,12 @@ __device__ __forceinline__ void rank_items(S &sm, const K (&key)[ITEMS], uint32_
     rank[i] = ((before + __popc(peers & lt_mask)) << 9) | d;
     __syncwarp();
   }
+}
+template <class K, int ITEMS, int RANK, class S>
+__device__ __forceinline__ void rank_items(S &sm, const K (&key)[ITEMS], uint32_t (&rank)[ITEMS], int nitems,
+                                           uint32_t wofs, uint32_t lim, int shift) {
+  rank_digits<ITEMS, RANK>(sm, rank, nitems, wofs, lim,
+                           [&](int i) { return KeyOps<K>::digit(key[i], shift, RADIX_BITS); });
 }
 
 // Turns the per-warp digit counts into each warp's first position per digit
@@ -250,7 +297,7 @@ __device__ __forceinline__ void seg_sort_tile(
     SegSortSmem<K, true, ITEMS, BLOCK> &sm, uint32_t tile, const K *__restrict__ kin, const uint32_t *__restrict__ vin,
     const uint64_t *__restrict__ bound, const uint32_t *__restrict__ osize, const uint64_t *__restrict__ ooff,
     const K *__restrict__ gk, const uint32_t *__restrict__ gv, K *__restrict__ kout, uint32_t *__restrict__ vout,
-    int low_bits, int key_bits) {
+    LowBits lb, ValOrder vo) {
   using S = SegSortSmem<K, true, ITEMS, BLOCK>;
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
   if (osize[tile]) {
@@ -263,7 +310,7 @@ __device__ __forceinline__ void seg_sort_tile(
   }
   for (int i = tid; i < S::WARPS * RADIX; i += BLOCK) (&sm.whist[0][0])[i] = 0;
   for (int i = tid; i < S::WARPS * (RADIX + 1); i += BLOCK) (&sm.match[0][0])[i] = 0;
-  seg_setup<K>(sm, kin, bound, tile, low_bits, key_bits);
+  seg_setup<K>(sm, kin, bound, tile, lb);
   const uint64_t s = sm.bound[0];
   const uint32_t cnt = (uint32_t)(sm.bound[1] - s);
   if (cnt == 0) return;
@@ -283,12 +330,18 @@ __device__ __forceinline__ void seg_sort_tile(
     key[i] = in ? KeyOps<K>::sub(kin[s + j], base) : KeyOps<K>::zero();
     val[i] = in ? vin[s + j] : 0u;
   }
-  for (int p = 0; p < passes; p++) {
+  // records that come in no order: their payloads' digits first
+  const int vpasses = vo.sort ? 4 : 0;
+  for (int p = 0; p < vpasses + passes; p++) {
     if (p > 0) {
       reload_items<K, true, ITEMS>(sm, key, val, ipw, wofs, cnt);
       __syncthreads();
     }
-    rank_items<K, ITEMS, RANK>(sm, key, rank, ipw, wofs, cnt, p * RADIX_BITS);
+    if (p < vpasses)
+      rank_digits<ITEMS, RANK>(sm, rank, ipw, wofs, cnt,
+                               [&](int i) { return ((val[i] << vo.shift) >> (p * RADIX_BITS)) & 0xffu; });
+    else
+      rank_items<K, ITEMS, RANK>(sm, key, rank, ipw, wofs, cnt, (p - vpasses) * RADIX_BITS);
     digit_positions(sm);
     scatter_items<K, true, ITEMS>(sm, key, val, rank, ipw);
   }
@@ -305,36 +358,35 @@ template <class K, int ITEMS, int RANK, int BLOCK = SEG_BLOCK>
 __global__ __launch_bounds__(BLOCK, 2) void k_seg_sort(
     const K *__restrict__ kin, const uint32_t *__restrict__ vin, const uint64_t *__restrict__ bound,
     const uint32_t *__restrict__ osize, const uint64_t *__restrict__ ooff, const K *__restrict__ gk,
-    const uint32_t *__restrict__ gv, K *__restrict__ kout, uint32_t *__restrict__ vout, int low_bits, int key_bits,
+    const uint32_t *__restrict__ gv, K *__restrict__ kout, uint32_t *__restrict__ vout, LowBits lb, ValOrder vo,
     const uint32_t *__restrict__ tile_list = nullptr, const uint32_t *__restrict__ list_count = nullptr) {
   using S = SegSortSmem<K, true, ITEMS, BLOCK>;
   extern __shared__ __align__(128) unsigned char smem_raw[];
   S &sm = *reinterpret_cast<S *>(smem_raw);
   if (!tile_list) {
-    seg_sort_tile<K, ITEMS, RANK, BLOCK>(sm, blockIdx.x, kin, vin, bound, osize, ooff, gk, gv, kout, vout, low_bits,
-                                         key_bits);
+    seg_sort_tile<K, ITEMS, RANK, BLOCK>(sm, blockIdx.x, kin, vin, bound, osize, ooff, gk, gv, kout, vout, lb, vo);
     return;
   }
   const uint32_t n = *list_count;
   for (uint32_t q = blockIdx.x; q < n; q += gridDim.x) {
     seg_sort_tile<K, ITEMS, RANK, BLOCK>(sm, tile_list[q], kin, vin, bound, osize, ooff, gk, gv, kout, vout,
-                                         low_bits, key_bits);
+                                         lb, vo);
     __syncthreads();
   }
 }
 
-// Records by ranking within groups.  The tile's keys are already ordered
-// by their high bits (from low_bits up), so a record's place in the sorted
-// tile is its group's start plus the number of records of its group that
-// precede it: those with a smaller key, or an equal key and an earlier
-// position (which keeps the sort stable).  A 64-bit record is staged in
-// shared memory as one word, (low bits << 13) | position, and ranked by
-// comparing that word with the group's others; a 128-bit record as its key,
-// compared whole with the position as tie-break.  No digit pass and no
-// block barrier is needed past the staging.  The work is the sum of the
-// squared group lengths, small when the global passes leave groups of a
-// few dozen records.  A tile with a group longer than RANK_GROUP_MAX is
-// listed in fb_list for the digit-pass kernel instead.
+// Records by ranking within small buckets.  The tile's records are spread
+// over 4096 buckets by the top bits of their key offsets (a counting sort in
+// shared memory: one atomic add per record, a scan, one scatter), and a
+// record's place in the sorted tile is its bucket's start plus the number of
+// the bucket's records that precede it: those with a smaller key, or an
+// equal key and a smaller payload.  A bucket holds a node's own records and
+// seldom another node's, so that is a few comparisons per record, and they
+// need no particular order on arrival.  A tile with a bucket longer than
+// RANK_GROUP_MAX is listed in fb_list for the digit-pass kernel instead.
+//
+// Bound by shared-memory traffic (about 20 bytes written and 60 read per
+// 12-byte record); two CTAs of 512 threads per SM.
 constexpr int RANK_BLOCK = 512;
 constexpr uint32_t RANK_GROUP_MAX = 512;
 
@@ -342,97 +394,111 @@ template <class K>
 struct SegRankSmem {
   static constexpr int CAP = SEG_BLOCK * (sizeof(K) == 8 ? 24 : 12);  // the digit-pass kernel's capacity
   static constexpr int ITEMS = CAP / RANK_BLOCK;
-  static_assert(CAP <= 8192, "positions fit 13 bits");
-  using W = std::conditional_t<sizeof(K) == 8, uint64_t, K>;
-  W pk[CAP];  // 64-bit: (low bits << 13) | position; 128-bit: the key
+  static constexpr int TBITS = 12, NB = 1 << TBITS, PER = NB / RANK_BLOCK;
+  K key[CAP];             // offsets from base, by bucket
   uint32_t val[CAP];
-  uint16_t ord[CAP];           // group of each record
-  uint16_t gstart[CAP + 1];    // first position of each group, then cnt
-  uint32_t cnt[ITEMS * (RANK_BLOCK / 32) + 1];
-  uint32_t maxg;
+  uint32_t start[NB + 1];  // records per bucket, then its first position
+  uint32_t wsum[RANK_BLOCK / 32];
+  uint64_t bound[2];
+  K base, range;
+  uint32_t passes, span_bits, maxg;
 };
 
 template <class K>
 __global__ __launch_bounds__(RANK_BLOCK, 2) void k_seg_rank(
     const K *__restrict__ kin, const uint32_t *__restrict__ vin, const uint64_t *__restrict__ bound,
     const uint32_t *__restrict__ osize, const uint64_t *__restrict__ ooff, const K *__restrict__ gk,
-    const uint32_t *__restrict__ gv, K *__restrict__ kout, uint32_t *__restrict__ vout, int low_bits,
+    const uint32_t *__restrict__ gv, K *__restrict__ kout, uint32_t *__restrict__ vout, LowBits lb, ValOrder vo,
     uint32_t *__restrict__ fb_list, uint32_t *__restrict__ fb_count) {
   using S = SegRankSmem<K>;
-  constexpr int ITEMS = S::ITEMS;
-  constexpr bool WIDE = sizeof(K) == 16;
+  constexpr int ITEMS = S::ITEMS, PER = S::PER;
   extern __shared__ __align__(128) unsigned char smem_raw[];
   S &sm = *reinterpret_cast<S *>(smem_raw);
-  const int tid = threadIdx.x;
+  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
   const uint32_t tile = blockIdx.x;
-  const uint64_t s = bound[tile];
   if (osize[tile]) {
-    const uint64_t o = ooff[tile];
+    const uint64_t s = bound[tile], o = ooff[tile];
     for (uint32_t j = tid; j < osize[tile]; j += RANK_BLOCK) {
       kout[s + j] = gk[o + j];
       vout[s + j] = gv[o + j];
     }
     return;
   }
+  const uint64_t s = bound[tile];
   const uint32_t cnt = (uint32_t)(bound[tile + 1] - s);
   if (cnt == 0) return;
+  K key[ITEMS];
+  uint32_t val[ITEMS], at[ITEMS];
+#pragma unroll
+  for (int i = 0; i < ITEMS; i++) {
+    const uint32_t j = (uint32_t)i * RANK_BLOCK + tid;
+    if (j < cnt) {
+      key[i] = kin[s + j];
+      val[i] = vin[s + j];
+    }
+  }
+  for (int j = tid; j < S::NB; j += RANK_BLOCK) sm.start[j] = 0;
   if (tid == 0) sm.maxg = 0;
-  // stage the records; a group starts where the high bits change
-  bool head[ITEMS];
-  uint32_t rk[ITEMS];
+  seg_setup<K>(sm, kin, bound, tile, lb);  // synchronises
+  const K base = sm.base;
+  const int bshift = (int)sm.span_bits > S::TBITS ? (int)sm.span_bits - S::TBITS : 0;
+  auto bucket = [&](const K &d) { return (uint32_t)KeyOps<K>::words_lo(KeyOps<K>::shr(d, bshift)); };
 #pragma unroll
-  for (int i = 0; i < ITEMS; i++) {
-    const uint32_t j = (uint32_t)i * RANK_BLOCK + tid;
-    head[i] = false;
-    if (j < cnt) {
-      const K x = kin[s + j];
-      head[i] = j == 0 || !KeyOps<K>::eq(KeyOps<K>::shr(x, low_bits), KeyOps<K>::shr(kin[s + j - 1], low_bits));
-      if constexpr (WIDE) {
-        sm.pk[j] = x;
-      } else {
-        sm.pk[j] = ((x & ((1ull << low_bits) - 1ull)) << 13) | j;
-      }
-      sm.val[j] = vin[s + j];
+  for (int i = 0; i < ITEMS; i++)
+    if ((uint32_t)i * RANK_BLOCK + tid < cnt) {
+      key[i] = KeyOps<K>::sub(key[i], base);
+      at[i] = atomicAdd(&sm.start[bucket(key[i])], 1u);
     }
-  }
-  const uint32_t G = tile_flag_ranks<RANK_BLOCK, ITEMS>(head, rk, sm.cnt);
+  __syncthreads();
+  // exclusive scan, PER consecutive buckets per thread
+  uint32_t c[PER], sum = 0, mx = 0;
 #pragma unroll
-  for (int i = 0; i < ITEMS; i++) {
-    const uint32_t j = (uint32_t)i * RANK_BLOCK + tid;
-    if (j < cnt) {
-      const uint32_t o = rk[i] + (head[i] ? 1u : 0u) - 1u;
-      sm.ord[j] = (uint16_t)o;
-      if (head[i]) sm.gstart[o] = (uint16_t)j;
-    }
+  for (int j = 0; j < PER; j++) {
+    c[j] = sm.start[tid * PER + j];
+    sum += c[j];
+    mx = max(mx, c[j]);
   }
-  if (tid == 0) sm.gstart[G] = (uint16_t)cnt;
+  const uint32_t incl = warp_incl_scan(sum);
+  if (lane == 31) sm.wsum[warp] = incl;
+  mx = __reduce_max_sync(0xffffffffu, mx);
+  if (lane == 0 && mx > RANK_GROUP_MAX) sm.maxg = mx;
   __syncthreads();
-  uint32_t mg = 0;
-  for (uint32_t o = tid; o < G; o += RANK_BLOCK) mg = max(mg, (uint32_t)sm.gstart[o + 1] - sm.gstart[o]);
-  mg = __reduce_max_sync(0xffffffffu, mg);
-  if ((tid & 31) == 0 && mg) atomicMax(&sm.maxg, mg);
-  __syncthreads();
-  if (sm.maxg > RANK_GROUP_MAX) {
+  if (sm.maxg) {
     if (tid == 0) fb_list[atomicAdd(fb_count, 1u)] = tile;
     return;
   }
-  for (uint32_t i = tid; i < cnt; i += RANK_BLOCK) {
-    const uint32_t o = sm.ord[i], a = sm.gstart[o], b = sm.gstart[o + 1];
-    uint32_t r = 0;
-    if constexpr (WIDE) {
-      const K x = sm.pk[i];
-      for (uint32_t t = a; t < b; t++) {
-        const K y = sm.pk[t];
-        r += (KeyOps<K>::less(y, x) || (t < i && KeyOps<K>::eq(y, x))) ? 1u : 0u;
-      }
-      kout[s + a + r] = x;
-    } else {
-      const uint64_t p = sm.pk[i];
-#pragma unroll 4
-      for (uint32_t t = a; t < b; t++) r += sm.pk[t] < p ? 1u : 0u;
-      kout[s + a + r] = kin[s + i];
+  uint32_t run = incl - sum;
+  for (int w = 0; w < warp; w++) run += sm.wsum[w];
+#pragma unroll
+  for (int j = 0; j < PER; j++) {
+    sm.start[tid * PER + j] = run;
+    run += c[j];
+  }
+  if (tid == RANK_BLOCK - 1) sm.start[S::NB] = run;
+  __syncthreads();
+#pragma unroll
+  for (int i = 0; i < ITEMS; i++)
+    if ((uint32_t)i * RANK_BLOCK + tid < cnt) {
+      const uint32_t q = sm.start[bucket(key[i])] + at[i];
+      sm.key[q] = key[i];
+      sm.val[q] = val[i];
     }
-    vout[s + a + r] = sm.val[i];
+  __syncthreads();
+  for (uint32_t q = tid; q < cnt; q += RANK_BLOCK) {
+    const K d = sm.key[q];
+    const uint32_t v = sm.val[q], o = bucket(d), a = sm.start[o], b = sm.start[o + 1];
+    uint32_t r = 0;
+    for (uint32_t t = a; t < b; t++) {
+      const K y = sm.key[t];
+      bool before = KeyOps<K>::less(y, d);
+      if (KeyOps<K>::eq(y, d)) {
+        const uint32_t w = sm.val[t] << vo.shift, mine = v << vo.shift;
+        before = w < mine || (w == mine && t < q);
+      }
+      r += before ? 1u : 0u;
+    }
+    kout[s + a + r] = KeyOps<K>::add(d, base);
+    vout[s + a + r] = v;
   }
 }
 
@@ -465,8 +531,8 @@ template <class K, int ITEMS, int RANK>
 __global__ __launch_bounds__(SEG_BLOCK, 2) void k_seg_rle(
     const K *__restrict__ kin, const uint64_t *__restrict__ bound, const uint32_t *__restrict__ osize,
     const uint64_t *__restrict__ ooff, const K *__restrict__ guniq, const uint32_t *__restrict__ gheads, uint32_t H,
-    K *__restrict__ ustage, uint32_t *__restrict__ mstage, uint32_t *__restrict__ tcount, int low_bits,
-    int key_bits, const uint32_t *__restrict__ tile_list) {
+    K *__restrict__ ustage, uint32_t *__restrict__ mstage, uint32_t *__restrict__ tcount, LowBits lb,
+    const uint32_t *__restrict__ tile_list) {
   using S = SegSortSmem<K, false, ITEMS>;
   extern __shared__ __align__(128) unsigned char smem_raw[];
   S &sm = *reinterpret_cast<S *>(smem_raw);
@@ -479,7 +545,7 @@ __global__ __launch_bounds__(SEG_BLOCK, 2) void k_seg_rle(
     }
     for (int i = tid; i < S::WARPS * RADIX; i += SEG_BLOCK) (&sm.whist[0][0])[i] = 0;
     for (int i = tid; i < S::WARPS * (RADIX + 1); i += SEG_BLOCK) (&sm.match[0][0])[i] = 0;
-    seg_setup<K>(sm, kin, bound, tile, low_bits, key_bits);
+    seg_setup<K>(sm, kin, bound, tile, lb);
     const uint64_t s = sm.bound[0];
     const uint32_t cnt = (uint32_t)(sm.bound[1] - s);
     const K base = sm.base;
@@ -545,15 +611,14 @@ __global__ __launch_bounds__(SEG_BLOCK, 2) void k_seg_rle(
 // over_list and sorted by k_seg_rle instead.
 //
 // Ordering the distinct keys.  With rank_groups set, the distinct keys are
-// bucketed by their high bits (from low_bits up) -- the tile's groups, in
-// order; where those bits span more than TBL values, by their top bits, so
-// that a bucket holds 2, 4, ... adjacent groups -- and each key goes to its
-// bucket's start plus the number of the bucket's keys below it; a tile
-// with a bucket of more than COUNT_GROUP_MAX distinct keys is radix-sorted
-// by the 8-bit passes instead (and counted in rank_fb).  (Packing a 64-bit
-// key's offset and its count into one slot word, counted by 64-bit shared
-// atomic adds, measured 1.9x slower: the hot slots of a 30x-covered key
-// serialise.)
+// bucketed by the top 11 bits of their offset from the tile's base (2048
+// buckets for a few hundred to 1500 keys, so that most hold one or none),
+// and each key goes to its bucket's start plus the number of the bucket's
+// keys below it; a tile with a bucket of more than COUNT_GROUP_MAX distinct
+// keys is radix-sorted by the 8-bit passes instead (and counted in rank_fb).
+// (Packing a 64-bit key's offset and its count into one slot word, counted
+// by 64-bit shared atomic adds, measured 1.9x slower: the hot slots of a
+// 30x-covered key serialise.)
 constexpr uint32_t COUNT_GROUP_MAX = 256;
 
 // Hash-table slots of the counting pass.  The empty mark is the all-ones
@@ -618,14 +683,14 @@ struct SegCountSmem {
   uint32_t cnt[ITEMS * WARPS + 1];
   uint32_t tmp[8];
   uint64_t bound[2];
-  K base;
-  uint32_t tile, passes, excl, total, spread_bits, overflow, maxg;
+  K base, range;
+  uint32_t tile, passes, excl, total, span_bits, overflow, maxg;
 };
 
-// high bits of a key offset, as a group index within the tile
+// high bits of a key offset, as a bucket index within the tile
 template <class K>
-__device__ __forceinline__ uint32_t group_of(K d, int low_bits) {
-  return (uint32_t)KeyOps<K>::words_lo(KeyOps<K>::shr(d, low_bits));
+__device__ __forceinline__ uint32_t group_of(K d, int bshift) {
+  return (uint32_t)KeyOps<K>::words_lo(KeyOps<K>::shr(d, bshift));
 }
 
 template <class K, int RANK>
@@ -633,8 +698,7 @@ __global__ __launch_bounds__(SEG_BLOCK, 4) void k_seg_count(
     const K *__restrict__ kin, const uint64_t *__restrict__ bound, const uint32_t *__restrict__ osize,
     const uint64_t *__restrict__ ooff, const K *__restrict__ guniq, const uint32_t *__restrict__ gheads, uint32_t H,
     K *__restrict__ ustage, uint32_t *__restrict__ mstage, uint32_t *__restrict__ tcount,
-    uint32_t *__restrict__ over_list, uint32_t *__restrict__ over_count, int low_bits, int key_bits,
-    int rank_groups, uint32_t *__restrict__ rank_fb) {
+    uint32_t *__restrict__ over_list, uint32_t *__restrict__ over_count, LowBits lb, int rank_groups, uint32_t *__restrict__ rank_fb) {
   using S = SegCountSmem<K, RANK>;
   using O = SlotOps<K>;
   constexpr int ITEMS = S::ITEMS;
@@ -654,13 +718,13 @@ __global__ __launch_bounds__(SEG_BLOCK, 4) void k_seg_count(
     sm.vals[j] = 0;
   }
   if (tid == 0) sm.overflow = 0;
-  seg_setup<K>(sm, kin, bound, tile, low_bits, key_bits);  // synchronises
+  seg_setup<K>(sm, kin, bound, tile, lb);  // synchronises
   const uint64_t s = sm.bound[0];
   const uint32_t cnt = (uint32_t)(sm.bound[1] - s);
   const K base = sm.base;
   // the tile's path (uniform): ranked by buckets of groups
   const bool by_groups = rank_groups && cnt > 0;
-  const int bshift = (int)sm.spread_bits > S::TBITS ? (int)sm.spread_bits - S::TBITS : 0;
+  const int bshift = (int)sm.span_bits > S::TBITS ? (int)sm.span_bits - S::TBITS : 0;
   // count: each key into its slot, LOAD keys per thread at a time
   for (uint32_t j0 = 0; j0 < cnt; j0 += S::LOAD * SEG_BLOCK) {
     K d[S::LOAD];
@@ -717,16 +781,15 @@ __global__ __launch_bounds__(SEG_BLOCK, 4) void k_seg_count(
     }
   }
   __syncthreads();
-  const int gshift = low_bits + bshift;  // a key offset's bucket bits
   bool ranked = false;
   if (by_groups && D > 0) {
     // bucket the distinct keys: counts, exclusive scan (ITEMS consecutive
     // buckets per thread), then placement
-    const uint32_t G = 1u << ((int)sm.spread_bits - bshift);
+    const uint32_t G = cnt > 0 ? group_of<K>(sm.range, bshift) + 1u : 0u;
     for (uint32_t o = tid; o < G; o += SEG_BLOCK) sm.gst[o] = 0;
     if (tid == 0) sm.maxg = 0;
     __syncthreads();
-    for (uint32_t r = tid; r < D; r += SEG_BLOCK) atomicAdd(&sm.gst[group_of<K>(sm.keys[r], gshift)], 1u);
+    for (uint32_t r = tid; r < D; r += SEG_BLOCK) atomicAdd(&sm.gst[group_of<K>(sm.keys[r], bshift)], 1u);
     __syncthreads();
     uint32_t gc[ITEMS], sum = 0, mx = 0;
 #pragma unroll
@@ -748,11 +811,11 @@ __global__ __launch_bounds__(SEG_BLOCK, 4) void k_seg_count(
     __syncthreads();
     if (sm.maxg <= COUNT_GROUP_MAX) {
       for (uint32_t r = tid; r < D; r += SEG_BLOCK)
-        sm.perm[atomicAdd(&sm.gst[group_of<K>(sm.keys[r], gshift)], 1u)] = (uint16_t)r;
+        sm.perm[atomicAdd(&sm.gst[group_of<K>(sm.keys[r], bshift)], 1u)] = (uint16_t)r;
       __syncthreads();
       // bucket o now spans [gst[o - 1], gst[o]) (from 0 for o = 0)
       for (uint32_t q = tid; q < D; q += SEG_BLOCK) {
-        const uint32_t r = sm.perm[q], o = group_of<K>(sm.keys[r], gshift);
+        const uint32_t r = sm.perm[q], o = group_of<K>(sm.keys[r], bshift);
         const uint32_t a = o ? sm.gst[o - 1] : 0u, b = sm.gst[o];
         const K x = sm.keys[r];
         uint32_t below = 0;
