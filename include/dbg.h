@@ -212,10 +212,12 @@ dbg_status dbg_compact(dbg_ctx *ctx, const dbg_graph *g, dbg_unitigs **out);
 
 /* How dbg_compact ranks the lists.  0 (the default): the meeting walks
  * with staged halves when every list is short and acyclic, with 32-bit walk
- * words up to 2^29 - 1 strand-nodes and 64-bit words up to 2^30, else
- * pointer jumping with cycle breaking; 1: the walks with 64-bit words at
- * any size they allow; 2: pointer jumping only.  The unitigs are the same
- * either way.  DBG_EINVAL for another mode. */
+ * words up to 2^29 - 1 strand-nodes and 64-bit words up to 2^30; few long
+ * lists by segments (pointer jumping over about one strand-node in 16); and
+ * pointer jumping over all of them with cycle breaking when there are cycles.
+ * 1: the same with 64-bit walk words at any size they allow; 2: pointer
+ * jumping only.  The unitigs are the same either way.  DBG_EINVAL for another
+ * mode. */
 dbg_status dbg_compact_mode_set(dbg_ctx *ctx, int mode);
 
 /* Streams over which the read-back of a graph (dbg_graph_*_async) or of

@@ -75,11 +75,11 @@ __global__ void k_side_links(const uint64_t *__restrict__ row_ptr, const uint32_
 
 // A meeting walk's word per strand-node: its successor (or "tail") and its
 // entry base -- the base a walk appends on arriving at it, the last base of
-// its k-mer on its strand -- or a mark (the head of the walker that took
-// the node on the other strand).  32-bit words for up to 2^29 - 1
-// strand-nodes (successor in bits 0-28, all ones for a tail; base in bits
-// 29-30; mark in bit 31), 64-bit words above (successor in the low word,
-// all ones for a tail; base in bits 32-33; a mark as 2^62 | head).
+// its k-mer on its strand -- or, once the walk that leads there has ended, the
+// number of a walker's record.  32-bit words for up to 2^29 - 1 strand-nodes
+// (successor in bits 0-28, all ones for a tail; base in bits 29-30), 64-bit
+// words above (successor in the low word, all ones for a tail; base in bits
+// 32-33).
 template <class W>
 struct WalkWord;
 template <>
@@ -88,9 +88,6 @@ struct WalkWord<uint32_t> {
   __host__ __device__ static uint32_t make(uint32_t next, uint32_t base) {
     return ((base & 3u) << 29) | (next == NONE32 ? 0x1fffffffu : next);
   }
-  __device__ static bool marked(uint32_t w) { return (w >> 31) != 0; }
-  __device__ static uint32_t mark(uint32_t head) { return 0x80000000u | head; }
-  __device__ static uint32_t head(uint32_t w) { return w & 0x7fffffffu; }
   __device__ static bool tail(uint32_t w) { return (w & 0x1fffffffu) == 0x1fffffffu; }
   __device__ static uint32_t next(uint32_t w) { return w & 0x1fffffffu; }
   __device__ static uint32_t base(uint32_t w) { return (w >> 29) & 3u; }
@@ -101,38 +98,56 @@ struct WalkWord<uint64_t> {
   __host__ __device__ static uint64_t make(uint32_t next, uint32_t base) {
     return ((uint64_t)(base & 3u) << 32) | next;
   }
-  __device__ static bool marked(uint64_t w) { return (w >> 62) == 1ull; }
-  __device__ static uint64_t mark(uint32_t head) { return (1ull << 62) | head; }
-  __device__ static uint32_t head(uint64_t w) { return (uint32_t)w; }
   __device__ static bool tail(uint64_t w) { return (uint32_t)w == NONE32; }
   __device__ static uint32_t next(uint64_t w) { return (uint32_t)w; }
   __device__ static uint32_t base(uint64_t w) { return (uint32_t)(w >> 32) & 3u; }
 };
 
+// *sum += the warps' (warp-uniform) counts, one atomic add per block.
+__device__ __forceinline__ void add_per_block(uint32_t *sum, uint32_t count) {
+  __shared__ uint32_t s_sum;
+  if (threadIdx.x == 0) s_sum = 0;
+  __syncthreads();
+  if ((threadIdx.x & 31) == 0 && count) atomicAdd(&s_sum, count);
+  __syncthreads();
+  if (threadIdx.x == 0 && s_sum) atomicAdd(sum, s_sum);
+}
+
 // ListRankingTransform arcs.  Strand-node x = 2v + s leaves v by its right
 // side (s = 0) or its left side (s = 1); the arc exists when the edge there
 // joins two distinct nodes and is alone on the far node's side too.  It
 // enters w on side sw: strand 0 when that is w's left side, 1 otherwise.
-// succ[x] = the successor or NONE; mk, when given, receives x's walk word
-// (the meeting walks' working copy, which they mark), with x's entry base
-// (entering v by side s).
+// succ[x] = the successor or NONE; mk and tails, when given, receive x's walk
+// word, with x's entry base (entering v by side s), and the bitmap of the strand-nodes
+// without a successor.
 template <class W>
 __global__ void k_successors(const uint32_t *__restrict__ link_node, const uint64_t *__restrict__ link_edge,
-                             uint64_t V, uint32_t *__restrict__ succ, W *__restrict__ mk) {
-  for (uint64_t x = (uint64_t)blockIdx.x * blockDim.x + threadIdx.x; x < 2 * V; x += (uint64_t)gridDim.x * blockDim.x) {
-    const uint64_t v = x >> 1;
-    const uint32_t leave = (x & 1) ? 0u : 1u;
-    const uint32_t ln = link_node[2 * v + leave];
+                             uint64_t V, uint32_t *__restrict__ succ, W *__restrict__ mk,
+                             uint32_t *__restrict__ tails, uint32_t *__restrict__ lists) {
+  const int lane = threadIdx.x & 31;
+  uint32_t count = 0;
+  for (uint64_t g = (uint64_t)blockIdx.x * blockDim.x + (threadIdx.x & ~31u); g < 2 * V;
+       g += (uint64_t)gridDim.x * blockDim.x) {
+    const uint64_t x = g + lane;
     uint32_t out = NONE32;
-    uint64_t far = 0;
-    if (ln != NONE32) {
-      const uint32_t w = ln >> 1, sw = ln & 1u;
-      far = link_edge[2 * (uint64_t)w + sw];
-      if (w != (uint32_t)v && (uint32_t)far == (uint32_t)link_edge[2 * v + leave]) out = 2 * w + (sw == 0 ? 0u : 1u);
+    if (x < 2 * V) {
+      const uint64_t v = x >> 1;
+      const uint32_t leave = (x & 1) ? 0u : 1u;
+      const uint32_t ln = link_node[2 * v + leave];
+      uint64_t far = 0;
+      if (ln != NONE32) {
+        const uint32_t w = ln >> 1, sw = ln & 1u;
+        far = link_edge[2 * (uint64_t)w + sw];
+        if (w != (uint32_t)v && (uint32_t)far == (uint32_t)link_edge[2 * v + leave]) out = 2 * w + (sw == 0 ? 0u : 1u);
+      }
+      succ[x] = out;
+      if (mk) mk[x] = WalkWord<W>::make(out, (uint32_t)(link_edge[2 * v + (x & 1)] >> 32));
     }
-    succ[x] = out;
-    if (mk) mk[x] = WalkWord<W>::make(out, (uint32_t)(link_edge[2 * v + (x & 1)] >> 32));
+    const unsigned t = __ballot_sync(0xffffffffu, x < 2 * V && out == NONE32);
+    if (tails && lane == 0) tails[g / 32] = t;
+    count += __popc(t);
   }
+  if (lists) add_per_block(lists, count);
 }
 
 // The same arcs, for up to 2^29 - 1 strand-nodes, through a bitmap small
@@ -197,25 +212,29 @@ __global__ void k_side_cand(const uint64_t *__restrict__ row_ptr, const uint32_t
   }
 }
 
-// Keeps the candidates whose successor's side is lone too: mk[x] (in
-// place) and succ[x].  Each thread takes SL_U strand-nodes a grid stride
-// apart, their candidate loads and then their bitmap lookups (L2 hits at
-// random) in flight together.
+// Keeps the candidates whose successor's side is lone too: mk[x] in place
+// (rewritten only where the candidate falls), the bitmap of the strand-nodes
+// left without a successor, their number, and, when given, succ[x].  Each thread takes SL_U
+// strand-nodes a grid stride apart, their candidate loads and then their
+// bitmap lookups (L2 hits at random) in flight together.
 constexpr int SL_U = 4;
 
 __global__ void k_succ_lone(uint32_t *__restrict__ mk, const uint32_t *__restrict__ lone, uint64_t n,
-                            uint32_t *__restrict__ succ) {
+                            uint32_t *__restrict__ tails, uint32_t *__restrict__ succ,
+                            uint32_t *__restrict__ lists) {
+  uint32_t count = 0;  // (lane 0) tails met
   const uint64_t stride = (uint64_t)gridDim.x * blockDim.x;
-  for (uint64_t x0 = (uint64_t)blockIdx.x * blockDim.x + threadIdx.x; x0 < n; x0 += stride * SL_U) {
+  const int lane = threadIdx.x & 31;
+  for (uint64_t g = (uint64_t)blockIdx.x * blockDim.x + (threadIdx.x & ~31u); g < n; g += stride * SL_U) {
     uint32_t c[SL_U], bits[SL_U];
 #pragma unroll
     for (int u = 0; u < SL_U; u++) {
-      const uint64_t x = x0 + (uint64_t)u * stride;
+      const uint64_t x = g + lane + (uint64_t)u * stride;
       c[u] = x < n ? mk[x] : 0u;
     }
 #pragma unroll
     for (int u = 0; u < SL_U; u++) {
-      const uint64_t x = x0 + (uint64_t)u * stride;
+      const uint64_t x = g + lane + (uint64_t)u * stride;
       bits[u] = 0;
       if (x < n && !WalkWord<uint32_t>::tail(c[u])) {
         const uint32_t y = WalkWord<uint32_t>::next(c[u]);
@@ -224,17 +243,18 @@ __global__ void k_succ_lone(uint32_t *__restrict__ mk, const uint32_t *__restric
     }
 #pragma unroll
     for (int u = 0; u < SL_U; u++) {
-      const uint64_t x = x0 + (uint64_t)u * stride;
-      if (x >= n) break;
-      uint32_t out = NONE32;
-      if (!WalkWord<uint32_t>::tail(c[u])) {
-        if (bits[u] & 1u) out = WalkWord<uint32_t>::next(c[u]);
-        else c[u] = WalkWord<uint32_t>::make(NONE32, WalkWord<uint32_t>::base(c[u]));
-      }
-      mk[x] = c[u];
-      succ[x] = out;
+      const uint64_t w = g + (uint64_t)u * stride, x = w + lane;
+      if (w >= n) break;  // warp-uniform
+      const bool was = x < n && !WalkWord<uint32_t>::tail(c[u]);
+      const bool keep = was && (bits[u] & 1u);
+      if (was && !keep) mk[x] = WalkWord<uint32_t>::make(NONE32, WalkWord<uint32_t>::base(c[u]));
+      if (succ && x < n) succ[x] = keep ? WalkWord<uint32_t>::next(c[u]) : NONE32;
+      const unsigned t = __ballot_sync(0xffffffffu, x < n && !keep);
+      if (lane == 0) tails[w / 32] = t;
+      count += __popc(t);
     }
   }
+  add_per_block(lists, count);
 }
 
 // The predecessor of a strand-node, from the mirror symmetry of the
@@ -266,6 +286,84 @@ __global__ void k_walk_lists(const uint32_t *__restrict__ succ, uint64_t n, uint
       if (ny == NONE32) break;
       y = ny;
     }
+  }
+}
+
+// List ranking by segments: every list is cut at its splitters (about one
+// node in 16, by a hash of its ID, on both strands).  A walker per segment --
+// from each list head and each splitter to the next splitter -- writes (start
+// of the segment, offset) to the strand-nodes after its start, so a splitter's
+// word leads to the start before it; pointer jumping then ranks the splitters
+// among themselves (a sixteenth of the strand-nodes, listed in `active`), and
+// k_resolve_segments adds their ranks to the offsets.  No walk is much longer
+// than a few hundred steps however long the lists are.  *total counts the
+// words written: fewer than n when a cycle holds no splitter.
+constexpr int SPLIT_BITS = 4;
+__device__ __forceinline__ bool is_splitter(uint32_t x) {
+  return ((x >> 1) * 0x9e3779b1u) >> (32 - SPLIT_BITS) == 0;
+}
+
+__global__ void k_walk_segments(const uint32_t *__restrict__ succ, uint64_t n, uint64_t *__restrict__ word,
+                                uint32_t *__restrict__ active, uint32_t *__restrict__ active_count,
+                                unsigned long long *__restrict__ total) {
+  constexpr int WARPS = 8, CHUNK = 1024;
+  __shared__ uint32_t s_q[WARPS][CHUNK];
+  __shared__ uint32_t s_next[WARPS];
+  const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
+  const uint64_t chunks = (n + CHUNK - 1) / CHUNK;
+  unsigned long long written = 0;
+  for (uint64_t c = (uint64_t)blockIdx.x * WARPS + w; c < chunks; c += (uint64_t)gridDim.x * WARPS) {
+    // bit j of lane r: strand-node 32 r + j of the chunk starts a segment /
+    // is a splitter inside a list
+    uint32_t start = 0, inner = 0;
+    for (int r = 0; r < 32; r++) {
+      const uint64_t x = c * CHUNK + r * 32 + lane;
+      const bool head = x < n && succ[x ^ 1] == NONE32, in = x < n && !head && is_splitter((uint32_t)x);
+      const unsigned bs = __ballot_sync(0xffffffffu, head || in), bi = __ballot_sync(0xffffffffu, in);
+      if (lane == r) {
+        start = bs;
+        inner = bi;
+      }
+    }
+    const uint32_t ns = __popc(start), is = warp_incl_scan(ns), cnt = __shfl_sync(0xffffffffu, is, 31);
+    const uint32_t ni = __popc(inner), ii = warp_incl_scan(ni), act = __shfl_sync(0xffffffffu, ii, 31);
+    uint32_t base = 0;
+    if (lane == 0) {
+      s_next[w] = 0;
+      if (act) base = atomicAdd(active_count, act);
+    }
+    base = __shfl_sync(0xffffffffu, base, 0);
+    const uint32_t x0 = (uint32_t)(c * CHUNK) + lane * 32;
+    for (uint32_t b = start, at = is - ns; b; b &= b - 1) s_q[w][at++] = x0 + __ffs(b) - 1;
+    for (uint32_t b = inner, at = base + ii - ni; b; b &= b - 1) active[at++] = x0 + __ffs(b) - 1;
+    __syncwarp();
+    for (;;) {
+      const uint32_t qi = atomicAdd(&s_next[w], 1u);
+      if (qi >= cnt) break;
+      const uint32_t s = s_q[w][qi];
+      if (succ[s ^ 1u] == NONE32) {
+        word[s] = pk(s, 0);
+        written++;
+      }
+      uint32_t i = 0;
+      for (uint32_t y = succ[s]; y != NONE32; y = succ[y]) {
+        word[y] = pk(s, ++i);
+        if (is_splitter(y)) break;
+      }
+      written += i;
+    }
+    __syncwarp();
+  }
+  written = __reduce_add_sync(0xffffffffu, (unsigned)written);
+  if (lane == 0 && written) atomicAdd(total, written);
+}
+
+// word[x] = (list head, rank) from (segment start, offset) and the start's
+// own word, which is final (a start's word resolves to itself).
+__global__ void k_resolve_segments(uint64_t n, uint64_t *word) {
+  for (uint64_t x = (uint64_t)blockIdx.x * blockDim.x + threadIdx.x; x < n; x += (uint64_t)gridDim.x * blockDim.x) {
+    const uint64_t w = word[x], ws = word[pk_a(w)];
+    if (pk_a(ws) != pk_a(w)) word[x] = pk(pk_a(ws), pk_d(ws) + pk_d(w));
   }
 }
 
@@ -443,36 +541,54 @@ __device__ __forceinline__ K strand_kmer(const uint64_t *node_keys, uint32_t x, 
   return (x & 1u) ? revcomp(km, k) : km;
 }
 
-// Walk scheduling: each warp takes a chunk of WALK_CHUNK indices, queues the
-// list heads it finds there in shared memory (ballots), and its lanes then
-// take heads from the queue one at a time, so no lane idles while another
-// finishes a long list.
+// Walk scheduling: each warp takes a chunk of WALK_CHUNK strand-nodes, queues
+// the list heads it finds there in shared memory, and its lanes then take
+// heads from the queue as their lists end.  (All 32 lanes in lockstep, each
+// taking a new head in the iteration after its list ended, keeps three times
+// the lanes busy and was slower: 10.7 ms against 9.2 for 200 M nodes.)
 constexpr int WALK_BLOCK = 256, WALK_WARPS = WALK_BLOCK / 32, WALK_CHUNK = 1024;
 
-template <class IsHead>
-__device__ __forceinline__ uint32_t queue_heads(uint64_t base, uint64_t n, uint32_t *q, IsHead is_head) {
+// The heads in chunk c: strand-node x heads a list when x ^ 1 has no
+// successor (the mirror symmetry of the transform), so 32 words of the
+// bitmap of tails, one per lane, with neighbouring bits swapped.
+__device__ __forceinline__ uint32_t queue_heads(uint64_t c, uint64_t words, const uint32_t *__restrict__ tails,
+                                                uint32_t *q) {
   const int lane = threadIdx.x & 31;
-  uint32_t cnt = 0;
-  for (int r = 0; r < WALK_CHUNK / 32; r++) {
-    const uint64_t x = base + r * 32 + lane;
-    const bool h = x < n && is_head(x);
-    const unsigned b = __ballot_sync(0xffffffffu, h);
-    if (h) q[cnt + __popc(b & ((1u << lane) - 1u))] = (uint32_t)x;
-    cnt += __popc(b);
+  const uint64_t i = c * (WALK_CHUNK / 32) + lane;
+  const uint32_t t = i < words ? tails[i] : 0u;
+  uint32_t h = (t >> 1 & 0x55555555u) | (t & 0x55555555u) << 1;
+  const uint32_t mine = __popc(h), incl = warp_incl_scan(mine);
+  uint32_t at = incl - mine;
+  while (h) {
+    q[at++] = (uint32_t)(i * 32) + (uint32_t)(__ffs(h) - 1);
+    h &= h - 1;
   }
   __syncwarp();
-  return cnt;
+  return __shfl_sync(0xffffffffu, incl, 31);
 }
 
-// The meeting walks.  A walker at strand-node y loads y's word from mk, the
-// working copy of the successor words; if the other walker has marked it
-// (with the other walker's head) the node is the other's and the walk
-// stops; else the walker marks the word the other walker would load at
-// this node, mk[y ^ 1], takes y and goes on.  Plain loads and stores: two
-// walkers arriving together may both take a few nodes, which the pairing
-// step measures.  hrec[x] = (nodes walker x took, its last strand-node, the
-// other walker's head, the index of its first staged entry); the walker
-// with the smaller head of each pair appends that head to `pairs`.
+// The meeting walks.  A walker at strand-node y claims y's node by an atomic
+// OR of its bit in `claimed` (one bit per node: 25 MB for 200 M nodes, which
+// stays in L2); if the other walker of the unitig claimed the node first, the
+// walk stops there, else the walker loads y's word from mk, takes y and goes
+// on to the word's successor.  So every node is taken by exactly one walker.
+//
+// Bound by random DRAM accesses: 42 G/s is what this part does, for chains and
+// for independent loads, whatever is fetched around the word (32, 64 or 128
+// bytes), so 4.8 ms for 200 M nodes; a claim in L2 costs 1/6 of one.
+// (With the load in flight during the claim, a load is lost per walker: 3 %
+// for 200 M nodes.)  The form before this one marked the word that the other
+// walker would load instead of a bit, a dirty DRAM sector per node: 11.4 ms
+// for 200 M nodes with its pairing; this one 10.2.
+//
+// rec[r] = (head, nodes taken, where it stopped, the index of its first
+// staged entry), r counting the heads.  Where it stopped: the strand-node
+// that was claimed, or the last strand-node taken | WALK_TAIL at the list's
+// end (the other walker then took none).  Of two walkers that were stopped by
+// each other, the one whose last node has the smaller ID leaves its record's
+// number (and WALK_LEFT in its own record) in the word that leads back to that
+// node, mk[last ^ 1], whose sector its walk has just loaded: the other
+// walker's stop, where k_walk_pair looks it up.
 //
 // Staging: each lane stages the strand-nodes its walks take, in walk order,
 // as entries (y << 2) | y's entry base (the base the arc into y appends), at
@@ -483,6 +599,7 @@ __device__ __forceinline__ uint32_t queue_heads(uint64_t base, uint64_t n, uint3
 // sectors half written in L2 under the walks' random traffic).  If the
 // staging area runs out, *overflow is set and the walks only measure.
 constexpr uint32_t STAGE_PAGE = 256;
+constexpr uint32_t WALK_TAIL = 0x80000000u, WALK_LEFT = 0x40000000u;  // (strand-nodes stay below 2^30)
 
 struct StageLane {
   uint32_t b[8];
@@ -514,50 +631,71 @@ __device__ __forceinline__ void stage_push(StageLane &ln, uint32_t e, uint32_t *
   ln.idx++;
   if (ln.nb == 8) {
     uint4 *dst = reinterpret_cast<uint4 *>(stage + (ln.idx - 8));
-    dst[0] = make_uint4(ln.b[0], ln.b[1], ln.b[2], ln.b[3]);
-    dst[1] = make_uint4(ln.b[4], ln.b[5], ln.b[6], ln.b[7]);
+    __stcs(dst, make_uint4(ln.b[0], ln.b[1], ln.b[2], ln.b[3]));
+    __stcs(dst + 1, make_uint4(ln.b[4], ln.b[5], ln.b[6], ln.b[7]));
     ln.nb = 0;
   }
 }
 
 template <class W>
-__global__ __launch_bounds__(WALK_BLOCK, 6) void k_mark_stage(W *__restrict__ mk,
-                                                           const uint32_t *__restrict__ succ, uint64_t n,
-                                                           uint32_t cap, uint4 *__restrict__ hrec,
-                                                           uint32_t *__restrict__ stage,
+__global__ __launch_bounds__(WALK_BLOCK, 6) void k_walk_claim(W *__restrict__ mk, const uint32_t *__restrict__ tails,
+                                                           uint64_t n, uint32_t cap, uint32_t *__restrict__ claimed,
+                                                           uint4 *__restrict__ rec, uint32_t *__restrict__ stage,
                                                            uint32_t *__restrict__ page_next,
                                                            unsigned long long *__restrict__ cursor,
                                                            uint64_t stage_cap, uint32_t *too_long,
-                                                           uint32_t *overflow, uint32_t *__restrict__ pairs,
-                                                           uint32_t *pair_count) {
+                                                           uint32_t *overflow, uint32_t *rec_count,
+                                                           const uint32_t *__restrict__ lists) {
   __shared__ uint32_t s_q[WALK_WARPS][WALK_CHUNK];
   __shared__ uint32_t s_next[WALK_WARPS];
   const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
-  const uint64_t chunks = (n + WALK_CHUNK - 1) / WALK_CHUNK;
+  const uint64_t chunks = (n + WALK_CHUNK - 1) / WALK_CHUNK, words = (n + 31) / 32;
   uint32_t lng = 0;
   StageLane ln;
+  // Few long lists are ranked by segments instead.  With H lists of n / H
+  // strand-nodes on average, the longest -- lengths falling off exponentially
+  // -- has n / H ln H, half of which its walker takes at 0.7 us a step: more
+  // than ranking by segments costs when that is over 250 us (its rounds of
+  // jumping) and over 0.12 ns a strand-node (H < 2^15).  And a list beyond
+  // twice the cap, of which H exp(-2 cap H / n) are expected, would be left to
+  // it after all.
+  const float H = (float)*lists, mean = (float)n / fmaxf(H, 1.f);
+  if ((H < 32768.f && mean * logf(fmaxf(H, 2.f)) > 700.f) || H * expf(-2.f * cap / mean) > 4.f ||
+      mean > 2.f * cap) {
+    if (blockIdx.x == 0 && threadIdx.x == 0) *too_long = 1;
+    return;
+  }
   for (uint64_t c = (uint64_t)blockIdx.x * WALK_WARPS + w; c < chunks; c += (uint64_t)gridDim.x * WALK_WARPS) {
-    const uint32_t cnt = queue_heads(c * WALK_CHUNK, n, s_q[w], [&](uint64_t x) { return succ[x ^ 1] == NONE32; });
-    if (lane == 0) s_next[w] = 0;
+    const uint32_t cnt = queue_heads(c, words, tails, s_q[w]);
+    uint32_t r0 = 0;
+    if (lane == 0) {
+      s_next[w] = 0;
+      if (cnt) r0 = atomicAdd(rec_count, cnt);
+    }
+    r0 = __shfl_sync(0xffffffffu, r0, 0);
     __syncwarp();
     for (;;) {
       const uint32_t qi = atomicAdd(&s_next[w], 1u);
       if (qi >= cnt) break;
-      const uint32_t x = s_q[w][qi];
-      uint32_t y = x, d = 0, last = NONE32, partner = NONE32, first = NONE32;
+      const uint32_t x = s_q[w][qi], r = r0 + qi;
+      uint32_t y = x, d = 0, last = NONE32, stop = NONE32, first = NONE32;
       for (;;) {
-        const W wd = __ldcg(mk + y);  // from L2: another SM's mark may be there
-        if (WalkWord<W>::marked(wd)) {
-          partner = WalkWord<W>::head(wd);
+        const uint32_t v = y >> 1, bit = 1u << (v & 31u);
+        if (atomicOr(claimed + (v >> 5), bit) & bit) {
+          stop = y;
+          if (d && last >> 1 < v) {
+            __stcg(mk + (last ^ 1u), (W)r);
+            stop |= WALK_LEFT;
+          }
           break;
         }
-        __stcg(mk + (y ^ 1u), WalkWord<W>::mark(x));
+        const W wd = __ldcg(mk + y);
         stage_push(ln, (y << 2) | WalkWord<W>::base(wd), stage, page_next, cursor, stage_cap, overflow);
         if (first == NONE32 && !ln.full) first = (uint32_t)(ln.idx - 1);
         d++;
         last = y;
         if (WalkWord<W>::tail(wd)) {
-          partner = y ^ 1u;
+          stop = y | WALK_TAIL;
           break;
         }
         if (d >= cap) {
@@ -566,19 +704,7 @@ __global__ __launch_bounds__(WALK_BLOCK, 6) void k_mark_stage(W *__restrict__ mk
         }
         y = WalkWord<W>::next(wd);
       }
-      hrec[x] = make_uint4(d, last, partner, first);
-      // append x when it is its pair's smaller head (one atomic per warp
-      // for the lanes here now)
-      const bool smaller = partner != NONE32 && partner > x;
-      const unsigned act = __activemask();
-      const unsigned want = __ballot_sync(act, smaller);
-      if (want) {
-        const int leader = __ffs(act) - 1;
-        uint32_t at = 0;
-        if (lane == leader) at = atomicAdd(pair_count, (uint32_t)__popc(want));
-        at = __shfl_sync(act, at, leader);
-        if (smaller) pairs[at + __popc(want & ((1u << lane) - 1u))] = x;
-      }
+      rec[r] = make_uint4(x, d, stop, first);
     }
     __syncwarp();
   }
@@ -595,53 +721,47 @@ __global__ __launch_bounds__(WALK_BLOCK, 6) void k_mark_stage(W *__restrict__ mk
   if (lane == 0 && lng) atomicAdd(too_long, lng);
 }
 
-// Per pair of walkers (listed by the smaller head): the unitig's length
-// L = d_a + d_b - o, o the nodes both took (found by stepping from the
-// second walker's last node, read on the first walker's strands, to the
-// first walker's last node); the copy kept (the one whose first k-mer is
-// smaller) and its first node's tables: its bit in the bitmap of unitig
-// heads, and the unitig's length << 1 | the kept copy's strand (one word,
-// one random store).
-template <class K>
-__global__ void k_mark_pair(const uint32_t *__restrict__ pairs, const uint32_t *__restrict__ pair_count,
-                            const uint32_t *__restrict__ succ, uint64_t n, const uint4 *__restrict__ hrec,
-                            const uint64_t *__restrict__ node_keys, int k, uint32_t cap,
-                            uint32_t *__restrict__ head_bits, uint32_t *__restrict__ len_at_head,
+// Per pair of walkers, by the record r that represents it -- the one that did
+// not leave its number, or the only one that took nodes: the copy kept (the one whose
+// first k-mer is smaller) and its first node's tables: its bit in the bitmap
+// of unitig heads, and in one word (one random store) r << 32 | the other
+// copy is kept << 31 | the unitig's length << 1 | the kept copy's strand.
+// rec[r].z becomes the other walker's record, or stays as it was where that
+// took no node.  (Lengths are at most twice the walks' cap.)
+template <class K, class W>
+__global__ void k_walk_pair(uint4 *__restrict__ rec, const uint32_t *__restrict__ rec_count,
+                            const W *__restrict__ mk, uint64_t n, const uint64_t *__restrict__ node_keys, int k,
+                            uint32_t *__restrict__ head_bits, uint64_t *__restrict__ at_head,
                             unsigned long long *covered, uint32_t *err) {
   unsigned long long cov = 0;
-  const uint32_t np = *pair_count;
-  for (uint64_t i = (uint64_t)blockIdx.x * blockDim.x + threadIdx.x; i < np; i += (uint64_t)gridDim.x * blockDim.x) {
-    const uint32_t x = pairs[i];
-    const uint4 ra = hrec[x];
-    const uint32_t p = ra.z;
-    if (p >= n || p <= x) {
-      atomicOr(err, ERR_INTERNAL);
-      continue;
-    }
-    const uint4 rb = hrec[p];
-    if (rb.z != x) {
-      atomicOr(err, ERR_INTERNAL);
-      continue;
-    }
-    uint32_t o = 0;
-    if (ra.x > 0 && rb.x > 0 && succ[ra.y] != (rb.y ^ 1u)) {
-      // the walks overlap: step from b's last node (on a's strands) to a's last
-      uint32_t y = rb.y ^ 1u, steps = 0;
-      while (y != ra.y && steps <= cap) {
-        y = succ[y];
-        steps++;
-      }
-      if (y != ra.y) {
+  const uint32_t nr = *rec_count;
+  for (uint64_t i = (uint64_t)blockIdx.x * blockDim.x + threadIdx.x; i < nr; i += (uint64_t)gridDim.x * blockDim.x) {
+    const uint4 ra = rec[i];
+    if (ra.y == 0) continue;
+    uint32_t L = ra.y, p;
+    if (ra.z & WALK_TAIL) {
+      p = (ra.z & ~WALK_TAIL) ^ 1u;  // the other copy's head is the last node's other strand
+    } else {
+      if (ra.z & WALK_LEFT) continue;
+      const uint32_t j = (uint32_t)mk[ra.z];
+      if (j >= nr || j == i) {
         atomicOr(err, ERR_INTERNAL);
         continue;
       }
-      o = steps + 1;
+      const uint4 rb = rec[j];
+      p = rb.x;
+      L += rb.y;
+      rec[i].z = j;
     }
-    const uint32_t L = ra.x + rb.x - o;
-    const uint32_t kept = KeyOps<K>::less(strand_kmer<K>(node_keys, p, k), strand_kmer<K>(node_keys, x, k)) ? p : x;
-    const uint32_t h = kept >> 1;
+    if (p >= n) {
+      atomicOr(err, ERR_INTERNAL);
+      continue;
+    }
+    const uint32_t x = ra.x;
+    const bool other = KeyOps<K>::less(strand_kmer<K>(node_keys, p, k), strand_kmer<K>(node_keys, x, k));
+    const uint32_t kept = other ? p : x, h = kept >> 1;
     atomicOr(head_bits + (h >> 5), 1u << (h & 31u));
-    len_at_head[h] = L << 1 | (kept & 1u);
+    at_head[h] = i << 32 | (other ? 1ull << 31 : 0ull) | L << 1 | (kept & 1u);
     cov += L;
   }
   cov = __reduce_add_sync(0xffffffffu, (unsigned)cov);
@@ -656,19 +776,18 @@ __global__ void k_head_popc(const uint32_t *__restrict__ head_bits, uint64_t nw,
 
 // The unitigs in the order of their first nodes: unitig u = the u-th set bit
 // of the head bitmap (wpre = the exclusive scan of the words' bit counts),
-// with its first strand-node uy[u] = 2v + the kept strand and its length
-// (from the head's word, length << 1 | strand).
+// with its length and its walkers' representative << 1 | the other copy is
+// kept (from the head's word).
 __global__ void k_head_list(const uint32_t *__restrict__ head_bits, uint64_t nw, const uint64_t *__restrict__ wpre,
-                            const uint32_t *__restrict__ len_at_head, uint32_t *__restrict__ uy,
+                            const uint64_t *__restrict__ at_head, uint32_t *__restrict__ urec,
                             uint32_t *__restrict__ ulen) {
   for (uint64_t i = (uint64_t)blockIdx.x * blockDim.x + threadIdx.x; i < nw; i += (uint64_t)gridDim.x * blockDim.x) {
     uint32_t b = head_bits[i];
     uint64_t u = wpre[i];
     while (b) {
-      const uint32_t v = (uint32_t)(i * 32) + (uint32_t)(__ffs(b) - 1);
-      const uint32_t w = len_at_head[v];
-      uy[u] = 2 * v + (w & 1u);
-      ulen[u] = w >> 1;
+      const uint64_t w = at_head[i * 32 + (uint32_t)(__ffs(b) - 1)];
+      urec[u] = (uint32_t)(w >> 31);
+      ulen[u] = (uint32_t)(w & 0x7fffffffu) >> 1;
       u++;
       b &= b - 1u;
     }
@@ -693,8 +812,7 @@ __device__ __forceinline__ char base_char(uint32_t b) { return (char)((0x5447434
 // Every kept unitig from its two staged halves.  With the kept walker's
 // head y (the unitig's first strand-node), a nodes taken by it and L in
 // all, the first a nodes are its entries in order; the other L - a are the
-// first L - a entries of the other walker, read backwards on the other
-// strand.  The string S (k + L - 1 bases) starts with y's k-mer, then the
+// entries of the other walker, read backwards on the other strand.  The string S (k + L - 1 bases) starts with y's k-mer, then the
 // bases the kept walker's arcs appended; the rest is the reverse complement
 // of the first L - a characters of the other walker's string T (its head's
 // k-mer, then its arcs' bases): S[k - 2 + L - m] is the complement of T[m].
@@ -706,8 +824,8 @@ constexpr int COPY_CHUNK = 64;  // unitigs per warp chunk (about as many nodes a
 
 template <class K>
 __global__ __launch_bounds__(WALK_BLOCK, 6) void k_stage_copy(
-    const uint32_t *__restrict__ uy, const uint32_t *__restrict__ ulen, const uint64_t *__restrict__ uoff,
-    const uint4 *__restrict__ hrec, const uint32_t *__restrict__ stage, const uint32_t *__restrict__ page_next,
+    const uint32_t *__restrict__ urec, const uint32_t *__restrict__ ulen, const uint64_t *__restrict__ uoff,
+    const uint4 *__restrict__ rec, const uint32_t *__restrict__ stage, const uint32_t *__restrict__ page_next,
     const uint64_t *__restrict__ node_keys, uint64_t V, uint64_t U, int k, uint64_t *__restrict__ nodes_out,
     char *__restrict__ seq, uint64_t *__restrict__ node_off, uint64_t *__restrict__ seq_off,
     uint8_t *__restrict__ circular) {
@@ -730,9 +848,17 @@ __global__ __launch_bounds__(WALK_BLOCK, 6) void k_stage_copy(
       qi = __shfl_sync(gmask, qi, 0, CG);
       if (qi >= cnt) break;
       const uint64_t u = u0 + qi;
-      const uint32_t y = uy[u];
-      const uint4 ra = hrec[y];
-      const uint32_t L = ulen[u], a = ra.x, bp = L - a;
+      const uint32_t ur = urec[u], L = ulen[u];
+      uint4 ra = rec[ur >> 1], rb;
+      // the other walker: its record, or its head alone where it took no node
+      if (ra.z & WALK_TAIL) rb = make_uint4((ra.z & ~WALK_TAIL) ^ 1u, 0u, 0u, 0u);
+      else rb = rec[ra.z];
+      if (ur & 1u) {
+        const uint4 t = ra;
+        ra = rb;
+        rb = t;
+      }
+      const uint32_t y = ra.x, a = ra.y, bp = L - a;
       const uint64_t off = uoff[u], so = off + u * (uint64_t)(k - 1);
       if (gl == 0) {
         node_off[u] = off;
@@ -751,12 +877,11 @@ __global__ __launch_bounds__(WALK_BLOCK, 6) void k_stage_copy(
         if (e + CG < a) q = stage_advance(page_next, q, CG);
       }
       if (bp > 0) {
-        const uint32_t zb = ra.z;
-        const K kb = strand_kmer<K>(node_keys, zb, k);
+        const K kb = strand_kmer<K>(node_keys, rb.x, k);
         const uint32_t mk_end = min((uint32_t)k, bp);
         for (uint32_t m = gl; m < mk_end; m += CG)
           seq[so + k - 2 + L - m] = base_char(3u - KeyOps<K>::digit(kb, 2 * (k - 1 - (int)m), 2));
-        q = (uint32_t)gl < bp ? stage_advance(page_next, hrec[zb].w, (uint32_t)gl) : 0;
+        q = (uint32_t)gl < bp ? stage_advance(page_next, rb.w, (uint32_t)gl) : 0;
         for (uint32_t e = gl; e < bp; e += CG) {
           const uint32_t t = stage[q];
           nodes_out[off + L - 1 - e] = (t >> 2) ^ 1u;
@@ -923,12 +1048,19 @@ static dbg_status compact_impl(dbg_ctx *ctx, const dbg_graph *g, dbg_unitigs *u,
     // up to 2^30 (their staged entries hold a strand-node in 30 bits)
     const bool fast = ctx->compact_mode != 2 && n <= WalkWord<uint64_t>::MAX_N;
     const bool w32 = fast && ctx->compact_mode == 0 && n <= WalkWord<uint32_t>::MAX_N;
-    DevBuf mk;
-    DBG_TRY(alloc_buf(ctx, succ, n1 * 4));
-    if (fast) DBG_TRY(alloc_buf(ctx, mk, n1 * (w32 ? 4 : 8)));
-    if (w32) {
-      // per side the lone end, a bitmap of the lone sides, the candidate
-      // words; then the arcs whose far side is lone too
+    DevBuf mk, tails;
+    const uint64_t tw = (n + 31) / 32;
+    // counters: 10 lists, 11 too_long, 12-13 covered, 14-15 page cursor,
+    // 16 overflow, 17 records
+    uint32_t *lists = ctx->d_counters + 10;
+    DBG_CUDA_TRY(cudaMemsetAsync(lists, 0, 8 * sizeof(uint32_t), s));
+    if (fast) {
+      DBG_TRY(alloc_buf(ctx, mk, n1 * (w32 ? 4 : 8)));
+      DBG_TRY(alloc_buf(ctx, tails, tw * 4));
+    }
+    // per side the lone end, a bitmap of the lone sides, the candidate words;
+    // then the arcs whose far side is lone too (succ: the general path's copy)
+    auto links_by_bitmap = [&](uint32_t *succ_out) -> dbg_status {
       DevBuf lone;
       DBG_TRY(alloc_buf(ctx, lone, (V / 16 + 2) * 4));
       DBG_LAUNCH(ctx, ST_COMPACT_LINKS,
@@ -938,10 +1070,15 @@ static dbg_status compact_impl(dbg_ctx *ctx, const dbg_graph *g, dbg_unitigs *u,
                                                            g->orient.as<uint8_t>(), g->adj_side.as<uint8_t>(),
                                                            g->node_keys.as<uint64_t>(), V, k, literal,
                                                            mk.as<uint32_t>(), lone.as<uint32_t>()));
-      DBG_LAUNCH(ctx, ST_COMPACT_LINKS, 12.0 * n,
+      DBG_LAUNCH(ctx, ST_COMPACT_LINKS, (succ_out ? 8.0 : 4.0) * n,
                  k_succ_lone<<<grid_of(n), 256, 0, s>>>(mk.as<uint32_t>(), lone.as<uint32_t>(), n,
-                                                        succ.as<uint32_t>()));
+                                                        tails.as<uint32_t>(), succ_out, lists));
+      return DBG_OK;
+    };
+    if (w32) {
+      DBG_TRY(links_by_bitmap(nullptr));
     } else {
+      DBG_TRY(alloc_buf(ctx, succ, n1 * 4));
       DBG_TRY(alloc_buf(ctx, link_node, n1 * 4));
       DBG_TRY(alloc_buf(ctx, link_edge, n1 * 8));
       DBG_LAUNCH(ctx, ST_COMPACT_LINKS, 16.0 * V + (double)E2 * 10 + 8.0 * V * g->key_words + 12.0 * n,
@@ -953,62 +1090,64 @@ static dbg_status compact_impl(dbg_ctx *ctx, const dbg_graph *g, dbg_unitigs *u,
       DBG_LAUNCH(ctx, ST_COMPACT_LINKS, 12.0 * n + 8.0 * n + (fast ? 12.0 : 4.0) * n,
                  k_successors<uint64_t><<<grid_of(n), 256, 0, s>>>(link_node.as<uint32_t>(), link_edge.as<uint64_t>(),
                                                                    V, succ.as<uint32_t>(),
-                                                                   fast ? mk.as<uint64_t>() : nullptr));
+                                                                   fast ? mk.as<uint64_t>() : nullptr,
+                                                                   fast ? tails.as<uint32_t>() : nullptr,
+                                                                   fast ? lists : nullptr));
       link_node.release();
       link_edge.release();
     }
     // ---- fast path: short acyclic lists only ----
     if (fast) {
-      // the heads of the unitigs as a bitmap over the nodes; their lengths
-      // and kept strands at the head nodes only
-      DevBuf f_bits, f_len, hrec, stage, page_next;
+      // the heads of the unitigs as a bitmap over the nodes; their words at
+      // the head nodes only
+      DevBuf f_bits, f_word, claimed, rec, stage, page_next;
       const uint64_t nw = (V + 31) / 32, nw1 = std::max<uint64_t>(1, nw);
       DBG_TRY(alloc_buf(ctx, f_bits, nw1 * 4));
-      DBG_TRY(alloc_buf(ctx, f_len, V1 * 4));
+      DBG_TRY(alloc_buf(ctx, f_word, V1 * 8));
+      DBG_TRY(alloc_buf(ctx, claimed, nw1 * 4));
       DBG_CUDA_TRY(cudaMemsetAsync(f_bits.p, 0, nw1 * 4, s));
+      DBG_CUDA_TRY(cudaMemsetAsync(claimed.p, 0, nw1 * 4, s));
       // the two walkers of each unitig meet half way and stage what they
-      // take (k_mark_stage); each pair gives its unitig's length and kept
-      // copy (k_mark_pair).  Staging room: every node once (the few that
-      // both walkers of a pair take within the margin), plus two partly
+      // take (k_walk_claim); each pair gives its unitig's length and kept
+      // copy (k_walk_pair).  Staging room: every node once, plus two partly
       // used pages per lane.
-      const unsigned wgrid = w32 ? walk_grid(ctx, n, k_mark_stage<uint32_t>) : walk_grid(ctx, n, k_mark_stage<uint64_t>);
+      const unsigned wgrid = w32 ? walk_grid(ctx, n, k_walk_claim<uint32_t>) : walk_grid(ctx, n, k_walk_claim<uint64_t>);
       const uint64_t lanes = (uint64_t)wgrid * WALK_BLOCK;
-      const uint64_t stage_cap = ((V + V / 4 + 2 * lanes * STAGE_PAGE) / STAGE_PAGE + 1) * STAGE_PAGE;
-      DBG_TRY(alloc_buf(ctx, hrec, n1 * sizeof(uint4)));
+      const uint64_t stage_cap = ((V + 2 * lanes * STAGE_PAGE) / STAGE_PAGE + 1) * STAGE_PAGE;
+      DBG_TRY(alloc_buf(ctx, rec, n1 * sizeof(uint4)));
       DBG_TRY(alloc_buf(ctx, stage, stage_cap * 4));
       DBG_TRY(alloc_buf(ctx, page_next, stage_cap / STAGE_PAGE * 4));
-      // counters: 11 too_long, 12-13 covered, 14-15 page cursor, 16 overflow,
-      // 17 pairs listed
-      DBG_CUDA_TRY(cudaMemsetAsync(ctx->d_counters + 10, 0, 8 * sizeof(uint32_t), s));
-      DevBuf pairs;
-      DBG_TRY(alloc_buf(ctx, pairs, V1 * 4));
       unsigned long long *cursor = reinterpret_cast<unsigned long long *>(ctx->d_counters + 14);
+      unsigned long long *d_covered = reinterpret_cast<unsigned long long *>(ctx->d_counters + 12);
+      uint32_t *nrec = ctx->d_counters + 17;
       if (w32)
-        DBG_LAUNCH(ctx, ST_COMPACT_RANK, 8.0 * n + 16.0 * V + 4.0 * V,
-                   k_mark_stage<uint32_t><<<wgrid, WALK_BLOCK, 0, s>>>(
-                       mk.as<uint32_t>(), succ.as<uint32_t>(), n, kWalkCap, hrec.as<uint4>(), stage.as<uint32_t>(),
-                       page_next.as<uint32_t>(), cursor, stage_cap, ctx->d_counters + 11, ctx->d_counters + 16,
-                       pairs.as<uint32_t>(), ctx->d_counters + 17));
+        DBG_LAUNCH(ctx, ST_COMPACT_RANK, 4.0 * V + n / 8.0 + V / 8.0 + 4.0 * V,
+                   k_walk_claim<uint32_t><<<wgrid, WALK_BLOCK, 0, s>>>(
+                       mk.as<uint32_t>(), tails.as<uint32_t>(), n, kWalkCap, claimed.as<uint32_t>(), rec.as<uint4>(),
+                       stage.as<uint32_t>(), page_next.as<uint32_t>(), cursor, stage_cap, ctx->d_counters + 11,
+                       ctx->d_counters + 16, nrec, lists));
       else
-        DBG_LAUNCH(ctx, ST_COMPACT_RANK, 8.0 * n + 24.0 * V + 4.0 * V,
-                   k_mark_stage<uint64_t><<<wgrid, WALK_BLOCK, 0, s>>>(
-                       mk.as<uint64_t>(), succ.as<uint32_t>(), n, kWalkCap, hrec.as<uint4>(), stage.as<uint32_t>(),
-                       page_next.as<uint32_t>(), cursor, stage_cap, ctx->d_counters + 11, ctx->d_counters + 16,
-                       pairs.as<uint32_t>(), ctx->d_counters + 17));
+        DBG_LAUNCH(ctx, ST_COMPACT_RANK, 8.0 * V + n / 8.0 + V / 8.0 + 4.0 * V,
+                   k_walk_claim<uint64_t><<<wgrid, WALK_BLOCK, 0, s>>>(
+                       mk.as<uint64_t>(), tails.as<uint32_t>(), n, kWalkCap, claimed.as<uint32_t>(), rec.as<uint4>(),
+                       stage.as<uint32_t>(), page_next.as<uint32_t>(), cursor, stage_cap, ctx->d_counters + 11,
+                       ctx->d_counters + 16, nrec, lists));
       DBG_CUDA_TRY(cudaGetLastError());
       uint32_t flags[6] = {0, 0, 0, 0, 0, 0};  // counters 11..16
       DBG_TRY(read_small(ctx, ctx->d_counters + 11, sizeof(flags), flags));
       const uint32_t too_long = flags[0], overflow = flags[5];
-      mk.release();
       uint64_t covered = 0;
       if (too_long == 0 && overflow == 0) {
-        DBG_LAUNCH(ctx, ST_COMPACT_RANK, 8.0 * n + 32.0 * V,
-                   k_mark_pair<K><<<grid_of(V), 256, 0, s>>>(pairs.as<uint32_t>(), ctx->d_counters + 17,
-                                                             succ.as<uint32_t>(), n, hrec.as<uint4>(),
-                                                             g->node_keys.as<uint64_t>(), k, kWalkCap,
-                                                             f_bits.as<uint32_t>(), f_len.as<uint32_t>(),
-                                                             reinterpret_cast<unsigned long long *>(ctx->d_counters + 12),
-                                                             ctx->d_err));
+        if (w32)
+          DBG_LAUNCH(ctx, ST_COMPACT_RANK, 16.0 * V,
+                     k_walk_pair<K, uint32_t><<<grid_of(V), 256, 0, s>>>(
+                         rec.as<uint4>(), nrec, mk.as<uint32_t>(), n, g->node_keys.as<uint64_t>(), k,
+                         f_bits.as<uint32_t>(), f_word.as<uint64_t>(), d_covered, ctx->d_err));
+        else
+          DBG_LAUNCH(ctx, ST_COMPACT_RANK, 16.0 * V,
+                     k_walk_pair<K, uint64_t><<<grid_of(V), 256, 0, s>>>(
+                         rec.as<uint4>(), nrec, mk.as<uint64_t>(), n, g->node_keys.as<uint64_t>(), k,
+                         f_bits.as<uint32_t>(), f_word.as<uint64_t>(), d_covered, ctx->d_err));
         DBG_CUDA_TRY(cudaGetLastError());
         DBG_TRY(read_small(ctx, ctx->d_counters + 12, sizeof(uint64_t), &covered));
         DBG_TRY(check_device_error(ctx));
@@ -1016,7 +1155,8 @@ static dbg_status compact_impl(dbg_ctx *ctx, const dbg_graph *g, dbg_unitigs *u,
       if (too_long == 0 && overflow == 0 && covered == V) {
         // the unitigs in the order of their first nodes: a scan over the
         // bitmap words, the list of heads, a scan over the unitigs' lengths
-        DevBuf wcnt, wpre, uy, ulen, uoff;
+        mk.release();
+        DevBuf wcnt, wpre, urec, ulen, uoff;
         DBG_TRY(alloc_buf(ctx, wcnt, nw1 * 4));
         DBG_TRY(alloc_buf(ctx, wpre, (nw + 1) * 8));
         DBG_LAUNCH(ctx, ST_COMPACT_OUTPUT, 8.0 * nw,
@@ -1024,12 +1164,12 @@ static dbg_status compact_impl(dbg_ctx *ctx, const dbg_graph *g, dbg_unitigs *u,
         uint32_t U32 = 0, total = 0;
         DBG_TRY(scan_excl(ctx, wcnt.as<uint32_t>(), nw, wpre.as<uint64_t>(), &U32));
         const uint64_t Uf = U32;
-        DBG_TRY(alloc_buf(ctx, uy, std::max<uint64_t>(1, Uf) * 4));
+        DBG_TRY(alloc_buf(ctx, urec, std::max<uint64_t>(1, Uf) * 4));
         DBG_TRY(alloc_buf(ctx, ulen, std::max<uint64_t>(1, Uf) * 4));
         DBG_TRY(alloc_buf(ctx, uoff, (Uf + 1) * 8));
         DBG_LAUNCH(ctx, ST_COMPACT_OUTPUT, 12.0 * nw + (double)Uf * (4 + 4 + 4),
                    k_head_list<<<grid_of(nw), 256, 0, s>>>(f_bits.as<uint32_t>(), nw, wpre.as<uint64_t>(),
-                                                           f_len.as<uint32_t>(), uy.as<uint32_t>(),
+                                                           f_word.as<uint64_t>(), urec.as<uint32_t>(),
                                                            ulen.as<uint32_t>()));
         DBG_TRY(scan_excl(ctx, ulen.as<uint32_t>(), Uf, uoff.as<uint64_t>(), &total));
         if (total != V) {
@@ -1046,7 +1186,7 @@ static dbg_status compact_impl(dbg_ctx *ctx, const dbg_graph *g, dbg_unitigs *u,
         DBG_LAUNCH(ctx, ST_COMPACT_OUTPUT,
                    (double)V * (4 + 8 + 1) + (double)Uf * (4 + 4 + 8 + 32 + 8 * g->key_words * 2 + 16 + k),
                    k_stage_copy<K><<<walk_grid(ctx, Uf, k_stage_copy<K>, COPY_CHUNK), WALK_BLOCK, 0, s>>>(
-                       uy.as<uint32_t>(), ulen.as<uint32_t>(), uoff.as<uint64_t>(), hrec.as<uint4>(),
+                       urec.as<uint32_t>(), ulen.as<uint32_t>(), uoff.as<uint64_t>(), rec.as<uint4>(),
                        stage.as<uint32_t>(), page_next.as<uint32_t>(), g->node_keys.as<uint64_t>(), V, Uf, k,
                        u->nodes.as<uint64_t>(), u->seq.as<char>(), u->node_off.as<uint64_t>(),
                        u->seq_off.as<uint64_t>(), u->circular.as<uint8_t>()));
@@ -1056,52 +1196,77 @@ static dbg_status compact_impl(dbg_ctx *ctx, const dbg_graph *g, dbg_unitigs *u,
       }
     }
     // ---- general path: long lists or cycles present ----
+    if (w32) {  // (walkers left their numbers in some words: the arcs again)
+      DBG_TRY(alloc_buf(ctx, succ, n1 * 4));
+      DBG_TRY(links_by_bitmap(succ.as<uint32_t>()));
+    }
     mk.release();
+    tails.release();
     DBG_TRY(alloc_buf(ctx, word, n1 * 8));
-    DBG_CUDA_TRY(cudaMemsetAsync(word.p, 0xff, n * 8, s));
-    DBG_LAUNCH(ctx, ST_COMPACT_RANK, 4.0 * n + 12.0 * n,
-               k_walk_lists<<<grid_of(n), 256, 0, s>>>(succ.as<uint32_t>(), n, kWalkCap,
-                                                       word.as<uint64_t>()));
-    DBG_CUDA_TRY(cudaGetLastError());
-    // what the walks left: tails of very long lists, and cycles
-    DBG_CUDA_TRY(cudaMemsetAsync(ctx->d_counters + 4, 0, sizeof(uint32_t), s));
     DBG_TRY(alloc_buf(ctx, active, n1 * 4));
-    DBG_LAUNCH(ctx, ST_COMPACT_RANK, 16.0 * n,
-               k_collect_active<<<grid_of(n), 256, 0, s>>>(succ.as<uint32_t>(), n, word.as<uint64_t>(),
-                                                           active.as<uint32_t>(), ctx->d_counters + 4));
-    uint32_t A = 0;
-    DBG_TRY(read_small(ctx, ctx->d_counters + 4, sizeof(uint32_t), &A));
-    if (A > 0) {
-      uint32_t left = 0;
-      DBG_TRY(jump_until_stable(ctx, active.as<uint32_t>(), A, word.as<uint64_t>(), &left));
-      if (left > 0) {
-        have_cycles = true;
-        DBG_TRY(alloc_buf(ctx, cycl, (uint64_t)A * 4));
-        DBG_TRY(alloc_buf(ctx, lab, n1 * 8));
-        DBG_TRY(alloc_buf(ctx, cyc, n1));
-        DBG_CUDA_TRY(cudaMemsetAsync(cyc.p, 0, n, s));
-        DBG_CUDA_TRY(cudaMemsetAsync(ctx->d_counters + 5, 0, sizeof(uint32_t), s));
-        DBG_LAUNCH(ctx, ST_COMPACT_CYCLES, 24.0 * A,
-                   k_collect_cycles<<<grid_of(A), 256, 0, s>>>(active.as<uint32_t>(), A, word.as<uint64_t>(),
-                                                               succ.as<uint32_t>(), cycl.as<uint32_t>(),
-                                                               lab.as<uint64_t>(), ctx->d_counters + 5));
-        uint32_t C = 0;
-        DBG_TRY(read_small(ctx, ctx->d_counters + 5, sizeof(uint32_t), &C));
-        int R = 2;
-        while ((1ull << (R - 2)) < C) R++;
-        for (int r = 0; r < R; r++)
-          DBG_LAUNCH(ctx, ST_COMPACT_CYCLES, 20.0 * C,
-                     k_cycle_min<<<grid_of(C), 256, 0, s>>>(cycl.as<uint32_t>(), C, lab.as<uint64_t>()));
-        DBG_LAUNCH(ctx, ST_COMPACT_CYCLES, 25.0 * C,
-                   k_cycle_break<<<grid_of(C), 256, 0, s>>>(cycl.as<uint32_t>(), C, lab.as<uint64_t>(),
-                                                            succ.as<uint32_t>(), cyc.as<uint8_t>(),
-                                                            word.as<uint64_t>()));
-        DBG_CUDA_TRY(cudaGetLastError());
-        uint32_t still = 0;
-        DBG_TRY(jump_until_stable(ctx, cycl.as<uint32_t>(), C, word.as<uint64_t>(), &still));
-        if (still != 0) {
-          set_error("%u strand-nodes stayed on cycles after they were opened", still);
-          return DBG_EINTERNAL;
+    bool ranked = false;
+    if (ctx->compact_mode != 2) {
+      // by segments, unless there are cycles
+      DBG_CUDA_TRY(cudaMemsetAsync(ctx->d_counters + 10, 0, 4 * sizeof(uint32_t), s));
+      DBG_LAUNCH(ctx, ST_COMPACT_RANK, 12.0 * n,
+                 k_walk_segments<<<walk_grid(ctx, n, k_walk_segments, 1024), 256, 0, s>>>(
+                     succ.as<uint32_t>(), n, word.as<uint64_t>(), active.as<uint32_t>(), ctx->d_counters + 10,
+                     reinterpret_cast<unsigned long long *>(ctx->d_counters + 12)));
+      DBG_CUDA_TRY(cudaGetLastError());
+      uint32_t got[4] = {0, 0, 0, 0}, left = 0;  // active; total
+      DBG_TRY(read_small(ctx, ctx->d_counters + 10, sizeof(got), got));
+      if (((uint64_t)got[3] << 32 | got[2]) == n) {
+        if (got[0] > 0) DBG_TRY(jump_until_stable(ctx, active.as<uint32_t>(), got[0], word.as<uint64_t>(), &left));
+        ranked = left == 0;
+      }
+      if (ranked)
+        DBG_LAUNCH(ctx, ST_COMPACT_RANK, 24.0 * n, k_resolve_segments<<<grid_of(n), 256, 0, s>>>(n, word.as<uint64_t>()));
+    }
+    if (!ranked) {
+      DBG_CUDA_TRY(cudaMemsetAsync(word.p, 0xff, n * 8, s));
+      DBG_LAUNCH(ctx, ST_COMPACT_RANK, 4.0 * n + 12.0 * n,
+                 k_walk_lists<<<grid_of(n), 256, 0, s>>>(succ.as<uint32_t>(), n, kWalkCap,
+                                                         word.as<uint64_t>()));
+      DBG_CUDA_TRY(cudaGetLastError());
+      // what the walks left: tails of very long lists, and cycles
+      DBG_CUDA_TRY(cudaMemsetAsync(ctx->d_counters + 4, 0, sizeof(uint32_t), s));
+      DBG_LAUNCH(ctx, ST_COMPACT_RANK, 16.0 * n,
+                 k_collect_active<<<grid_of(n), 256, 0, s>>>(succ.as<uint32_t>(), n, word.as<uint64_t>(),
+                                                             active.as<uint32_t>(), ctx->d_counters + 4));
+      uint32_t A = 0;
+      DBG_TRY(read_small(ctx, ctx->d_counters + 4, sizeof(uint32_t), &A));
+      if (A > 0) {
+        uint32_t left = 0;
+        DBG_TRY(jump_until_stable(ctx, active.as<uint32_t>(), A, word.as<uint64_t>(), &left));
+        if (left > 0) {
+          have_cycles = true;
+          DBG_TRY(alloc_buf(ctx, cycl, (uint64_t)A * 4));
+          DBG_TRY(alloc_buf(ctx, lab, n1 * 8));
+          DBG_TRY(alloc_buf(ctx, cyc, n1));
+          DBG_CUDA_TRY(cudaMemsetAsync(cyc.p, 0, n, s));
+          DBG_CUDA_TRY(cudaMemsetAsync(ctx->d_counters + 5, 0, sizeof(uint32_t), s));
+          DBG_LAUNCH(ctx, ST_COMPACT_CYCLES, 24.0 * A,
+                     k_collect_cycles<<<grid_of(A), 256, 0, s>>>(active.as<uint32_t>(), A, word.as<uint64_t>(),
+                                                                 succ.as<uint32_t>(), cycl.as<uint32_t>(),
+                                                                 lab.as<uint64_t>(), ctx->d_counters + 5));
+          uint32_t C = 0;
+          DBG_TRY(read_small(ctx, ctx->d_counters + 5, sizeof(uint32_t), &C));
+          int R = 2;
+          while ((1ull << (R - 2)) < C) R++;
+          for (int r = 0; r < R; r++)
+            DBG_LAUNCH(ctx, ST_COMPACT_CYCLES, 20.0 * C,
+                       k_cycle_min<<<grid_of(C), 256, 0, s>>>(cycl.as<uint32_t>(), C, lab.as<uint64_t>()));
+          DBG_LAUNCH(ctx, ST_COMPACT_CYCLES, 25.0 * C,
+                     k_cycle_break<<<grid_of(C), 256, 0, s>>>(cycl.as<uint32_t>(), C, lab.as<uint64_t>(),
+                                                              succ.as<uint32_t>(), cyc.as<uint8_t>(),
+                                                              word.as<uint64_t>()));
+          DBG_CUDA_TRY(cudaGetLastError());
+          uint32_t still = 0;
+          DBG_TRY(jump_until_stable(ctx, cycl.as<uint32_t>(), C, word.as<uint64_t>(), &still));
+          if (still != 0) {
+            set_error("%u strand-nodes stayed on cycles after they were opened", still);
+            return DBG_EINTERNAL;
+          }
         }
       }
     }
@@ -1282,7 +1447,7 @@ static dbg_status compact_bucketed_impl(dbg_ctx *ctx, const dbg_graph *g, uint64
                                                           false, link_node.as<uint32_t>(), link_edge.as<uint64_t>()));
     DBG_LAUNCH(ctx, ST_COMPACT_LINKS, 24.0 * n,
                k_successors<uint64_t><<<grid_of(n), 256, 0, s>>>(link_node.as<uint32_t>(), link_edge.as<uint64_t>(),
-                                                                 V, succ.as<uint32_t>(), nullptr));
+                                                                 V, succ.as<uint32_t>(), nullptr, nullptr, nullptr));
     DBG_CUDA_TRY(cudaGetLastError());
   }
   PinnedBuf h_succ, h_W, h_lab, h_req, h_out, h_moved;
