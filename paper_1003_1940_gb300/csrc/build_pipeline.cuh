@@ -557,6 +557,14 @@ dbg_status msd_sort(dbg_ctx *ctx, K **keys, K **alt_keys, uint32_t **vals, uint3
   return DBG_OK;
 }
 
+// The local pass's tiles and, sorted over every digit, the keys of the
+// oversize ones.
+struct TileSet {
+  uint64_t tiles = 0;
+  uint32_t gathered = 0;
+  DevBuf bound, osize, ooff, gk, gv;
+};
+
 // The records' order by payload: *out = n words whose low halves list the
 // records by ascending payload << shift.  (64-bit keys' sort: build_u64.cu.)
 dbg_status order_by_payload(dbg_ctx *ctx, const uint32_t *v, uint64_t n, int shift, DevBuf &buf,
@@ -565,14 +573,17 @@ dbg_status order_by_payload(dbg_ctx *ctx, const uint32_t *v, uint64_t n, int shi
 // Tile bounds of the local pass over n keys in the groups gr (sorted by
 // their bits from gr.lb up), and the oversize tiles (longer than the
 // shared-memory capacity) gathered into *gk / *gv and sorted over every
-// digit.  Returns the number of gathered keys in *G (0: none).
+// digit.
 template <class K, bool HAS_VAL>
 dbg_status seg_prepare(dbg_ctx *ctx, const K *kin, const uint32_t *vin, uint64_t n, Groups &gr, ValOrder vo,
-                       int key_bits, DevBuf &bound, DevBuf &osize, DevBuf &ooff, DevBuf &gk, DevBuf &gv, uint32_t *G, int stage) {
+                       int key_bits, TileSet &ts, int stage) {
   using Sh = SegShape<K>;
   cudaStream_t s = ctx->stream;
   const uint64_t tiles = (n + Sh::TILE - 1) / Sh::TILE;
   if (tiles > 0x7fffffffull) return DBG_EOVERFLOW;
+  ts.tiles = tiles;
+  DevBuf &bound = ts.bound, &osize = ts.osize, &ooff = ts.ooff, &gk = ts.gk, &gv = ts.gv;
+  uint32_t *G = &ts.gathered;
   DBG_TRY(alloc_buf(ctx, osize, tiles * 4));
   DBG_TRY(alloc_buf(ctx, ooff, (tiles + 1) * 8));
   if (gr.ng) DBG_TRY(msd_bounds<K>(ctx, gr, n, nullptr, stage));
@@ -629,49 +640,73 @@ dbg_status seg_prepare(dbg_ctx *ctx, const K *kin, const uint32_t *vin, uint64_t
   return DBG_OK;
 }
 
-// The local pass over node records in the groups gr: the fully sorted
-// records (equal keys by payload, in the order vo) to kout / vout.
+// The listed tiles of k_seg_rank, sorted by the digit passes.
+template <class K>
+dbg_status seg_sort_listed(dbg_ctx *ctx, const K *kin, const uint32_t *vin, K *kout, uint32_t *vout, Groups &gr,
+                           ValOrder vo, TileSet &ts, const uint32_t *fb_list, const uint32_t *fb_count,
+                           uint32_t nfb) {
+  using Sh = SegShape<K>;
+  const int rank = local_rank_method(ctx, sizeof(K) == 16);
+  auto kern = rank == RANK_MATCH    ? k_seg_sort<K, Sh::ITEMS, RANK_MATCH>
+              : rank == RANK_ATOMIC ? k_seg_sort<K, Sh::ITEMS, RANK_ATOMIC>
+                                    : k_seg_sort<K, Sh::ITEMS, RANK_BALLOT>;
+  constexpr size_t smem = sizeof(SegSortSmem<K, true, Sh::ITEMS>);
+  set_smem_attrs(kern, smem);
+  const unsigned grid = (unsigned)std::min<uint64_t>(nfb, 2ull * (uint64_t)std::max(1, ctx->num_sms));
+  DBG_LAUNCH(ctx, ST_LOCAL_SORT_NODES, 0.0,
+             kern<<<grid, SEG_BLOCK, smem, ctx->stream>>>(
+                 kin, vin, ts.bound.as<uint64_t>(), ts.osize.as<uint32_t>(), ts.ooff.as<uint64_t>(), ts.gk.as<K>(),
+                 ts.gv.as<uint32_t>(), kout, vout, gr.lb, vo, fb_list, fb_count));
+  DBG_CUDA_TRY(cudaGetLastError());
+  return DBG_OK;
+}
+
+// k_seg_rank over every tile (FUSED: heads and tcount), then the digit passes
+// for the tiles that it listed.
+template <class K, bool FUSED>
+dbg_status seg_rank_tiles(dbg_ctx *ctx, const K *kin, const uint32_t *vin, K *kout, uint32_t *vout, uint64_t n,
+                          Groups &gr, ValOrder vo, TileSet &ts, uint32_t *heads, uint32_t *tcount) {
+  static_assert(SegRankSmem<K>::CAP == SEG_BLOCK * SegShape<K>::ITEMS, "same tile capacity as the digit-pass kernel");
+  auto kern = k_seg_rank<K, FUSED>;
+  set_smem_attrs(kern, sizeof(SegRankSmem<K>));
+  DevBuf fb;
+  // the tiles listed for the digit passes, and from the other end the oversize
+  // ones; their numbers first
+  DBG_TRY(alloc_buf(ctx, fb, (ts.tiles + 2) * 4));
+  uint32_t *fb_count = fb.as<uint32_t>(), *fb_list = fb_count + 2;
+  DBG_CUDA_TRY(cudaMemsetAsync(fb_count, 0, 8, ctx->stream));
+  DBG_LAUNCH(ctx, ST_LOCAL_SORT_NODES, 2.0 * (double)n * (sizeof(K) + 4),
+             kern<<<(unsigned)ts.tiles, RANK_BLOCK, sizeof(SegRankSmem<K>), ctx->stream>>>(
+                 kin, vin, ts.bound.as<uint64_t>(), ts.osize.as<uint32_t>(), ts.ooff.as<uint64_t>(), ts.gk.as<K>(),
+                 ts.gv.as<uint32_t>(), kout, vout, gr.lb, vo, fb_list, fb_count, heads, tcount));
+  DBG_CUDA_TRY(cudaGetLastError());
+  uint32_t listed[2] = {0, 0};
+  DBG_TRY(read_small(ctx, fb_count, sizeof(listed), listed));
+  const uint32_t nfb = listed[0], n_over = listed[1];
+  ctx->rank_fallback_tiles += nfb;
+  if (nfb) DBG_TRY(seg_sort_listed<K>(ctx, kin, vin, kout, vout, gr, vo, ts, fb_list, fb_count, nfb));
+  if (FUSED && nfb + n_over > 0) {
+    const unsigned grid = (unsigned)std::min<uint64_t>(nfb + n_over, 4ull * (uint64_t)std::max(1, ctx->num_sms));
+    DBG_LAUNCH(ctx, ST_LOCAL_SORT_NODES, 0.0,
+               k_tile_heads<K><<<grid, RANK_BLOCK, 0, ctx->stream>>>(kout, ts.bound.as<uint64_t>(),
+                                                                     (uint32_t)ts.tiles, fb_list, nfb, n_over, heads,
+                                                                     tcount));
+    DBG_CUDA_TRY(cudaGetLastError());
+  }
+  return DBG_OK;
+}
+
+// The local pass over records in the groups gr: the fully sorted records
+// (equal keys by payload, in the order vo) to kout / vout.
 template <class K>
 dbg_status seg_sort_records(dbg_ctx *ctx, const K *kin, const uint32_t *vin, K *kout, uint32_t *vout, uint64_t n,
-                            Groups &gr, ValOrder vo, int key_bits) {
+                            Groups &gr, ValOrder vo, TileSet &ts) {
   using Sh = SegShape<K>;
-  DevBuf bound, osize, ooff, gk, gv;
-  uint32_t G = 0;
-  DBG_TRY((seg_prepare<K, true>(ctx, kin, vin, n, gr, vo, key_bits, bound, osize, ooff, gk, gv, &G,
-                                ST_LOCAL_SORT_NODES)));
+  if (ctx->seg_rank)
+    return seg_rank_tiles<K, false>(ctx, kin, vin, kout, vout, n, gr, vo, ts, nullptr, nullptr);
   const int rank = local_rank_method(ctx, sizeof(K) == 16);
-  const uint64_t tiles = (n + Sh::TILE - 1) / Sh::TILE;
-  if (ctx->seg_rank) {
-    // ranking within buckets; tiles with a long bucket are listed and
-    // sorted by the digit passes
-    static_assert(SegRankSmem<K>::CAP == SEG_BLOCK * Sh::ITEMS, "same tile capacity as the digit-pass kernel");
-    set_smem_attrs(k_seg_rank<K>, sizeof(SegRankSmem<K>));
-    DevBuf fb;
-    DBG_TRY(alloc_buf(ctx, fb, (tiles + 1) * 4));
-    uint32_t *fb_count = fb.as<uint32_t>(), *fb_list = fb_count + 1;
-    DBG_CUDA_TRY(cudaMemsetAsync(fb_count, 0, 4, ctx->stream));
-    DBG_LAUNCH(ctx, ST_LOCAL_SORT_NODES, 2.0 * (double)n * (sizeof(K) + 4),
-               k_seg_rank<K><<<(unsigned)tiles, RANK_BLOCK, sizeof(SegRankSmem<K>), ctx->stream>>>(
-                   kin, vin, bound.as<uint64_t>(), osize.as<uint32_t>(), ooff.as<uint64_t>(), gk.as<K>(),
-                   gv.as<uint32_t>(), kout, vout, gr.lb, vo, fb_list, fb_count));
-    DBG_CUDA_TRY(cudaGetLastError());
-    uint32_t nfb = 0;
-    DBG_TRY(read_small(ctx, fb_count, sizeof(uint32_t), &nfb));
-    ctx->rank_fallback_tiles += nfb;
-    if (nfb == 0) return DBG_OK;
-    auto kern = rank == RANK_MATCH    ? k_seg_sort<K, Sh::ITEMS, RANK_MATCH>
-                : rank == RANK_ATOMIC ? k_seg_sort<K, Sh::ITEMS, RANK_ATOMIC>
-                                      : k_seg_sort<K, Sh::ITEMS, RANK_BALLOT>;
-    constexpr size_t smem = sizeof(SegSortSmem<K, true, Sh::ITEMS>);
-    set_smem_attrs(kern, smem);
-    const unsigned grid = (unsigned)std::min<uint64_t>(nfb, 2ull * (uint64_t)std::max(1, ctx->num_sms));
-    DBG_LAUNCH(ctx, ST_LOCAL_SORT_NODES, 0.0,
-               kern<<<grid, SEG_BLOCK, smem, ctx->stream>>>(
-                   kin, vin, bound.as<uint64_t>(), osize.as<uint32_t>(), ooff.as<uint64_t>(), gk.as<K>(),
-                   gv.as<uint32_t>(), kout, vout, gr.lb, vo, fb_list, fb_count));
-    DBG_CUDA_TRY(cudaGetLastError());
-    return DBG_OK;
-  }
+  const uint64_t tiles = ts.tiles;
+  const DevBuf &bound = ts.bound, &osize = ts.osize, &ooff = ts.ooff, &gk = ts.gk, &gv = ts.gv;
   const int v = ctx->sort_variant[sizeof(K) == 16 ? 5 : 4];
   if (v >= 3) {
     // the wide form: 384 threads x (2/3 of the items), the same capacity
@@ -709,10 +744,11 @@ dbg_status seg_rle(dbg_ctx *ctx, K *kin, K *kstage, uint64_t n, Groups &gr, int 
                    uint64_t *E) {
   using Sh = SegShape<K>;
   cudaStream_t s = ctx->stream;
-  DevBuf bound, osize, ooff, gk, gv, gheads, guniq;
-  uint32_t G = 0;
-  DBG_TRY((seg_prepare<K, false>(ctx, kin, nullptr, n, gr, ValOrder{}, key_bits, bound, osize, ooff, gk, gv, &G,
-                                 ST_LOCAL_SORT_EDGES)));
+  TileSet ts;
+  DBG_TRY((seg_prepare<K, false>(ctx, kin, nullptr, n, gr, ValOrder{}, key_bits, ts, ST_LOCAL_SORT_EDGES)));
+  DevBuf gheads, guniq;
+  const DevBuf &bound = ts.bound, &osize = ts.osize, &ooff = ts.ooff, &gk = ts.gk;
+  const uint32_t G = ts.gathered;
   uint64_t H = 0;
   if (G > 0) {
     DBG_TRY(alloc_buf(ctx, guniq, (uint64_t)G * sizeof(K)));
@@ -804,16 +840,14 @@ dbg_status sort_count_keys(dbg_ctx *ctx, K **kp, K **alt, uint64_t n, const Sort
   return DBG_OK;
 }
 
-// STEP-3's sort of R records by key, equal keys by payload << vshift, by
-// plan p.  The records come in payload order, which the least-significant-
-// first passes keep and the local pass restores after the MSD passes.
+// STEP-3's sort of R records by key, equal keys by payload, by plan p: the
+// global passes and the local pass's tiles (p.local()).  The records come in
+// payload order, which the least-significant-first passes keep and the local
+// pass restores after the MSD passes.
 template <class K>
-dbg_status sort_records(dbg_ctx *ctx, K **rk, K **rk_alt, uint32_t **rv, uint32_t **rv_alt, uint64_t R,
-                        const SortPlan<K> &p, int vshift, unsigned long long *d_hist, uint64_t *d_digit_base) {
-  if (!p.local() || R <= 1) return radix_sort<K, true>(ctx, rk, rk_alt, rv, rv_alt, R, p.bits, d_hist, d_digit_base);
-  Groups gr;
-  ValOrder vo;
-  vo.shift = vshift;
+dbg_status sort_records_global(dbg_ctx *ctx, K **rk, K **rk_alt, uint32_t **rv, uint32_t **rv_alt, uint64_t R,
+                               const SortPlan<K> &p, ValOrder &vo, unsigned long long *d_hist,
+                               uint64_t *d_digit_base, Groups &gr, TileSet &ts) {
   if (p.msd) {
     DBG_TRY((msd_sort<K, true>(ctx, rk, rk_alt, rv, rv_alt, R, p, d_hist, gr)));
     vo.sort = p.passes > 0;
@@ -821,10 +855,42 @@ dbg_status sort_records(dbg_ctx *ctx, K **rk, K **rk_alt, uint32_t **rv, uint32_
     DBG_TRY((radix_sort<K, true>(ctx, rk, rk_alt, rv, rv_alt, R, p.bits, d_hist, d_digit_base, p.first_pass, p.adj)));
     gr.lb.fixed = RADIX_BITS * p.first_pass - p.adj;
   }
-  DBG_TRY(seg_sort_records<K>(ctx, *rk, *rv, *rk_alt, *rv_alt, R, gr, vo, p.bits));
+  return seg_prepare<K, true>(ctx, *rk, *rv, R, gr, vo, p.bits, ts, ST_LOCAL_SORT_NODES);
+}
+
+// The whole sort, the sorted records in *rk / *rv.
+template <class K>
+dbg_status sort_records(dbg_ctx *ctx, K **rk, K **rk_alt, uint32_t **rv, uint32_t **rv_alt, uint64_t R,
+                        const SortPlan<K> &p, ValOrder vo, unsigned long long *d_hist, uint64_t *d_digit_base) {
+  if (!p.local() || R <= 1) return radix_sort<K, true>(ctx, rk, rk_alt, rv, rv_alt, R, p.bits, d_hist, d_digit_base);
+  Groups gr;
+  TileSet ts;
+  DBG_TRY(sort_records_global<K>(ctx, rk, rk_alt, rv, rv_alt, R, p, vo, d_hist, d_digit_base, gr, ts));
+  DBG_TRY(seg_sort_records<K>(ctx, *rk, *rv, *rk_alt, *rv_alt, R, gr, vo, ts));
   std::swap(*rk, *rk_alt);
   std::swap(*rv, *rv_alt);
   return DBG_OK;
+}
+
+// The payload order of node records: (e << 1 | role) of `edges` edges, the
+// side bits on top or not, with or without reads of exactly k bases; or of
+// read numbers below `reads`.
+inline int bit_length(uint64_t x) {
+  int b = 0;
+  while (x >> b) b++;
+  return b;
+}
+inline ValOrder edge_end_order(uint64_t edges, bool sides, bool isolated) {
+  ValOrder vo;
+  vo.shift = sides ? 2 : 0;
+  vo.pb = std::max(1, std::min(31, bit_length(edges)));
+  vo.dups = isolated;
+  return vo;
+}
+inline ValOrder read_order(uint64_t reads) {
+  ValOrder vo;
+  vo.pb = std::max(1, std::min(31, bit_length(reads / 2 + 1)));
+  return vo;
 }
 
 // The plan of a record sort.  Least significant first, with records ranked
@@ -905,6 +971,58 @@ dbg_status assign_node_ids(dbg_ctx *ctx, const K *rk, const uint32_t *rv, uint64
   DBG_CUDA_TRY(cudaGetLastError());
   *V = nv;
   *ends = ne;
+  return DBG_OK;
+}
+
+// The local pass over R node records in the groups gr, fused with the node-ID
+// pass: the graph's node keys, row_ptr, adjacency and edge ends.  Returns
+// |V| and the number of edge ends.  make_room allocates the adjacency.
+template <class K, class Room>
+dbg_status rank_and_assign(dbg_ctx *ctx, const K *rk, const uint32_t *rv, K *ukeys, uint32_t *vals, uint64_t R,
+                           uint64_t E, uint64_t I, Groups &gr, ValOrder vo, TileSet &ts, Room make_room, dbg_graph *g,
+                           uint64_t *V, uint64_t *ends) {
+  cudaStream_t s = ctx->stream;
+  const uint64_t tiles = ts.tiles;
+  DevBuf heads, tcount, hoff, ecount, eoff;
+  DBG_TRY(alloc_buf(ctx, heads, (R / 32 + tiles + 2) * 4));
+  DBG_TRY(alloc_buf(ctx, tcount, tiles * 4));
+  DBG_TRY(alloc_buf(ctx, hoff, (tiles + 1) * 8));
+  DBG_TRY((seg_rank_tiles<K, true>(ctx, rk, rv, ukeys, vals, R, gr, vo, ts, heads.as<uint32_t>(),
+                                   tcount.as<uint32_t>())));
+  uint32_t nv = 0, ne = (uint32_t)R;
+  if (I > 0) {
+    DBG_TRY(alloc_buf(ctx, ecount, tiles * 4));
+    DBG_TRY(alloc_buf(ctx, eoff, (tiles + 1) * 8));
+    DBG_LAUNCH(ctx, ST_NODE_IDS, 4.0 * R,
+               k_tile_ends<<<(unsigned)std::min<uint64_t>(tiles, 152ull * 16), 256, 0, s>>>(
+                   ts.bound.as<uint64_t>(), (uint32_t)tiles, vals, ecount.as<uint32_t>()));
+    DBG_TRY(scan_u32(ctx, ecount.as<uint32_t>(), tiles, eoff.as<uint64_t>(), &ne, ST_NODE_IDS));
+  }
+  DBG_TRY(scan_u32(ctx, tcount.as<uint32_t>(), tiles, hoff.as<uint64_t>(), &nv, ST_NODE_IDS));
+  *V = nv;
+  *ends = ne;
+  if (ne != 2 * E) return DBG_OK;  // (the caller reports it)
+  DBG_TRY(make_room());
+  DBG_TRY(alloc_buf(ctx, g->node_keys, std::max<uint64_t>(1, nv) * sizeof(K)));
+  DBG_TRY(alloc_buf(ctx, g->row_ptr, ((uint64_t)nv + 1) * sizeof(uint64_t)));
+  int bshift = 10;
+  while ((E + (1ull << bshift) - 1) >> bshift > 256) bshift++;
+  DevBuf part, fill;
+  DBG_TRY(alloc_buf(ctx, part, 2 * E * 8));
+  DBG_TRY(alloc_buf(ctx, fill, 256 * 4));
+  DBG_CUDA_TRY(cudaMemsetAsync(fill.p, 0, 256 * 4, s));
+  auto kern = I > 0 ? k_node_tiles<K, true> : k_node_tiles<K, false>;
+  DBG_LAUNCH(ctx, ST_NODE_IDS,
+             4.0 * R + R / 8.0 + (double)nv * (2 * sizeof(K) + 8) + (double)ne * (g->adj_side.p ? 14 : 13),
+             kern<<<(unsigned)std::min<uint64_t>(tiles, 3ull * (uint64_t)std::max(1, ctx->num_sms)), RANK_BLOCK, 0, s>>>(
+                 ts.bound.as<uint64_t>(), (uint32_t)tiles, ukeys, vals, heads.as<uint32_t>(), tcount.as<uint32_t>(),
+                 hoff.as<uint64_t>(), eoff.as<uint64_t>(), g->node_keys.as<K>(), g->row_ptr.as<uint64_t>(),
+                 g->adj_edge.as<uint32_t>(), g->adj_role.as<uint8_t>(), g->adj_side.as<uint8_t>(),
+                 part.as<uint64_t>(), fill.as<uint32_t>(), bshift));
+  DBG_LAUNCH(ctx, ST_NODE_IDS, 2.0 * E * (8 + 4),
+             k_scatter_ends<<<grid_for(2 * E, 256 * 16), 256, 0, s>>>(part.as<uint64_t>(), 2 * E,
+                                                                      g->src.as<uint32_t>(), g->dst.as<uint32_t>()));
+  DBG_CUDA_TRY(cudaGetLastError());
   return DBG_OK;
 }
 
@@ -1014,7 +1132,7 @@ dbg_status count_node_reads(dbg_ctx *ctx, const DevBuf &packed, const DevBuf &ba
   koff.release();
   K *kp = ka.as<K>(), *kalt = kb.as<K>();
   uint32_t *vp = va.as<uint32_t>(), *valt = vb.as<uint32_t>();
-  DBG_TRY(sort_records<K>(ctx, &kp, &kalt, &vp, &valt, M, plan, 0, d_hist, d_digit_base));
+  DBG_TRY(sort_records<K>(ctx, &kp, &kalt, &vp, &valt, M, plan, read_order(n), d_hist, d_digit_base));
   // flags into the free payload buffer, their scan, the key runs
   DBG_LAUNCH(ctx, ST_NODE_MULT, (double)M * (2 * sizeof(K) + 12),
              k_read_change_flags<K><<<grid_for(M, 256 * 8), 256, 0, s>>>(kp, vp, M, valt));
@@ -1224,22 +1342,54 @@ dbg_status build_graph_impl(dbg_ctx *ctx, const BuildInput &in, dbg_graph *g) {
   base_off.release();
   edge_off.release();
 
-  // ---- STEP-3 sort of the node records (stable: payload order kept) ----
+  // ---- STEP-3 sort of the node records (payload order kept), K6 node IDs +
+  // adjacency rows, K7 neighbours ----
   K *rk = rk_a.as<K>(), *rk_alt = rk_b.as<K>();
   uint32_t *rv = rv_a.as<uint32_t>(), *rv_alt = rv_b.as<uint32_t>();
-  DBG_TRY(sort_records<K>(ctx, &rk, &rk_alt, &rv, &rv_alt, R, rplan, sides ? 2 : 0, d_hist, d_digit_base));
-
-  // ---- K6 node IDs + adjacency rows, K7 neighbours ----
+  const ValOrder vo = edge_end_order(E, sides, I > 0);
   DevBuf row_tmp;
-  DBG_TRY(alloc_buf(ctx, row_tmp, (R + 1) * sizeof(uint64_t)));
-  DBG_TRY(alloc_buf(ctx, g->src, std::max<uint64_t>(1, E) * sizeof(uint32_t)));
-  DBG_TRY(alloc_buf(ctx, g->dst, std::max<uint64_t>(1, E) * sizeof(uint32_t)));
-  DBG_TRY(alloc_buf(ctx, g->adj_edge, std::max<uint64_t>(1, 2 * E) * sizeof(uint32_t)));
-  DBG_TRY(alloc_buf(ctx, g->adj_role, std::max<uint64_t>(1, 2 * E)));
-  DBG_TRY(alloc_buf(ctx, g->adj_nbr, std::max<uint64_t>(1, 2 * E) * sizeof(uint32_t)));
-  if (sides) DBG_TRY(alloc_buf(ctx, g->adj_side, 2 * E));
+  auto alloc_adjacency = [&]() -> dbg_status {
+    DBG_TRY(alloc_buf(ctx, g->src, std::max<uint64_t>(1, E) * sizeof(uint32_t)));
+    DBG_TRY(alloc_buf(ctx, g->dst, std::max<uint64_t>(1, E) * sizeof(uint32_t)));
+    DBG_TRY(alloc_buf(ctx, g->adj_edge, std::max<uint64_t>(1, 2 * E) * sizeof(uint32_t)));
+    DBG_TRY(alloc_buf(ctx, g->adj_role, std::max<uint64_t>(1, 2 * E)));
+    DBG_TRY(alloc_buf(ctx, g->adj_nbr, std::max<uint64_t>(1, 2 * E) * sizeof(uint32_t)));
+    if (sides) DBG_TRY(alloc_buf(ctx, g->adj_side, 2 * E));
+    return DBG_OK;
+  };
   uint64_t V = 0;
-  if (R > 0) {
+  // The local pass hands the node-ID pass the tiles' distinct keys and head
+  // bits instead of sorted keys -- unless many records are in oversize tiles,
+  // which one CTA each would go through (a million records: about 0.3 ms).
+  bool fused = false;
+  if (E > 0 && rplan.local() && ctx->seg_rank) {
+    Groups gr;
+    TileSet ts;
+    ValOrder fvo = vo;
+    DBG_TRY(sort_records_global<K>(ctx, &rk, &rk_alt, &rv, &rv_alt, R, rplan, fvo, d_hist, d_digit_base, gr, ts));
+    fused = ts.gathered <= 1u << 20;
+    if (fused) {
+      uint64_t ends = 0;
+      DBG_TRY(rank_and_assign<K>(ctx, rk, rv, rk_alt, rv_alt, R, E, I, gr, fvo, ts, alloc_adjacency, g, &V, &ends));
+      DBG_TRY(check_device_error(ctx));
+      if (ends != 2 * E) {
+        set_error("adjacency holds %llu edge ends, expected %llu", (unsigned long long)ends,
+                  (unsigned long long)(2 * E));
+        return DBG_EINTERNAL;
+      }
+    } else {
+      DBG_TRY(seg_sort_records<K>(ctx, rk, rv, rk_alt, rv_alt, R, gr, fvo, ts));
+      std::swap(rk, rk_alt);
+      std::swap(rv, rv_alt);
+    }
+  } else {
+    DBG_TRY(sort_records<K>(ctx, &rk, &rk_alt, &rv, &rv_alt, R, rplan, vo, d_hist, d_digit_base));
+  }
+  if (!fused) {
+    DBG_TRY(alloc_buf(ctx, row_tmp, (R + 1) * sizeof(uint64_t)));
+    DBG_TRY(alloc_adjacency());
+  }
+  if (R > 0 && !fused) {
     // node keys go to the free record buffer first (|V| is known only after)
     uint64_t ends = 0;
     DBG_TRY(assign_node_ids<K>(ctx, rk, rv, R, rk_alt, row_tmp.as<uint64_t>(), g, 0u, 0ull, &V, &ends, E,
@@ -1270,9 +1420,13 @@ dbg_status build_graph_impl(dbg_ctx *ctx, const BuildInput &in, dbg_graph *g) {
     if (V == 0) DBG_TRY(alloc_buf(ctx, read_counts, sizeof(uint32_t)));
     g->node_reads = std::move(read_counts);
   }
-  DBG_TRY(alloc_buf(ctx, g->node_keys, std::max<uint64_t>(1, V) * sizeof(K)));
-  DBG_TRY(alloc_buf(ctx, g->row_ptr, (V + 1) * sizeof(uint64_t)));
-  if (V > 0) {
+  if (!fused) {
+    DBG_TRY(alloc_buf(ctx, g->node_keys, std::max<uint64_t>(1, V) * sizeof(K)));
+    DBG_TRY(alloc_buf(ctx, g->row_ptr, (V + 1) * sizeof(uint64_t)));
+  }
+  if (fused) {
+    // written in place
+  } else if (V > 0) {
     Span sp(ctx, ST_COPIES, 2.0 * V * (sizeof(K) + 8), 0);
     DBG_CUDA_TRY(cudaMemcpyAsync(g->node_keys.p, rk_alt, V * sizeof(K), cudaMemcpyDeviceToDevice, s));
     DBG_CUDA_TRY(cudaMemcpyAsync(g->row_ptr.p, row_tmp.p, (V + 1) * sizeof(uint64_t), cudaMemcpyDeviceToDevice, s));
@@ -1674,7 +1828,8 @@ dbg_status build_bucketed_impl(dbg_ctx *ctx, const BucketInput &in, uint64_t bud
     if (R == 0) continue;
     K *rk = ra.as<K>(), *rk_alt = rb.as<K>();
     uint32_t *rv = va.as<uint32_t>(), *rv_alt = vb.as<uint32_t>();
-    DBG_TRY(sort_records<K>(ctx, &rk, &rk_alt, &rv, &rv_alt, R, rplan, 0, d_hist, d_digit_base));
+    DBG_TRY(sort_records<K>(ctx, &rk, &rk_alt, &rv, &rv_alt, R, rplan, edge_end_order(E, false, I > 0), d_hist,
+                            d_digit_base));
     DBG_TRY(alloc_buf(ctx, row_tmp, (R + 1) * 8));
     uint64_t tot[2] = {0, 0};
     DBG_TRY(assign_node_ids<K>(ctx, rk, rv, R, rk_alt, row_tmp.as<uint64_t>(), g, (uint32_t)base_v, base_slot,

@@ -65,9 +65,13 @@ struct LowBits {
 // shift drops the side bits that a node record's payload carries on top).
 // sort: they come in no particular order and payload digits take part in the
 // digit passes; otherwise they come in that order and stable passes keep it.
+// pb: enough bits for every (payload << shift >> shift) >> 1 of a record that
+// is an edge end, with all ones left for REC_NONE.  dups: records may be equal.
 struct ValOrder {
   int shift = 0;
   int sort = 0;
+  int pb = 32;
+  int dups = 1;
 };
 
 // bound[t] for t in [0, tiles]: the first index of the group holding
@@ -376,7 +380,8 @@ __global__ __launch_bounds__(BLOCK, 2) void k_seg_sort(
 }
 
 // Records by ranking within small buckets.  The tile's records are spread
-// over 4096 buckets by the top bits of their key offsets (a counting sort in
+// over 8192 buckets (4096 for 128-bit keys, whose tiles are half as long) by
+// the top bits of their key offsets (a counting sort in
 // shared memory: one atomic add per record, a scan, one scatter), and a
 // record's place in the sorted tile is its bucket's start plus the number of
 // the bucket's records that precede it: those with a smaller key, or an
@@ -385,78 +390,111 @@ __global__ __launch_bounds__(BLOCK, 2) void k_seg_sort(
 // need no particular order on arrival.  A tile with a bucket longer than
 // RANK_GROUP_MAX is listed in fb_list for the digit-pass kernel instead.
 //
-// Bound by shared-memory traffic (about 20 bytes written and 60 read per
-// 12-byte record); two CTAs of 512 threads per SM.
+// Bound by instruction issue.  Where a record's bits below its bucket's and
+// its payload's upper bits fit 64 bits (vo.pb of them; nearly every tile of
+// 64-bit keys), they form one word that a single comparison orders; the
+// bucket, the payload's lowest bit (an edge end's role: the tie-break where it
+// has no room in the word) and its side bits are in 16 bits beside it.  Two CTAs of 512 threads per SM.
+//
+// FUSED (STEP-3's node records): instead of the sorted keys, the tile's
+// distinct keys go to the front of its own range of kout, with their number
+// in tcount, and a bit per record that starts a node to `heads` -- record j
+// of tile t at bit j % 32 of word (first record of t) / 32 + t + j / 32.
 constexpr int RANK_BLOCK = 512;
 constexpr uint32_t RANK_GROUP_MAX = 512;
+
+__device__ __forceinline__ uint32_t *head_words(uint32_t *heads, uint64_t first, uint32_t tile) {
+  return heads + (first >> 5) + tile;
+}
 
 template <class K>
 struct SegRankSmem {
   static constexpr int CAP = SEG_BLOCK * (sizeof(K) == 8 ? 24 : 12);  // the digit-pass kernel's capacity
   static constexpr int ITEMS = CAP / RANK_BLOCK;
-  static constexpr int TBITS = 12, NB = 1 << TBITS, PER = NB / RANK_BLOCK;
-  K key[CAP];             // offsets from base, by bucket
-  uint32_t val[CAP];
-  uint32_t start[NB + 1];  // records per bucket, then its first position
+  static constexpr int TBITS = sizeof(K) == 8 ? 13 : 12, NB = 1 << TBITS, PER = NB / 2 / RANK_BLOCK;
+  union {
+    struct {
+      K key[CAP];  // offsets from base
+      uint32_t val[CAP];
+    } g;
+    struct {
+      uint64_t word[CAP];
+      uint16_t ord[CAP];
+    } n;
+  };
+  uint32_t start2[NB / 2 + 1];  // 16 bits per bucket: its records, then its first position
   uint32_t wsum[RANK_BLOCK / 32];
+  uint32_t cnt[ITEMS * (RANK_BLOCK / 32) + 1];
   uint64_t bound[2];
   K base, range;
   uint32_t passes, span_bits, maxg;
 };
 
-template <class K>
+template <class K, bool FUSED>
 __global__ __launch_bounds__(RANK_BLOCK, 2) void k_seg_rank(
     const K *__restrict__ kin, const uint32_t *__restrict__ vin, const uint64_t *__restrict__ bound,
     const uint32_t *__restrict__ osize, const uint64_t *__restrict__ ooff, const K *__restrict__ gk,
     const uint32_t *__restrict__ gv, K *__restrict__ kout, uint32_t *__restrict__ vout, LowBits lb, ValOrder vo,
-    uint32_t *__restrict__ fb_list, uint32_t *__restrict__ fb_count) {
+    uint32_t *__restrict__ fb_list, uint32_t *__restrict__ fb_count, uint32_t *__restrict__ heads,
+    uint32_t *__restrict__ tcount) {
   using S = SegRankSmem<K>;
   constexpr int ITEMS = S::ITEMS, PER = S::PER;
   extern __shared__ __align__(128) unsigned char smem_raw[];
   S &sm = *reinterpret_cast<S *>(smem_raw);
+  uint16_t *const start = reinterpret_cast<uint16_t *>(sm.start2);
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
   const uint32_t tile = blockIdx.x;
+  const uint64_t s = bound[tile];
   if (osize[tile]) {
-    const uint64_t s = bound[tile], o = ooff[tile];
+    const uint64_t o = ooff[tile];
     for (uint32_t j = tid; j < osize[tile]; j += RANK_BLOCK) {
       kout[s + j] = gk[o + j];
       vout[s + j] = gv[o + j];
     }
+    if (FUSED && tid == 0) fb_list[gridDim.x - 1 - atomicAdd(fb_count + 1, 1u)] = tile;
     return;
   }
-  const uint64_t s = bound[tile];
   const uint32_t cnt = (uint32_t)(bound[tile + 1] - s);
-  if (cnt == 0) return;
+  if (cnt == 0) {
+    if (FUSED && tid == 0) tcount[tile] = 0;
+    return;
+  }
+  const int items = (int)((cnt + RANK_BLOCK - 1) / RANK_BLOCK);  // of each thread
   K key[ITEMS];
-  uint32_t val[ITEMS], at[ITEMS];
+  uint32_t val[ITEMS], oa[ITEMS];  // bucket, place on arrival << 13
 #pragma unroll
   for (int i = 0; i < ITEMS; i++) {
+    if (i >= items) break;
     const uint32_t j = (uint32_t)i * RANK_BLOCK + tid;
     if (j < cnt) {
       key[i] = kin[s + j];
       val[i] = vin[s + j];
     }
   }
-  for (int j = tid; j < S::NB; j += RANK_BLOCK) sm.start[j] = 0;
+  for (int j = tid; j <= S::NB / 2; j += RANK_BLOCK) sm.start2[j] = 0;
   if (tid == 0) sm.maxg = 0;
   seg_setup<K>(sm, kin, bound, tile, lb);  // synchronises
   const K base = sm.base;
   const int bshift = (int)sm.span_bits > S::TBITS ? (int)sm.span_bits - S::TBITS : 0;
-  auto bucket = [&](const K &d) { return (uint32_t)KeyOps<K>::words_lo(KeyOps<K>::shr(d, bshift)); };
+  const bool narrow = sizeof(K) == 8 && bshift + vo.pb <= 64;
 #pragma unroll
-  for (int i = 0; i < ITEMS; i++)
+  for (int i = 0; i < ITEMS; i++) {
+    if (i >= items) break;
     if ((uint32_t)i * RANK_BLOCK + tid < cnt) {
       key[i] = KeyOps<K>::sub(key[i], base);
-      at[i] = atomicAdd(&sm.start[bucket(key[i])], 1u);
+      const uint32_t o = (uint32_t)KeyOps<K>::words_lo(KeyOps<K>::shr(key[i], bshift)), h = 16 * (o & 1u);
+      oa[i] = o | ((atomicAdd(&sm.start2[o >> 1], 1u << h) >> h) & 0xffffu) << S::TBITS;
     }
+  }
   __syncthreads();
-  // exclusive scan, PER consecutive buckets per thread
+  // exclusive scan, 2 PER consecutive buckets per thread
   uint32_t c[PER], sum = 0, mx = 0;
 #pragma unroll
   for (int j = 0; j < PER; j++) {
-    c[j] = sm.start[tid * PER + j];
-    sum += c[j];
-    mx = max(mx, c[j]);
+    c[j] = sm.start2[tid * PER + j];
+    const uint32_t c0 = c[j] & 0xffffu, c1 = c[j] >> 16;
+    sum += c0 + c1;
+    mx = max(mx, max(c0, c1));
   }
   const uint32_t incl = warp_incl_scan(sum);
   if (lane == 31) sm.wsum[warp] = incl;
@@ -471,34 +509,341 @@ __global__ __launch_bounds__(RANK_BLOCK, 2) void k_seg_rank(
   for (int w = 0; w < warp; w++) run += sm.wsum[w];
 #pragma unroll
   for (int j = 0; j < PER; j++) {
-    sm.start[tid * PER + j] = run;
-    run += c[j];
+    const uint32_t c0 = c[j] & 0xffffu, c1 = c[j] >> 16;
+    sm.start2[tid * PER + j] = run | (run + c0) << 16;
+    run += c0 + c1;
   }
-  if (tid == RANK_BLOCK - 1) sm.start[S::NB] = run;
+  if (tid == RANK_BLOCK - 1) sm.start2[S::NB / 2] = run;
+  __syncthreads();
+  // the output, from the sorted tile in shared memory
+  auto write_out = [&](auto key_at, auto val_at, auto is_head) {
+    if (FUSED) {
+      unsigned hb[ITEMS];
+#pragma unroll
+      for (int i = 0; i < ITEMS; i++) {
+        if (i >= items) break;
+        const uint32_t j = (uint32_t)i * RANK_BLOCK + tid;
+        hb[i] = __ballot_sync(0xffffffffu, j < cnt && is_head(j));
+        if (lane == 0) {
+          sm.cnt[i * (RANK_BLOCK / 32) + warp] = __popc(hb[i]);
+          if (j < cnt) head_words(heads, s, tile)[j >> 5] = hb[i];
+        }
+      }
+      __syncthreads();
+      // heads before each warp's 32 records: scanned by one warp
+      if (warp == 0) {
+        constexpr int NW = ITEMS * (RANK_BLOCK / 32), EACH = (NW + 31) / 32;
+        const int nw = items * (RANK_BLOCK / 32);
+        uint32_t x[EACH], sum = 0;
+#pragma unroll
+        for (int j = 0; j < EACH; j++) {
+          x[j] = lane * EACH + j < nw ? sm.cnt[lane * EACH + j] : 0u;
+          sum += x[j];
+        }
+        const uint32_t incl = warp_incl_scan(sum);
+        uint32_t run = incl - sum;
+#pragma unroll
+        for (int j = 0; j < EACH; j++) {
+          if (lane * EACH + j < nw) sm.cnt[lane * EACH + j] = run;
+          run += x[j];
+        }
+        if (lane == 31) tcount[tile] = incl;
+      }
+      __syncthreads();
+#pragma unroll
+      for (int i = 0; i < ITEMS; i++) {
+        if (i >= items) break;
+        const uint32_t j = (uint32_t)i * RANK_BLOCK + tid;
+        if (j < cnt) vout[s + j] = val_at(j);
+        if (hb[i] >> lane & 1u)
+          kout[s + sm.cnt[i * (RANK_BLOCK / 32) + warp] + __popc(hb[i] & ((1u << lane) - 1u))] = key_at(j);
+      }
+    } else {
+      for (uint32_t j = tid; j < cnt; j += RANK_BLOCK) {
+        kout[s + j] = key_at(j);
+        vout[s + j] = val_at(j);
+      }
+    }
+  };
+  if constexpr (sizeof(K) == 8) {
+    if (narrow) {
+      // word: the bits below the bucket's at the top, the payload's upper pb
+      // bits -- and its lowest, where there is room -- at the bottom
+      const int up = 64 - bshift;                      // (64: no bit below the bucket's)
+      const int role = up > vo.pb ? 1 : 0;
+      const int pbits = vo.pb + role;
+      const uint32_t pmask = pbits >= 32 ? 0xffffffffu : (1u << pbits) - 1u, obits = S::NB - 1;
+#pragma unroll
+      for (int i = 0; i < ITEMS; i++) {
+        if (i >= items) break;
+        if ((uint32_t)i * RANK_BLOCK + tid < cnt) {
+          const uint32_t o = oa[i] & obits, q = start[o] + (oa[i] >> S::TBITS);
+          const uint32_t p = val[i] << vo.shift >> vo.shift;
+          const uint64_t low = bshift ? key[i] << up : 0ull;
+          sm.n.word[q] = low | min(p >> (1 - role), pmask);  // (no edge: all ones, last)
+          sm.n.ord[q] = (uint16_t)(o | (p & 1u) << 13 | (vo.shift ? val[i] >> 30 : 0u) << 14);
+        }
+      }
+      __syncthreads();
+      const bool ties = vo.dups || !role;
+      uint64_t wd[ITEMS];
+      uint32_t po[ITEMS];
+#pragma unroll
+      for (int i = 0; i < ITEMS; i++) {
+        if (i >= items) break;
+        const uint32_t q = (uint32_t)i * RANK_BLOCK + tid;
+        if (q < cnt) {
+          const uint64_t d = sm.n.word[q];
+          const uint32_t od = sm.n.ord[q], o = od & obits, a = start[o], b = start[o + 1];
+          uint32_t r = a;
+          if (!ties) {
+#pragma unroll 2
+            for (uint32_t t = a; t < b; t++) r += sm.n.word[t] < d ? 1u : 0u;
+          } else {
+            for (uint32_t t = a; t < b; t++) {
+              const uint64_t y = sm.n.word[t];
+              r += y < d ? 1u : 0u;
+              if (y == d && t != q) {  // one edge's two ends at a node, or equal records
+                const uint32_t bt = sm.n.ord[t] >> 13 & 1u, bq = od >> 13 & 1u;
+                r += bt < bq || (bt == bq && t < q) ? 1u : 0u;
+              }
+            }
+          }
+          wd[i] = d;
+          po[i] = od | r << 16;
+        }
+      }
+      __syncthreads();
+#pragma unroll
+      for (int i = 0; i < ITEMS; i++) {
+        if (i >= items) break;
+        if ((uint32_t)i * RANK_BLOCK + tid < cnt) {
+          sm.n.word[po[i] >> 16] = wd[i];
+          sm.n.ord[po[i] >> 16] = (uint16_t)po[i];
+        }
+      }
+      __syncthreads();
+      write_out(
+          [&](uint32_t j) {
+            return base + ((uint64_t)(sm.n.ord[j] & obits) << bshift | (bshift ? sm.n.word[j] >> up : 0ull));
+          },
+          [&](uint32_t j) {
+            const uint32_t e = (uint32_t)sm.n.word[j] & pmask, od = sm.n.ord[j];
+            const uint32_t v = (role ? e : e << 1 | (od >> 13 & 1u)) | (vo.shift ? (od >> 14) << 30 : 0u);
+            return e == pmask ? REC_NONE : v;
+          },
+          [&](uint32_t j) {
+            if (j == 0) return true;
+            const uint64_t x = sm.n.word[j] ^ sm.n.word[j - 1];
+            return ((uint32_t)(x >> 32) | ((uint32_t)x & ~pmask) |
+                    ((uint32_t)(sm.n.ord[j] ^ sm.n.ord[j - 1]) & obits)) != 0;
+          });
+      return;
+    }
+  }
+#pragma unroll
+  for (int i = 0; i < ITEMS; i++)
+    if ((uint32_t)i * RANK_BLOCK + tid < cnt) {
+      const uint32_t q = start[oa[i] & (S::NB - 1)] + (oa[i] >> S::TBITS);
+      sm.g.key[q] = key[i];
+      sm.g.val[q] = val[i];
+    }
+  __syncthreads();
+#pragma unroll
+  for (int i = 0; i < ITEMS; i++) {
+    const uint32_t q = (uint32_t)i * RANK_BLOCK + tid;
+    if (q < cnt) {
+      const K d = sm.g.key[q];
+      const uint32_t v = sm.g.val[q], o = (uint32_t)KeyOps<K>::words_lo(KeyOps<K>::shr(d, bshift));
+      const uint32_t a = start[o], b = start[o + 1];
+      uint32_t r = a;
+      for (uint32_t t = a; t < b; t++) {
+        const K y = sm.g.key[t];
+        bool before = KeyOps<K>::less(y, d);
+        if (KeyOps<K>::eq(y, d)) {
+          const uint32_t w = sm.g.val[t] << vo.shift, mine = v << vo.shift;
+          before = w < mine || (w == mine && t < q);
+        }
+        r += before ? 1u : 0u;
+      }
+      key[i] = d;
+      val[i] = v;
+      oa[i] = r;
+    }
+  }
   __syncthreads();
 #pragma unroll
   for (int i = 0; i < ITEMS; i++)
     if ((uint32_t)i * RANK_BLOCK + tid < cnt) {
-      const uint32_t q = sm.start[bucket(key[i])] + at[i];
-      sm.key[q] = key[i];
-      sm.val[q] = val[i];
+      sm.g.key[oa[i]] = key[i];
+      sm.g.val[oa[i]] = val[i];
     }
   __syncthreads();
-  for (uint32_t q = tid; q < cnt; q += RANK_BLOCK) {
-    const K d = sm.key[q];
-    const uint32_t v = sm.val[q], o = bucket(d), a = sm.start[o], b = sm.start[o + 1];
-    uint32_t r = 0;
-    for (uint32_t t = a; t < b; t++) {
-      const K y = sm.key[t];
-      bool before = KeyOps<K>::less(y, d);
-      if (KeyOps<K>::eq(y, d)) {
-        const uint32_t w = sm.val[t] << vo.shift, mine = v << vo.shift;
-        before = w < mine || (w == mine && t < q);
+  write_out([&](uint32_t j) { return KeyOps<K>::add(sm.g.key[j], base); }, [&](uint32_t j) { return sm.g.val[j]; },
+            [&](uint32_t j) { return j == 0 || !KeyOps<K>::eq(sm.g.key[j], sm.g.key[j - 1]); });
+}
+
+// FUSED's outputs for tiles that other kernels sorted into keys / vals (the
+// first n_fb of fb_list, and the oversize ones: the last n_over): the heads, their number,
+// and the distinct keys moved to the front of the tile.  One CTA per tile at a
+// time; a chunk's keys are all in registers before its distinct ones, which
+// lie at or before them, are written.
+template <class K>
+__global__ __launch_bounds__(RANK_BLOCK) void k_tile_heads(K *__restrict__ keys, const uint64_t *__restrict__ bound,
+                                                           uint32_t tiles, const uint32_t *__restrict__ fb_list,
+                                                           uint32_t n_fb, uint32_t n_over,
+                                                           uint32_t *__restrict__ heads,
+                                                           uint32_t *__restrict__ tcount) {
+  constexpr int ITEMS = 8;
+  constexpr uint32_t CHUNK = RANK_BLOCK * ITEMS;
+  __shared__ uint32_t s_cnt[ITEMS * (RANK_BLOCK / 32) + 1];
+  __shared__ K s_last;
+  const int tid = threadIdx.x, lane = tid & 31;
+  for (uint32_t q = blockIdx.x; q < n_fb + n_over; q += gridDim.x) {
+    const uint32_t tile = fb_list[q < n_fb ? q : tiles - 1 - (q - n_fb)];
+    const uint64_t s = bound[tile], n = bound[tile + 1] - s;
+    uint32_t *hw = head_words(heads, s, tile);
+    uint64_t out = 0;
+    for (uint64_t c = 0; c < n; c += CHUNK) {
+      K k[ITEMS];
+      bool head[ITEMS];
+      uint32_t rk[ITEMS];
+#pragma unroll
+      for (int i = 0; i < ITEMS; i++) {
+        const uint64_t j = c + (uint64_t)i * RANK_BLOCK + tid;
+        head[i] = false;
+        if (j < n) {
+          k[i] = keys[s + j];
+          head[i] = j == 0 || !KeyOps<K>::eq(k[i], j == c ? s_last : keys[s + j - 1]);
+        }
+        const unsigned b = __ballot_sync(0xffffffffu, head[i]);
+        if (lane == 0 && j < n) hw[j >> 5] = b;
       }
-      r += before ? 1u : 0u;
+      const uint32_t count = tile_flag_ranks<RANK_BLOCK, ITEMS>(head, rk, s_cnt);  // synchronises
+      if (c + CHUNK - 1 < n && tid == RANK_BLOCK - 1) s_last = k[ITEMS - 1];
+#pragma unroll
+      for (int i = 0; i < ITEMS; i++)
+        if (head[i]) keys[s + out + rk[i]] = k[i];
+      out += count;
+      __syncthreads();
     }
-    kout[s + a + r] = KeyOps<K>::add(d, base);
-    vout[s + a + r] = v;
+    if (tid == 0) tcount[tile] = (uint32_t)out;
+  }
+}
+
+// STEP-3 / STEP-4 from FUSED's outputs: tile t's records, hoff[t] the ID of
+// its first node, (ISO) eoff[t] the adjacency slot of its first edge end --
+// without reads of exactly k bases every record is an edge end, and a record's
+// slot is its own index.  Writes the tile's node keys and row starts, the
+// adjacency entries, and the edge ends partitioned by edge range (see
+// k_write_nodes).  Reads 4 bytes and a bit per record and 8 or 16 per node.
+template <class K, bool ISO>
+__global__ __launch_bounds__(RANK_BLOCK, ISO ? 2 : 3) void k_node_tiles(
+    const uint64_t *__restrict__ bound, uint32_t tiles, const K *__restrict__ ukeys, const uint32_t *__restrict__ vals,
+    const uint32_t *__restrict__ heads, const uint32_t *__restrict__ tcount, const uint64_t *__restrict__ hoff,
+    const uint64_t *__restrict__ eoff, K *__restrict__ node_keys, uint64_t *__restrict__ row_ptr,
+    uint32_t *__restrict__ adj_edge, uint8_t *__restrict__ adj_role, uint8_t *__restrict__ adj_side,
+    uint64_t *__restrict__ ends, uint32_t *__restrict__ bucket_fill, int bshift) {
+  constexpr int ITEMS = 12, WARPS = RANK_BLOCK / 32;
+  constexpr uint32_t CHUNK = RANK_BLOCK * ITEMS;
+  __shared__ uint32_t s_word[ITEMS * WARPS], s_pre[ITEMS * WARPS + 1], s_cnt[ISO ? ITEMS * WARPS + 1 : 1];
+  __shared__ uint32_t s_bcnt[256], s_bbase[256], s_w[WARPS];
+  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+  for (uint32_t tile = blockIdx.x; tile < tiles; tile += gridDim.x) {
+    const uint64_t s = bound[tile], n = bound[tile + 1] - s;
+    const uint32_t *hw = heads + (s >> 5) + tile;
+    uint64_t id0 = hoff[tile], slot0 = ISO ? eoff[tile] : s;
+    for (uint32_t u = tid; u < tcount[tile]; u += RANK_BLOCK) node_keys[id0 + u] = ukeys[s + u];
+    for (uint64_t c = 0; c < n; c += CHUNK) {
+      const uint32_t cnt = (uint32_t)min((uint64_t)CHUNK, n - c);
+      const int items = (int)((cnt + RANK_BLOCK - 1) / RANK_BLOCK);
+      uint32_t val[ITEMS];
+#pragma unroll
+      for (int i = 0; i < ITEMS; i++) {
+        const uint32_t j = (uint32_t)i * RANK_BLOCK + tid;
+        val[i] = j < cnt ? vals[s + c + j] : REC_NONE;
+      }
+      // heads before each word of 32 records
+      uint32_t w = 0, pc = 0;
+      if (tid < ITEMS * WARPS) {
+        w = (uint32_t)tid * 32 < cnt ? hw[(c >> 5) + tid] : 0u;
+        pc = __popc(w);
+        s_word[tid] = w;
+      }
+      if (tid < 256) s_bcnt[tid] = 0;
+      const uint32_t incl = warp_incl_scan(pc);
+      if (lane == 31) s_w[warp] = incl;
+      __syncthreads();
+      uint32_t pre = incl - pc;
+      for (int x = 0; x < warp; x++) pre += s_w[x];
+      if (tid < ITEMS * WARPS) s_pre[tid] = pre;
+      if (tid == ITEMS * WARPS - 1) s_pre[ITEMS * WARPS] = pre + pc;
+      uint32_t rk[ITEMS];  // an edge end's slot, then its rank in its bucket
+      uint32_t n_end = cnt;
+      if (ISO) {
+        bool end[ITEMS];
+#pragma unroll
+        for (int i = 0; i < ITEMS; i++) end[i] = val[i] != REC_NONE;
+        n_end = tile_flag_ranks<RANK_BLOCK, ITEMS>(end, rk, s_cnt);  // synchronises
+      } else {
+        __syncthreads();
+      }
+      auto id_of = [&](int i, uint32_t hb) {
+        return (uint32_t)id0 + s_pre[i * WARPS + warp] + __popc(hb & (0xffffffffu >> (31 - lane))) - 1u;
+      };
+#pragma unroll
+      for (int i = 0; i < ITEMS; i++) {
+        if (i >= items) break;
+        const uint32_t j = (uint32_t)i * RANK_BLOCK + tid;
+        if (j < cnt) {
+          const uint32_t hb = s_word[i * WARPS + warp];
+          const uint64_t slot = slot0 + (ISO ? rk[i] : j);
+          if (hb >> lane & 1u) row_ptr[id_of(i, hb)] = slot;
+          if (!ISO || val[i] != REC_NONE) {
+            if (adj_side) {  // the two side bits on top of the payload
+              adj_side[slot] = (uint8_t)(val[i] >> 30);
+              val[i] &= 0x3fffffffu;
+            }
+            adj_edge[slot] = val[i] >> 1;
+            adj_role[slot] = (uint8_t)(val[i] & 1u);
+            rk[i] = atomicAdd(&s_bcnt[val[i] >> 1 >> bshift], 1u);
+          }
+        }
+      }
+      __syncthreads();
+      if (tid < 256 && s_bcnt[tid]) s_bbase[tid] = atomicAdd(bucket_fill + tid, s_bcnt[tid]);
+      __syncthreads();
+#pragma unroll
+      for (int i = 0; i < ITEMS; i++) {
+        if (i >= items) break;
+        if ((uint32_t)i * RANK_BLOCK + tid < cnt && (!ISO || val[i] != REC_NONE)) {
+          const uint32_t bk = val[i] >> 1 >> bshift;
+          ends[((uint64_t)bk << (bshift + 1)) + s_bbase[bk] + rk[i]] =
+              (uint64_t)val[i] << 32 | id_of(i, s_word[i * WARPS + warp]);
+        }
+      }
+      id0 += s_pre[ITEMS * WARPS];
+      slot0 += n_end;
+      __syncthreads();
+    }
+    if (tile == tiles - 1 && tid == 0) row_ptr[id0] = slot0;
+  }
+}
+
+// Edge ends (records that are not REC_NONE) of each tile.
+static __global__ __launch_bounds__(256) void k_tile_ends(const uint64_t *__restrict__ bound, uint32_t tiles,
+                                                          const uint32_t *__restrict__ vals,
+                                                          uint32_t *__restrict__ ecount) {
+  __shared__ uint32_t s_sum;
+  for (uint32_t tile = blockIdx.x; tile < tiles; tile += gridDim.x) {
+    if (threadIdx.x == 0) s_sum = 0;
+    __syncthreads();
+    uint32_t c = 0;
+    for (uint64_t j = bound[tile] + threadIdx.x; j < bound[tile + 1]; j += 256) c += vals[j] != REC_NONE;
+    c = __reduce_add_sync(0xffffffffu, c);
+    if ((threadIdx.x & 31) == 0 && c) atomicAdd(&s_sum, c);
+    __syncthreads();
+    if (threadIdx.x == 0) ecount[tile] = s_sum;
   }
 }
 
@@ -652,7 +997,9 @@ struct SlotOps<Key128> {
     return (uint32_t)(((d.lo ^ (d.hi * 0x9e3779b97f4a7c15ull)) * 0xc2b2ae3d27d4eb4full) >> 32);
   }
   // every probe is a 128-bit compare-and-swap, which also reads the slot
-  // whole (two 64-bit loads could see a slot half written)
+  // whole (two 64-bit loads could see a slot half written; trusting halves
+  // that are not empty's and swapping only otherwise was slower, 2.4 instead of
+  // 1.0 ms for 9 M keys nearly all distinct and no gain at 30x coverage)
   __device__ static Key128 claim(Key128 *p, Key128 d) {
     Key128 old;
     asm volatile(
