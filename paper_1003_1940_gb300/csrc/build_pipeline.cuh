@@ -1061,11 +1061,12 @@ dbg_status count_node_kmers(dbg_ctx *ctx, const DevBuf &packed, const DevBuf &ba
   DBG_TRY(alloc_buf(ctx, ka, M * sizeof(K) + MSD_PAD));
   DBG_TRY(alloc_buf(ctx, kb, M * sizeof(K) + MSD_PAD));
   DBG_CUDA_TRY(cudaMemsetAsync(d_hist, 0, MAX_PASSES * RADIX * sizeof(unsigned long long), s));
+  const DigitSpec digits = plan.digits();
   // emitting with k - 1 gives windows of k bases at the k-mer offsets
   DBG_LAUNCH(ctx, ST_NODE_MULT, 8.0 * n + (double)M * sizeof(K),
-             k_emit<K><<<(unsigned)std::min<uint64_t>(grid_for(n, EMIT_BLOCK / 32), 152ull * 64), EMIT_BLOCK, 0, s>>>(
+             (digits.wide ? k_emit<K, true> : k_emit<K, false>)<<<(unsigned)std::min<uint64_t>(grid_for(n, EMIT_BLOCK / 32), 152ull * 64), EMIT_BLOCK, 0, s>>>(
                  packed.as<uint64_t>(), base_off.as<uint64_t>(), koff.as<uint64_t>(), n, k - 1, ka.as<K>(),
-                 plan.digits(), d_hist, nullptr));
+                 digits, d_hist, nullptr, nullptr));
   DBG_CUDA_TRY(cudaGetLastError());
   K *kp = ka.as<K>(), *alt = kb.as<K>();
   uint32_t *vn = nullptr, *van = nullptr;
@@ -1123,11 +1124,12 @@ dbg_status count_node_reads(dbg_ctx *ctx, const DevBuf &packed, const DevBuf &ba
   DBG_TRY(alloc_buf(ctx, va, M * sizeof(uint32_t) + MSD_PAD));
   DBG_TRY(alloc_buf(ctx, vb, M * sizeof(uint32_t) + MSD_PAD));
   DBG_CUDA_TRY(cudaMemsetAsync(d_hist, 0, MAX_PASSES * RADIX * sizeof(unsigned long long), s));
+  const DigitSpec digits = plan.digits();
   // windows of k bases at the k-mer offsets, each with its read index
   DBG_LAUNCH(ctx, ST_NODE_MULT, 8.0 * n + (double)M * (sizeof(K) + 4),
-             k_emit<K><<<(unsigned)std::min<uint64_t>(grid_for(n, EMIT_BLOCK / 32), 152ull * 64), EMIT_BLOCK, 0, s>>>(
+             (digits.wide ? k_emit<K, true> : k_emit<K, false>)<<<(unsigned)std::min<uint64_t>(grid_for(n, EMIT_BLOCK / 32), 152ull * 64), EMIT_BLOCK, 0, s>>>(
                  packed.as<uint64_t>(), base_off.as<uint64_t>(), koff.as<uint64_t>(), n, k - 1, ka.as<K>(),
-                 plan.digits(), d_hist, nullptr, va.as<uint32_t>()));
+                 digits, d_hist, nullptr, va.as<uint32_t>()));
   DBG_CUDA_TRY(cudaGetLastError());
   koff.release();
   K *kp = ka.as<K>(), *kalt = kb.as<K>();
@@ -1210,11 +1212,12 @@ dbg_status build_graph_impl(dbg_ctx *ctx, const BuildInput &in, dbg_graph *g) {
   DevBuf packed;
   const uint64_t nwords = (total_bases + 31) / 32;
   // K2 emit over the keys [krange[0], krange[1]) (all of them: nullptr)
+  const DigitSpec digits = plan.digits();
   auto emit = [&](const uint64_t *krange, double bytes) -> dbg_status {
     DBG_LAUNCH(ctx, ST_EMIT, bytes,
-               k_emit<K><<<(unsigned)std::min<uint64_t>(grid_for(n, EMIT_BLOCK / 32), 152ull * 64), EMIT_BLOCK, 0,
+               (digits.wide ? k_emit<K, true> : k_emit<K, false>)<<<(unsigned)std::min<uint64_t>(grid_for(n, EMIT_BLOCK / 32), 152ull * 64), EMIT_BLOCK, 0,
                            s>>>(packed.as<uint64_t>(), base_off.as<uint64_t>(), edge_off.as<uint64_t>(), n, k,
-                                keys_a.as<K>(), plan.digits(), d_hist, krange));
+                                keys_a.as<K>(), digits, d_hist, krange, nullptr));
     DBG_CUDA_TRY(cudaGetLastError());
     return DBG_OK;
   };

@@ -303,7 +303,45 @@ __device__ __forceinline__ uint64_t last_le(const uint64_t *__restrict__ a, uint
   return lo;
 }
 
-template <class K>
+// The 32 bits x with the order of its 2-bit codes reversed and every code
+// complemented: bit reversal also swaps the two bits of a code, which taking
+// the odd bits from one place down and the even bits from one place up undoes.
+__device__ __forceinline__ uint32_t rev_comp16(uint32_t x) {
+  const uint32_t y = ~__brev(x);
+  return ((y >> 1) & 0x55555555u) | ((y << 1) & 0xaaaaaaaau);
+}
+
+// The canonical form of the m bases whose first lies in the 32-bit half `odd`
+// (0: the upper) of the 64-bit word *w, o bits (twice the base's place in the
+// half) below its top.  Whole 32-bit words are funnel-shifted into place.
+template <class K> __device__ __forceinline__ K canonical_window(const uint64_t *w, uint32_t o, bool odd, int m);
+
+template <>
+__device__ __forceinline__ uint64_t canonical_window<uint64_t>(const uint64_t *w, uint32_t o, bool odd, int m) {
+  const uint64_t a = __ldg(w), b = __ldg(w + 1);
+  const uint32_t x0 = odd ? (uint32_t)a : (uint32_t)(a >> 32), x1 = odd ? (uint32_t)(b >> 32) : (uint32_t)a,
+                 x2 = odd ? (uint32_t)b : (uint32_t)(b >> 32);
+  const uint32_t hi = __funnelshift_l(x1, x0, o), lo = __funnelshift_l(x2, x1, o);
+  const uint64_t z = ((uint64_t)hi << 32 | lo) >> (64 - 2 * m);
+  const uint64_t rc = ((uint64_t)rev_comp16((uint32_t)z) << 32 | rev_comp16((uint32_t)(z >> 32))) >> (64 - 2 * m);
+  return min(z, rc);
+}
+
+template <>
+__device__ __forceinline__ Key128 canonical_window<Key128>(const uint64_t *w, uint32_t o, bool odd, int m) {
+  const uint64_t a = __ldg(w), b = __ldg(w + 1), c = __ldg(w + 2);
+  const uint32_t x0 = odd ? (uint32_t)a : (uint32_t)(a >> 32), x1 = odd ? (uint32_t)(b >> 32) : (uint32_t)a,
+                 x2 = odd ? (uint32_t)b : (uint32_t)(b >> 32), x3 = odd ? (uint32_t)(c >> 32) : (uint32_t)b,
+                 x4 = odd ? (uint32_t)c : (uint32_t)(c >> 32);
+  const Key128 top{(uint64_t)__funnelshift_l(x1, x0, o) << 32 | __funnelshift_l(x2, x1, o),
+                   (uint64_t)__funnelshift_l(x3, x2, o) << 32 | __funnelshift_l(x4, x3, o)};
+  const Key128 z = KeyOps<Key128>::shr(top, 128 - 2 * m);
+  auto rev = [](uint64_t x) { return (uint64_t)rev_comp16((uint32_t)x) << 32 | rev_comp16((uint32_t)(x >> 32)); };
+  return kmin(z, KeyOps<Key128>::shr(Key128{rev(z.lo), rev(z.hi)}, 128 - 2 * m));
+}
+
+// WIDE: the keys' one digit of ds.wide bits is counted (see DigitSpec).
+template <class K, bool WIDE>
 __global__ __launch_bounds__(EMIT_BLOCK) void k_emit(const uint64_t *__restrict__ packed,
                                                      const uint64_t *__restrict__ base_off,
                                                      const uint64_t *__restrict__ edge_off, uint64_t n_reads,
@@ -316,7 +354,10 @@ __global__ __launch_bounds__(EMIT_BLOCK) void k_emit(const uint64_t *__restrict_
   // krange is given), so lanes stay busy across read ends and every
   // warp-wide store writes 32 consecutive keys.  A lane follows the
   // read that holds its key: one binary search per warp, then a step to the
-  // next read when the key passes the current one's end.
+  // next read when the key passes the current one's end.  From one of its keys
+  // to the next a lane moves 32 bases, one packed word, so its place within
+  // the word only changes with the read.  Key numbers fit 32 bits (one build
+  // has fewer than 2^32 instances).  Instruction-bound: @@
   __shared__ uint32_t s_hist[MAX_PASSES * RADIX];
   for (int i = threadIdx.x; i < ds.entries(); i += EMIT_BLOCK) s_hist[i] = 0;
   __syncthreads();
@@ -324,36 +365,43 @@ __global__ __launch_bounds__(EMIT_BLOCK) void k_emit(const uint64_t *__restrict_
   const uint64_t warps = (uint64_t)gridDim.x * (EMIT_BLOCK / 32);
   const uint64_t wid = (uint64_t)blockIdx.x * (EMIT_BLOCK / 32) + (threadIdx.x >> 5);
   const int m = (int)k + 1;
-  const int G = ds.passes - ds.first;  // histogrammed passes
-  uint32_t *hbase = s_hist + ds.first * RADIX;
   const uint64_t lo = krange ? krange[0] : 0, hi = krange ? krange[1] : __ldg(edge_off + n_reads);
   const uint64_t per = ((hi - lo + warps - 1) / warps + 31) & ~31ull;
-  const uint64_t a = lo + wid * per, b = min(a + per, hi);
-  if (a < b) {
-    // the read holding key a + lane: the last read starting at or before a,
-    // then forward (reads without keys are stepped over)
-    uint64_t r = last_le(edge_off, 0, n_reads, a);
-    uint64_t e_hi = __ldg(edge_off + r + 1), pos = __ldg(base_off + r) - __ldg(edge_off + r);
-    for (uint64_t i = a + lane; i < b; i += 32) {
-      while (i >= e_hi) {
-        r++;
-        const uint64_t e_lo = e_hi;
-        e_hi = __ldg(edge_off + r + 1);
-        pos = __ldg(base_off + r) - e_lo;
+  const uint64_t a64 = lo + wid * per;
+  if (a64 < hi) {
+    const uint32_t a = (uint32_t)a64, b = (uint32_t)min(a64 + per, hi);
+    const uint32_t *const edge32 = reinterpret_cast<const uint32_t *>(edge_off);  // (the low halves)
+    // the read holding key a: the last one starting at or before it
+    uint32_t r = (uint32_t)last_le(edge_off, 0, n_reads, a64);
+    uint32_t i = a + lane, end = __ldg(edge32 + 2 * (size_t)(r + 1));  // the first key behind the read
+    const uint64_t *w = nullptr;
+    uint32_t o = 0;
+    bool odd = false;
+    auto place = [&](uint32_t e_lo) {
+      const uint64_t p = __ldg(base_off + r) + (i - e_lo);
+      w = packed + (p >> 5);
+      o = (uint32_t)p * 2 & 30u;
+      odd = (uint32_t)p & 16u;
+    };
+    place(__ldg(edge32 + 2 * (size_t)r));
+    // (b <= 2^32 - 1 and i advances by 32: the count of rows, not i, ends the loop)
+    for (uint32_t rows = i < b ? (b - i + 31) / 32 : 0; rows > 0; rows--) {
+      if (i >= end) {
+        uint32_t e_lo;
+        do {  // (reads without keys are stepped over)
+          e_lo = end;
+          r++;
+          end = __ldg(edge32 + 2 * (size_t)(r + 1));
+        } while (i >= end);
+        place(e_lo);
       }
-      const K z = load_window<K>(packed, pos + i, m);
-      const K key = kmin(z, revcomp(z, m));
+      const K key = canonical_window<K>(w, o, odd, m);
+      w++;
       keys[i] = key;
-      if (read_of) read_of[i] = (uint32_t)r;
-      if (!ds.wide && G <= 4) {
-        // the histogrammed digits are the low bytes of one shifted word
-        const uint32_t w = (uint32_t)KeyOps<K>::words_lo(KeyOps<K>::shr(key, ds.first * RADIX_BITS));
-#pragma unroll
-        for (int g = 0; g < 4; g++)
-          if (g < G) atomicAdd(hbase + g * RADIX + ((w >> (8 * g)) & 0xffu), 1u);
-      } else {
-        ds.count(s_hist, key);
-      }
+      if (read_of) read_of[i] = r;
+      if (WIDE) atomicAdd(&s_hist[KeyOps<K>::digit(key, ds.first, ds.wide)], 1u);
+      else ds.count(s_hist, key);
+      i += 32;
     }
   }
   __syncthreads();
