@@ -357,7 +357,8 @@ __global__ __launch_bounds__(EMIT_BLOCK) void k_emit(const uint64_t *__restrict_
   // next read when the key passes the current one's end.  From one of its keys
   // to the next a lane moves 32 bases, one packed word, so its place within
   // the word only changes with the read.  Key numbers fit 32 bits (one build
-  // has fewer than 2^32 instances).  Instruction-bound: @@
+  // has fewer than 2^32 instances).  Instruction-bound: 3.04 ms for 1.035 G
+  // keys (8.3 GB written); with 64-bit shifts and key numbers 3.45.
   __shared__ uint32_t s_hist[MAX_PASSES * RADIX];
   for (int i = threadIdx.x; i < ds.entries(); i += EMIT_BLOCK) s_hist[i] = 0;
   __syncthreads();
