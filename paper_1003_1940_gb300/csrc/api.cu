@@ -46,12 +46,87 @@ void Allocator::put(void *p, size_t bytes) {
 dbg_status alloc_buf(dbg_ctx *ctx, DevBuf &b, size_t bytes) {
   b.release();
   b.al = &ctx->al;
+  b.ar = nullptr;
   b.p = ctx->al.get(bytes);
+  if (!b.p && ctx->scratch.drop(ctx->al)) b.p = ctx->al.get(bytes);
   if (!b.p) {
     set_error("device allocation of %zu bytes failed", bytes);
     return DBG_ENOMEM;
   }
   b.bytes = bytes;
+  return DBG_OK;
+}
+
+void *Scratch::get(Allocator &al, size_t bytes) {
+  bytes = (std::max<size_t>(bytes, 1) + 255) & ~(size_t)255;
+  if (bytes > MOST || short_of_memory) return nullptr;
+  if (!base) {
+    base = static_cast<char *>(al.get(CAP));
+    short_of_memory = !base;
+    if (!base) return nullptr;
+    pieces.assign(1, Piece{0, CAP, false});
+  }
+  for (size_t i = 0; i < pieces.size(); i++) {
+    if (pieces[i].used || pieces[i].bytes < bytes) continue;
+    if (pieces[i].bytes > bytes)
+      pieces.insert(pieces.begin() + i + 1, Piece{pieces[i].off + bytes, pieces[i].bytes - bytes, false});
+    pieces[i].bytes = bytes;
+    pieces[i].used = true;
+    return base + pieces[i].off;
+  }
+  return nullptr;
+}
+
+void Scratch::put(void *p) {
+  const size_t off = static_cast<size_t>(static_cast<char *>(p) - base);
+  size_t i = 0;
+  while (i < pieces.size() && pieces[i].off != off) i++;
+  if (i == pieces.size()) return;
+  pieces[i].used = false;
+  if (i + 1 < pieces.size() && !pieces[i + 1].used) {
+    pieces[i].bytes += pieces[i + 1].bytes;
+    pieces.erase(pieces.begin() + i + 1);
+  }
+  if (i > 0 && !pieces[i - 1].used) {
+    pieces[i - 1].bytes += pieces[i].bytes;
+    pieces.erase(pieces.begin() + i);
+  }
+}
+
+bool Scratch::drop(Allocator &al) {
+  short_of_memory = true;
+  if (!base || pieces.size() != 1 || pieces[0].used) return false;
+  al.put(base, CAP);
+  base = nullptr;
+  return true;
+}
+
+dbg_status alloc_tmp(dbg_ctx *ctx, DevBuf &b, size_t bytes) {
+  b.release();
+  if (void *p = ctx->scratch.get(ctx->al, bytes)) {
+    b.al = nullptr;
+    b.ar = &ctx->scratch;
+    b.p = p;
+    b.bytes = bytes;
+    return DBG_OK;
+  }
+  return alloc_buf(ctx, b, bytes);
+}
+
+dbg_status alloc_block(dbg_ctx *ctx, DevBuf &block, std::initializer_list<BlockPart> parts) {
+  auto padded = [](size_t b) { return (std::max<size_t>(b, 1) + 255) & ~(size_t)255; };
+  size_t total = 0;
+  for (const BlockPart &x : parts) total += padded(x.bytes);
+  DBG_TRY(alloc_buf(ctx, block, total));
+  char *at = static_cast<char *>(block.p);
+  for (const BlockPart &x : parts) {
+    x.buf->release();
+    x.buf->al = nullptr;
+    x.buf->ar = nullptr;
+    x.buf->p = at;
+    x.buf->bytes = x.bytes;
+    at += padded(x.bytes);
+  }
   return DBG_OK;
 }
 
@@ -95,10 +170,23 @@ dbg_status next_epoch(dbg_ctx *ctx, uint32_t *epoch) {
   return DBG_OK;
 }
 
+static dbg_status status_of_error(dbg_ctx *ctx, uint32_t e);
+
 dbg_status check_device_error(dbg_ctx *ctx) {
   DBG_CUDA_TRY(cudaMemcpyAsync(ctx->h_pinned, ctx->d_err, sizeof(uint32_t), cudaMemcpyDeviceToHost, ctx->stream));
   DBG_CUDA_TRY(cudaStreamSynchronize(ctx->stream));
-  uint32_t e = ctx->h_pinned[0];
+  return status_of_error(ctx, ctx->h_pinned[0]);
+}
+
+dbg_status read_counters(dbg_ctx *ctx, uint32_t *counters) {
+  // the error word and the counters are one 256-byte block
+  DBG_CUDA_TRY(cudaMemcpyAsync(ctx->h_pinned, ctx->d_err, 256, cudaMemcpyDeviceToHost, ctx->stream));
+  DBG_CUDA_TRY(cudaStreamSynchronize(ctx->stream));
+  std::memcpy(counters, ctx->h_pinned + (ctx->d_counters - ctx->d_err), (CT_LAST + 1) * sizeof(uint32_t));
+  return status_of_error(ctx, ctx->h_pinned[0]);
+}
+
+static dbg_status status_of_error(dbg_ctx *ctx, uint32_t e) {
   if (e == 0) return DBG_OK;
   DBG_CUDA_TRY(cudaMemsetAsync(ctx->d_err, 0, sizeof(uint32_t), ctx->stream));
   if (e & ERR_BAD_BASE) {
@@ -316,6 +404,7 @@ void dbg_destroy(dbg_ctx *ctx) {
   prof_resolve(ctx);
   for (cudaEvent_t e : ctx->ev_pool) cudaEventDestroy(e);
   if (ctx->d_status) cudaFreeAsync(ctx->d_status, ctx->stream);
+  if (ctx->scratch.base) ctx->al.put(ctx->scratch.base, Scratch::CAP);
   if (ctx->stream) cudaStreamSynchronize(ctx->stream);
   if (ctx->d_err) cudaFree(ctx->d_err);
   if (ctx->h_pinned) cudaFreeHost(ctx->h_pinned);
@@ -359,7 +448,9 @@ dbg_status dbg_build(dbg_ctx *ctx, const char *reads, const uint32_t *lengths, u
   g->device = ctx->device;
   g->n_copy = ctx->copy_streams;
   // graph arrays must be freed through the graph's own allocator copy
-  auto rebind = [&](DevBuf &b) { b.al = &g->al; };
+  auto rebind = [&](DevBuf &b) {
+    if (b.al) b.al = &g->al;
+  };
 
   dbg_status st = DBG_OK;
   DevBuf d_len;
@@ -368,7 +459,7 @@ dbg_status dbg_build(dbg_ctx *ctx, const char *reads, const uint32_t *lengths, u
   if (n > 0) {
     reads_on_dev = is_device_ptr(reads);
     if (!is_device_ptr(lengths)) {
-      st = alloc_buf(ctx, d_len, n * sizeof(uint32_t));
+      st = alloc_tmp(ctx, d_len, n * sizeof(uint32_t));
       if (st == DBG_OK && cudaMemcpyAsync(d_len.p, lengths, n * sizeof(uint32_t), cudaMemcpyHostToDevice, s) != cudaSuccess) {
         set_error("copy of the read lengths to the device failed");
         st = DBG_ECUDA;
@@ -381,8 +472,9 @@ dbg_status dbg_build(dbg_ctx *ctx, const char *reads, const uint32_t *lengths, u
     BuildInput in{reinterpret_cast<const uint8_t *>(reads), len_dev, n, !reads_on_dev, k};
     st = k <= 31 ? build_graph_u64(ctx, in, g) : build_graph_u128(ctx, in, g);
   }
-  for (DevBuf *b : {&g->node_keys, &g->edge_keys, &g->src, &g->dst, &g->orient, &g->mult, &g->row_ptr,
-                    &g->adj_nbr, &g->adj_edge, &g->adj_role, &g->adj_side, &g->node_mult, &g->node_reads})
+  for (DevBuf *b : {&g->block[0], &g->block[1], &g->node_keys, &g->edge_keys, &g->src, &g->dst, &g->orient, &g->mult,
+                    &g->row_ptr, &g->adj_nbr, &g->adj_edge, &g->adj_role, &g->adj_side, &g->node_mult,
+                    &g->node_reads})
     rebind(*b);
   d_len.release();
   cudaStreamSynchronize(s);
@@ -437,7 +529,7 @@ dbg_status dbg_build_bucketed(dbg_ctx *ctx, const char *reads, const uint32_t *l
   const uint32_t *len_dev = lengths;
   const bool reads_on_dev = n > 0 && is_device_ptr(reads);
   if (n > 0 && !is_device_ptr(lengths)) {
-    st = alloc_buf(ctx, d_len, n * sizeof(uint32_t));
+    st = alloc_tmp(ctx, d_len, n * sizeof(uint32_t));
     if (st == DBG_OK && cudaMemcpyAsync(d_len.p, lengths, n * 4, cudaMemcpyHostToDevice, s) != cudaSuccess) {
       set_error("copy of the read lengths to the device failed");
       st = DBG_ECUDA;

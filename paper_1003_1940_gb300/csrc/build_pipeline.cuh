@@ -387,8 +387,10 @@ inline unsigned grid_for(uint64_t n, int per_block) {
   return (unsigned)std::max<uint64_t>(1, std::min<uint64_t>(g, 0x7fffffffull));
 }
 
-// Exclusive scan of n u32 values into n + 1 u64 (the last is the total).
-inline dbg_status scan_u32_async(dbg_ctx *ctx, const uint32_t *in, uint64_t n, uint64_t *out, int stage) {
+// Exclusive scan of n u32 values into n + 1 u64 (the last is the total, which
+// also goes to counter `total`).
+inline dbg_status scan_u32_async(dbg_ctx *ctx, const uint32_t *in, uint64_t n, uint64_t *out, int stage,
+                                 int total = 1) {
   cudaStream_t s = ctx->stream;
   const uint64_t tiles = (n + SCAN_TILE - 1) / SCAN_TILE;
   DBG_TRY(ensure_status(ctx, tiles));
@@ -397,7 +399,7 @@ inline dbg_status scan_u32_async(dbg_ctx *ctx, const uint32_t *in, uint64_t n, u
   DBG_CUDA_TRY(cudaMemsetAsync(ctx->d_counters, 0, 2 * sizeof(uint32_t), s));
   DBG_LAUNCH(ctx, stage, 12.0 * n,
              k_scan_excl<<<(unsigned)tiles, SCAN_BLOCK, 0, s>>>(in, n, out, ctx->d_status, ctx->d_counters, epoch,
-                                                                ctx->spin_limit, ctx->d_err, ctx->d_counters + 1));
+                                                                ctx->spin_limit, ctx->d_err, ctx->d_counters + total));
   DBG_CUDA_TRY(cudaGetLastError());
   return DBG_OK;
 }
@@ -413,8 +415,8 @@ dbg_status run_length_reduce(dbg_ctx *ctx, const K *sorted, uint64_t n, K *uniq,
   cudaStream_t s = ctx->stream;
   const uint64_t tiles = (n + RS_TILE - 1) / RS_TILE;
   DevBuf counts, toff;
-  DBG_TRY(alloc_buf(ctx, counts, tiles * 4));
-  DBG_TRY(alloc_buf(ctx, toff, (tiles + 1) * 8));
+  DBG_TRY(alloc_tmp(ctx, counts, tiles * 4));
+  DBG_TRY(alloc_tmp(ctx, toff, (tiles + 1) * 8));
   DBG_LAUNCH(ctx, ST_RLE, (double)n * sizeof(K),
              k_count_heads<K><<<(unsigned)tiles, SCAN_BLOCK, 0, s>>>(sorted, nullptr, n, counts.as<uint32_t>(),
                                                                    nullptr));
@@ -444,7 +446,7 @@ template <class K>
 dbg_status msd_bounds(dbg_ctx *ctx, Groups &gr, uint64_t n, uint32_t *cursor, int stage) {
   constexpr uint64_t T = SegShape<K>::TILE;
   const uint64_t tiles = (n + T - 1) / T;
-  DBG_TRY(alloc_buf(ctx, gr.bound, (tiles + 1) * 8));
+  DBG_TRY(alloc_tmp(ctx, gr.bound, (tiles + 1) * 8));
   const uint64_t *places = gr.ng ? gr.tables.as<uint64_t>() : gr.goff.as<uint64_t>();
   DBG_LAUNCH(ctx, stage, 0.0,
              k_msd_bounds<<<std::min(grid_for(gr.ng_max, 256), 152u * 8), 256, 0, ctx->stream>>>(
@@ -500,7 +502,7 @@ dbg_status msd_sort(dbg_ctx *ctx, K **keys, K **alt_keys, uint32_t **vals, uint3
   gr.ng_max = two ? (uint32_t)(2 * (n / msd_mean<K>()) + W) : W;
   // [start: W + 1] u64, [cursor: W][gfirst: W + 1][tfirst: W + 1] u32, [tmap] u16, [w2][low] u8
   const size_t bytes = (size_t)(W + 1) * 8 + (size_t)(3 * W + 2) * 4 + (two ? tiles2 * 2 : 0) + 2 * (size_t)W + 16;
-  DBG_TRY(alloc_buf(ctx, gr.tables, bytes));
+  DBG_TRY(alloc_tmp(ctx, gr.tables, bytes));
   MsdTables tb{};
   tb.start = gr.tables.as<uint64_t>();
   uint32_t *cursor = reinterpret_cast<uint32_t *>(tb.start + W + 1);
@@ -533,8 +535,8 @@ dbg_status msd_sort(dbg_ctx *ctx, K **keys, K **alt_keys, uint32_t **vals, uint3
   // the groups' sizes, their places, and the second pass
   DevBuf gcount;
   const uint64_t NG = gr.ng_max;
-  DBG_TRY(alloc_buf(ctx, gcount, NG * 4));
-  DBG_TRY(alloc_buf(ctx, gr.goff, (NG + 1) * 8));
+  DBG_TRY(alloc_tmp(ctx, gcount, NG * 4));
+  DBG_TRY(alloc_tmp(ctx, gr.goff, (NG + 1) * 8));
   DBG_CUDA_TRY(cudaMemsetAsync(gcount.p, 0, NG * 4, s));
   DBG_LAUNCH(ctx, stage, (double)n * sizeof(K),
              k_msd_count<K><<<(unsigned)std::min<uint64_t>(tiles2, 4ull * std::max(1, ctx->num_sms)), MSD_BLOCK,
@@ -561,8 +563,10 @@ dbg_status msd_sort(dbg_ctx *ctx, K **keys, K **alt_keys, uint32_t **vals, uint3
 // oversize ones.
 struct TileSet {
   uint64_t tiles = 0;
-  uint32_t gathered = 0;
-  DevBuf bound, osize, ooff, gk, gv;
+  uint32_t gathered = 0;         // keys in oversize tiles, once known
+  uint32_t oversize = 0;         // and those tiles' number,
+  DevBuf bound, osize, olist;    // which olist lists
+  DevBuf ooff, gk, gv;           // (seg_gather)
 };
 
 // The records' order by payload: *out = n words whose low halves list the
@@ -572,41 +576,55 @@ dbg_status order_by_payload(dbg_ctx *ctx, const uint32_t *v, uint64_t n, int shi
 
 // Tile bounds of the local pass over n keys in the groups gr (sorted by
 // their bits from gr.lb up), and the oversize tiles (longer than the
-// shared-memory capacity) gathered into *gk / *gv and sorted over every
-// digit.
-template <class K, bool HAS_VAL>
-dbg_status seg_prepare(dbg_ctx *ctx, const K *kin, const uint32_t *vin, uint64_t n, Groups &gr, ValOrder vo,
-                       int key_bits, TileSet &ts, int stage) {
+// shared-memory capacity): their sizes, a list of them, and in the counters
+// their keys and number.
+template <class K>
+dbg_status seg_tiles(dbg_ctx *ctx, const K *kin, uint64_t n, Groups &gr, TileSet &ts, int stage) {
   using Sh = SegShape<K>;
   cudaStream_t s = ctx->stream;
   const uint64_t tiles = (n + Sh::TILE - 1) / Sh::TILE;
   if (tiles > 0x7fffffffull) return DBG_EOVERFLOW;
   ts.tiles = tiles;
-  DevBuf &bound = ts.bound, &osize = ts.osize, &ooff = ts.ooff, &gk = ts.gk, &gv = ts.gv;
-  uint32_t *G = &ts.gathered;
-  DBG_TRY(alloc_buf(ctx, osize, tiles * 4));
-  DBG_TRY(alloc_buf(ctx, ooff, (tiles + 1) * 8));
+  DBG_TRY(alloc_tmp(ctx, ts.osize, tiles * 4));
+  DBG_TRY(alloc_tmp(ctx, ts.olist, tiles * 4));
   if (gr.ng) DBG_TRY(msd_bounds<K>(ctx, gr, n, nullptr, stage));
   if (gr.bound.p) {
-    bound = std::move(gr.bound);
+    ts.bound = std::move(gr.bound);
   } else {
-    DBG_TRY(alloc_buf(ctx, bound, (tiles + 1) * 8));
+    DBG_TRY(alloc_tmp(ctx, ts.bound, (tiles + 1) * 8));
     DBG_LAUNCH(ctx, stage, 0.0,
                k_seg_bounds<K><<<grid_for(tiles + 1, 256), 256, 0, s>>>(kin, n, gr.lb.fixed, Sh::TILE, tiles,
-                                                                       bound.as<uint64_t>()));
+                                                                       ts.bound.as<uint64_t>()));
   }
+  DBG_CUDA_TRY(cudaMemsetAsync(ctx->d_counters + CT_GATHERED, 0, (CT_ENDS - CT_GATHERED + 1) * 4, s));
   DBG_LAUNCH(ctx, stage, 0.0,
-             k_seg_oversize<<<grid_for(tiles, 256), 256, 0, s>>>(bound.as<uint64_t>(), tiles,
+             k_seg_oversize<<<grid_for(tiles, 256), 256, 0, s>>>(ts.bound.as<uint64_t>(), tiles,
                                                                  (uint32_t)(SEG_BLOCK * Sh::ITEMS),
-                                                                 osize.as<uint32_t>()));
-  DBG_TRY(scan_u32(ctx, osize.as<uint32_t>(), tiles, ooff.as<uint64_t>(), G, stage));
-  if (*G == 0) return DBG_OK;
+                                                                 ts.osize.as<uint32_t>(), ts.olist.as<uint32_t>(),
+                                                                 ctx->d_counters + CT_GATHERED,
+                                                                 ctx->d_counters + CT_OVERSIZE));
+  DBG_CUDA_TRY(cudaGetLastError());
+  return DBG_OK;
+}
+
+// The keys (and payloads) of the oversize tiles, gathered and sorted over
+// every digit, once ts.gathered says that there are some.
+template <class K, bool HAS_VAL>
+dbg_status seg_gather(dbg_ctx *ctx, const K *kin, const uint32_t *vin, ValOrder vo, int key_bits, TileSet &ts,
+                      int stage) {
+  if (ts.gathered == 0) return DBG_OK;
+  cudaStream_t s = ctx->stream;
+  const uint64_t tiles = ts.tiles;
+  const uint32_t *G = &ts.gathered;
+  DevBuf &bound = ts.bound, &osize = ts.osize, &ooff = ts.ooff, &gk = ts.gk, &gv = ts.gv;
+  DBG_TRY(alloc_tmp(ctx, ooff, (tiles + 1) * 8));
+  DBG_TRY(scan_u32_async(ctx, osize.as<uint32_t>(), tiles, ooff.as<uint64_t>(), stage));
   // the oversize tiles, gathered in order and sorted over every digit
   const uint64_t g = *G;
   DevBuf galt, gvalt, small;
-  DBG_TRY(alloc_buf(ctx, gk, g * sizeof(K)));
-  if (HAS_VAL) DBG_TRY(alloc_buf(ctx, gv, g * 4));
-  DBG_TRY(alloc_buf(ctx, small, MAX_PASSES * RADIX * 16));
+  DBG_TRY(alloc_tmp(ctx, gk, g * sizeof(K)));
+  if (HAS_VAL) DBG_TRY(alloc_tmp(ctx, gv, g * 4));
+  DBG_TRY(alloc_tmp(ctx, small, MAX_PASSES * RADIX * 16));
   unsigned long long *hist = small.as<unsigned long long>();
   uint64_t *dbase = reinterpret_cast<uint64_t *>(hist + MAX_PASSES * RADIX);
   const int passes = passes_for_bits(key_bits);
@@ -617,8 +635,8 @@ dbg_status seg_prepare(dbg_ctx *ctx, const K *kin, const uint32_t *vin, uint64_t
   DevBuf order;  // for records in no order: the words that order them by payload
   const uint64_t *words = nullptr;
   if (HAS_VAL && vo.sort) DBG_TRY(order_by_payload(ctx, gv.as<uint32_t>(), g, vo.shift, order, &words));
-  DBG_TRY(alloc_buf(ctx, galt, g * sizeof(K)));
-  if (HAS_VAL) DBG_TRY(alloc_buf(ctx, gvalt, g * 4));
+  DBG_TRY(alloc_tmp(ctx, galt, g * sizeof(K)));
+  if (HAS_VAL) DBG_TRY(alloc_tmp(ctx, gvalt, g * 4));
   if (words) {
     DBG_LAUNCH(ctx, stage, 2.0 * g * (sizeof(K) + 4),
                k_permute<K><<<grid_for(g, 256 * 8), 256, 0, s>>>(words, g, gk.as<K>(), gv.as<uint32_t>(),
@@ -661,38 +679,27 @@ dbg_status seg_sort_listed(dbg_ctx *ctx, const K *kin, const uint32_t *vin, K *k
   return DBG_OK;
 }
 
-// k_seg_rank over every tile (FUSED: heads and tcount), then the digit passes
-// for the tiles that it listed.
-template <class K, bool FUSED>
+// k_seg_rank over every tile, then the digit passes for the tiles that it
+// listed: the sorted records.
+template <class K>
 dbg_status seg_rank_tiles(dbg_ctx *ctx, const K *kin, const uint32_t *vin, K *kout, uint32_t *vout, uint64_t n,
-                          Groups &gr, ValOrder vo, TileSet &ts, uint32_t *heads, uint32_t *tcount) {
-  static_assert(SegRankSmem<K>::CAP == SEG_BLOCK * SegShape<K>::ITEMS, "same tile capacity as the digit-pass kernel");
-  auto kern = k_seg_rank<K, FUSED>;
+                          Groups &gr, ValOrder vo, TileSet &ts) {
+  auto kern = k_seg_rank<K, false>;
   set_smem_attrs(kern, sizeof(SegRankSmem<K>));
   DevBuf fb;
-  // the tiles listed for the digit passes, and from the other end the oversize
-  // ones; their numbers first
-  DBG_TRY(alloc_buf(ctx, fb, (ts.tiles + 2) * 4));
-  uint32_t *fb_count = fb.as<uint32_t>(), *fb_list = fb_count + 2;
-  DBG_CUDA_TRY(cudaMemsetAsync(fb_count, 0, 8, ctx->stream));
+  DBG_TRY(alloc_tmp(ctx, fb, ts.tiles * 4));
+  uint32_t *nlisted = ctx->d_counters + CT_LISTED;
+  DBG_CUDA_TRY(cudaMemsetAsync(nlisted, 0, 4, ctx->stream));
   DBG_LAUNCH(ctx, ST_LOCAL_SORT_NODES, 2.0 * (double)n * (sizeof(K) + 4),
              kern<<<(unsigned)ts.tiles, RANK_BLOCK, sizeof(SegRankSmem<K>), ctx->stream>>>(
                  kin, vin, ts.bound.as<uint64_t>(), ts.osize.as<uint32_t>(), ts.ooff.as<uint64_t>(), ts.gk.as<K>(),
-                 ts.gv.as<uint32_t>(), kout, vout, gr.lb, vo, fb_list, fb_count, heads, tcount));
+                 ts.gv.as<uint32_t>(), kout, vout, gr.lb, vo, fb.as<uint32_t>(), nlisted, nullptr, nullptr));
   DBG_CUDA_TRY(cudaGetLastError());
-  uint32_t listed[2] = {0, 0};
-  DBG_TRY(read_small(ctx, fb_count, sizeof(listed), listed));
-  const uint32_t nfb = listed[0], n_over = listed[1];
-  ctx->rank_fallback_tiles += nfb;
-  if (nfb) DBG_TRY(seg_sort_listed<K>(ctx, kin, vin, kout, vout, gr, vo, ts, fb_list, fb_count, nfb));
-  if (FUSED && nfb + n_over > 0) {
-    const unsigned grid = (unsigned)std::min<uint64_t>(nfb + n_over, 4ull * (uint64_t)std::max(1, ctx->num_sms));
-    DBG_LAUNCH(ctx, ST_LOCAL_SORT_NODES, 0.0,
-               k_tile_heads<K><<<grid, RANK_BLOCK, 0, ctx->stream>>>(kout, ts.bound.as<uint64_t>(),
-                                                                     (uint32_t)ts.tiles, fb_list, nfb, n_over, heads,
-                                                                     tcount));
-    DBG_CUDA_TRY(cudaGetLastError());
-  }
+  uint32_t c[CT_LAST + 1];
+  DBG_TRY(read_counters(ctx, c));
+  ctx->rank_fallback_tiles += c[CT_LISTED];
+  if (c[CT_LISTED])
+    DBG_TRY(seg_sort_listed<K>(ctx, kin, vin, kout, vout, gr, vo, ts, fb.as<uint32_t>(), nlisted, c[CT_LISTED]));
   return DBG_OK;
 }
 
@@ -703,7 +710,7 @@ dbg_status seg_sort_records(dbg_ctx *ctx, const K *kin, const uint32_t *vin, K *
                             Groups &gr, ValOrder vo, TileSet &ts) {
   using Sh = SegShape<K>;
   if (ctx->seg_rank)
-    return seg_rank_tiles<K, false>(ctx, kin, vin, kout, vout, n, gr, vo, ts, nullptr, nullptr);
+    return seg_rank_tiles<K>(ctx, kin, vin, kout, vout, n, gr, vo, ts);
   const int rank = local_rank_method(ctx, sizeof(K) == 16);
   const uint64_t tiles = ts.tiles;
   const DevBuf &bound = ts.bound, &osize = ts.osize, &ooff = ts.ooff, &gk = ts.gk, &gv = ts.gv;
@@ -745,72 +752,83 @@ dbg_status seg_rle(dbg_ctx *ctx, K *kin, K *kstage, uint64_t n, Groups &gr, int 
   using Sh = SegShape<K>;
   cudaStream_t s = ctx->stream;
   TileSet ts;
-  DBG_TRY((seg_prepare<K, false>(ctx, kin, nullptr, n, gr, ValOrder{}, key_bits, ts, ST_LOCAL_SORT_EDGES)));
-  DevBuf gheads, guniq;
-  const DevBuf &bound = ts.bound, &osize = ts.osize, &ooff = ts.ooff, &gk = ts.gk;
-  const uint32_t G = ts.gathered;
+  DevBuf gheads, guniq, mstage, tcount, toff, over;
   uint64_t H = 0;
-  if (G > 0) {
-    DBG_TRY(alloc_buf(ctx, guniq, (uint64_t)G * sizeof(K)));
-    DBG_TRY(alloc_buf(ctx, gheads, ((uint64_t)G + 1) * 4));
-    DBG_TRY(run_length_reduce<K>(ctx, gk.as<K>(), G, guniq.as<K>(), gheads.as<uint32_t>(), &H));
-  }
-  const uint64_t tiles = (n + Sh::TILE - 1) / Sh::TILE;
-  DevBuf mstage, tcount, toff;
-  DBG_TRY(alloc_buf(ctx, mstage, n * 4));
-  DBG_TRY(alloc_buf(ctx, tcount, tiles * 4));
-  DBG_TRY(alloc_buf(ctx, toff, (tiles + 1) * 8));
+  DBG_TRY(seg_tiles<K>(ctx, kin, n, gr, ts, ST_LOCAL_SORT_EDGES));
+  const uint64_t tiles = ts.tiles;
+  DBG_TRY(alloc_tmp(ctx, mstage, n * 4));
+  DBG_TRY(alloc_tmp(ctx, tcount, tiles * 4));
+  DBG_TRY(alloc_tmp(ctx, toff, (tiles + 1) * 8));
   const int rank = local_rank_method(ctx, sizeof(K) == 16);
-  auto radix = rank == RANK_MATCH    ? k_seg_rle<K, Sh::ITEMS, RANK_MATCH>
-               : rank == RANK_ATOMIC ? k_seg_rle<K, Sh::ITEMS, RANK_ATOMIC>
-                                     : k_seg_rle<K, Sh::ITEMS, RANK_BALLOT>;
-  constexpr size_t rsmem = sizeof(SegSortSmem<K, false, Sh::ITEMS>);
-  set_smem_attrs(radix, rsmem);
-  bool counted = false;
-  {
-    if (ctx->count_first) {
-      // count-first; the tiles that overflow their table are listed (after
-      // a counter word) and sorted copy by copy
-      auto count = rank == RANK_MATCH    ? k_seg_count<K, RANK_MATCH>
-                   : rank == RANK_ATOMIC ? k_seg_count<K, RANK_ATOMIC>
-                                         : k_seg_count<K, RANK_BALLOT>;
-      const size_t csmem = rank == RANK_MATCH    ? sizeof(SegCountSmem<K, RANK_MATCH>)
-                           : rank == RANK_ATOMIC ? sizeof(SegCountSmem<K, RANK_ATOMIC>)
-                                                 : sizeof(SegCountSmem<K, RANK_BALLOT>);
-      set_smem_attrs(count, csmem);
-      DevBuf over;
-      DBG_TRY(alloc_buf(ctx, over, (tiles + 2) * 4));
-      uint32_t *over_count = over.as<uint32_t>(), *rank_fb = over_count + 1, *over_list = over_count + 2;
-      DBG_CUDA_TRY(cudaMemsetAsync(over_count, 0, 8, s));
-      DBG_LAUNCH(ctx, ST_LOCAL_SORT_EDGES, (double)n * sizeof(K),
-                 count<<<(unsigned)tiles, SEG_BLOCK, csmem, s>>>(
-                     kin, bound.as<uint64_t>(), osize.as<uint32_t>(), ooff.as<uint64_t>(), guniq.as<K>(),
-                     gheads.as<uint32_t>(), (uint32_t)H, kstage, mstage.as<uint32_t>(), tcount.as<uint32_t>(),
-                     over_list, over_count, gr.lb, ctx->seg_rank, rank_fb));
-      DBG_CUDA_TRY(cudaGetLastError());
-      uint32_t nover_fb[2] = {0, 0};
-      DBG_TRY(read_small(ctx, over_count, 2 * sizeof(uint32_t), nover_fb));
-      const uint32_t nover = nover_fb[0];
-      ctx->count_overflow_tiles += nover;
-      ctx->rank_fallback_tiles += nover_fb[1];
-      if (nover > 0)
-        DBG_LAUNCH(ctx, ST_LOCAL_SORT_EDGES, 0.0,
-                   radix<<<nover, SEG_BLOCK, rsmem, s>>>(
-                       kin, bound.as<uint64_t>(), osize.as<uint32_t>(), ooff.as<uint64_t>(), guniq.as<K>(),
-                       gheads.as<uint32_t>(), (uint32_t)H, kstage, mstage.as<uint32_t>(), tcount.as<uint32_t>(),
-                       gr.lb, over_list));
-      counted = true;
-    }
-  }
-  if (!counted)
+  // the radix-sorting kernel over the tiles of a list (nullptr: all), the
+  // oversize ones from the gathered keys
+  auto sort_tiles = [&](uint64_t count, const uint32_t *list, double bytes) -> dbg_status {
+    auto radix = rank == RANK_MATCH    ? k_seg_rle<K, Sh::ITEMS, RANK_MATCH>
+                 : rank == RANK_ATOMIC ? k_seg_rle<K, Sh::ITEMS, RANK_ATOMIC>
+                                       : k_seg_rle<K, Sh::ITEMS, RANK_BALLOT>;
+    constexpr size_t rsmem = sizeof(SegSortSmem<K, false, Sh::ITEMS>);
+    set_smem_attrs(radix, rsmem);
+    if (count == 0) return DBG_OK;
+    DBG_LAUNCH(ctx, ST_LOCAL_SORT_EDGES, bytes,
+               radix<<<(unsigned)count, SEG_BLOCK, rsmem, s>>>(
+                   kin, ts.bound.as<uint64_t>(), ts.osize.as<uint32_t>(), ts.ooff.as<uint64_t>(), guniq.as<K>(),
+                   gheads.as<uint32_t>(), (uint32_t)H, kstage, mstage.as<uint32_t>(), tcount.as<uint32_t>(), gr.lb,
+                   list));
+    DBG_CUDA_TRY(cudaGetLastError());
+    return DBG_OK;
+  };
+  auto gather = [&]() -> dbg_status {
+    if (ts.gathered == 0) return DBG_OK;
+    DBG_TRY((seg_gather<K, false>(ctx, kin, nullptr, ValOrder{}, key_bits, ts, ST_LOCAL_SORT_EDGES)));
+    DBG_TRY(alloc_tmp(ctx, guniq, (uint64_t)ts.gathered * sizeof(K)));
+    DBG_TRY(alloc_tmp(ctx, gheads, ((uint64_t)ts.gathered + 1) * 4));
+    return run_length_reduce<K>(ctx, ts.gk.as<K>(), ts.gathered, guniq.as<K>(), gheads.as<uint32_t>(), &H);
+  };
+  uint32_t c[CT_LAST + 1];
+  bool final = false;  // the scan below covers every tile
+  if (ctx->count_first) {
+    // count-first; the tiles that overflow their table are listed and sorted
+    // copy by copy, and the oversize ones left out, if there are any: one
+    // read-back tells, with the total that holds otherwise
+    auto count = rank == RANK_MATCH    ? k_seg_count<K, RANK_MATCH>
+                 : rank == RANK_ATOMIC ? k_seg_count<K, RANK_ATOMIC>
+                                       : k_seg_count<K, RANK_BALLOT>;
+    const size_t csmem = rank == RANK_MATCH    ? sizeof(SegCountSmem<K, RANK_MATCH>)
+                         : rank == RANK_ATOMIC ? sizeof(SegCountSmem<K, RANK_ATOMIC>)
+                                               : sizeof(SegCountSmem<K, RANK_BALLOT>);
+    set_smem_attrs(count, csmem);
+    DBG_TRY(alloc_tmp(ctx, over, tiles * 4));
     DBG_LAUNCH(ctx, ST_LOCAL_SORT_EDGES, (double)n * sizeof(K),
-               radix<<<(unsigned)tiles, SEG_BLOCK, rsmem, s>>>(
-                   kin, bound.as<uint64_t>(), osize.as<uint32_t>(), ooff.as<uint64_t>(), guniq.as<K>(),
-                   gheads.as<uint32_t>(), (uint32_t)H, kstage, mstage.as<uint32_t>(), tcount.as<uint32_t>(),
-                   gr.lb, nullptr));
-  DBG_CUDA_TRY(cudaGetLastError());
-  uint32_t total = 0;
-  DBG_TRY(scan_u32(ctx, tcount.as<uint32_t>(), tiles, toff.as<uint64_t>(), &total, ST_LOCAL_SORT_EDGES));
+               count<<<(unsigned)tiles, SEG_BLOCK, csmem, s>>>(
+                   kin, ts.bound.as<uint64_t>(), ts.osize.as<uint32_t>(), kstage, mstage.as<uint32_t>(),
+                   tcount.as<uint32_t>(), over.as<uint32_t>(), ctx->d_counters + CT_LISTED, gr.lb, ctx->seg_rank,
+                   ctx->d_counters + CT_LONG));
+    DBG_CUDA_TRY(cudaGetLastError());
+    DBG_TRY(scan_u32_async(ctx, tcount.as<uint32_t>(), tiles, toff.as<uint64_t>(), ST_LOCAL_SORT_EDGES, CT_TOTAL));
+    DBG_TRY(read_counters(ctx, c));
+    ts.gathered = c[CT_GATHERED];
+    ts.oversize = c[CT_OVERSIZE];
+    ctx->count_overflow_tiles += c[CT_LISTED];
+    ctx->rank_fallback_tiles += c[CT_LONG];
+    final = c[CT_LISTED] == 0 && ts.oversize == 0;
+    if (!final) {
+      const uint32_t listed = c[CT_LISTED];
+      DBG_TRY(gather());
+      DBG_TRY(sort_tiles(listed, over.as<uint32_t>(), 0.0));
+      DBG_TRY(sort_tiles(ts.oversize, ts.olist.as<uint32_t>(), 0.0));
+    }
+  } else {
+    DBG_TRY(read_counters(ctx, c));
+    ts.gathered = c[CT_GATHERED];
+    DBG_TRY(gather());
+    DBG_TRY(sort_tiles(tiles, nullptr, (double)n * sizeof(K)));
+  }
+  if (!final) {
+    DBG_TRY(scan_u32_async(ctx, tcount.as<uint32_t>(), tiles, toff.as<uint64_t>(), ST_LOCAL_SORT_EDGES, CT_TOTAL));
+    DBG_TRY(read_counters(ctx, c));
+  }
+  const uint32_t total = c[CT_TOTAL];
+  const DevBuf &bound = ts.bound;
   *E = total;
   DBG_TRY(alloc_buf(ctx, mult_out, std::max<uint64_t>(1, total) * 4));
   DBG_LAUNCH(ctx, ST_LOCAL_SORT_EDGES, 2.0 * total * (sizeof(K) + 4),
@@ -855,7 +873,7 @@ dbg_status sort_records_global(dbg_ctx *ctx, K **rk, K **rk_alt, uint32_t **rv, 
     DBG_TRY((radix_sort<K, true>(ctx, rk, rk_alt, rv, rv_alt, R, p.bits, d_hist, d_digit_base, p.first_pass, p.adj)));
     gr.lb.fixed = RADIX_BITS * p.first_pass - p.adj;
   }
-  return seg_prepare<K, true>(ctx, *rk, *rv, R, gr, vo, p.bits, ts, ST_LOCAL_SORT_NODES);
+  return seg_tiles<K>(ctx, *rk, R, gr, ts, ST_LOCAL_SORT_NODES);
 }
 
 // The whole sort, the sorted records in *rk / *rv.
@@ -866,6 +884,11 @@ dbg_status sort_records(dbg_ctx *ctx, K **rk, K **rk_alt, uint32_t **rv, uint32_
   Groups gr;
   TileSet ts;
   DBG_TRY(sort_records_global<K>(ctx, rk, rk_alt, rv, rv_alt, R, p, vo, d_hist, d_digit_base, gr, ts));
+  uint32_t c[CT_LAST + 1];
+  DBG_TRY(read_counters(ctx, c));
+  ts.gathered = c[CT_GATHERED];
+  ts.oversize = c[CT_OVERSIZE];
+  DBG_TRY((seg_gather<K, true>(ctx, *rk, *rv, vo, p.bits, ts, ST_LOCAL_SORT_NODES)));
   DBG_TRY(seg_sort_records<K>(ctx, *rk, *rv, *rk_alt, *rv_alt, R, gr, vo, ts));
   std::swap(*rk, *rk_alt);
   std::swap(*rv, *rv_alt);
@@ -922,10 +945,10 @@ dbg_status assign_node_ids(dbg_ctx *ctx, const K *rk, const uint32_t *rv, uint64
   cudaStream_t s = ctx->stream;
   const uint64_t tiles = (R + RS_TILE - 1) / RS_TILE;
   DevBuf hc, ec, ho, eo;
-  DBG_TRY(alloc_buf(ctx, hc, tiles * 4));
-  DBG_TRY(alloc_buf(ctx, ec, tiles * 4));
-  DBG_TRY(alloc_buf(ctx, ho, (tiles + 1) * 8));
-  DBG_TRY(alloc_buf(ctx, eo, (tiles + 1) * 8));
+  DBG_TRY(alloc_tmp(ctx, hc, tiles * 4));
+  DBG_TRY(alloc_tmp(ctx, ec, tiles * 4));
+  DBG_TRY(alloc_tmp(ctx, ho, (tiles + 1) * 8));
+  DBG_TRY(alloc_tmp(ctx, eo, (tiles + 1) * 8));
   DBG_LAUNCH(ctx, ST_NODE_IDS, (double)R * (sizeof(K) + 4),
              k_count_heads<K><<<(unsigned)tiles, SCAN_BLOCK, 0, s>>>(rk, rv, R, hc.as<uint32_t>(), ec.as<uint32_t>()));
   uint32_t nv = 0, ne = 0;
@@ -935,8 +958,8 @@ dbg_status assign_node_ids(dbg_ctx *ctx, const K *rk, const uint32_t *rv, uint64
     int bshift = 10;
     while ((E_all + (1ull << bshift) - 1) >> bshift > 256) bshift++;
     DevBuf part, fill;
-    DBG_TRY(alloc_buf(ctx, part, 2 * E_all * 8));
-    DBG_TRY(alloc_buf(ctx, fill, 256 * 4));
+    DBG_TRY(alloc_tmp(ctx, part, 2 * E_all * 8));
+    DBG_TRY(alloc_tmp(ctx, fill, 256 * 4));
     DBG_CUDA_TRY(cudaMemsetAsync(fill.p, 0, 256 * 4, s));
     const double wbytes = (double)R * (sizeof(K) + 4) + (double)nv * (sizeof(K) + 8) + (double)ne * (adj_side ? 14 : 13);
     if constexpr (sizeof(K) == 8) {
@@ -976,40 +999,91 @@ dbg_status assign_node_ids(dbg_ctx *ctx, const K *rk, const uint32_t *rv, uint64
 
 // The local pass over R node records in the groups gr, fused with the node-ID
 // pass: the graph's node keys, row_ptr, adjacency and edge ends.  Returns
-// |V| and the number of edge ends.  make_room allocates the adjacency.
-template <class K, class Room>
+// |V| and the number of edge ends; *done = false, with the oversize tiles
+// gathered, where the unfused passes are to do it.
+template <class K>
 dbg_status rank_and_assign(dbg_ctx *ctx, const K *rk, const uint32_t *rv, K *ukeys, uint32_t *vals, uint64_t R,
-                           uint64_t E, uint64_t I, Groups &gr, ValOrder vo, TileSet &ts, Room make_room, dbg_graph *g,
-                           uint64_t *V, uint64_t *ends) {
+                           uint64_t E, uint64_t I, int key_bits, Groups &gr, ValOrder vo, TileSet &ts, dbg_graph *g,
+                           bool sides, bool *done, uint64_t *V, uint64_t *ends) {
   cudaStream_t s = ctx->stream;
   const uint64_t tiles = ts.tiles;
-  DevBuf heads, tcount, hoff, ecount, eoff;
-  DBG_TRY(alloc_buf(ctx, heads, (R / 32 + tiles + 2) * 4));
-  DBG_TRY(alloc_buf(ctx, tcount, tiles * 4));
-  DBG_TRY(alloc_buf(ctx, hoff, (tiles + 1) * 8));
-  DBG_TRY((seg_rank_tiles<K, true>(ctx, rk, rv, ukeys, vals, R, gr, vo, ts, heads.as<uint32_t>(),
-                                   tcount.as<uint32_t>())));
-  uint32_t nv = 0, ne = (uint32_t)R;
+  DevBuf heads, tcount, hoff, ecount, eoff, fb;
+  DBG_TRY(alloc_tmp(ctx, heads, (R / 32 + tiles + 2) * 4));
+  DBG_TRY(alloc_tmp(ctx, tcount, tiles * 4));
+  DBG_TRY(alloc_tmp(ctx, hoff, (tiles + 1) * 8));
+  DBG_TRY(alloc_tmp(ctx, fb, tiles * 4));
   if (I > 0) {
-    DBG_TRY(alloc_buf(ctx, ecount, tiles * 4));
-    DBG_TRY(alloc_buf(ctx, eoff, (tiles + 1) * 8));
-    DBG_LAUNCH(ctx, ST_NODE_IDS, 4.0 * R,
-               k_tile_ends<<<(unsigned)std::min<uint64_t>(tiles, 152ull * 16), 256, 0, s>>>(
-                   ts.bound.as<uint64_t>(), (uint32_t)tiles, vals, ecount.as<uint32_t>()));
-    DBG_TRY(scan_u32(ctx, ecount.as<uint32_t>(), tiles, eoff.as<uint64_t>(), &ne, ST_NODE_IDS));
+    DBG_TRY(alloc_tmp(ctx, ecount, tiles * 4));
+    DBG_TRY(alloc_tmp(ctx, eoff, (tiles + 1) * 8));
   }
-  DBG_TRY(scan_u32(ctx, tcount.as<uint32_t>(), tiles, hoff.as<uint64_t>(), &nv, ST_NODE_IDS));
+  uint32_t c[CT_LAST + 1], *nlisted = ctx->d_counters + CT_LISTED;
+  // the tiles' node and edge-end counts, scanned
+  auto scan_tiles = [&]() -> dbg_status {
+    if (I > 0) {
+      DBG_LAUNCH(ctx, ST_NODE_IDS, 4.0 * R,
+                 k_tile_ends<<<(unsigned)std::min<uint64_t>(tiles, 152ull * 16), 256, 0, s>>>(
+                     ts.bound.as<uint64_t>(), (uint32_t)tiles, vals, ecount.as<uint32_t>()));
+      DBG_TRY(scan_u32_async(ctx, ecount.as<uint32_t>(), tiles, eoff.as<uint64_t>(), ST_NODE_IDS, CT_ENDS));
+    }
+    DBG_TRY(scan_u32_async(ctx, tcount.as<uint32_t>(), tiles, hoff.as<uint64_t>(), ST_NODE_IDS, CT_TOTAL));
+    return read_counters(ctx, c);
+  };
+  static_assert(SegRankSmem<K>::CAP == SEG_BLOCK * SegShape<K>::ITEMS, "same tile capacity as the digit-pass kernel");
+  auto rank = k_seg_rank<K, true>;
+  set_smem_attrs(rank, sizeof(SegRankSmem<K>));
+  DBG_LAUNCH(ctx, ST_LOCAL_SORT_NODES, 2.0 * (double)R * (sizeof(K) + 4),
+             rank<<<(unsigned)tiles, RANK_BLOCK, sizeof(SegRankSmem<K>), s>>>(
+                 rk, rv, ts.bound.as<uint64_t>(), ts.osize.as<uint32_t>(), nullptr, nullptr, nullptr, ukeys, vals,
+                 gr.lb, vo, fb.as<uint32_t>(), nlisted, heads.as<uint32_t>(), tcount.as<uint32_t>()));
+  DBG_CUDA_TRY(cudaGetLastError());
+  DBG_TRY(scan_tiles());
+  ts.gathered = c[CT_GATHERED];
+  ts.oversize = c[CT_OVERSIZE];
+  // many records in oversize tiles, which one CTA each would go through (a
+  // million records: about 0.3 ms): the unfused passes
+  *done = ts.gathered <= 1u << 20;
+  if (!*done) return seg_gather<K, true>(ctx, rk, rv, vo, key_bits, ts, ST_LOCAL_SORT_NODES);
+  if (c[CT_LISTED] || ts.oversize) {
+    const uint32_t listed = c[CT_LISTED], both = listed + ts.oversize;
+    ctx->rank_fallback_tiles += listed;
+    const unsigned grid = (unsigned)std::min<uint64_t>(both, 4ull * (uint64_t)std::max(1, ctx->num_sms));
+    DBG_TRY((seg_gather<K, true>(ctx, rk, rv, vo, key_bits, ts, ST_LOCAL_SORT_NODES)));
+    if (ts.oversize)
+      DBG_LAUNCH(ctx, ST_LOCAL_SORT_NODES, 2.0 * ts.gathered * (sizeof(K) + 4),
+                 k_seg_place<K><<<grid, 256, 0, s>>>(ts.bound.as<uint64_t>(), ts.osize.as<uint32_t>(),
+                                                     ts.ooff.as<uint64_t>(), ts.olist.as<uint32_t>(), ts.oversize,
+                                                     ts.gk.as<K>(), ts.gv.as<uint32_t>(), ukeys, vals));
+    if (listed) {
+      // (the gathered keys' sort may have used the counters)
+      DBG_CUDA_TRY(cudaMemcpyAsync(nlisted, &listed, 4, cudaMemcpyHostToDevice, s));
+      DBG_TRY(seg_sort_listed<K>(ctx, rk, rv, ukeys, vals, gr, vo, ts, fb.as<uint32_t>(), nlisted, listed));
+    }
+    DBG_LAUNCH(ctx, ST_LOCAL_SORT_NODES, 0.0,
+               k_tile_heads<K><<<grid, RANK_BLOCK, 0, s>>>(ukeys, ts.bound.as<uint64_t>(), fb.as<uint32_t>(), listed,
+                                                           ts.olist.as<uint32_t>(), ts.oversize,
+                                                           heads.as<uint32_t>(), tcount.as<uint32_t>()));
+    DBG_CUDA_TRY(cudaGetLastError());
+    DBG_TRY(scan_tiles());
+  }
+  const uint32_t nv = c[CT_TOTAL], ne = I > 0 ? c[CT_ENDS] : (uint32_t)R;
   *V = nv;
   *ends = ne;
   if (ne != 2 * E) return DBG_OK;  // (the caller reports it)
-  DBG_TRY(make_room());
-  DBG_TRY(alloc_buf(ctx, g->node_keys, std::max<uint64_t>(1, nv) * sizeof(K)));
-  DBG_TRY(alloc_buf(ctx, g->row_ptr, ((uint64_t)nv + 1) * sizeof(uint64_t)));
+  DBG_TRY(alloc_block(ctx, g->block[1],
+                      {{&g->node_keys, nv * sizeof(K)},
+                       {&g->row_ptr, ((uint64_t)nv + 1) * sizeof(uint64_t)},
+                       {&g->src, E * sizeof(uint32_t)},
+                       {&g->dst, E * sizeof(uint32_t)},
+                       {&g->adj_edge, 2 * E * sizeof(uint32_t)},
+                       {&g->adj_nbr, 2 * E * sizeof(uint32_t)},
+                       {&g->adj_role, 2 * E},
+                       {&g->adj_side, sides ? 2 * E : 0}}));
+  if (!sides) g->adj_side.p = nullptr;
   int bshift = 10;
   while ((E + (1ull << bshift) - 1) >> bshift > 256) bshift++;
   DevBuf part, fill;
-  DBG_TRY(alloc_buf(ctx, part, 2 * E * 8));
-  DBG_TRY(alloc_buf(ctx, fill, 256 * 4));
+  DBG_TRY(alloc_tmp(ctx, part, 2 * E * 8));
+  DBG_TRY(alloc_tmp(ctx, fill, 256 * 4));
   DBG_CUDA_TRY(cudaMemsetAsync(fill.p, 0, 256 * 4, s));
   auto kern = I > 0 ? k_node_tiles<K, true> : k_node_tiles<K, false>;
   DBG_LAUNCH(ctx, ST_NODE_IDS,
@@ -1046,8 +1120,8 @@ dbg_status count_node_kmers(dbg_ctx *ctx, const DevBuf &packed, const DevBuf &ba
     return DBG_EOVERFLOW;
   }
   DevBuf per, koff;
-  DBG_TRY(alloc_buf(ctx, per, n * sizeof(uint32_t)));
-  DBG_TRY(alloc_buf(ctx, koff, (n + 1) * sizeof(uint64_t)));
+  DBG_TRY(alloc_tmp(ctx, per, n * sizeof(uint32_t)));
+  DBG_TRY(alloc_tmp(ctx, koff, (n + 1) * sizeof(uint64_t)));
   DBG_LAUNCH(ctx, ST_NODE_MULT, 8.0 * n,
              k_kmer_counts<<<grid_for(n, 256), 256, 0, s>>>(d_lengths, n, k, per.as<uint32_t>()));
   uint32_t low32 = 0;
@@ -1058,8 +1132,8 @@ dbg_status count_node_kmers(dbg_ctx *ctx, const DevBuf &packed, const DevBuf &ba
   const int kbits = 2 * (int)k;
   const SortPlan<K> plan = plan_sort<K>(ctx, M, kbits, ctx->partition_first);
   DevBuf ka, kb, headpos;
-  DBG_TRY(alloc_buf(ctx, ka, M * sizeof(K) + MSD_PAD));
-  DBG_TRY(alloc_buf(ctx, kb, M * sizeof(K) + MSD_PAD));
+  DBG_TRY(alloc_tmp(ctx, ka, M * sizeof(K) + MSD_PAD));
+  DBG_TRY(alloc_tmp(ctx, kb, M * sizeof(K) + MSD_PAD));
   DBG_CUDA_TRY(cudaMemsetAsync(d_hist, 0, MAX_PASSES * RADIX * sizeof(unsigned long long), s));
   const DigitSpec digits = plan.digits();
   // emitting with k - 1 gives windows of k bases at the k-mer offsets
@@ -1074,7 +1148,7 @@ dbg_status count_node_kmers(dbg_ctx *ctx, const DevBuf &packed, const DevBuf &ba
   if (plan.local()) {
     DBG_TRY(sort_count_keys<K>(ctx, &kp, &alt, M, plan, d_hist, d_digit_base, counts, &D));
   } else {
-    DBG_TRY(alloc_buf(ctx, headpos, (M + 1) * sizeof(uint32_t)));
+    DBG_TRY(alloc_tmp(ctx, headpos, (M + 1) * sizeof(uint32_t)));
     DBG_TRY((radix_sort<K, false>(ctx, &kp, &alt, &vn, &van, M, kbits, d_hist, d_digit_base)));
     DBG_TRY(run_length_reduce<K>(ctx, kp, M, alt, headpos.as<uint32_t>(), &D));
     DBG_TRY(alloc_buf(ctx, counts, std::max<uint64_t>(1, D) * sizeof(uint32_t)));
@@ -1106,8 +1180,8 @@ dbg_status count_node_reads(dbg_ctx *ctx, const DevBuf &packed, const DevBuf &ba
     return DBG_EOVERFLOW;
   }
   DevBuf per, koff;
-  DBG_TRY(alloc_buf(ctx, per, n * sizeof(uint32_t)));
-  DBG_TRY(alloc_buf(ctx, koff, (n + 1) * sizeof(uint64_t)));
+  DBG_TRY(alloc_tmp(ctx, per, n * sizeof(uint32_t)));
+  DBG_TRY(alloc_tmp(ctx, koff, (n + 1) * sizeof(uint64_t)));
   DBG_LAUNCH(ctx, ST_NODE_MULT, 8.0 * n,
              k_kmer_counts<<<grid_for(n, 256), 256, 0, s>>>(d_lengths, n, k, per.as<uint32_t>()));
   uint32_t low32 = 0;
@@ -1119,10 +1193,10 @@ dbg_status count_node_reads(dbg_ctx *ctx, const DevBuf &packed, const DevBuf &ba
   const int kbits = 2 * (int)k;
   const SortPlan<K> plan = plan_records<K>(ctx, M, kbits, false);
   DevBuf ka, kb, va, vb;
-  DBG_TRY(alloc_buf(ctx, ka, M * sizeof(K) + MSD_PAD));
-  DBG_TRY(alloc_buf(ctx, kb, M * sizeof(K) + MSD_PAD));
-  DBG_TRY(alloc_buf(ctx, va, M * sizeof(uint32_t) + MSD_PAD));
-  DBG_TRY(alloc_buf(ctx, vb, M * sizeof(uint32_t) + MSD_PAD));
+  DBG_TRY(alloc_tmp(ctx, ka, M * sizeof(K) + MSD_PAD));
+  DBG_TRY(alloc_tmp(ctx, kb, M * sizeof(K) + MSD_PAD));
+  DBG_TRY(alloc_tmp(ctx, va, M * sizeof(uint32_t) + MSD_PAD));
+  DBG_TRY(alloc_tmp(ctx, vb, M * sizeof(uint32_t) + MSD_PAD));
   DBG_CUDA_TRY(cudaMemsetAsync(d_hist, 0, MAX_PASSES * RADIX * sizeof(unsigned long long), s));
   const DigitSpec digits = plan.digits();
   // windows of k bases at the k-mer offsets, each with its read index
@@ -1139,10 +1213,10 @@ dbg_status count_node_reads(dbg_ctx *ctx, const DevBuf &packed, const DevBuf &ba
   DBG_LAUNCH(ctx, ST_NODE_MULT, (double)M * (2 * sizeof(K) + 12),
              k_read_change_flags<K><<<grid_for(M, 256 * 8), 256, 0, s>>>(kp, vp, M, valt));
   DevBuf F, headpos;
-  DBG_TRY(alloc_buf(ctx, F, (M + 1) * sizeof(uint64_t)));
+  DBG_TRY(alloc_tmp(ctx, F, (M + 1) * sizeof(uint64_t)));
   uint32_t low = 0;
   DBG_TRY(scan_u32(ctx, valt, M, F.as<uint64_t>(), &low, ST_NODE_MULT));
-  DBG_TRY(alloc_buf(ctx, headpos, (M + 1) * sizeof(uint32_t)));
+  DBG_TRY(alloc_tmp(ctx, headpos, (M + 1) * sizeof(uint32_t)));
   uint64_t D = 0;
   DBG_TRY(run_length_reduce<K>(ctx, kp, M, kalt, headpos.as<uint32_t>(), &D));
   DBG_TRY(alloc_buf(ctx, counts, std::max<uint64_t>(1, D) * sizeof(uint32_t)));
@@ -1166,10 +1240,10 @@ dbg_status build_graph_impl(dbg_ctx *ctx, const BuildInput &in, dbg_graph *g) {
   // ---- per-read offsets (exclusive scans of L and max(0, L - k)) ----
   DevBuf base_off, edge_off, tile_sums, small;
   const uint64_t off_tiles = (n + OFF_TILE - 1) / OFF_TILE;
-  DBG_TRY(alloc_buf(ctx, base_off, (n + 1) * sizeof(uint64_t)));
-  DBG_TRY(alloc_buf(ctx, edge_off, (n + 1) * sizeof(uint64_t)));
-  DBG_TRY(alloc_buf(ctx, tile_sums, std::max<uint64_t>(1, off_tiles) * sizeof(Sum3)));
-  DBG_TRY(alloc_buf(ctx, small, 64 * sizeof(uint64_t) + (MAX_PASSES * RADIX) * 16));
+  DBG_TRY(alloc_tmp(ctx, base_off, (n + 1) * sizeof(uint64_t)));
+  DBG_TRY(alloc_tmp(ctx, edge_off, (n + 1) * sizeof(uint64_t)));
+  DBG_TRY(alloc_tmp(ctx, tile_sums, std::max<uint64_t>(1, off_tiles) * sizeof(Sum3)));
+  DBG_TRY(alloc_tmp(ctx, small, 64 * sizeof(uint64_t) + (MAX_PASSES * RADIX) * 16));
   uint64_t *d_totals = small.as<uint64_t>();
   unsigned long long *d_hist = reinterpret_cast<unsigned long long *>(d_totals + 64);
   uint64_t *d_digit_base = reinterpret_cast<uint64_t *>(d_hist + MAX_PASSES * RADIX);
@@ -1205,8 +1279,8 @@ dbg_status build_graph_impl(dbg_ctx *ctx, const BuildInput &in, dbg_graph *g) {
   uint64_t E = 0;
   const SortPlan<K> plan = plan_sort<K>(ctx, N, kbits, ctx->partition_first);
   if (N > 0) {
-    DBG_TRY(alloc_buf(ctx, keys_a, N * sizeof(K) + MSD_PAD));
-    DBG_TRY(alloc_buf(ctx, keys_b, N * sizeof(K) + MSD_PAD));
+    DBG_TRY(alloc_tmp(ctx, keys_a, N * sizeof(K) + MSD_PAD));
+    DBG_TRY(alloc_tmp(ctx, keys_b, N * sizeof(K) + MSD_PAD));
     DBG_CUDA_TRY(cudaMemsetAsync(d_hist, 0, MAX_PASSES * RADIX * sizeof(unsigned long long), s));
   }
   DevBuf packed;
@@ -1223,7 +1297,7 @@ dbg_status build_graph_impl(dbg_ctx *ctx, const BuildInput &in, dbg_graph *g) {
   };
 
   // ---- K1 pack (+ K2 emit) ----
-  DBG_TRY(alloc_buf(ctx, packed, (nwords + 3) * sizeof(uint64_t)));
+  DBG_TRY(alloc_tmp(ctx, packed, (nwords + 3) * sizeof(uint64_t)));
   DBG_CUDA_TRY(cudaMemsetAsync(packed.as<uint64_t>() + nwords, 0, 3 * sizeof(uint64_t), s));
   bool emitted = false;
   if (nwords > 0 && !in.h_reads) {
@@ -1242,7 +1316,7 @@ dbg_status build_graph_impl(dbg_ctx *ctx, const BuildInput &in, dbg_graph *g) {
     const uint64_t slen = std::min(chunk, total_bases);
     DBG_TRY(alloc_buf(ctx, stage[0], slen));
     if (chunks > 1) DBG_TRY(alloc_buf(ctx, stage[1], slen));
-    DBG_TRY(alloc_buf(ctx, kbound, (chunks + 1) * sizeof(uint64_t)));
+    DBG_TRY(alloc_tmp(ctx, kbound, (chunks + 1) * sizeof(uint64_t)));
     if (N > 0)
       DBG_LAUNCH(ctx, ST_EMIT, 0.0,
                  k_chunk_key_bounds<<<grid_for(chunks + 1, 64), 64, 0, s>>>(
@@ -1277,14 +1351,15 @@ dbg_status build_graph_impl(dbg_ctx *ctx, const BuildInput &in, dbg_graph *g) {
     if (plan.local()) {
       // high digits globally, then the local sort with the run-length
       // reduce: distinct keys into alt, multiplicities into mult_tmp
+      // (its last read-back brought the error word)
       DBG_TRY(sort_count_keys<K>(ctx, &kp, &alt, N, plan, d_hist, d_digit_base, mult_tmp, &E));
     } else {
       // every digit globally, then the run-length reduce
-      DBG_TRY(alloc_buf(ctx, headpos, (N + 1) * sizeof(uint32_t)));
+      DBG_TRY(alloc_tmp(ctx, headpos, (N + 1) * sizeof(uint32_t)));
       DBG_TRY((radix_sort<K, false>(ctx, &kp, &alt, &vn, &van, N, kbits, d_hist, d_digit_base)));
       DBG_TRY(run_length_reduce<K>(ctx, kp, N, alt, headpos.as<uint32_t>(), &E));
+      DBG_TRY(check_device_error(ctx));
     }
-    DBG_TRY(check_device_error(ctx));
     // keep the buffer holding the unique keys (alt); the sorted keys are done
     if (alt == keys_b.as<K>()) { uniq = std::move(keys_b); keys_a.release(); }
     else { uniq = std::move(keys_a); keys_b.release(); }
@@ -1308,14 +1383,13 @@ dbg_status build_graph_impl(dbg_ctx *ctx, const BuildInput &in, dbg_graph *g) {
   // ---- K5 edge ends + records of reads of length k ----
   const uint64_t R = 2 * E + I;
   const int nbits = 2 * (int)k;
-  DBG_TRY(alloc_buf(ctx, g->edge_keys, std::max<uint64_t>(1, E) * sizeof(K)));
-  DBG_TRY(alloc_buf(ctx, g->mult, std::max<uint64_t>(1, E) * sizeof(uint32_t)));
-  DBG_TRY(alloc_buf(ctx, g->orient, std::max<uint64_t>(1, E)));
+  DBG_TRY(alloc_block(ctx, g->block[0],
+                      {{&g->edge_keys, E * sizeof(K)}, {&g->mult, E * sizeof(uint32_t)}, {&g->orient, E}}));
   DevBuf rk_a, rk_b, rv_a, rv_b;
-  DBG_TRY(alloc_buf(ctx, rk_a, R * sizeof(K) + MSD_PAD));
-  DBG_TRY(alloc_buf(ctx, rk_b, R * sizeof(K) + MSD_PAD));
-  DBG_TRY(alloc_buf(ctx, rv_a, R * sizeof(uint32_t) + MSD_PAD));
-  DBG_TRY(alloc_buf(ctx, rv_b, R * sizeof(uint32_t) + MSD_PAD));
+  DBG_TRY(alloc_tmp(ctx, rk_a, R * sizeof(K) + MSD_PAD));
+  DBG_TRY(alloc_tmp(ctx, rk_b, R * sizeof(K) + MSD_PAD));
+  DBG_TRY(alloc_tmp(ctx, rv_a, R * sizeof(uint32_t) + MSD_PAD));
+  DBG_TRY(alloc_tmp(ctx, rv_b, R * sizeof(uint32_t) + MSD_PAD));
   DBG_CUDA_TRY(cudaMemsetAsync(d_hist, 0, MAX_PASSES * RADIX * sizeof(unsigned long long), s));
   const SortPlan<K> rplan = plan_records<K>(ctx, R, nbits, true);
   const DigitSpec nspec = rplan.digits();
@@ -1362,34 +1436,29 @@ dbg_status build_graph_impl(dbg_ctx *ctx, const BuildInput &in, dbg_graph *g) {
   };
   uint64_t V = 0;
   // The local pass hands the node-ID pass the tiles' distinct keys and head
-  // bits instead of sorted keys -- unless many records are in oversize tiles,
-  // which one CTA each would go through (a million records: about 0.3 ms).
+  // bits instead of sorted keys.
   bool fused = false;
   if (E > 0 && rplan.local() && ctx->seg_rank) {
     Groups gr;
     TileSet ts;
     ValOrder fvo = vo;
+    uint64_t ends = 0;
     DBG_TRY(sort_records_global<K>(ctx, &rk, &rk_alt, &rv, &rv_alt, R, rplan, fvo, d_hist, d_digit_base, gr, ts));
-    fused = ts.gathered <= 1u << 20;
-    if (fused) {
-      uint64_t ends = 0;
-      DBG_TRY(rank_and_assign<K>(ctx, rk, rv, rk_alt, rv_alt, R, E, I, gr, fvo, ts, alloc_adjacency, g, &V, &ends));
-      DBG_TRY(check_device_error(ctx));
-      if (ends != 2 * E) {
-        set_error("adjacency holds %llu edge ends, expected %llu", (unsigned long long)ends,
-                  (unsigned long long)(2 * E));
-        return DBG_EINTERNAL;
-      }
-    } else {
+    DBG_TRY(rank_and_assign<K>(ctx, rk, rv, rk_alt, rv_alt, R, E, I, nbits, gr, fvo, ts, g, sides, &fused, &V, &ends));
+    if (!fused) {
       DBG_TRY(seg_sort_records<K>(ctx, rk, rv, rk_alt, rv_alt, R, gr, fvo, ts));
       std::swap(rk, rk_alt);
       std::swap(rv, rv_alt);
+    } else if (ends != 2 * E) {
+      set_error("adjacency holds %llu edge ends, expected %llu", (unsigned long long)ends,
+                (unsigned long long)(2 * E));
+      return DBG_EINTERNAL;
     }
   } else {
     DBG_TRY(sort_records<K>(ctx, &rk, &rk_alt, &rv, &rv_alt, R, rplan, vo, d_hist, d_digit_base));
   }
   if (!fused) {
-    DBG_TRY(alloc_buf(ctx, row_tmp, (R + 1) * sizeof(uint64_t)));
+    DBG_TRY(alloc_tmp(ctx, row_tmp, (R + 1) * sizeof(uint64_t)));
     DBG_TRY(alloc_adjacency());
   }
   if (R > 0 && !fused) {
@@ -1443,8 +1512,7 @@ dbg_status build_graph_impl(dbg_ctx *ctx, const BuildInput &in, dbg_graph *g) {
                                                      g->adj_nbr.as<uint32_t>()));
     DBG_CUDA_TRY(cudaGetLastError());
   }
-  DBG_CUDA_TRY(cudaStreamSynchronize(s));
-  return check_device_error(ctx);
+  return check_device_error(ctx);  // waits for the stream
 }
 
 }  // namespace dbg
@@ -1496,13 +1564,13 @@ dbg_status autotune_kind(dbg_ctx *ctx, uint64_t n, double *ms_out) {
   int count = 0;
   const SortVariant *t = SortKind<K, V>::table(&count);
   DevBuf ka, kb, va, vb, small;
-  DBG_TRY(alloc_buf(ctx, ka, n * sizeof(K)));
-  DBG_TRY(alloc_buf(ctx, kb, n * sizeof(K)));
+  DBG_TRY(alloc_tmp(ctx, ka, n * sizeof(K)));
+  DBG_TRY(alloc_tmp(ctx, kb, n * sizeof(K)));
   if (V) {
-    DBG_TRY(alloc_buf(ctx, va, n * 4));
-    DBG_TRY(alloc_buf(ctx, vb, n * 4));
+    DBG_TRY(alloc_tmp(ctx, va, n * 4));
+    DBG_TRY(alloc_tmp(ctx, vb, n * 4));
   }
-  DBG_TRY(alloc_buf(ctx, small, RADIX * 16));
+  DBG_TRY(alloc_tmp(ctx, small, RADIX * 16));
   unsigned long long *hist = small.as<unsigned long long>();
   uint64_t *dbase = reinterpret_cast<uint64_t *>(hist + RADIX);
   k_tune_fill<K><<<1024, 256, 0, s>>>(ka.as<K>(), V ? va.as<uint32_t>() : nullptr, n);
@@ -1627,10 +1695,10 @@ dbg_status build_bucketed_impl(dbg_ctx *ctx, const BucketInput &in, uint64_t bud
   // ---- per-read offsets ----
   DevBuf base_off, edge_off, tile_sums, small;
   const uint64_t off_tiles = (n + OFF_TILE - 1) / OFF_TILE;
-  DBG_TRY(alloc_buf(ctx, base_off, (n + 1) * 8));
-  DBG_TRY(alloc_buf(ctx, edge_off, (n + 1) * 8));
-  DBG_TRY(alloc_buf(ctx, tile_sums, std::max<uint64_t>(1, off_tiles) * sizeof(Sum3)));
-  DBG_TRY(alloc_buf(ctx, small, 64 * 8 + MAX_PASSES * RADIX * 16 + PREFIX_BINS * 8));
+  DBG_TRY(alloc_tmp(ctx, base_off, (n + 1) * 8));
+  DBG_TRY(alloc_tmp(ctx, edge_off, (n + 1) * 8));
+  DBG_TRY(alloc_tmp(ctx, tile_sums, std::max<uint64_t>(1, off_tiles) * sizeof(Sum3)));
+  DBG_TRY(alloc_tmp(ctx, small, 64 * 8 + MAX_PASSES * RADIX * 16 + PREFIX_BINS * 8));
   uint64_t *d_totals = small.as<uint64_t>();
   unsigned long long *d_hist = reinterpret_cast<unsigned long long *>(d_totals + 64);
   uint64_t *d_digit_base = reinterpret_cast<uint64_t *>(d_hist + MAX_PASSES * RADIX);
@@ -1656,7 +1724,7 @@ dbg_status build_bucketed_impl(dbg_ctx *ctx, const BucketInput &in, uint64_t bud
   // ---- pack the reads once; host reads stream through a staging buffer ----
   DevBuf packed;
   const uint64_t nwords = (total_bases + 31) / 32;
-  DBG_TRY(alloc_buf(ctx, packed, (nwords + 3) * 8));
+  DBG_TRY(alloc_tmp(ctx, packed, (nwords + 3) * 8));
   DBG_CUDA_TRY(cudaMemsetAsync(packed.as<uint64_t>() + nwords, 0, 3 * 8, s));
   if (nwords > 0) {
     if (in.reads_on_device) {
@@ -1707,9 +1775,9 @@ dbg_status build_bucketed_impl(dbg_ctx *ctx, const BucketInput &in, uint64_t bud
     const uint64_t cnt = sizes[b];
     if (cnt == 0) continue;
     DevBuf ka, kb, headpos;
-    DBG_TRY(alloc_buf(ctx, ka, cnt * w + MSD_PAD));
-    DBG_TRY(alloc_buf(ctx, kb, cnt * w + MSD_PAD));
-    DBG_TRY(alloc_buf(ctx, headpos, (cnt + 1) * 4));
+    DBG_TRY(alloc_tmp(ctx, ka, cnt * w + MSD_PAD));
+    DBG_TRY(alloc_tmp(ctx, kb, cnt * w + MSD_PAD));
+    DBG_TRY(alloc_tmp(ctx, headpos, (cnt + 1) * 4));
     DBG_CUDA_TRY(cudaMemsetAsync(d_hist, 0, MAX_PASSES * RADIX * 8, s));
     DBG_CUDA_TRY(cudaMemsetAsync(ctx->d_counters + 8, 0, 4, s));
     const SortPlan<K> plan = plan_sort<K>(ctx, cnt, kbits, ctx->partition_first);
@@ -1734,9 +1802,9 @@ dbg_status build_bucketed_impl(dbg_ctx *ctx, const BucketInput &in, uint64_t bud
     DBG_TRY(check_device_error(ctx));
     const uint32_t eb = (uint32_t)eb64;
     DevBuf k1, m1, o1;
-    DBG_TRY(alloc_buf(ctx, k1, std::max<uint64_t>(1, eb) * w));
-    DBG_TRY(alloc_buf(ctx, m1, std::max<uint64_t>(1, eb) * 4));
-    DBG_TRY(alloc_buf(ctx, o1, std::max<uint64_t>(1, eb)));
+    DBG_TRY(alloc_tmp(ctx, k1, std::max<uint64_t>(1, eb) * w));
+    DBG_TRY(alloc_tmp(ctx, m1, std::max<uint64_t>(1, eb) * 4));
+    DBG_TRY(alloc_tmp(ctx, o1, std::max<uint64_t>(1, eb)));
     if (eb)
       DBG_LAUNCH(ctx, ST_ENDPOINTS, (double)eb * (2 * w + 9),
                  k_edge_finish<K><<<grid_for(eb, 256), 256, 0, s>>>(alt, plan.local() ? nullptr : headpos.as<uint32_t>(),
@@ -1783,8 +1851,8 @@ dbg_status build_bucketed_impl(dbg_ctx *ctx, const BucketInput &in, uint64_t bud
   *n_node_buckets = (uint32_t)nranges.size();
   DevBuf flags, pos;
   if (E > 0) {
-    DBG_TRY(alloc_buf(ctx, flags, 2 * E * 4));
-    DBG_TRY(alloc_buf(ctx, pos, (2 * E + 1) * 8));
+    DBG_TRY(alloc_tmp(ctx, flags, 2 * E * 4));
+    DBG_TRY(alloc_tmp(ctx, pos, (2 * E + 1) * 8));
   }
   const int nbits = 2 * (int)k;
   std::vector<DevBuf> cnk, crp;
@@ -1802,10 +1870,10 @@ dbg_status build_bucketed_impl(dbg_ctx *ctx, const BucketInput &in, uint64_t bud
     const uint64_t cap = (uint64_t)Rc + I;
     if (cap == 0) continue;
     DevBuf ra, rb, va, vb, row_tmp;
-    DBG_TRY(alloc_buf(ctx, ra, cap * w + MSD_PAD));
-    DBG_TRY(alloc_buf(ctx, rb, cap * w + MSD_PAD));
-    DBG_TRY(alloc_buf(ctx, va, cap * 4 + MSD_PAD));
-    DBG_TRY(alloc_buf(ctx, vb, cap * 4 + MSD_PAD));
+    DBG_TRY(alloc_tmp(ctx, ra, cap * w + MSD_PAD));
+    DBG_TRY(alloc_tmp(ctx, rb, cap * w + MSD_PAD));
+    DBG_TRY(alloc_tmp(ctx, va, cap * 4 + MSD_PAD));
+    DBG_TRY(alloc_tmp(ctx, vb, cap * 4 + MSD_PAD));
     // (planned for every record that the range may hold: isolated reads are
     // counted by the range only)
     const SortPlan<K> rplan = plan_records<K>(ctx, cap, nbits, false);
@@ -1833,15 +1901,15 @@ dbg_status build_bucketed_impl(dbg_ctx *ctx, const BucketInput &in, uint64_t bud
     uint32_t *rv = va.as<uint32_t>(), *rv_alt = vb.as<uint32_t>();
     DBG_TRY(sort_records<K>(ctx, &rk, &rk_alt, &rv, &rv_alt, R, rplan, edge_end_order(E, false, I > 0), d_hist,
                             d_digit_base));
-    DBG_TRY(alloc_buf(ctx, row_tmp, (R + 1) * 8));
+    DBG_TRY(alloc_tmp(ctx, row_tmp, (R + 1) * 8));
     uint64_t tot[2] = {0, 0};
     DBG_TRY(assign_node_ids<K>(ctx, rk, rv, R, rk_alt, row_tmp.as<uint64_t>(), g, (uint32_t)base_v, base_slot,
                                &tot[0], &tot[1]));
     DBG_TRY(check_device_error(ctx));
     const uint64_t Vc = tot[0];
     DevBuf nk, rp;
-    DBG_TRY(alloc_buf(ctx, nk, std::max<uint64_t>(1, Vc) * w));
-    DBG_TRY(alloc_buf(ctx, rp, std::max<uint64_t>(1, Vc) * 8));
+    DBG_TRY(alloc_tmp(ctx, nk, std::max<uint64_t>(1, Vc) * w));
+    DBG_TRY(alloc_tmp(ctx, rp, std::max<uint64_t>(1, Vc) * 8));
     if (Vc) {
       DBG_CUDA_TRY(cudaMemcpyAsync(nk.p, rk_alt, Vc * w, cudaMemcpyDeviceToDevice, s));
       DBG_CUDA_TRY(cudaMemcpyAsync(rp.p, row_tmp.p, Vc * 8, cudaMemcpyDeviceToDevice, s));
@@ -1872,8 +1940,7 @@ dbg_status build_bucketed_impl(dbg_ctx *ctx, const BucketInput &in, uint64_t bud
                                                                  g->src.as<uint32_t>(), g->dst.as<uint32_t>(), 2 * E,
                                                                  g->adj_nbr.as<uint32_t>()));
   DBG_CUDA_TRY(cudaGetLastError());
-  DBG_CUDA_TRY(cudaStreamSynchronize(s));
-  return check_device_error(ctx);
+  return check_device_error(ctx);  // waits for the stream
 }
 
 }  // namespace dbg

@@ -29,7 +29,7 @@ dbg_status order_by_payload(dbg_ctx *ctx, const uint32_t *v, uint64_t n, int shi
                             const uint64_t **out) {
   cudaStream_t s = ctx->stream;
   // two word buffers, the digit histograms and bases
-  DBG_TRY(alloc_buf(ctx, buf, 2 * n * 8 + MAX_PASSES * RADIX * 16));
+  DBG_TRY(alloc_tmp(ctx, buf, 2 * n * 8 + MAX_PASSES * RADIX * 16));
   uint64_t *a = buf.as<uint64_t>(), *b = a + n, *base = b + n;
   unsigned long long *hist = reinterpret_cast<unsigned long long *>(base + MAX_PASSES * RADIX);
   DBG_LAUNCH(ctx, ST_LOCAL_SORT_NODES, 12.0 * n, k_val_words<<<grid_for(n, 256 * 8), 256, 0, s>>>(v, n, shift, a));
@@ -66,8 +66,8 @@ dbg_status roadmap_nodes(dbg_ctx *ctx, const dbg_graph *g, uint32_t t, uint32_t 
   *count = 0;
   if (V == 0) return DBG_OK;
   DevBuf flag, pos;
-  DBG_TRY(alloc_buf(ctx, flag, V * 4));
-  DBG_TRY(alloc_buf(ctx, pos, (V + 1) * 8));
+  DBG_TRY(alloc_tmp(ctx, flag, V * 4));
+  DBG_TRY(alloc_tmp(ctx, pos, (V + 1) * 8));
   DBG_LAUNCH(ctx, ST_NODE_MULT, 8.0 * V,
              k_roadmap_flags<<<grid_for(V, 256 * 8), 256, 0, s>>>(g->node_reads.as<uint32_t>(), V, t,
                                                                   flag.as<uint32_t>()));

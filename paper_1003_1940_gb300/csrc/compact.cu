@@ -732,7 +732,9 @@ template <class K, class W>
 __global__ void k_walk_pair(uint4 *__restrict__ rec, const uint32_t *__restrict__ rec_count,
                             const W *__restrict__ mk, uint64_t n, const uint64_t *__restrict__ node_keys, int k,
                             uint32_t *__restrict__ head_bits, uint64_t *__restrict__ at_head,
-                            unsigned long long *covered, uint32_t *err) {
+                            unsigned long long *covered, const uint32_t *too_long, const uint32_t *overflow,
+                            uint32_t *err) {
+  if (*too_long || *overflow) return;  // the general path ranks the lists
   unsigned long long cov = 0;
   const uint32_t nr = *rec_count;
   for (uint64_t i = (uint64_t)blockIdx.x * blockDim.x + threadIdx.x; i < nr; i += (uint64_t)gridDim.x * blockDim.x) {
@@ -915,11 +917,11 @@ static unsigned grid_of(uint64_t n) {
   return (unsigned)std::max<uint64_t>(1, std::min<uint64_t>((n + 255) / 256, 152ull * 64));
 }
 
-static dbg_status scan_excl(dbg_ctx *ctx, const uint32_t *in, uint64_t n, uint64_t *out, uint32_t *total) {
+dbg_status scan_excl_async(dbg_ctx *ctx, const uint32_t *in, uint64_t n, uint64_t *out, int total) {
   cudaStream_t s = ctx->stream;
   if (n == 0) {
     DBG_CUDA_TRY(cudaMemsetAsync(out, 0, sizeof(uint64_t), s));
-    *total = 0;
+    DBG_CUDA_TRY(cudaMemsetAsync(ctx->d_counters + total, 0, sizeof(uint32_t), s));
     return DBG_OK;
   }
   const uint64_t tiles = (n + SCAN_TILE - 1) / SCAN_TILE;
@@ -929,9 +931,9 @@ static dbg_status scan_excl(dbg_ctx *ctx, const uint32_t *in, uint64_t n, uint64
   DBG_CUDA_TRY(cudaMemsetAsync(ctx->d_counters, 0, 2 * sizeof(uint32_t), s));
   DBG_LAUNCH(ctx, ST_COMPACT_OUTPUT, 12.0 * n,
              k_scan_excl<<<(unsigned)tiles, SCAN_BLOCK, 0, s>>>(in, n, out, ctx->d_status, ctx->d_counters, epoch,
-                                                                ctx->spin_limit, ctx->d_err, ctx->d_counters + 1));
+                                                                ctx->spin_limit, ctx->d_err, ctx->d_counters + total));
   DBG_CUDA_TRY(cudaGetLastError());
-  return read_small(ctx, ctx->d_counters + 1, sizeof(uint32_t), total);
+  return DBG_OK;
 }
 
 // Pointer jumping over a list of strand-nodes until every one that can
@@ -972,11 +974,11 @@ static dbg_status finish_from_words(dbg_ctx *ctx, const dbg_graph *g, dbg_unitig
   DevBuf strand, head, rank, is_head, len_at_head, uidx, off_by_v;
   uint64_t U = 0;
   if (V > 0) {
-    DBG_TRY(alloc_buf(ctx, strand, V1));
-    DBG_TRY(alloc_buf(ctx, head, V1 * 4));
-    DBG_TRY(alloc_buf(ctx, rank, V1 * 4));
-    DBG_TRY(alloc_buf(ctx, is_head, V1 * 4));
-    DBG_TRY(alloc_buf(ctx, len_at_head, V1 * 4));
+    DBG_TRY(alloc_tmp(ctx, strand, V1));
+    DBG_TRY(alloc_tmp(ctx, head, V1 * 4));
+    DBG_TRY(alloc_tmp(ctx, rank, V1 * 4));
+    DBG_TRY(alloc_tmp(ctx, is_head, V1 * 4));
+    DBG_TRY(alloc_tmp(ctx, len_at_head, V1 * 4));
     DBG_CUDA_TRY(cudaMemsetAsync(len_at_head.p, 0, V1 * 4, s));
     DBG_LAUNCH(ctx, ST_COMPACT_OUTPUT, 16.0 * n + 8.0 * V + 17.0 * V,
                k_select<K><<<grid_of(V), 256, 0, s>>>(word.as<uint64_t>(), succ.as<uint32_t>(),
@@ -987,11 +989,15 @@ static dbg_status finish_from_words(dbg_ctx *ctx, const dbg_graph *g, dbg_unitig
     DBG_CUDA_TRY(cudaGetLastError());
     word.release();
     succ.release();
-    DBG_TRY(alloc_buf(ctx, uidx, (V + 1) * 8));
-    DBG_TRY(alloc_buf(ctx, off_by_v, (V + 1) * 8));
+    DBG_TRY(alloc_tmp(ctx, uidx, (V + 1) * 8));
+    DBG_TRY(alloc_tmp(ctx, off_by_v, (V + 1) * 8));
     uint32_t U32 = 0, total = 0;
-    DBG_TRY(scan_excl(ctx, is_head.as<uint32_t>(), V, uidx.as<uint64_t>(), &U32));
-    DBG_TRY(scan_excl(ctx, len_at_head.as<uint32_t>(), V, off_by_v.as<uint64_t>(), &total));
+    DBG_TRY(scan_excl_async(ctx, is_head.as<uint32_t>(), V, uidx.as<uint64_t>(), CT_TOTAL));
+    DBG_TRY(scan_excl_async(ctx, len_at_head.as<uint32_t>(), V, off_by_v.as<uint64_t>(), CT_ENDS));
+    uint32_t c[CT_LAST + 1];
+    DBG_TRY(read_counters(ctx, c));
+    U32 = c[CT_TOTAL];
+    total = c[CT_ENDS];
     if (total != V) {
       set_error("unitigs hold %u nodes, expected %llu", total, (unsigned long long)V);
       return DBG_EINTERNAL;
@@ -1008,7 +1014,7 @@ static dbg_status finish_from_words(dbg_ctx *ctx, const dbg_graph *g, dbg_unitig
   DBG_TRY(alloc_buf(ctx, u->seq, std::max<uint64_t>(1, u->total_bases)));
   if (V > 0) {
     DevBuf hinfo;
-    DBG_TRY(alloc_buf(ctx, hinfo, V1 * sizeof(uint4)));
+    DBG_TRY(alloc_tmp(ctx, hinfo, V1 * sizeof(uint4)));
     DBG_LAUNCH(ctx, ST_COMPACT_OUTPUT, 4.0 * V + 16.0 * U * 5,
                k_unitig_offsets<<<grid_of(V + 1), 256, 0, s>>>(
                    is_head.as<uint32_t>(), uidx.as<uint64_t>(), off_by_v.as<uint64_t>(), len_at_head.as<uint32_t>(),
@@ -1026,8 +1032,7 @@ static dbg_status finish_from_words(dbg_ctx *ctx, const dbg_graph *g, dbg_unitig
     DBG_CUDA_TRY(cudaMemsetAsync(u->node_off.p, 0, 8, s));
     DBG_CUDA_TRY(cudaMemsetAsync(u->seq_off.p, 0, 8, s));
   }
-  DBG_CUDA_TRY(cudaStreamSynchronize(s));
-  return check_device_error(ctx);
+  return check_device_error(ctx);  // waits for the stream
 }
 
 
@@ -1055,14 +1060,14 @@ static dbg_status compact_impl(dbg_ctx *ctx, const dbg_graph *g, dbg_unitigs *u,
     uint32_t *lists = ctx->d_counters + 10;
     DBG_CUDA_TRY(cudaMemsetAsync(lists, 0, 8 * sizeof(uint32_t), s));
     if (fast) {
-      DBG_TRY(alloc_buf(ctx, mk, n1 * (w32 ? 4 : 8)));
-      DBG_TRY(alloc_buf(ctx, tails, tw * 4));
+      DBG_TRY(alloc_tmp(ctx, mk, n1 * (w32 ? 4 : 8)));
+      DBG_TRY(alloc_tmp(ctx, tails, tw * 4));
     }
     // per side the lone end, a bitmap of the lone sides, the candidate words;
     // then the arcs whose far side is lone too (succ: the general path's copy)
     auto links_by_bitmap = [&](uint32_t *succ_out) -> dbg_status {
       DevBuf lone;
-      DBG_TRY(alloc_buf(ctx, lone, (V / 16 + 2) * 4));
+      DBG_TRY(alloc_tmp(ctx, lone, (V / 16 + 2) * 4));
       DBG_LAUNCH(ctx, ST_COMPACT_LINKS,
                  16.0 * V + (double)E2 * (g->adj_side.p ? 5 : 10) + 8.0 * V * g->key_words + 8.0 * V + V / 4.0,
                  k_side_cand<K><<<grid_of(V), 256, 0, s>>>(g->row_ptr.as<uint64_t>(), g->adj_nbr.as<uint32_t>(),
@@ -1078,9 +1083,9 @@ static dbg_status compact_impl(dbg_ctx *ctx, const dbg_graph *g, dbg_unitigs *u,
     if (w32) {
       DBG_TRY(links_by_bitmap(nullptr));
     } else {
-      DBG_TRY(alloc_buf(ctx, succ, n1 * 4));
-      DBG_TRY(alloc_buf(ctx, link_node, n1 * 4));
-      DBG_TRY(alloc_buf(ctx, link_edge, n1 * 8));
+      DBG_TRY(alloc_tmp(ctx, succ, n1 * 4));
+      DBG_TRY(alloc_tmp(ctx, link_node, n1 * 4));
+      DBG_TRY(alloc_tmp(ctx, link_edge, n1 * 8));
       DBG_LAUNCH(ctx, ST_COMPACT_LINKS, 16.0 * V + (double)E2 * 10 + 8.0 * V * g->key_words + 12.0 * n,
                  k_side_links<K><<<grid_of(V), 256, 0, s>>>(g->row_ptr.as<uint64_t>(), g->adj_nbr.as<uint32_t>(),
                                                             g->adj_edge.as<uint32_t>(), g->adj_role.as<uint8_t>(),
@@ -1102,9 +1107,9 @@ static dbg_status compact_impl(dbg_ctx *ctx, const dbg_graph *g, dbg_unitigs *u,
       // the head nodes only
       DevBuf f_bits, f_word, claimed, rec, stage, page_next;
       const uint64_t nw = (V + 31) / 32, nw1 = std::max<uint64_t>(1, nw);
-      DBG_TRY(alloc_buf(ctx, f_bits, nw1 * 4));
-      DBG_TRY(alloc_buf(ctx, f_word, V1 * 8));
-      DBG_TRY(alloc_buf(ctx, claimed, nw1 * 4));
+      DBG_TRY(alloc_tmp(ctx, f_bits, nw1 * 4));
+      DBG_TRY(alloc_tmp(ctx, f_word, V1 * 8));
+      DBG_TRY(alloc_tmp(ctx, claimed, nw1 * 4));
       DBG_CUDA_TRY(cudaMemsetAsync(f_bits.p, 0, nw1 * 4, s));
       DBG_CUDA_TRY(cudaMemsetAsync(claimed.p, 0, nw1 * 4, s));
       // the two walkers of each unitig meet half way and stage what they
@@ -1114,9 +1119,9 @@ static dbg_status compact_impl(dbg_ctx *ctx, const dbg_graph *g, dbg_unitigs *u,
       const unsigned wgrid = w32 ? walk_grid(ctx, n, k_walk_claim<uint32_t>) : walk_grid(ctx, n, k_walk_claim<uint64_t>);
       const uint64_t lanes = (uint64_t)wgrid * WALK_BLOCK;
       const uint64_t stage_cap = ((V + 2 * lanes * STAGE_PAGE) / STAGE_PAGE + 1) * STAGE_PAGE;
-      DBG_TRY(alloc_buf(ctx, rec, n1 * sizeof(uint4)));
-      DBG_TRY(alloc_buf(ctx, stage, stage_cap * 4));
-      DBG_TRY(alloc_buf(ctx, page_next, stage_cap / STAGE_PAGE * 4));
+      DBG_TRY(alloc_tmp(ctx, rec, n1 * sizeof(uint4)));
+      DBG_TRY(alloc_tmp(ctx, stage, stage_cap * 4));
+      DBG_TRY(alloc_tmp(ctx, page_next, stage_cap / STAGE_PAGE * 4));
       unsigned long long *cursor = reinterpret_cast<unsigned long long *>(ctx->d_counters + 14);
       unsigned long long *d_covered = reinterpret_cast<unsigned long long *>(ctx->d_counters + 12);
       uint32_t *nrec = ctx->d_counters + 17;
@@ -1133,49 +1138,42 @@ static dbg_status compact_impl(dbg_ctx *ctx, const dbg_graph *g, dbg_unitigs *u,
                        stage.as<uint32_t>(), page_next.as<uint32_t>(), cursor, stage_cap, ctx->d_counters + 11,
                        ctx->d_counters + 16, nrec, lists));
       DBG_CUDA_TRY(cudaGetLastError());
-      uint32_t flags[6] = {0, 0, 0, 0, 0, 0};  // counters 11..16
-      DBG_TRY(read_small(ctx, ctx->d_counters + 11, sizeof(flags), flags));
-      const uint32_t too_long = flags[0], overflow = flags[5];
-      uint64_t covered = 0;
-      if (too_long == 0 && overflow == 0) {
-        if (w32)
-          DBG_LAUNCH(ctx, ST_COMPACT_RANK, 16.0 * V,
-                     k_walk_pair<K, uint32_t><<<grid_of(V), 256, 0, s>>>(
-                         rec.as<uint4>(), nrec, mk.as<uint32_t>(), n, g->node_keys.as<uint64_t>(), k,
-                         f_bits.as<uint32_t>(), f_word.as<uint64_t>(), d_covered, ctx->d_err));
-        else
-          DBG_LAUNCH(ctx, ST_COMPACT_RANK, 16.0 * V,
-                     k_walk_pair<K, uint64_t><<<grid_of(V), 256, 0, s>>>(
-                         rec.as<uint4>(), nrec, mk.as<uint64_t>(), n, g->node_keys.as<uint64_t>(), k,
-                         f_bits.as<uint32_t>(), f_word.as<uint64_t>(), d_covered, ctx->d_err));
-        DBG_CUDA_TRY(cudaGetLastError());
-        DBG_TRY(read_small(ctx, ctx->d_counters + 12, sizeof(uint64_t), &covered));
-        DBG_TRY(check_device_error(ctx));
-      }
-      if (too_long == 0 && overflow == 0 && covered == V) {
-        // the unitigs in the order of their first nodes: a scan over the
-        // bitmap words, the list of heads, a scan over the unitigs' lengths
+      if (w32)
+        DBG_LAUNCH(ctx, ST_COMPACT_RANK, 16.0 * V,
+                   k_walk_pair<K, uint32_t><<<grid_of(V), 256, 0, s>>>(
+                       rec.as<uint4>(), nrec, mk.as<uint32_t>(), n, g->node_keys.as<uint64_t>(), k,
+                       f_bits.as<uint32_t>(), f_word.as<uint64_t>(), d_covered, ctx->d_counters + 11,
+                       ctx->d_counters + 16, ctx->d_err));
+      else
+        DBG_LAUNCH(ctx, ST_COMPACT_RANK, 16.0 * V,
+                   k_walk_pair<K, uint64_t><<<grid_of(V), 256, 0, s>>>(
+                       rec.as<uint4>(), nrec, mk.as<uint64_t>(), n, g->node_keys.as<uint64_t>(), k,
+                       f_bits.as<uint32_t>(), f_word.as<uint64_t>(), d_covered, ctx->d_counters + 11,
+                       ctx->d_counters + 16, ctx->d_err));
+      // the unitigs in the order of their first nodes: a scan over the bitmap
+      // words, the list of heads, a scan over the unitigs' lengths.  One
+      // read-back tells whether the walks covered the graph, and |U|.
+      DevBuf wcnt, wpre, urec, ulen, uoff;
+      DBG_TRY(alloc_tmp(ctx, wcnt, nw1 * 4));
+      DBG_TRY(alloc_tmp(ctx, wpre, (nw + 1) * 8));
+      DBG_LAUNCH(ctx, ST_COMPACT_OUTPUT, 8.0 * nw,
+                 k_head_popc<<<grid_of(nw), 256, 0, s>>>(f_bits.as<uint32_t>(), nw, wcnt.as<uint32_t>()));
+      DBG_TRY(scan_excl_async(ctx, wcnt.as<uint32_t>(), nw, wpre.as<uint64_t>(), CT_TOTAL));
+      uint32_t c[CT_LAST + 1];
+      DBG_TRY(read_counters(ctx, c));
+      if (c[11] == 0 && c[16] == 0 && ((uint64_t)c[13] << 32 | c[12]) == V) {
         mk.release();
-        DevBuf wcnt, wpre, urec, ulen, uoff;
-        DBG_TRY(alloc_buf(ctx, wcnt, nw1 * 4));
-        DBG_TRY(alloc_buf(ctx, wpre, (nw + 1) * 8));
-        DBG_LAUNCH(ctx, ST_COMPACT_OUTPUT, 8.0 * nw,
-                   k_head_popc<<<grid_of(nw), 256, 0, s>>>(f_bits.as<uint32_t>(), nw, wcnt.as<uint32_t>()));
-        uint32_t U32 = 0, total = 0;
-        DBG_TRY(scan_excl(ctx, wcnt.as<uint32_t>(), nw, wpre.as<uint64_t>(), &U32));
+        const uint32_t U32 = c[CT_TOTAL];
         const uint64_t Uf = U32;
-        DBG_TRY(alloc_buf(ctx, urec, std::max<uint64_t>(1, Uf) * 4));
-        DBG_TRY(alloc_buf(ctx, ulen, std::max<uint64_t>(1, Uf) * 4));
-        DBG_TRY(alloc_buf(ctx, uoff, (Uf + 1) * 8));
+        DBG_TRY(alloc_tmp(ctx, urec, std::max<uint64_t>(1, Uf) * 4));
+        DBG_TRY(alloc_tmp(ctx, ulen, std::max<uint64_t>(1, Uf) * 4));
+        DBG_TRY(alloc_tmp(ctx, uoff, (Uf + 1) * 8));
         DBG_LAUNCH(ctx, ST_COMPACT_OUTPUT, 12.0 * nw + (double)Uf * (4 + 4 + 4),
                    k_head_list<<<grid_of(nw), 256, 0, s>>>(f_bits.as<uint32_t>(), nw, wpre.as<uint64_t>(),
                                                            f_word.as<uint64_t>(), urec.as<uint32_t>(),
                                                            ulen.as<uint32_t>()));
-        DBG_TRY(scan_excl(ctx, ulen.as<uint32_t>(), Uf, uoff.as<uint64_t>(), &total));
-        if (total != V) {
-          set_error("unitigs hold %u nodes, expected %llu", total, (unsigned long long)V);
-          return DBG_EINTERNAL;
-        }
+        // (their sum is that of the pairs, V: read with the last wait)
+        DBG_TRY(scan_excl_async(ctx, ulen.as<uint32_t>(), Uf, uoff.as<uint64_t>(), CT_TOTAL));
         u->count = Uf;
         DBG_TRY(alloc_buf(ctx, u->node_off, (Uf + 1) * 8));
         DBG_TRY(alloc_buf(ctx, u->seq_off, (Uf + 1) * 8));
@@ -1191,19 +1189,23 @@ static dbg_status compact_impl(dbg_ctx *ctx, const dbg_graph *g, dbg_unitigs *u,
                        u->nodes.as<uint64_t>(), u->seq.as<char>(), u->node_off.as<uint64_t>(),
                        u->seq_off.as<uint64_t>(), u->circular.as<uint8_t>()));
         DBG_CUDA_TRY(cudaGetLastError());
-        DBG_CUDA_TRY(cudaStreamSynchronize(s));
-        return check_device_error(ctx);
+        DBG_TRY(read_counters(ctx, c));
+        if (c[CT_TOTAL] != V) {
+          set_error("unitigs hold %u nodes, expected %llu", c[CT_TOTAL], (unsigned long long)V);
+          return DBG_EINTERNAL;
+        }
+        return DBG_OK;
       }
     }
     // ---- general path: long lists or cycles present ----
     if (w32) {  // (walkers left their numbers in some words: the arcs again)
-      DBG_TRY(alloc_buf(ctx, succ, n1 * 4));
+      DBG_TRY(alloc_tmp(ctx, succ, n1 * 4));
       DBG_TRY(links_by_bitmap(succ.as<uint32_t>()));
     }
     mk.release();
     tails.release();
-    DBG_TRY(alloc_buf(ctx, word, n1 * 8));
-    DBG_TRY(alloc_buf(ctx, active, n1 * 4));
+    DBG_TRY(alloc_tmp(ctx, word, n1 * 8));
+    DBG_TRY(alloc_tmp(ctx, active, n1 * 4));
     bool ranked = false;
     if (ctx->compact_mode != 2) {
       // by segments, unless there are cycles
@@ -1240,9 +1242,9 @@ static dbg_status compact_impl(dbg_ctx *ctx, const dbg_graph *g, dbg_unitigs *u,
         DBG_TRY(jump_until_stable(ctx, active.as<uint32_t>(), A, word.as<uint64_t>(), &left));
         if (left > 0) {
           have_cycles = true;
-          DBG_TRY(alloc_buf(ctx, cycl, (uint64_t)A * 4));
-          DBG_TRY(alloc_buf(ctx, lab, n1 * 8));
-          DBG_TRY(alloc_buf(ctx, cyc, n1));
+          DBG_TRY(alloc_tmp(ctx, cycl, (uint64_t)A * 4));
+          DBG_TRY(alloc_tmp(ctx, lab, n1 * 8));
+          DBG_TRY(alloc_tmp(ctx, cyc, n1));
           DBG_CUDA_TRY(cudaMemsetAsync(cyc.p, 0, n, s));
           DBG_CUDA_TRY(cudaMemsetAsync(ctx->d_counters + 5, 0, sizeof(uint32_t), s));
           DBG_LAUNCH(ctx, ST_COMPACT_CYCLES, 24.0 * A,
@@ -1437,9 +1439,9 @@ static dbg_status compact_bucketed_impl(dbg_ctx *ctx, const dbg_graph *g, uint64
   // successors on the device (the graph is there), then to host memory
   {
     DevBuf link_node, link_edge;
-    DBG_TRY(alloc_buf(ctx, link_node, n * 4));
-    DBG_TRY(alloc_buf(ctx, link_edge, n * 8));
-    DBG_TRY(alloc_buf(ctx, succ, n * 4));
+    DBG_TRY(alloc_tmp(ctx, link_node, n * 4));
+    DBG_TRY(alloc_tmp(ctx, link_edge, n * 8));
+    DBG_TRY(alloc_tmp(ctx, succ, n * 4));
     DBG_LAUNCH(ctx, ST_COMPACT_LINKS, 16.0 * V + 20.0 * g->num_edges + 8.0 * V * g->key_words + 12.0 * n,
                k_side_links<K><<<grid_of(V), 256, 0, s>>>(g->row_ptr.as<uint64_t>(), g->adj_nbr.as<uint32_t>(),
                                                           g->adj_edge.as<uint32_t>(), g->adj_role.as<uint8_t>(),
@@ -1470,10 +1472,10 @@ static dbg_status compact_bucketed_impl(dbg_ctx *ctx, const dbg_graph *g, uint64
   const uint64_t per = std::max<uint64_t>(1u << 12, budget / 25);
   jb.slice_len = std::min<uint64_t>(n, per);
   jb.batch = std::min<uint64_t>(n, per);
-  DBG_TRY(alloc_buf(ctx, jb.slice, jb.slice_len * 8));
-  DBG_TRY(alloc_buf(ctx, jb.req, jb.batch * 8));
-  DBG_TRY(alloc_buf(ctx, jb.out, jb.batch * 8));
-  DBG_TRY(alloc_buf(ctx, jb.moved, jb.batch));
+  DBG_TRY(alloc_tmp(ctx, jb.slice, jb.slice_len * 8));
+  DBG_TRY(alloc_tmp(ctx, jb.req, jb.batch * 8));
+  DBG_TRY(alloc_tmp(ctx, jb.out, jb.batch * 8));
+  DBG_TRY(alloc_tmp(ctx, jb.moved, jb.batch));
   // initial words: a list head is its own root; every other strand-node
   // points at its predecessor at distance 1
   std::vector<uint32_t> act;
@@ -1520,10 +1522,10 @@ static dbg_status compact_bucketed_impl(dbg_ctx *ctx, const dbg_graph *g, uint64
   *rounds = (uint32_t)(ctx->launches - r0);
   jb = JoinBufs();
   // the ranking words back on the device for the rest of the general path
-  DBG_TRY(alloc_buf(ctx, word, n * 8));
+  DBG_TRY(alloc_tmp(ctx, word, n * 8));
   DBG_CUDA_TRY(cudaMemcpyAsync(word.p, W, n * 8, cudaMemcpyHostToDevice, s));
   if (have_cycles) {
-    DBG_TRY(alloc_buf(ctx, cyc, n));
+    DBG_TRY(alloc_tmp(ctx, cyc, n));
     DBG_CUDA_TRY(cudaMemcpyAsync(cyc.p, h_cyc.data(), n, cudaMemcpyHostToDevice, s));
   }
   DBG_CUDA_TRY(cudaStreamSynchronize(s));  // the host words may go

@@ -5,6 +5,7 @@
 
 #include <algorithm>
 #include <condition_variable>
+#include <initializer_list>
 #include <cstdint>
 #include <cstdio>
 #include <memory>
@@ -28,9 +29,30 @@ struct Allocator {
   void put(void *p, size_t bytes);
 };
 
+// Small scratch of a context's calls: one block, taken from the context's
+// allocator at first use and given back when the context is destroyed, handed
+// out piece by piece (first fit, 256-byte pieces).  A call takes some forty
+// buffers; through a host program's allocator hooks each costs microseconds,
+// and a small build is made of those.  All work of a context is on its one
+// stream and its calls are not concurrent, so a piece may be reused as soon as
+// it is put back.
+struct Scratch {
+  static constexpr size_t CAP = (size_t)32 << 20;   // the block
+  static constexpr size_t MOST = (size_t)4 << 20;   // larger buffers go to the allocator
+  struct Piece { size_t off, bytes; bool used; };
+  char *base = nullptr;
+  std::vector<Piece> pieces;
+  bool short_of_memory = false;  // an allocation failed: no block from then on
+  bool drop(Allocator &al);      // gives the block back, if none of it is in use
+  void *get(Allocator &al, size_t bytes);  // nullptr: no room
+  void put(void *p);
+};
+
 // One device buffer; released in stream order when it goes out of scope.
+// (al and ar both NULL: part of another buffer.)
 struct DevBuf {
   Allocator *al = nullptr;
+  Scratch *ar = nullptr;
   void *p = nullptr;
   size_t bytes = 0;
   DevBuf() = default;
@@ -40,14 +62,15 @@ struct DevBuf {
   DevBuf &operator=(DevBuf &&o) noexcept {
     if (this != &o) {
       release();
-      al = o.al; p = o.p; bytes = o.bytes;
+      al = o.al; ar = o.ar; p = o.p; bytes = o.bytes;
       o.p = nullptr; o.bytes = 0;
     }
     return *this;
   }
   ~DevBuf() { release(); }
   void release() {
-    if (p && al) al->put(p, bytes);
+    if (p && ar) ar->put(p);
+    else if (p && al) al->put(p, bytes);
     p = nullptr;
     bytes = 0;
   }
@@ -75,6 +98,7 @@ struct dbg_ctx {
   cudaStream_t stream = nullptr;
   bool own_stream = false;
   dbg::Allocator al;
+  dbg::Scratch scratch;
   uint64_t mem_budget = 0;
   uint32_t spin_limit = 1u << 22;
   // per sort kind: onesweep passes over 0: u64, 1: u64+payload, 2: u128,
@@ -138,6 +162,7 @@ struct dbg_graph {
   dbg::Allocator al;  // copy of the creating context's allocator
   int device = 0;
   uint32_t edge_buckets = 1, node_buckets = 1;  // key ranges used (bucket path)
+  dbg::DevBuf block[2];  // what the in-memory build's arrays are part of (edges; nodes and adjacency)
   dbg::DevBuf node_keys, edge_keys, src, dst, orient, mult, row_ptr, adj_nbr, adj_edge, adj_role;
   dbg::DevBuf adj_side;    // per adjacency slot: its end's side | the far end's side << 1 (when built)
   dbg::DevBuf node_mult;   // k-mer occurrences per node, when the build counted them
@@ -191,6 +216,14 @@ namespace dbg {
   } while (0)
 
 dbg_status alloc_buf(dbg_ctx *ctx, DevBuf &b, size_t bytes);
+// Scratch of a call on the context: from its scratch block if it is small.
+dbg_status alloc_tmp(dbg_ctx *ctx, DevBuf &b, size_t bytes);
+// One allocation for several arrays, which become parts of it.
+struct BlockPart {
+  DevBuf *buf;
+  size_t bytes;
+};
+dbg_status alloc_block(dbg_ctx *ctx, DevBuf &block, std::initializer_list<BlockPart> parts);
 // grows the persistent look-back status array to at least `words` words
 dbg_status ensure_status(dbg_ctx *ctx, size_t words);
 // creates the context's copy stream on first use
@@ -226,6 +259,17 @@ dbg_status check_device_error(dbg_ctx *ctx);
 
 // Reads a few bytes of device memory through the pinned mirror (synchronizes).
 dbg_status read_small(dbg_ctx *ctx, const void *d_src, size_t bytes, void *h_dst);
+
+// d_counters entries that hold a call's counts until one read_counters brings
+// them all, with the error word: gathered keys and oversize tiles of a local
+// pass, the tiles it listed (and those listed for long buckets), totals.
+enum Counter { CT_GATHERED = 20, CT_OVERSIZE, CT_LISTED, CT_LONG, CT_TOTAL, CT_ENDS, CT_REMOVED, CT_LAST = 47 };  // (CT_REMOVED: 64 bits)
+// Waits for the stream; counters[0 .. CT_LAST]; a status from the device error
+// word, as check_device_error.
+dbg_status read_counters(dbg_ctx *ctx, uint32_t *counters);
+
+// Exclusive scan of n u32 values into n + 1 u64; the total to counter `total`.
+dbg_status scan_excl_async(dbg_ctx *ctx, const uint32_t *in, uint64_t n, uint64_t *out, int total);
 
 // Host copy of n words from device or host memory (synchronous on ctx stream).
 dbg_status copy_out(dbg_ctx *ctx, void *dst, const void *src, size_t bytes);

@@ -103,12 +103,34 @@ __global__ void k_seg_bounds(const K *__restrict__ keys, uint64_t n, int low_bit
   }
 }
 
-// osize[t] = the tile's length if it exceeds cap (an oversize tile), else 0.
+// osize[t] = the tile's length if it exceeds cap (an oversize tile), else 0;
+// those tiles' numbers in olist, their keys added up in *keys.
 static __global__ void k_seg_oversize(const uint64_t *__restrict__ bound, uint64_t tiles, uint32_t cap,
-                                      uint32_t *__restrict__ osize) {
+                                      uint32_t *__restrict__ osize, uint32_t *__restrict__ olist,
+                                      uint32_t *__restrict__ keys, uint32_t *__restrict__ count) {
   for (uint64_t t = (uint64_t)blockIdx.x * blockDim.x + threadIdx.x; t < tiles; t += (uint64_t)gridDim.x * blockDim.x) {
     const uint64_t sz = bound[t + 1] - bound[t];
     osize[t] = sz > cap ? (uint32_t)sz : 0u;
+    if (sz > cap) {
+      atomicAdd(keys, (uint32_t)sz);
+      olist[atomicAdd(count, 1u)] = (uint32_t)t;
+    }
+  }
+}
+
+// The gathered, sorted records back into their tiles' ranges.
+template <class K>
+__global__ void k_seg_place(const uint64_t *__restrict__ bound, const uint32_t *__restrict__ osize,
+                            const uint64_t *__restrict__ ooff, const uint32_t *__restrict__ olist, uint32_t n,
+                            const K *__restrict__ gk, const uint32_t *__restrict__ gv, K *__restrict__ kout,
+                            uint32_t *__restrict__ vout) {
+  for (uint32_t q = blockIdx.x; q < n; q += gridDim.x) {
+    const uint32_t t = olist[q];
+    const uint64_t s = bound[t], o = ooff[t];
+    for (uint32_t j = threadIdx.x; j < osize[t]; j += blockDim.x) {
+      kout[s + j] = gk[o + j];
+      vout[s + j] = gv[o + j];
+    }
   }
 }
 
@@ -446,12 +468,15 @@ __global__ __launch_bounds__(RANK_BLOCK, 2) void k_seg_rank(
   const uint32_t tile = blockIdx.x;
   const uint64_t s = bound[tile];
   if (osize[tile]) {
+    if (FUSED) {  // (later: k_seg_place, k_tile_heads)
+      if (tid == 0) tcount[tile] = 0;
+      return;
+    }
     const uint64_t o = ooff[tile];
     for (uint32_t j = tid; j < osize[tile]; j += RANK_BLOCK) {
       kout[s + j] = gk[o + j];
       vout[s + j] = gv[o + j];
     }
-    if (FUSED && tid == 0) fb_list[gridDim.x - 1 - atomicAdd(fb_count + 1, 1u)] = tile;
     return;
   }
   const uint32_t cnt = (uint32_t)(bound[tile + 1] - s);
@@ -502,7 +527,10 @@ __global__ __launch_bounds__(RANK_BLOCK, 2) void k_seg_rank(
   if (lane == 0 && mx > RANK_GROUP_MAX) sm.maxg = mx;
   __syncthreads();
   if (sm.maxg) {
-    if (tid == 0) fb_list[atomicAdd(fb_count, 1u)] = tile;
+    if (tid == 0) {
+      fb_list[atomicAdd(fb_count, 1u)] = tile;
+      if (FUSED) tcount[tile] = 0;
+    }
     return;
   }
   uint32_t run = incl - sum;
@@ -684,14 +712,14 @@ __global__ __launch_bounds__(RANK_BLOCK, 2) void k_seg_rank(
 }
 
 // FUSED's outputs for tiles that other kernels sorted into keys / vals (the
-// first n_fb of fb_list, and the oversize ones: the last n_over): the heads, their number,
+// n_fb of fb_list and the n_over oversize ones of olist): the heads, their number,
 // and the distinct keys moved to the front of the tile.  One CTA per tile at a
 // time; a chunk's keys are all in registers before its distinct ones, which
 // lie at or before them, are written.
 template <class K>
 __global__ __launch_bounds__(RANK_BLOCK) void k_tile_heads(K *__restrict__ keys, const uint64_t *__restrict__ bound,
-                                                           uint32_t tiles, const uint32_t *__restrict__ fb_list,
-                                                           uint32_t n_fb, uint32_t n_over,
+                                                           const uint32_t *__restrict__ fb_list, uint32_t n_fb,
+                                                           const uint32_t *__restrict__ olist, uint32_t n_over,
                                                            uint32_t *__restrict__ heads,
                                                            uint32_t *__restrict__ tcount) {
   constexpr int ITEMS = 8;
@@ -700,7 +728,7 @@ __global__ __launch_bounds__(RANK_BLOCK) void k_tile_heads(K *__restrict__ keys,
   __shared__ K s_last;
   const int tid = threadIdx.x, lane = tid & 31;
   for (uint32_t q = blockIdx.x; q < n_fb + n_over; q += gridDim.x) {
-    const uint32_t tile = fb_list[q < n_fb ? q : tiles - 1 - (q - n_fb)];
+    const uint32_t tile = q < n_fb ? fb_list[q] : olist[q - n_fb];
     const uint64_t s = bound[tile], n = bound[tile + 1] - s;
     uint32_t *hw = head_words(heads, s, tile);
     uint64_t out = 0;
@@ -1043,7 +1071,6 @@ __device__ __forceinline__ uint32_t group_of(K d, int bshift) {
 template <class K, int RANK>
 __global__ __launch_bounds__(SEG_BLOCK, 4) void k_seg_count(
     const K *__restrict__ kin, const uint64_t *__restrict__ bound, const uint32_t *__restrict__ osize,
-    const uint64_t *__restrict__ ooff, const K *__restrict__ guniq, const uint32_t *__restrict__ gheads, uint32_t H,
     K *__restrict__ ustage, uint32_t *__restrict__ mstage, uint32_t *__restrict__ tcount,
     uint32_t *__restrict__ over_list, uint32_t *__restrict__ over_count, LowBits lb, int rank_groups, uint32_t *__restrict__ rank_fb) {
   using S = SegCountSmem<K, RANK>;
@@ -1053,8 +1080,8 @@ __global__ __launch_bounds__(SEG_BLOCK, 4) void k_seg_count(
   S &sm = *reinterpret_cast<S *>(smem_raw);
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
   const uint32_t tile = blockIdx.x;
-  if (osize[tile]) {
-    seg_rle_gathered<K>(tile, bound, osize, ooff, guniq, gheads, H, ustage, mstage, tcount);
+  if (osize[tile]) {  // (later: k_seg_rle, from the gathered keys)
+    if (tid == 0) tcount[tile] = 0;
     return;
   }
   for (int i = tid; i < S::WARPS * RADIX; i += SEG_BLOCK) (&sm.whist[0][0])[i] = 0;
@@ -1100,7 +1127,10 @@ __global__ __launch_bounds__(SEG_BLOCK, 4) void k_seg_count(
   }
   __syncthreads();
   if (sm.overflow) {
-    if (tid == 0) over_list[atomicAdd(over_count, 1u)] = tile;
+    if (tid == 0) {
+      over_list[atomicAdd(over_count, 1u)] = tile;
+      tcount[tile] = 0;
+    }
     return;
   }
   // pack the occupied slots to the front in slot order: a slot moves to its

@@ -32,26 +32,6 @@ unsigned grid_n(uint64_t n) {
   return (unsigned)std::max<uint64_t>(1, std::min<uint64_t>((n + 255) / 256, 152ull * 64));
 }
 
-// exclusive scan of n flags into n + 1 positions; returns the total
-dbg_status scan_flags_u32(dbg_ctx *ctx, const uint32_t *in, uint64_t n, uint64_t *out, uint64_t *total) {
-  cudaStream_t s = ctx->stream;
-  if (n == 0) {
-    DBG_CUDA_TRY(cudaMemsetAsync(out, 0, sizeof(uint64_t), s));
-    *total = 0;
-    return DBG_OK;
-  }
-  const uint64_t tiles = (n + SCAN_TILE - 1) / SCAN_TILE;
-  DBG_TRY(ensure_status(ctx, tiles));
-  uint32_t epoch;
-  DBG_TRY(next_epoch(ctx, &epoch));
-  DBG_CUDA_TRY(cudaMemsetAsync(ctx->d_counters, 0, 2 * sizeof(uint32_t), s));
-  DBG_LAUNCH(ctx, ST_COMPACT_OUTPUT, 12.0 * n,
-             k_scan_excl<<<(unsigned)tiles, SCAN_BLOCK, 0, s>>>(in, n, out, ctx->d_status, ctx->d_counters, epoch,
-                                                                ctx->spin_limit, ctx->d_err, ctx->d_counters + 1));
-  DBG_CUDA_TRY(cudaGetLastError());
-  return read_small(ctx, out + n, sizeof(uint64_t), total);
-}
-
 // Per entry p of the chains' node list: the unit its node belongs to (by
 // the unit's first node), its position and strand there.  A chain of at
 // least min_nodes nodes is one unit; the nodes of a shorter one are units
@@ -241,14 +221,14 @@ static dbg_status simplify_impl(dbg_ctx *ctx, const dbg_graph *g, uint32_t min_n
   DBG_TRY(compact_chains(ctx, g, &ch, true));
   for (DevBuf *b : {&ch.node_off, &ch.nodes, &ch.seq_off, &ch.seq, &ch.circular}) b->al = &ch.al;
   DevBuf unit_head, upos, ustrand, ustart, ulen, ucirc, uidx, uoff;
-  DBG_TRY(alloc_buf(ctx, unit_head, V1 * 4));
-  DBG_TRY(alloc_buf(ctx, upos, V1 * 4));
-  DBG_TRY(alloc_buf(ctx, ustrand, V1));
-  DBG_TRY(alloc_buf(ctx, ustart, V1 * 4));
-  DBG_TRY(alloc_buf(ctx, ulen, V1 * 4));
-  DBG_TRY(alloc_buf(ctx, ucirc, V1));
-  DBG_TRY(alloc_buf(ctx, uidx, (V + 1) * 8));
-  DBG_TRY(alloc_buf(ctx, uoff, (V + 1) * 8));
+  DBG_TRY(alloc_tmp(ctx, unit_head, V1 * 4));
+  DBG_TRY(alloc_tmp(ctx, upos, V1 * 4));
+  DBG_TRY(alloc_tmp(ctx, ustrand, V1));
+  DBG_TRY(alloc_tmp(ctx, ustart, V1 * 4));
+  DBG_TRY(alloc_tmp(ctx, ulen, V1 * 4));
+  DBG_TRY(alloc_tmp(ctx, ucirc, V1));
+  DBG_TRY(alloc_tmp(ctx, uidx, (V + 1) * 8));
+  DBG_TRY(alloc_tmp(ctx, uoff, (V + 1) * 8));
   DBG_CUDA_TRY(cudaMemsetAsync(ustart.p, 0, V1 * 4, s));
   DBG_CUDA_TRY(cudaMemsetAsync(ulen.p, 0, V1 * 4, s));
   uint64_t U = 0, total = 0;
@@ -261,8 +241,12 @@ static dbg_status simplify_impl(dbg_ctx *ctx, const dbg_graph *g, uint32_t min_n
                                                         ulen.as<uint32_t>(), ucirc.as<uint8_t>()));
     DBG_CUDA_TRY(cudaGetLastError());
   }
-  DBG_TRY(scan_flags_u32(ctx, ustart.as<uint32_t>(), V, uidx.as<uint64_t>(), &U));
-  DBG_TRY(scan_flags_u32(ctx, ulen.as<uint32_t>(), V, uoff.as<uint64_t>(), &total));
+  DBG_TRY(scan_excl_async(ctx, ustart.as<uint32_t>(), V, uidx.as<uint64_t>(), CT_TOTAL));
+  DBG_TRY(scan_excl_async(ctx, ulen.as<uint32_t>(), V, uoff.as<uint64_t>(), CT_ENDS));
+  uint32_t c[CT_LAST + 1];
+  DBG_TRY(read_counters(ctx, c));
+  U = c[CT_TOTAL];
+  total = c[CT_ENDS];
   if (total != V) {
     set_error("units hold %llu nodes, expected %llu", (unsigned long long)total, (unsigned long long)V);
     return DBG_EINTERNAL;
@@ -289,13 +273,13 @@ static dbg_status simplify_impl(dbg_ctx *ctx, const dbg_graph *g, uint32_t min_n
   // the edges: inside reported chains dropped, inconsistent ones counted,
   // the rest relabelled in edge order
   const uint64_t E1 = std::max<uint64_t>(1, E);
-  DevBuf deg, keep, pos, removed;
-  DBG_TRY(alloc_buf(ctx, deg, 2 * V1 * 4));
-  DBG_TRY(alloc_buf(ctx, keep, E1 * 4));
-  DBG_TRY(alloc_buf(ctx, pos, (E + 1) * 8));
-  DBG_TRY(alloc_buf(ctx, removed, 8));
+  DevBuf deg, keep, pos;
+  DBG_TRY(alloc_tmp(ctx, deg, 2 * V1 * 4));
+  DBG_TRY(alloc_tmp(ctx, keep, E1 * 4));
+  DBG_TRY(alloc_tmp(ctx, pos, (E + 1) * 8));
   DBG_CUDA_TRY(cudaMemsetAsync(deg.p, 0, 2 * V1 * 4, s));
-  DBG_CUDA_TRY(cudaMemsetAsync(removed.p, 0, 8, s));
+  unsigned long long *removed = reinterpret_cast<unsigned long long *>(ctx->d_counters + CT_REMOVED);
+  DBG_CUDA_TRY(cudaMemsetAsync(removed, 0, 8, s));
   uint64_t M = 0;
   if (E > 0) {
     DBG_LAUNCH(ctx, ST_COMPACT_LINKS, 9.0 * E,
@@ -305,11 +289,13 @@ static dbg_status simplify_impl(dbg_ctx *ctx, const dbg_graph *g, uint32_t min_n
                k_simple_edge_flags<<<grid_n(E), 256, 0, s>>>(
                    g->src.as<uint32_t>(), g->dst.as<uint32_t>(), g->orient.as<uint8_t>(), E, deg.as<uint32_t>(),
                    unit_head.as<uint32_t>(), upos.as<uint32_t>(), ustrand.as<uint8_t>(), ulen.as<uint32_t>(),
-                   ucirc.as<uint8_t>(), keep.as<uint32_t>(), removed.as<unsigned long long>()));
+                   ucirc.as<uint8_t>(), keep.as<uint32_t>(), removed));
     DBG_CUDA_TRY(cudaGetLastError());
   }
-  DBG_TRY(scan_flags_u32(ctx, keep.as<uint32_t>(), E, pos.as<uint64_t>(), &M));
-  DBG_TRY(read_small(ctx, removed.p, 8, &out->removed));
+  DBG_TRY(scan_excl_async(ctx, keep.as<uint32_t>(), E, pos.as<uint64_t>(), CT_TOTAL));
+  DBG_TRY(read_counters(ctx, c));
+  M = c[CT_TOTAL];
+  out->removed = (uint64_t)c[CT_REMOVED + 1] << 32 | c[CT_REMOVED];
   out->num_edges = M;
   const uint64_t M1 = std::max<uint64_t>(1, M);
   DBG_TRY(alloc_buf(ctx, out->unit_a, M1 * 4));
@@ -326,8 +312,7 @@ static dbg_status simplify_impl(dbg_ctx *ctx, const dbg_graph *g, uint32_t min_n
                    out->side_a.as<uint8_t>(), out->unit_b.as<uint32_t>(), out->side_b.as<uint8_t>(),
                    out->edge.as<uint32_t>()));
   DBG_CUDA_TRY(cudaGetLastError());
-  DBG_CUDA_TRY(cudaStreamSynchronize(s));
-  return check_device_error(ctx);
+  return check_device_error(ctx);  // waits for the stream
 }
 
 }  // namespace dbg
