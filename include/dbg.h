@@ -465,8 +465,8 @@ uint64_t dbg_sort_fallbacks(const dbg_ctx *ctx);
  * of the hybrid edge-key sort counts each tile's copies of every key in a
  * shared-memory hash table of 2048 slots and sorts only the distinct keys,
  * which at read coverage c are about 1/c of them; a tile whose distinct
- * keys do not fit (about 1500 and up) is sorted copy by copy instead, and
- * dbg_sort_count_overflows counts such tiles over the context's builds.
+ * keys do not fit (about 1500 and up), or whose first keys are nearly all
+ * distinct, is sorted copy by copy instead, and dbg_sort_count_overflows counts such tiles over the context's builds.
  * Off, every tile is sorted copy by copy.  The edge list is the same
  * either way.
  * -------------------------------------------------------------------- */

@@ -752,7 +752,7 @@ dbg_status seg_rle(dbg_ctx *ctx, K *kin, K *kstage, uint64_t n, Groups &gr, int 
   using Sh = SegShape<K>;
   cudaStream_t s = ctx->stream;
   TileSet ts;
-  DevBuf gheads, guniq, mstage, tcount, toff, over;
+  DevBuf gheads, guniq, mstage, tcount, toff, over, crowded;
   uint64_t H = 0;
   DBG_TRY(seg_tiles<K>(ctx, kin, n, gr, ts, ST_LOCAL_SORT_EDGES));
   const uint64_t tiles = ts.tiles;
@@ -760,20 +760,21 @@ dbg_status seg_rle(dbg_ctx *ctx, K *kin, K *kstage, uint64_t n, Groups &gr, int 
   DBG_TRY(alloc_tmp(ctx, tcount, tiles * 4));
   DBG_TRY(alloc_tmp(ctx, toff, (tiles + 1) * 8));
   const int rank = local_rank_method(ctx, sizeof(K) == 16);
-  // the radix-sorting kernel over the tiles of a list (nullptr: all), the
-  // oversize ones from the gathered keys
-  auto sort_tiles = [&](uint64_t count, const uint32_t *list, double bytes) -> dbg_status {
+  // the radix-sorting kernel over `count` tiles: all of them, those of a
+  // list, or as many of the list as the device has counted in *dcount
+  auto sort_tiles = [&](uint64_t count, const uint32_t *list, const uint32_t *dcount, double bytes) -> dbg_status {
     auto radix = rank == RANK_MATCH    ? k_seg_rle<K, Sh::ITEMS, RANK_MATCH>
                  : rank == RANK_ATOMIC ? k_seg_rle<K, Sh::ITEMS, RANK_ATOMIC>
                                        : k_seg_rle<K, Sh::ITEMS, RANK_BALLOT>;
     constexpr size_t rsmem = sizeof(SegSortSmem<K, false, Sh::ITEMS>);
     set_smem_attrs(radix, rsmem);
     if (count == 0) return DBG_OK;
+    if (dcount) count = std::min<uint64_t>(count, 2ull * (uint64_t)std::max(1, ctx->num_sms));
     DBG_LAUNCH(ctx, ST_LOCAL_SORT_EDGES, bytes,
                radix<<<(unsigned)count, SEG_BLOCK, rsmem, s>>>(
                    kin, ts.bound.as<uint64_t>(), ts.osize.as<uint32_t>(), ts.ooff.as<uint64_t>(), guniq.as<K>(),
                    gheads.as<uint32_t>(), (uint32_t)H, kstage, mstage.as<uint32_t>(), tcount.as<uint32_t>(), gr.lb,
-                   list));
+                   list, dcount));
     DBG_CUDA_TRY(cudaGetLastError());
     return DBG_OK;
   };
@@ -787,9 +788,10 @@ dbg_status seg_rle(dbg_ctx *ctx, K *kin, K *kstage, uint64_t n, Groups &gr, int 
   uint32_t c[CT_LAST + 1];
   bool final = false;  // the scan below covers every tile
   if (ctx->count_first) {
-    // count-first; the tiles that overflow their table are listed and sorted
-    // copy by copy, and the oversize ones left out, if there are any: one
-    // read-back tells, with the total that holds otherwise
+    // count-first; the tiles that overflow their table, or would, are listed
+    // and ordered copy by copy.  Those with crowded buckets (by digits) and the
+    // oversize ones follow if one read-back, with the total that holds
+    // otherwise, says that there are some.
     auto count = rank == RANK_MATCH    ? k_seg_count<K, RANK_MATCH>
                  : rank == RANK_ATOMIC ? k_seg_count<K, RANK_ATOMIC>
                                        : k_seg_count<K, RANK_BALLOT>;
@@ -804,24 +806,37 @@ dbg_status seg_rle(dbg_ctx *ctx, K *kin, K *kstage, uint64_t n, Groups &gr, int 
                    tcount.as<uint32_t>(), over.as<uint32_t>(), ctx->d_counters + CT_LISTED, gr.lb, ctx->seg_rank,
                    ctx->d_counters + CT_LONG));
     DBG_CUDA_TRY(cudaGetLastError());
+    uint32_t *listed = ctx->d_counters + CT_LISTED;
+    if (ctx->seg_rank) {
+      DBG_TRY(alloc_tmp(ctx, crowded, tiles * 4));
+      set_smem_attrs(k_rank_rle<K>, sizeof(RankRleSmem<K>));
+      DBG_LAUNCH(ctx, ST_LOCAL_SORT_EDGES, 0.0,
+                 k_rank_rle<K><<<(unsigned)std::min<uint64_t>(tiles, 2ull * (uint64_t)std::max(1, ctx->num_sms)),
+                                 RANK_BLOCK, sizeof(RankRleSmem<K>), s>>>(
+                     kin, ts.bound.as<uint64_t>(), kstage, mstage.as<uint32_t>(), tcount.as<uint32_t>(), gr.lb,
+                     over.as<uint32_t>(), listed, crowded.as<uint32_t>(), ctx->d_counters + CT_CROWDED));
+      DBG_CUDA_TRY(cudaGetLastError());
+    } else {
+      DBG_TRY(sort_tiles(tiles, over.as<uint32_t>(), listed, 0.0));
+    }
     DBG_TRY(scan_u32_async(ctx, tcount.as<uint32_t>(), tiles, toff.as<uint64_t>(), ST_LOCAL_SORT_EDGES, CT_TOTAL));
     DBG_TRY(read_counters(ctx, c));
     ts.gathered = c[CT_GATHERED];
     ts.oversize = c[CT_OVERSIZE];
     ctx->count_overflow_tiles += c[CT_LISTED];
-    ctx->rank_fallback_tiles += c[CT_LONG];
-    final = c[CT_LISTED] == 0 && ts.oversize == 0;
+    ctx->rank_fallback_tiles += c[CT_LONG] + c[CT_CROWDED];
+    final = ts.oversize == 0 && c[CT_CROWDED] == 0;
     if (!final) {
-      const uint32_t listed = c[CT_LISTED];
+      const uint32_t n_crowded = c[CT_CROWDED];
       DBG_TRY(gather());
-      DBG_TRY(sort_tiles(listed, over.as<uint32_t>(), 0.0));
-      DBG_TRY(sort_tiles(ts.oversize, ts.olist.as<uint32_t>(), 0.0));
+      DBG_TRY(sort_tiles(n_crowded, crowded.as<uint32_t>(), nullptr, 0.0));
+      DBG_TRY(sort_tiles(ts.oversize, ts.olist.as<uint32_t>(), nullptr, 0.0));
     }
   } else {
     DBG_TRY(read_counters(ctx, c));
     ts.gathered = c[CT_GATHERED];
     DBG_TRY(gather());
-    DBG_TRY(sort_tiles(tiles, nullptr, (double)n * sizeof(K)));
+    DBG_TRY(sort_tiles(tiles, nullptr, nullptr, (double)n * sizeof(K)));
   }
   if (!final) {
     DBG_TRY(scan_u32_async(ctx, tcount.as<uint32_t>(), tiles, toff.as<uint64_t>(), ST_LOCAL_SORT_EDGES, CT_TOTAL));

@@ -898,24 +898,27 @@ __device__ __forceinline__ void seg_rle_gathered(uint32_t tile, const uint64_t *
   if (threadIdx.x == 0) tcount[tile] = h1 - h0;
 }
 
-// Block radix local sort + RLE, one CTA per tile (every tile, or the tiles
-// of tile_list when it is not null).
+// Block radix local sort + RLE: one CTA per tile (every tile, or the tiles of
+// tile_list when it is not null), or a grid of CTAs that take the *list_count
+// listed tiles in turn.
 template <class K, int ITEMS, int RANK>
 __global__ __launch_bounds__(SEG_BLOCK, 2) void k_seg_rle(
     const K *__restrict__ kin, const uint64_t *__restrict__ bound, const uint32_t *__restrict__ osize,
     const uint64_t *__restrict__ ooff, const K *__restrict__ guniq, const uint32_t *__restrict__ gheads, uint32_t H,
     K *__restrict__ ustage, uint32_t *__restrict__ mstage, uint32_t *__restrict__ tcount, LowBits lb,
-    const uint32_t *__restrict__ tile_list) {
+    const uint32_t *__restrict__ tile_list, const uint32_t *__restrict__ list_count) {
   using S = SegSortSmem<K, false, ITEMS>;
   extern __shared__ __align__(128) unsigned char smem_raw[];
   S &sm = *reinterpret_cast<S *>(smem_raw);
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
-  const uint32_t tile = tile_list ? tile_list[blockIdx.x] : blockIdx.x;
-  {
+  const uint32_t todo = list_count ? *list_count : gridDim.x;
+  for (uint32_t q = blockIdx.x; q < todo; q += gridDim.x) {
+    const uint32_t tile = tile_list ? tile_list[q] : q;
     if (osize[tile]) {
       seg_rle_gathered<K>(tile, bound, osize, ooff, guniq, gheads, H, ustage, mstage, tcount);
-      return;
+      continue;
     }
+    __syncthreads();  // the previous tile's shared memory is read
     for (int i = tid; i < S::WARPS * RADIX; i += SEG_BLOCK) (&sm.whist[0][0])[i] = 0;
     for (int i = tid; i < S::WARPS * (RADIX + 1); i += SEG_BLOCK) (&sm.match[0][0])[i] = 0;
     seg_setup<K>(sm, kin, bound, tile, lb);
@@ -980,8 +983,9 @@ __global__ __launch_bounds__(SEG_BLOCK, 2) void k_seg_rle(
 // only the distinct keys.  The output is that of k_seg_rle: each distinct
 // key once, in order, with its multiplicity (STEP-2), staged in the tile's
 // own range.  The table is small so that several CTAs share an SM; a tile
-// whose keys do not fit (a probe longer than PROBES slots) is listed in
-// over_list and sorted by k_seg_rle instead.
+// whose keys do not fit (a probe longer than PROBES slots), or would not, is
+// listed in over_list and ordered copy by copy instead (k_rank_rle, or
+// k_seg_rle without rank_groups).
 //
 // Ordering the distinct keys.  With rank_groups set, the distinct keys are
 // bucketed by the top 11 bits of their offset from the tile's base (2048
@@ -993,6 +997,16 @@ __global__ __launch_bounds__(SEG_BLOCK, 2) void k_seg_rle(
 // by 64-bit shared atomic adds, measured 1.9x slower: the hot slots of a
 // 30x-covered key serialise.)
 constexpr uint32_t COUNT_GROUP_MAX = 256;
+
+// Of the first 256 keys of a tile of n with c copies each, about
+// 1 - 128 c / n are the first of their key: 96 % (64-bit keys, n = 4096) or
+// 92 % (128-bit, n = 2048) at c = 1.3, 50 % and 25 % at c = 30, and 40 to 60 %
+// where half a percent of errors adds its own keys.  At 1.3 copies of 28.5 M
+// 128-bit keys every tile passes 65 %, and the edge list's local pass takes
+// 0.89 ms; at 80 % 12143 of 13923 do, 0.98; at 90 % 6448, 1.27; without the
+// sample, sorting the 6465 tiles that overflow by digits, 2.17.  At 30 copies
+// the sample itself costs 1 % (1.035 G keys: 7.87 -> 7.97 ms).
+constexpr int COUNT_FRESH_PCT = 65;
 
 // Hash-table slots of the counting pass.  The empty mark is the all-ones
 // key, which no key offset reaches: an offset is key - base <= key, and the
@@ -1059,7 +1073,7 @@ struct SegCountSmem {
   uint32_t tmp[8];
   uint64_t bound[2];
   K base, range;
-  uint32_t tile, passes, excl, total, span_bits, overflow, maxg;
+  uint32_t tile, passes, excl, total, span_bits, overflow, fresh, maxg;
 };
 
 // high bits of a key offset, as a bucket index within the tile
@@ -1091,7 +1105,7 @@ __global__ __launch_bounds__(SEG_BLOCK, 4) void k_seg_count(
     sm.keys[j] = O::empty();
     sm.vals[j] = 0;
   }
-  if (tid == 0) sm.overflow = 0;
+  if (tid == 0) sm.overflow = sm.fresh = 0;
   seg_setup<K>(sm, kin, bound, tile, lb);  // synchronises
   const uint64_t s = sm.bound[0];
   const uint32_t cnt = (uint32_t)(sm.bound[1] - s);
@@ -1099,7 +1113,10 @@ __global__ __launch_bounds__(SEG_BLOCK, 4) void k_seg_count(
   // the tile's path (uniform): ranked by buckets of groups
   const bool by_groups = rank_groups && cnt > 0;
   const int bshift = (int)sm.span_bits > S::TBITS ? (int)sm.span_bits - S::TBITS : 0;
-  // count: each key into its slot, LOAD keys per thread at a time
+  // count: each key into its slot, LOAD keys per thread at a time.  A tile
+  // that could fill more than half the table and whose first keys are nearly
+  // all distinct (see COUNT_FRESH_PCT) is listed at once.
+  bool sample = rank_groups && cnt > S::TBL / 2;
   for (uint32_t j0 = 0; j0 < cnt; j0 += S::LOAD * SEG_BLOCK) {
     K d[S::LOAD];
 #pragma unroll
@@ -1110,19 +1127,30 @@ __global__ __launch_bounds__(SEG_BLOCK, 4) void k_seg_count(
     if (*reinterpret_cast<volatile uint32_t *>(&sm.overflow)) break;
 #pragma unroll
     for (int i = 0; i < S::LOAD; i++) {
-      if (KeyOps<K>::eq(d[i], O::empty())) continue;
-      uint32_t h = O::hash(d[i]) >> (32 - S::TBITS);
-      bool done = false;
-      for (uint32_t probe = 0; probe < S::PROBES; probe++) {
-        const K cur = O::claim(&sm.keys[h], d[i]);
-        if (KeyOps<K>::eq(cur, O::empty()) || KeyOps<K>::eq(cur, d[i])) {
-          atomicAdd(&sm.vals[h], 1u);
-          done = true;
-          break;
+      // (128-bit tiles are one batch long; in 64-bit ones, of two, a test here
+      // costs every tile 8 %)
+      if (sizeof(K) == 16 && i == 2 && *reinterpret_cast<volatile uint32_t *>(&sm.overflow)) break;
+      uint32_t fresh = 0;
+      if (!KeyOps<K>::eq(d[i], O::empty())) {
+        uint32_t h = O::hash(d[i]) >> (32 - S::TBITS);
+        bool done = false;
+        for (uint32_t probe = 0; probe < S::PROBES; probe++) {
+          const K cur = O::claim(&sm.keys[h], d[i]);
+          if (KeyOps<K>::eq(cur, O::empty()) || KeyOps<K>::eq(cur, d[i])) {
+            atomicAdd(&sm.vals[h], 1u);
+            if (i == 0) fresh = KeyOps<K>::eq(cur, d[i]) ? 0 : 1;
+            done = true;
+            break;
+          }
+          h = (h + 1) & (S::TBL - 1);
         }
-        h = (h + 1) & (S::TBL - 1);
+        if (!done) sm.overflow = 1;
       }
-      if (!done) sm.overflow = 1;
+      if (i == 0 && sample) {
+        const uint32_t f = __popc(__ballot_sync(0xffffffffu, fresh));
+        if (lane == 0 && atomicAdd(&sm.fresh, f) + f > SEG_BLOCK * COUNT_FRESH_PCT / 100) sm.overflow = 1;
+        sample = false;
+      }
     }
   }
   __syncthreads();
@@ -1248,6 +1276,172 @@ __global__ void k_seg_compact(const uint64_t *__restrict__ bound, const uint32_t
     for (uint32_t r = threadIdx.x; r < c; r += blockDim.x) {
       uniq[o + r] = ustage[s + r];
       mult[o + r] = mstage[s + r];
+    }
+  }
+}
+
+// Edge keys of a tile with few copies each: every copy is ranked, as the
+// records are by k_seg_rank, by a counting sort over buckets of the top bits
+// of the key offsets and comparisons within the bucket; then the runs of equal
+// keys are counted.  Bound by instruction issue: 0.27 ms for 6448 tiles of 2048
+// 128-bit keys, where k_seg_rle's digit passes take 0.89.
+// A grid of CTAs takes the *list_count tiles of `list` in turn (two of 512
+// threads per SM); a tile with a bucket longer than RANK_GROUP_MAX goes to
+// fb_list, for k_seg_rle.
+template <class K>
+struct RankRleSmem {
+  static constexpr int CAP = SegRankSmem<K>::CAP, ITEMS = SegRankSmem<K>::ITEMS;
+  static constexpr int TBITS = SegRankSmem<K>::TBITS, NB = 1 << TBITS, PER = NB / 2 / RANK_BLOCK;
+  static_assert(NB > CAP, "the run starts take the buckets' place");
+  K key[CAP];                   // offsets from base
+  uint32_t start2[NB / 2 + 1];  // 16 bits per bucket: its keys, then its first position; then where each run starts
+  uint32_t wsum[RANK_BLOCK / 32];
+  uint32_t cnt[ITEMS * (RANK_BLOCK / 32) + 1], head[ITEMS * (RANK_BLOCK / 32)];
+  uint64_t bound[2];
+  K base, range;
+  uint32_t passes, span_bits, maxg, distinct;
+};
+
+template <class K>
+__global__ __launch_bounds__(RANK_BLOCK, 2) void k_rank_rle(
+    const K *__restrict__ kin, const uint64_t *__restrict__ bound, K *__restrict__ ustage,
+    uint32_t *__restrict__ mstage, uint32_t *__restrict__ tcount, LowBits lb, const uint32_t *__restrict__ list,
+    const uint32_t *__restrict__ list_count, uint32_t *__restrict__ fb_list, uint32_t *__restrict__ fb_count) {
+  using S = RankRleSmem<K>;
+  constexpr int ITEMS = S::ITEMS, PER = S::PER;
+  extern __shared__ __align__(128) unsigned char smem_raw[];
+  S &sm = *reinterpret_cast<S *>(smem_raw);
+  uint16_t *const start = reinterpret_cast<uint16_t *>(sm.start2);
+  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+  const uint32_t todo = *list_count;
+  for (uint32_t next = blockIdx.x; next < todo; next += gridDim.x) {
+    const uint32_t tile = list[next];
+    __syncthreads();  // the previous tile's shared memory is read
+    for (int j = tid; j <= S::NB / 2; j += RANK_BLOCK) sm.start2[j] = 0;
+    if (tid == 0) sm.maxg = 0;
+    seg_setup<K>(sm, kin, bound, tile, lb);  // synchronises
+    const uint64_t s = sm.bound[0];
+    const uint32_t cnt = (uint32_t)(sm.bound[1] - s);
+    const int items = (int)((cnt + RANK_BLOCK - 1) / RANK_BLOCK);  // of each thread
+    const K base = sm.base;
+    const int bshift = (int)sm.span_bits > S::TBITS ? (int)sm.span_bits - S::TBITS : 0;
+    K key[ITEMS];
+    uint32_t oa[ITEMS];  // bucket, place on arrival << 13; then place
+#pragma unroll
+    for (int i = 0; i < ITEMS; i++) {
+      if (i >= items) break;
+      const uint32_t j = (uint32_t)i * RANK_BLOCK + tid;
+      if (j < cnt) key[i] = KeyOps<K>::sub(kin[s + j], base);
+    }
+#pragma unroll
+    for (int i = 0; i < ITEMS; i++) {
+      if (i >= items) break;
+      if ((uint32_t)i * RANK_BLOCK + tid < cnt) {
+        const uint32_t o = group_of<K>(key[i], bshift), h = 16 * (o & 1u);
+        oa[i] = o | ((atomicAdd(&sm.start2[o >> 1], 1u << h) >> h) & 0xffffu) << S::TBITS;
+      }
+    }
+    __syncthreads();
+    // exclusive scan, 2 PER consecutive buckets per thread
+    uint32_t c[PER], sum = 0, mx = 0;
+#pragma unroll
+    for (int j = 0; j < PER; j++) {
+      c[j] = sm.start2[tid * PER + j];
+      const uint32_t c0 = c[j] & 0xffffu, c1 = c[j] >> 16;
+      sum += c0 + c1;
+      mx = max(mx, max(c0, c1));
+    }
+    const uint32_t incl = warp_incl_scan(sum);
+    if (lane == 31) sm.wsum[warp] = incl;
+    mx = __reduce_max_sync(0xffffffffu, mx);
+    if (lane == 0 && mx > RANK_GROUP_MAX) sm.maxg = mx;
+    __syncthreads();
+    if (sm.maxg) {  // (tcount is 0 from the listing)
+      if (tid == 0) fb_list[atomicAdd(fb_count, 1u)] = tile;
+      continue;
+    }
+    uint32_t run = incl - sum;
+    for (int w = 0; w < warp; w++) run += sm.wsum[w];
+#pragma unroll
+    for (int j = 0; j < PER; j++) {
+      const uint32_t c0 = c[j] & 0xffffu, c1 = c[j] >> 16;
+      sm.start2[tid * PER + j] = run | (run + c0) << 16;
+      run += c0 + c1;
+    }
+    if (tid == RANK_BLOCK - 1) sm.start2[S::NB / 2] = run;
+    __syncthreads();
+#pragma unroll
+    for (int i = 0; i < ITEMS; i++) {
+      if (i >= items) break;
+      if ((uint32_t)i * RANK_BLOCK + tid < cnt) {
+        oa[i] = start[oa[i] & (S::NB - 1)] + (oa[i] >> S::TBITS);
+        sm.key[oa[i]] = key[i];
+      }
+    }
+    __syncthreads();
+#pragma unroll
+    for (int i = 0; i < ITEMS; i++) {
+      if (i >= items) break;
+      if ((uint32_t)i * RANK_BLOCK + tid < cnt) {
+        // place: the bucket's smaller keys, and its equal ones before this
+        const uint32_t q = oa[i], o = group_of<K>(key[i], bshift), a = start[o], b = start[o + 1];
+        uint32_t r = a;
+#pragma unroll 1
+        for (uint32_t t = a; t < q; t++) r += KeyOps<K>::less(key[i], sm.key[t]) ? 0u : 1u;
+#pragma unroll 1
+        for (uint32_t t = q + 1; t < b; t++) r += KeyOps<K>::less(sm.key[t], key[i]) ? 1u : 0u;
+        oa[i] = r;
+      }
+    }
+    __syncthreads();
+#pragma unroll
+    for (int i = 0; i < ITEMS; i++) {
+      if (i >= items) break;
+      if ((uint32_t)i * RANK_BLOCK + tid < cnt) sm.key[oa[i]] = key[i];
+    }
+    __syncthreads();
+    // the runs' first positions, in the buckets' place
+    for (int i = 0; i < items; i++) {
+      const uint32_t j = (uint32_t)i * RANK_BLOCK + tid;
+      const unsigned hb = __ballot_sync(0xffffffffu, j < cnt && (j == 0 || !KeyOps<K>::eq(sm.key[j], sm.key[j - 1])));
+      if (lane == 0) {
+        sm.head[i * (RANK_BLOCK / 32) + warp] = hb;
+        sm.cnt[i * (RANK_BLOCK / 32) + warp] = __popc(hb);
+      }
+    }
+    __syncthreads();
+    if (warp == 0) {
+      constexpr int NW = ITEMS * (RANK_BLOCK / 32), EACH = (NW + 31) / 32;
+      const int nw = items * (RANK_BLOCK / 32);
+      uint32_t x[EACH], sum = 0;
+#pragma unroll
+      for (int j = 0; j < EACH; j++) {
+        x[j] = lane * EACH + j < nw ? sm.cnt[lane * EACH + j] : 0u;
+        sum += x[j];
+      }
+      const uint32_t incl = warp_incl_scan(sum);
+      uint32_t run = incl - sum;
+#pragma unroll
+      for (int j = 0; j < EACH; j++) {
+        if (lane * EACH + j < nw) sm.cnt[lane * EACH + j] = run;
+        run += x[j];
+      }
+      if (lane == 31) {
+        sm.distinct = incl;
+        start[incl] = (uint16_t)cnt;
+        tcount[tile] = incl;
+      }
+    }
+    __syncthreads();
+    for (int i = 0; i < items; i++) {
+      const int w = i * (RANK_BLOCK / 32) + warp;
+      if (sm.head[w] >> lane & 1u)
+        start[sm.cnt[w] + __popc(sm.head[w] & ((1u << lane) - 1u))] = (uint16_t)(i * RANK_BLOCK + tid);
+    }
+    __syncthreads();
+    for (uint32_t r = tid; r < sm.distinct; r += RANK_BLOCK) {
+      ustage[s + r] = KeyOps<K>::add(sm.key[start[r]], base);
+      mstage[s + r] = (uint32_t)start[r + 1] - start[r];
     }
   }
 }
