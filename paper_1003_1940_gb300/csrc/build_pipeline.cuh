@@ -1667,20 +1667,6 @@ inline std::vector<std::pair<uint32_t, uint32_t>> plan_ranges(const uint64_t *hi
   return out;
 }
 
-static dbg_status scan_flags(dbg_ctx *ctx, const uint32_t *in, uint64_t n, uint64_t *out, uint32_t *total) {
-  cudaStream_t s = ctx->stream;
-  const uint64_t tiles = (n + SCAN_TILE - 1) / SCAN_TILE;
-  DBG_TRY(ensure_status(ctx, tiles));
-  uint32_t epoch;
-  DBG_TRY(next_epoch(ctx, &epoch));
-  DBG_CUDA_TRY(cudaMemsetAsync(ctx->d_counters, 0, 2 * sizeof(uint32_t), s));
-  DBG_LAUNCH(ctx, ST_NODE_IDS, 12.0 * n,
-             k_scan_excl<<<(unsigned)tiles, SCAN_BLOCK, 0, s>>>(in, n, out, ctx->d_status, ctx->d_counters, epoch,
-                                                                ctx->spin_limit, ctx->d_err, ctx->d_counters + 1));
-  DBG_CUDA_TRY(cudaGetLastError());
-  return read_small(ctx, ctx->d_counters + 1, sizeof(uint32_t), total);
-}
-
 template <class K>
 dbg_status concat_chunks(dbg_ctx *ctx, std::vector<DevBuf> &chunks, const std::vector<uint64_t> &counts,
                          size_t elem, void *dst) {
@@ -1797,7 +1783,7 @@ dbg_status build_bucketed_impl(dbg_ctx *ctx, const BucketInput &in, uint64_t bud
     DBG_CUDA_TRY(cudaMemsetAsync(ctx->d_counters + 8, 0, 4, s));
     const SortPlan<K> plan = plan_sort<K>(ctx, cnt, kbits, ctx->partition_first);
     DBG_LAUNCH(ctx, ST_EMIT, 8.0 * nwords + 16.0 * n + (double)cnt * w,
-               k_emit_range<K><<<emit_grid, EMIT_BLOCK, 0, s>>>(packed.as<uint64_t>(), base_off.as<uint64_t>(),
+               k_emit_range<K><<<emit_grid, EMIT_BLOCK, EMIT_BLOCK / 32 * EMIT_BUF<K> * sizeof(K), s>>>(packed.as<uint64_t>(), base_off.as<uint64_t>(),
                                                                 edge_off.as<uint64_t>(), n, k, ranges[b].first,
                                                                 ranges[b].second, ka.as<K>(), ctx->d_counters + 8,
                                                                 plan.digits(), d_hist));
@@ -1864,10 +1850,11 @@ dbg_status build_bucketed_impl(dbg_ctx *ctx, const BucketInput &in, uint64_t bud
   sizes.clear();
   auto nranges = plan_ranges(hist.data(), rec_cap, &sizes);
   *n_node_buckets = (uint32_t)nranges.size();
-  DevBuf flags, pos;
+  const uint64_t etiles = (E + ENDS_TILE - 1) / ENDS_TILE;
+  DevBuf tcount, toff;
   if (E > 0) {
-    DBG_TRY(alloc_tmp(ctx, flags, 2 * E * 4));
-    DBG_TRY(alloc_tmp(ctx, pos, (2 * E + 1) * 8));
+    DBG_TRY(alloc_tmp(ctx, tcount, etiles * 4));
+    DBG_TRY(alloc_tmp(ctx, toff, (etiles + 1) * 8));
   }
   const int nbits = 2 * (int)k;
   std::vector<DevBuf> cnk, crp;
@@ -1877,10 +1864,10 @@ dbg_status build_bucketed_impl(dbg_ctx *ctx, const BucketInput &in, uint64_t bud
     const uint32_t lo = nranges[c].first, hi = nranges[c].second;
     uint32_t Rc = 0;
     if (E > 0) {
-      DBG_LAUNCH(ctx, ST_ENDPOINTS, (double)E * w + 8.0 * E,
-                 k_flag_ends<K><<<grid_for(E, 256 * 8), 256, 0, s>>>(g->edge_keys.as<K>(), E, k, lo, hi,
-                                                                    flags.as<uint32_t>()));
-      DBG_TRY(scan_flags(ctx, flags.as<uint32_t>(), 2 * E, pos.as<uint64_t>(), &Rc));
+      DBG_LAUNCH(ctx, ST_ENDPOINTS, (double)E * w,
+                 k_count_ends<K><<<(unsigned)etiles, ENDS_BLOCK, 0, s>>>(g->edge_keys.as<K>(), E, k, lo, hi,
+                                                                         tcount.as<uint32_t>()));
+      DBG_TRY(scan_u32(ctx, tcount.as<uint32_t>(), etiles, toff.as<uint64_t>(), &Rc, ST_ENDPOINTS));
     }
     const uint64_t cap = (uint64_t)Rc + I;
     if (cap == 0) continue;
@@ -1894,11 +1881,10 @@ dbg_status build_bucketed_impl(dbg_ctx *ctx, const BucketInput &in, uint64_t bud
     const SortPlan<K> rplan = plan_records<K>(ctx, cap, nbits, false);
     DBG_CUDA_TRY(cudaMemsetAsync(d_hist, 0, MAX_PASSES * RADIX * 8, s));
     if (Rc > 0)
-      DBG_LAUNCH(ctx, ST_ENDPOINTS, (double)E * (w + 8) + (double)Rc * (w + 4),
-                 k_gather_ends<K><<<grid_for(E, 256 * 8), 256, 0, s>>>(g->edge_keys.as<K>(), E, k,
-                                                                      flags.as<uint32_t>(), pos.as<uint64_t>(),
-                                                                      ra.as<K>(), va.as<uint32_t>(),
-                                                                      rplan.digits(), d_hist));
+      DBG_LAUNCH(ctx, ST_ENDPOINTS, (double)E * w + (double)Rc * (w + 4),
+                 k_gather_ends<K><<<(unsigned)std::min<uint64_t>(etiles, 152ull * 8), ENDS_BLOCK, 0, s>>>(
+                     g->edge_keys.as<K>(), E, k, lo, hi, toff.as<uint64_t>(), etiles, ra.as<K>(), va.as<uint32_t>(),
+                     rplan.digits(), d_hist));
     uint64_t R = Rc;
     if (I > 0) {
       DBG_CUDA_TRY(cudaMemsetAsync(ctx->d_counters + 9, 0, 4, s));

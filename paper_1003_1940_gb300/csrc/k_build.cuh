@@ -1442,14 +1442,16 @@ __global__ __launch_bounds__(EMIT_BLOCK) void k_emit_prefix_hist(const uint64_t 
   __shared__ uint32_t s_hist[PREFIX_BINS];
   for (int i = threadIdx.x; i < PREFIX_BINS; i += EMIT_BLOCK) s_hist[i] = 0;
   __syncthreads();
-  const int lane = threadIdx.x & 31, m = (int)k + 1;
+  const int m = (int)k + 1;
+  const uint32_t lane = threadIdx.x & 31;
   const uint64_t warps = (uint64_t)gridDim.x * (EMIT_BLOCK / 32);
   for (uint64_t r = (uint64_t)blockIdx.x * (EMIT_BLOCK / 32) + (threadIdx.x >> 5); r < n_reads; r += warps) {
-    const uint64_t e0 = __ldg(edge_off + r), cnt = __ldg(edge_off + r + 1) - e0, p0 = __ldg(base_off + r);
-    for (uint64_t j = lane; j < cnt; j += 32) {
-      const K z = load_window<K>(packed, p0 + j, m);
-      atomicAdd(&s_hist[key_prefix(kmin(z, revcomp(z, m)), 2 * m)], 1u);
-    }
+    const uint64_t e0 = __ldg(edge_off + r), p = __ldg(base_off + r) + lane;
+    const uint32_t cnt = (uint32_t)(__ldg(edge_off + r + 1) - e0);
+    const uint64_t *w = packed + (p >> 5);
+    for (uint32_t j0 = 0; j0 < cnt; j0 += 32, w++)
+      if (cnt - j0 > lane)
+        atomicAdd(&s_hist[key_prefix(canonical_window<K>(w, (uint32_t)p * 2 & 30u, (uint32_t)p & 16u, m), 2 * m)], 1u);
   }
   __syncthreads();
   for (int i = threadIdx.x; i < PREFIX_BINS; i += EMIT_BLOCK)
@@ -1458,7 +1460,14 @@ __global__ __launch_bounds__(EMIT_BLOCK) void k_emit_prefix_hist(const uint64_t 
 
 // STEP-1 restricted to keys whose prefix lies in [lo, hi): the keys of one
 // bucket, appended in any order (the sort that follows orders them), with
-// the digit histograms of its radix passes.
+// the digit histograms of its radix passes.  A warp per read (the instances
+// may number more than 2^32).  A warp collects its keys in shared memory and
+// appends a bufferful at a time: one atomic add on the bucket's count per some
+// 240 keys (112 of 128 bits) instead of one per row of 32 windows, which
+// bounded the kernel: 0.32 ms for a third of 69 M windows (k = 31), was 1.83.
+template <class K>
+constexpr int EMIT_BUF = sizeof(K) == 8 ? 256 : 128;  // keys per warp
+
 template <class K>
 __global__ __launch_bounds__(EMIT_BLOCK) void k_emit_range(const uint64_t *__restrict__ packed,
                                                            const uint64_t *__restrict__ base_off,
@@ -1466,34 +1475,47 @@ __global__ __launch_bounds__(EMIT_BLOCK) void k_emit_range(const uint64_t *__res
                                                            uint32_t k, uint32_t lo, uint32_t hi,
                                                            K *__restrict__ keys, uint32_t *count, DigitSpec ds,
                                                            unsigned long long *__restrict__ hist) {
+  extern __shared__ __align__(16) unsigned char emit_buf[];
+  K *const buf = reinterpret_cast<K *>(emit_buf) + (threadIdx.x >> 5) * EMIT_BUF<K>;
   __shared__ uint32_t s_hist[MAX_PASSES * RADIX];
   for (int i = threadIdx.x; i < ds.entries(); i += EMIT_BLOCK) s_hist[i] = 0;
   __syncthreads();
-  const int lane = threadIdx.x & 31, m = (int)k + 1;
+  const int m = (int)k + 1;
+  const uint32_t lane = threadIdx.x & 31, lt = (1u << lane) - 1u;
   const uint64_t warps = (uint64_t)gridDim.x * (EMIT_BLOCK / 32);
+  uint32_t held = 0;
+  auto flush = [&]() {
+    uint32_t base = 0;
+    if (lane == 0) base = atomicAdd(count, held);
+    base = __shfl_sync(0xffffffffu, base, 0);
+    for (uint32_t i = lane; i < held; i += 32) {
+      const K key = buf[i];
+      keys[(uint64_t)base + i] = key;
+      ds.count(s_hist, key);
+    }
+    held = 0;
+    __syncwarp();
+  };
   for (uint64_t r = (uint64_t)blockIdx.x * (EMIT_BLOCK / 32) + (threadIdx.x >> 5); r < n_reads; r += warps) {
-    const uint64_t e0 = __ldg(edge_off + r), cnt = __ldg(edge_off + r + 1) - e0, p0 = __ldg(base_off + r);
-    for (uint64_t j0 = 0; j0 < cnt; j0 += 32) {
-      const uint64_t j = j0 + lane;
+    const uint64_t e0 = __ldg(edge_off + r), p = __ldg(base_off + r) + lane;
+    const uint32_t cnt = (uint32_t)(__ldg(edge_off + r + 1) - e0);
+    const uint64_t *w = packed + (p >> 5);
+    for (uint32_t j0 = 0; j0 < cnt; j0 += 32, w++) {
       K key = KeyOps<K>::zero();
       bool in = false;
-      if (j < cnt) {
-        const K z = load_window<K>(packed, p0 + j, m);
-        key = kmin(z, revcomp(z, m));
+      if (cnt - j0 > lane) {
+        key = canonical_window<K>(w, (uint32_t)p * 2 & 30u, (uint32_t)p & 16u, m);
         const uint32_t pf = key_prefix(key, 2 * m);
         in = pf >= lo && pf < hi;
       }
       const unsigned b = __ballot_sync(0xffffffffu, in);
-      if (!b) continue;
-      uint32_t base = 0;
-      if (lane == 0) base = atomicAdd(count, (uint32_t)__popc(b));
-      base = __shfl_sync(0xffffffffu, base, 0);
-      if (in) {
-        keys[base + __popc(b & ((1u << lane) - 1u))] = key;
-        ds.count(s_hist, key);
-      }
+      if (held + __popc(b) > EMIT_BUF<K>) flush();
+      if (in) buf[held + __popc(b & lt)] = key;
+      held += __popc(b);
+      __syncwarp();
     }
   }
+  if (held) flush();
   __syncthreads();
   for (int i = threadIdx.x; i < ds.entries(); i += EMIT_BLOCK)
     if (s_hist[i]) atomicAdd(hist + i, (unsigned long long)s_hist[i]);
@@ -1551,44 +1573,96 @@ __global__ void k_node_prefix_hist(const K *__restrict__ edge_keys, uint64_t E, 
     if (s_hist[i]) atomicAdd(hist + i, (unsigned long long)s_hist[i]);
 }
 
-// 1 for every edge end (slot 2e + role) whose node key prefix is in [lo, hi).
+// The edge ends whose node key's prefix is in [lo, hi), ENDS_TILE edges at a
+// time: their number per tile, and, given its scan, the ends as node records
+// in (e, role) order with the node-sort digit histograms.  Deriving an edge's
+// ends twice, from 8 or 16 bytes, costs less than a flag and a 64-bit position
+// per end in memory: 48 and 104 us for
+// a seventh of 13.6 M edges' ends, where flags, their scan and the gather took 50,
+// 190 and 73.
+constexpr int ENDS_BLOCK = 256, ENDS_ITEMS = 8, ENDS_TILE = ENDS_BLOCK * ENDS_ITEMS;
+
 template <class K>
-__global__ void k_flag_ends(const K *__restrict__ edge_keys, uint64_t E, uint32_t k, uint32_t lo, uint32_t hi,
-                            uint32_t *__restrict__ flags) {
-  for (uint64_t e = (uint64_t)blockIdx.x * blockDim.x + threadIdx.x; e < E; e += (uint64_t)gridDim.x * blockDim.x) {
-    K s, d;
-    uint32_t o;
-    edge_ends(edge_keys[e], (int)k, s, d, o);
-    const uint32_t ps = key_prefix(s, 2 * (int)k), pd = key_prefix(d, 2 * (int)k);
-    flags[2 * e] = ps >= lo && ps < hi;
-    flags[2 * e + 1] = pd >= lo && pd < hi;
-  }
+__device__ __forceinline__ uint32_t ends_in_range(const K &edge, uint32_t k, uint32_t lo, uint32_t hi, K &s, K &d) {
+  uint32_t o;
+  edge_ends(edge, (int)k, s, d, o);
+  const uint32_t ps = key_prefix(s, 2 * (int)k), pd = key_prefix(d, 2 * (int)k);
+  return (ps >= lo && ps < hi ? 1u : 0u) | (pd >= lo && pd < hi ? 2u : 0u);
 }
 
-// The flagged edge ends as node records, in (e, role) order (positions from
-// an exclusive scan of the flags), with the node-sort digit histograms.
 template <class K>
-__global__ void k_gather_ends(const K *__restrict__ edge_keys, uint64_t E, uint32_t k,
-                              const uint32_t *__restrict__ flags, const uint64_t *__restrict__ pos,
-                              K *__restrict__ rkeys, uint32_t *__restrict__ rvals, DigitSpec ds,
-                              unsigned long long *__restrict__ hist) {
-  __shared__ uint32_t s_hist[MAX_PASSES * RADIX];
-  for (int i = threadIdx.x; i < ds.entries(); i += blockDim.x) s_hist[i] = 0;
+__global__ __launch_bounds__(ENDS_BLOCK) void k_count_ends(const K *__restrict__ edge_keys, uint64_t E, uint32_t k,
+                                                           uint32_t lo, uint32_t hi, uint32_t *__restrict__ tcount) {
+  __shared__ uint32_t total;
+  if (threadIdx.x == 0) total = 0;
   __syncthreads();
-  for (uint64_t e = (uint64_t)blockIdx.x * blockDim.x + threadIdx.x; e < E; e += (uint64_t)gridDim.x * blockDim.x) {
-    const uint32_t f0 = flags[2 * e], f1 = flags[2 * e + 1];
-    if (!f0 && !f1) continue;
+  const uint64_t first = (uint64_t)blockIdx.x * ENDS_TILE + threadIdx.x;
+  uint32_t sum = 0;
+#pragma unroll
+  for (int i = 0; i < ENDS_ITEMS; i++) {
+    const uint64_t e = first + (uint64_t)i * ENDS_BLOCK;
     K s, d;
-    uint32_t o;
-    edge_ends(edge_keys[e], (int)k, s, d, o);
-    for (int role = 0; role < 2; role++) {
-      if (!(role ? f1 : f0)) continue;
-      const K nk = role ? d : s;
-      const uint64_t p = pos[2 * e + role];
-      rkeys[p] = nk;
-      rvals[p] = (uint32_t)(e << 1) | (uint32_t)role;
-      ds.count(s_hist, nk);
+    if (e < E) sum += __popc(ends_in_range<K>(edge_keys[e], k, lo, hi, s, d));
+  }
+  sum = __reduce_add_sync(0xffffffffu, sum);
+  if ((threadIdx.x & 31) == 0) atomicAdd(&total, sum);
+  __syncthreads();
+  if (threadIdx.x == 0) tcount[blockIdx.x] = total;
+}
+
+template <class K>
+__global__ __launch_bounds__(ENDS_BLOCK) void k_gather_ends(const K *__restrict__ edge_keys, uint64_t E, uint32_t k,
+                                                            uint32_t lo, uint32_t hi,
+                                                            const uint64_t *__restrict__ toff, uint64_t tiles,
+                                                            K *__restrict__ rkeys, uint32_t *__restrict__ rvals,
+                                                            DigitSpec ds, unsigned long long *__restrict__ hist) {
+  constexpr int WARPS = ENDS_BLOCK / 32;
+  __shared__ uint32_t s_hist[MAX_PASSES * RADIX];
+  __shared__ uint32_t s_cnt[ENDS_ITEMS * WARPS];
+  for (int i = threadIdx.x; i < ds.entries(); i += ENDS_BLOCK) s_hist[i] = 0;
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  const unsigned lt = (1u << lane) - 1u;
+  for (uint64_t t = blockIdx.x; t < tiles; t += gridDim.x) {
+    const uint64_t first = t * ENDS_TILE + threadIdx.x;
+    uint32_t at[ENDS_ITEMS];  // ends before the lane's in its warp's row << 2 | the lane's
+#pragma unroll
+    for (int i = 0; i < ENDS_ITEMS; i++) {
+      const uint64_t e = first + (uint64_t)i * ENDS_BLOCK;
+      K s, d;
+      const uint32_t f = e < E ? ends_in_range<K>(edge_keys[e], k, lo, hi, s, d) : 0u;
+      const unsigned b0 = __ballot_sync(0xffffffffu, f & 1u), b1 = __ballot_sync(0xffffffffu, f & 2u);
+      at[i] = (uint32_t)(__popc(b0 & lt) + __popc(b1 & lt)) << 2 | f;
+      if (lane == 0) s_cnt[i * WARPS + warp] = __popc(b0) + __popc(b1);
     }
+    __syncthreads();
+    if (warp == 0) {
+      static_assert(ENDS_ITEMS * WARPS == 64, "two counts per lane");
+      const uint32_t x = s_cnt[2 * lane], y = s_cnt[2 * lane + 1], before = warp_incl_scan(x + y) - x - y;
+      s_cnt[2 * lane] = before;
+      s_cnt[2 * lane + 1] = before + x;
+    }
+    __syncthreads();
+    const uint64_t base = toff[t];
+#pragma unroll
+    for (int i = 0; i < ENDS_ITEMS; i++) {
+      if (!(at[i] & 3u)) continue;
+      const uint64_t e = first + (uint64_t)i * ENDS_BLOCK;
+      K s, d;
+      uint32_t o;
+      edge_ends(edge_keys[e], (int)k, s, d, o);
+      uint64_t p = base + s_cnt[i * WARPS + warp] + (at[i] >> 2);
+      if (at[i] & 1u) {
+        rkeys[p] = s;
+        rvals[p++] = (uint32_t)(e << 1);
+        ds.count(s_hist, s);
+      }
+      if (at[i] & 2u) {
+        rkeys[p] = d;
+        rvals[p] = (uint32_t)(e << 1) | 1u;
+        ds.count(s_hist, d);
+      }
+    }
+    __syncthreads();  // s_cnt is read
   }
   __syncthreads();
   for (int i = threadIdx.x; i < ds.entries(); i += blockDim.x)
