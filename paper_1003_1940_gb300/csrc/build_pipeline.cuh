@@ -744,11 +744,23 @@ dbg_status seg_sort_records(dbg_ctx *ctx, const K *kin, const uint32_t *vin, K *
   return DBG_OK;
 }
 
-// The local pass of STEP-2 over n edge keys in the groups gr.  Leaves the E distinct keys in kin[0, E) and their
-// multiplicities in mult_out (allocated here); kstage (n keys) is scratch.
+// The tiles of STEP-2's local pass: tile t's tcount[t] distinct keys start at
+// bound[t] of the key buffer that they were staged in, their multiplicities
+// there in mult; toff numbers them.
+struct EdgeTiles {
+  uint64_t tiles = 0;
+  DevBuf bound, tcount, toff, mult;
+  void release() {
+    for (DevBuf *b : {&bound, &tcount, &toff, &mult}) b->release();
+  }
+};
+
+// The local pass of STEP-2 over n edge keys in the groups gr.  Leaves the E
+// distinct keys in kin[0, E) and their multiplicities in mult_out (allocated
+// here), kstage (n keys) being scratch; or, with `staged`, in kstage by tiles.
 template <class K>
-dbg_status seg_rle(dbg_ctx *ctx, K *kin, K *kstage, uint64_t n, Groups &gr, int key_bits, DevBuf &mult_out,
-                   uint64_t *E) {
+dbg_status seg_rle(dbg_ctx *ctx, K *kin, K *kstage, uint64_t n, Groups &gr, int key_bits, DevBuf *mult_out,
+                   EdgeTiles *staged, uint64_t *E) {
   using Sh = SegShape<K>;
   cudaStream_t s = ctx->stream;
   TileSet ts;
@@ -845,21 +857,30 @@ dbg_status seg_rle(dbg_ctx *ctx, K *kin, K *kstage, uint64_t n, Groups &gr, int 
   const uint32_t total = c[CT_TOTAL];
   const DevBuf &bound = ts.bound;
   *E = total;
-  DBG_TRY(alloc_buf(ctx, mult_out, std::max<uint64_t>(1, total) * 4));
+  if (staged) {
+    staged->tiles = tiles;
+    staged->bound = std::move(ts.bound);
+    staged->tcount = std::move(tcount);
+    staged->toff = std::move(toff);
+    staged->mult = std::move(mstage);
+    return DBG_OK;
+  }
+  DBG_TRY(alloc_buf(ctx, *mult_out, std::max<uint64_t>(1, total) * 4));
   DBG_LAUNCH(ctx, ST_LOCAL_SORT_EDGES, 2.0 * total * (sizeof(K) + 4),
              k_seg_compact<K><<<(unsigned)std::min<uint64_t>(tiles, 152ull * 16), 256, 0, s>>>(
                  bound.as<uint64_t>(), tcount.as<uint32_t>(), toff.as<uint64_t>(), tiles, kstage,
-                 mstage.as<uint32_t>(), kin, mult_out.as<uint32_t>()));
+                 mstage.as<uint32_t>(), kin, mult_out->as<uint32_t>()));
   DBG_CUDA_TRY(cudaGetLastError());
   return DBG_OK;
 }
 
 // STEP-2 over n edge keys by plan p (p.local()): the global passes, then the
 // local pass with the run-length reduce.  The E distinct keys end in *alt,
-// their multiplicities in mult.
+// their multiplicities in *mult, or (mult == nullptr) both as *staged tells.
 template <class K>
 dbg_status sort_count_keys(dbg_ctx *ctx, K **kp, K **alt, uint64_t n, const SortPlan<K> &p,
-                           const unsigned long long *d_hist, uint64_t *d_digit_base, DevBuf &mult, uint64_t *E) {
+                           const unsigned long long *d_hist, uint64_t *d_digit_base, DevBuf *mult, EdgeTiles *staged,
+                           uint64_t *E) {
   uint32_t *vn = nullptr, *van = nullptr;
   Groups gr;
   if (p.msd) {
@@ -868,8 +889,8 @@ dbg_status sort_count_keys(dbg_ctx *ctx, K **kp, K **alt, uint64_t n, const Sort
     DBG_TRY((radix_sort<K, false>(ctx, kp, alt, &vn, &van, n, p.bits, d_hist, d_digit_base, p.first_pass)));
     gr.lb.fixed = RADIX_BITS * p.first_pass;
   }
-  DBG_TRY(seg_rle<K>(ctx, *kp, *alt, n, gr, p.bits, mult, E));
-  std::swap(*kp, *alt);
+  DBG_TRY(seg_rle<K>(ctx, *kp, *alt, n, gr, p.bits, mult, staged, E));
+  if (!staged) std::swap(*kp, *alt);
   return DBG_OK;
 }
 
@@ -1161,7 +1182,7 @@ dbg_status count_node_kmers(dbg_ctx *ctx, const DevBuf &packed, const DevBuf &ba
   uint32_t *vn = nullptr, *van = nullptr;
   uint64_t D = 0;
   if (plan.local()) {
-    DBG_TRY(sort_count_keys<K>(ctx, &kp, &alt, M, plan, d_hist, d_digit_base, counts, &D));
+    DBG_TRY(sort_count_keys<K>(ctx, &kp, &alt, M, plan, d_hist, d_digit_base, &counts, nullptr, &D));
   } else {
     DBG_TRY(alloc_tmp(ctx, headpos, (M + 1) * sizeof(uint32_t)));
     DBG_TRY((radix_sort<K, false>(ctx, &kp, &alt, &vn, &van, M, kbits, d_hist, d_digit_base)));
@@ -1290,7 +1311,8 @@ dbg_status build_graph_impl(dbg_ctx *ctx, const BuildInput &in, dbg_graph *g) {
   // ---- K2 set-up: key buffers and histograms come first, so that host
   // reads can be emitted chunk by chunk as they are packed ----
   const int kbits = 2 * ((int)k + 1);
-  DevBuf keys_a, keys_b, headpos, mult_tmp, uniq;
+  DevBuf keys_a, keys_b, headpos, uniq;
+  EdgeTiles edge_tiles;  // the distinct keys in uniq, unless its run heads are in headpos
   uint64_t E = 0;
   const SortPlan<K> plan = plan_sort<K>(ctx, N, kbits, ctx->partition_first);
   if (N > 0) {
@@ -1365,9 +1387,9 @@ dbg_status build_graph_impl(dbg_ctx *ctx, const BuildInput &in, dbg_graph *g) {
     uint32_t *vn = nullptr, *van = nullptr;
     if (plan.local()) {
       // high digits globally, then the local sort with the run-length
-      // reduce: distinct keys into alt, multiplicities into mult_tmp
+      // reduce: distinct keys into alt, by tiles
       // (its last read-back brought the error word)
-      DBG_TRY(sort_count_keys<K>(ctx, &kp, &alt, N, plan, d_hist, d_digit_base, mult_tmp, &E));
+      DBG_TRY(sort_count_keys<K>(ctx, &kp, &alt, N, plan, d_hist, d_digit_base, nullptr, &edge_tiles, &E));
     } else {
       // every digit globally, then the run-length reduce
       DBG_TRY(alloc_tmp(ctx, headpos, (N + 1) * sizeof(uint32_t)));
@@ -1402,9 +1424,7 @@ dbg_status build_graph_impl(dbg_ctx *ctx, const BuildInput &in, dbg_graph *g) {
                       {{&g->edge_keys, E * sizeof(K)}, {&g->mult, E * sizeof(uint32_t)}, {&g->orient, E}}));
   DevBuf rk_a, rk_b, rv_a, rv_b;
   DBG_TRY(alloc_tmp(ctx, rk_a, R * sizeof(K) + MSD_PAD));
-  DBG_TRY(alloc_tmp(ctx, rk_b, R * sizeof(K) + MSD_PAD));
   DBG_TRY(alloc_tmp(ctx, rv_a, R * sizeof(uint32_t) + MSD_PAD));
-  DBG_TRY(alloc_tmp(ctx, rv_b, R * sizeof(uint32_t) + MSD_PAD));
   DBG_CUDA_TRY(cudaMemsetAsync(d_hist, 0, MAX_PASSES * RADIX * sizeof(unsigned long long), s));
   const SortPlan<K> rplan = plan_records<K>(ctx, R, nbits, true);
   const DigitSpec nspec = rplan.digits();
@@ -1412,11 +1432,22 @@ dbg_status build_graph_impl(dbg_ctx *ctx, const BuildInput &in, dbg_graph *g) {
   // the node IDs pass stores them per adjacency slot (for the compaction)
   const bool sides = E > 0 && E < (1ull << 29);
   if (E > 0) {
-    DBG_LAUNCH(ctx, ST_ENDPOINTS, (double)E * (3 * sizeof(K) + 4 + 4 + 1 + 8),
-               k_endpoints<K><<<grid_for(E, EMIT_TILE), EMIT_BLOCK, 0, s>>>(
-        uniq.as<K>(), headpos.p ? headpos.as<uint32_t>() : nullptr, mult_tmp.as<uint32_t>(), E, k,
-        g->edge_keys.as<K>(), g->mult.as<uint32_t>(),
-        g->orient.as<uint8_t>(), rk_a.as<K>(), rv_a.as<uint32_t>(), nspec, d_hist, sides));
+    const EdgeOut<K> out{g->edge_keys.as<K>(), g->mult.as<uint32_t>(), g->orient.as<uint8_t>(),
+                         rk_a.as<K>(),         rv_a.as<uint32_t>(),    sides};
+    const double bytes = (double)E * (4 * sizeof(K) + 4 + 4 + 1 + 8);
+    if (headpos.p)
+      DBG_LAUNCH(ctx, ST_ENDPOINTS, bytes,
+                 k_endpoints<K><<<grid_for(E, EMIT_TILE), EMIT_BLOCK, 0, s>>>(uniq.as<K>(), headpos.as<uint32_t>(), E,
+                                                                             k, out, nspec, d_hist));
+    else
+    {
+      const uint64_t per = std::min<uint64_t>(4, edge_tiles.tiles / (152 * 8) + 1);
+      DBG_LAUNCH(ctx, ST_ENDPOINTS, bytes,
+                 k_endpoints_tiles<K><<<(unsigned)((edge_tiles.tiles + per - 1) / per), EMIT_BLOCK, 0, s>>>(
+                     edge_tiles.bound.as<uint64_t>(), edge_tiles.tcount.as<uint32_t>(),
+                     edge_tiles.toff.as<uint64_t>(), (uint32_t)edge_tiles.tiles, (uint32_t)per, uniq.as<K>(),
+                     edge_tiles.mult.as<uint32_t>(), k, out, nspec, d_hist));
+    }
   }
   if (I > 0) {
     DBG_CUDA_TRY(cudaMemsetAsync(ctx->d_counters + 2, 0, sizeof(uint32_t), s));
@@ -1429,10 +1460,12 @@ dbg_status build_graph_impl(dbg_ctx *ctx, const BuildInput &in, dbg_graph *g) {
   DBG_CUDA_TRY(cudaGetLastError());
   uniq.release();
   headpos.release();
-  mult_tmp.release();
+  edge_tiles.release();
   packed.release();
   base_off.release();
   edge_off.release();
+  DBG_TRY(alloc_tmp(ctx, rk_b, R * sizeof(K) + MSD_PAD));
+  DBG_TRY(alloc_tmp(ctx, rv_b, R * sizeof(uint32_t) + MSD_PAD));
 
   // ---- STEP-3 sort of the node records (payload order kept), K6 node IDs +
   // adjacency rows, K7 neighbours ----
@@ -1794,7 +1827,7 @@ dbg_status build_bucketed_impl(dbg_ctx *ctx, const BucketInput &in, uint64_t bud
     if (plan.local()) {
       // multiplicities go where the run heads would (headpos is cnt + 1 long)
       DevBuf mdense;
-      DBG_TRY(sort_count_keys<K>(ctx, &kp, &alt, cnt, plan, d_hist, d_digit_base, mdense, &eb64));
+      DBG_TRY(sort_count_keys<K>(ctx, &kp, &alt, cnt, plan, d_hist, d_digit_base, &mdense, nullptr, &eb64));
       if (eb64) DBG_CUDA_TRY(cudaMemcpyAsync(headpos.p, mdense.p, eb64 * 4, cudaMemcpyDeviceToDevice, s));
     } else {
       DBG_TRY((radix_sort<K, false>(ctx, &kp, &alt, &vn, &van, cnt, kbits, d_hist, d_digit_base)));

@@ -1308,8 +1308,7 @@ static __global__ __launch_bounds__(SCAN_BLOCK) void k_scan_excl(const uint32_t 
 // negative strand, STEP-1's table gives (x^, y^, o1, o2) if x^ <= y^ and
 // (y^, x^, not o2, not o1) otherwise.  Writes orient, mult, a copy of the
 // key into the graph, and two node records per edge (payload e<<1 | role),
-// and accumulates the digit histograms of the node sort.  The multiplicity comes from the run heads
-// (headpos) or directly from mult_in.  With `sides` (E < 2^29), each payload
+// and accumulates the digit histograms of the node sort.  With `sides` (E < 2^29), each payload
 // also carries the side of its own end (bit 30) and of the edge's other end
 // (bit 31), for k_write_nodes to store per adjacency slot.
 // ---------------------------------------------------------------------------
@@ -1323,22 +1322,16 @@ __device__ __forceinline__ uint32_t end_side(uint8_t orient, uint32_t role) {
 }
 
 template <class K>
-__global__ __launch_bounds__(EMIT_BLOCK) void k_endpoints(const K *__restrict__ uniq,
-                                                          const uint32_t *__restrict__ headpos,
-                                                          const uint32_t *__restrict__ mult_in, uint64_t E,
-                                                          uint32_t k, K *__restrict__ edge_keys,
-                                                          uint32_t *__restrict__ mult,
-                                                          uint8_t *__restrict__ orient, K *__restrict__ rkeys,
-                                                          uint32_t *__restrict__ rvals, DigitSpec ds,
-                                                          unsigned long long *__restrict__ hist,
-                                                          bool sides = false) {
-  __shared__ uint32_t s_hist[MAX_PASSES * RADIX];
-  for (int i = threadIdx.x; i < ds.entries(); i += EMIT_BLOCK) s_hist[i] = 0;
-  __syncthreads();
-  const int kk = (int)k;
-  for (uint64_t e = (uint64_t)blockIdx.x * EMIT_TILE + threadIdx.x; e < min(E, (uint64_t)(blockIdx.x + 1) * EMIT_TILE);
-       e += EMIT_BLOCK) {
-    const K z = uniq[e];
+struct EdgeOut {
+  K *__restrict__ edge_keys;
+  uint32_t *__restrict__ mult;
+  uint8_t *__restrict__ orient;
+  K *__restrict__ rkeys;
+  uint32_t *__restrict__ rvals;
+  bool sides;
+  // edge e, with key z and multiplicity c
+  __device__ __forceinline__ void put(uint64_t e, const K &z, uint32_t c, int kk, const DigitSpec &ds,
+                                      uint32_t *s_hist) const {
     const K x = KeyOps<K>::shr(z, 2);
     const K y = KeyOps<K>::mask_low(z, 2 * kk);
     const K xh = kmin(x, revcomp(x, kk));
@@ -1351,14 +1344,86 @@ __global__ __launch_bounds__(EMIT_BLOCK) void k_endpoints(const K *__restrict__ 
     edge_keys[e] = z;
     const uint8_t o = (uint8_t)((a << 1) | b);
     orient[e] = o;
-    mult[e] = headpos ? headpos[e + 1] - headpos[e] : mult_in[e];
+    mult[e] = c;
     const uint32_t s0 = sides ? end_side(o, 0) : 0u, s1 = sides ? end_side(o, 1) : 0u;
-    rkeys[2 * e] = s;
-    rvals[2 * e] = (uint32_t)(e << 1) | s0 << 30 | s1 << 31;
-    rkeys[2 * e + 1] = d;
-    rvals[2 * e + 1] = (uint32_t)(e << 1) | 1u | s1 << 30 | s0 << 31;
+    const uint32_t v = (uint32_t)(e << 1);
+    if constexpr (sizeof(K) == 8) {
+      reinterpret_cast<ulonglong2 *>(rkeys)[e] = make_ulonglong2(s, d);
+    } else {
+      rkeys[2 * e] = s;
+      rkeys[2 * e + 1] = d;
+    }
+    reinterpret_cast<uint2 *>(rvals)[e] = make_uint2(v | s0 << 30 | s1 << 31, v | 1u | s1 << 30 | s0 << 31);
     ds.count(s_hist, s);
     ds.count(s_hist, d);
+  }
+};
+
+template <class K>
+__global__ __launch_bounds__(EMIT_BLOCK) void k_endpoints(const K *__restrict__ uniq,
+                                                          const uint32_t *__restrict__ headpos, uint64_t E,
+                                                          uint32_t k, EdgeOut<K> out, DigitSpec ds,
+                                                          unsigned long long *__restrict__ hist) {
+  __shared__ uint32_t s_hist[MAX_PASSES * RADIX];
+  for (int i = threadIdx.x; i < ds.entries(); i += EMIT_BLOCK) s_hist[i] = 0;
+  __syncthreads();
+  for (uint64_t e = (uint64_t)blockIdx.x * EMIT_TILE + threadIdx.x; e < min(E, (uint64_t)(blockIdx.x + 1) * EMIT_TILE);
+       e += EMIT_BLOCK)
+    out.put(e, uniq[e], headpos[e + 1] - headpos[e], (int)k, ds, s_hist);
+  __syncthreads();
+  for (int i = threadIdx.x; i < ds.entries(); i += EMIT_BLOCK)
+    if (s_hist[i]) atomicAdd(hist + i, (unsigned long long)s_hist[i]);
+}
+
+// The same from the local pass's tiles, where tile t's tcount[t] distinct keys
+// and their multiplicities start at bound[t] and its edges at toff[t]: they
+// need no dense copy in between.  A CTA takes `per` consecutive tiles, so that
+// what the chip writes at one time lies together.  Bound by memory: 1.57 ms
+// for 190 M edges (49 bytes each); with a dense copy first 1.57 + 0.96.
+// (per = 24: 1.79; a resident grid that takes every 1216th tile: 2.1.)
+template <class K>
+__global__ __launch_bounds__(EMIT_BLOCK) void k_endpoints_tiles(
+    const uint64_t *__restrict__ bound, const uint32_t *__restrict__ tcount, const uint64_t *__restrict__ toff,
+    uint32_t tiles, uint32_t per, const K *__restrict__ ustage, const uint32_t *__restrict__ mstage, uint32_t k, EdgeOut<K> out,
+    DigitSpec ds, unsigned long long *__restrict__ hist) {
+  __shared__ uint32_t s_hist[MAX_PASSES * RADIX];
+  for (int i = threadIdx.x; i < ds.entries(); i += EMIT_BLOCK) s_hist[i] = 0;
+  __syncthreads();
+  constexpr int ROWS = 4;  // loads in flight
+  uint32_t t = blockIdx.x * per, n = tcount[t];
+  uint64_t s = bound[t], o = toff[t];
+  const uint32_t last = min(tiles, t + per);
+  while (true) {
+    const uint32_t next = t + 1;
+    uint32_t n_next = 0;
+    uint64_t s_next = 0, o_next = 0;
+    if (next < last) {
+      n_next = tcount[next];
+      s_next = bound[next];
+      o_next = toff[next];
+    }
+    for (uint32_t r0 = threadIdx.x; r0 < n; r0 += ROWS * EMIT_BLOCK) {
+      K z[ROWS];
+      uint32_t c[ROWS];
+#pragma unroll
+      for (int i = 0; i < ROWS; i++) {
+        const uint32_t r = r0 + i * EMIT_BLOCK;
+        if (r < n) {
+          z[i] = ustage[s + r];
+          c[i] = mstage[s + r];
+        }
+      }
+#pragma unroll
+      for (int i = 0; i < ROWS; i++) {
+        const uint32_t r = r0 + i * EMIT_BLOCK;
+        if (r < n) out.put(o + r, z[i], c[i], (int)k, ds, s_hist);
+      }
+    }
+    if (next >= last) break;
+    t = next;
+    n = n_next;
+    s = s_next;
+    o = o_next;
   }
   __syncthreads();
   for (int i = threadIdx.x; i < ds.entries(); i += EMIT_BLOCK)
