@@ -1124,7 +1124,7 @@ dbg_status rank_and_assign(dbg_ctx *ctx, const K *rk, const uint32_t *rv, K *uke
   auto kern = I > 0 ? k_node_tiles<K, true> : k_node_tiles<K, false>;
   DBG_LAUNCH(ctx, ST_NODE_IDS,
              4.0 * R + R / 8.0 + (double)nv * (2 * sizeof(K) + 8) + (double)ne * (g->adj_side.p ? 14 : 13),
-             kern<<<(unsigned)std::min<uint64_t>(tiles, 3ull * (uint64_t)std::max(1, ctx->num_sms)), RANK_BLOCK, 0, s>>>(
+             kern<<<(unsigned)tiles, RANK_BLOCK, 0, s>>>(
                  ts.bound.as<uint64_t>(), (uint32_t)tiles, ukeys, vals, heads.as<uint32_t>(), tcount.as<uint32_t>(),
                  hoff.as<uint64_t>(), eoff.as<uint64_t>(), g->node_keys.as<K>(), g->row_ptr.as<uint64_t>(),
                  g->adj_edge.as<uint32_t>(), g->adj_role.as<uint8_t>(), g->adj_side.as<uint8_t>(),

@@ -765,6 +765,9 @@ __global__ __launch_bounds__(RANK_BLOCK) void k_tile_heads(K *__restrict__ keys,
 // slot is its own index.  Writes the tile's node keys and row starts, the
 // adjacency entries, and the edge ends partitioned by edge range (see
 // k_write_nodes).  Reads 4 bytes and a bit per record and 8 or 16 per node.
+// Launched with a CTA per tile, so that what the chip writes at one time lies
+// together: 2.6 ms for 380 M records (a resident grid that takes every 456th
+// tile: 2.9; without the loop the compiler's code is 3 to 6 % slower).
 template <class K, bool ISO>
 __global__ __launch_bounds__(RANK_BLOCK, ISO ? 2 : 3) void k_node_tiles(
     const uint64_t *__restrict__ bound, uint32_t tiles, const K *__restrict__ ukeys, const uint32_t *__restrict__ vals,
@@ -1098,9 +1101,6 @@ __global__ __launch_bounds__(SEG_BLOCK, 4) void k_seg_count(
     if (tid == 0) tcount[tile] = 0;
     return;
   }
-  for (int i = tid; i < S::WARPS * RADIX; i += SEG_BLOCK) (&sm.whist[0][0])[i] = 0;
-  if (RANK == RANK_ATOMIC)
-    for (int i = tid; i < S::WARPS * (RADIX + 1); i += SEG_BLOCK) (&sm.match[0][0])[i] = 0;
   for (int j = tid; j < S::TBL; j += SEG_BLOCK) {
     sm.keys[j] = O::empty();
     sm.vals[j] = 0;
@@ -1234,6 +1234,10 @@ __global__ __launch_bounds__(SEG_BLOCK, 4) void k_seg_count(
   if (!ranked && D > 0) {
     if (rank_groups && tid == 0) atomicAdd(rank_fb, 1u);
     // sort the D distinct keys (with their counts) by their offset bits
+    for (int i = tid; i < S::WARPS * RADIX; i += SEG_BLOCK) (&sm.whist[0][0])[i] = 0;
+    if (RANK == RANK_ATOMIC)
+      for (int i = tid; i < S::WARPS * (RADIX + 1); i += SEG_BLOCK) (&sm.match[0][0])[i] = 0;
+    __syncthreads();
     const int passes = (int)sm.passes;
     const int ipw = (int)((D + SEG_BLOCK - 1) / SEG_BLOCK);
     const uint32_t wofs = (uint32_t)warp * 32u * ipw;
