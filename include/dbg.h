@@ -520,7 +520,8 @@ dbg_status dbg_selftest_wait(dbg_ctx *ctx, uint32_t spin_limit);
  * adjacency, copies, compact_links, compact_rank, compact_cycles,
  * compact_output, local_sort_edges, local_sort_nodes, partition_edges
  * (the edge keys' first global pass when it is a partition; sort_edges
- * then holds their stable onesweep passes), node_mult (the k-mer counting
+ * then holds what follows: the counts and the second partition pass, or the
+ * stable onesweep passes), node_mult (the k-mer counting
  * for node multiplicities, whose sort passes count under the edge-key
  * sort stages).
  * -------------------------------------------------------------------- */

@@ -1,29 +1,25 @@
 // k_segsort.cuh -- the local half of the hybrid radix sort (K3 / STEP-2 and
-// STEP-3).  The global onesweep passes sort the keys by their high bits only
-// (the digits at and above bit `low_bits`), which leaves every group of keys
-// with equal high bits contiguous.  One CTA then finishes a run of whole
-// groups in shared memory: tile t covers [bound[t], bound[t+1]), where
-// bound[t] is the start of the group holding position t * TILE_T (found by
-// binary search, the high bits being sorted), so no group is split between
-// CTAs, and the keys are sorted by their remaining bits with an in-shared-
-// memory LSD radix sort.  Because the global passes are stable and the local
-// passes are stable, the result equals a full stable LSD sort.
+// STEP-3).  The global passes (unordered partitions, k_msd.cuh, or ordered
+// onesweep passes) bring the keys into groups that share their high bits, in
+// ascending order of those bits.  One CTA then finishes a run of whole groups
+// in shared memory: tile t covers [bound[t], bound[t+1]), where bound[t] is
+// the start of the group holding position t * TILE_T, so no group is split
+// between CTAs and no run of equal keys crosses a tile boundary.
 //
 // A tile longer than the shared-memory capacity (it holds a group of more
-// keys than that, e.g. a tandem repeat's (k+1)-mer) is "oversize": the host
-// gathers all oversize tiles into one buffer, sorts it with the global
-// passes over every digit, and the local kernels copy those results into
-// place instead of sorting.
+// keys than that, e.g. a tandem repeat's (k+1)-mer) is "oversize": all
+// oversize tiles are gathered into one buffer, which is sorted over every
+// digit by the ordered global passes; the results then go back into place.
 //
-// k_seg_sort sorts (key, payload) records (STEP-3's node records), with 256
-// threads of 24 items (126 registers, 2 CTAs per SM) or, in its wide form,
-// 384 threads of 16 items: the same capacity with half again the warps.
-// k_seg_rle finishes STEP-2 on the edge keys: it sorts them and writes each
-// distinct key once with the length of its run (its multiplicity) into the
-// tile's own range; k_seg_compact then packs the tiles' outputs.  Equal keys share their high bits, so no run of
-// equal keys crosses a tile boundary.  k_seg_count does the same work by
-// counting each tile's copies in a hash table first and sorting only the
-// distinct keys.
+// Edge keys (STEP-2): k_seg_count counts a tile's copies in a hash table and
+// orders the distinct keys; a tile with few copies of each key is ranked copy
+// by copy (k_rank_rle); k_seg_rle, by 8-bit digit passes, takes what neither
+// can.  Each writes the tile's distinct keys and multiplicities at the front
+// of its own range, from where k_endpoints_tiles reads them (or k_seg_compact
+// packs them).
+// Node records (STEP-3): k_seg_rank ranks records within small buckets, by
+// key and payload; k_seg_sort, by digit passes, takes tiles with crowded
+// buckets (256 threads of 24 items, or 384 of 16 in its wide form).
 #pragma once
 
 #include "k_build.cuh"
