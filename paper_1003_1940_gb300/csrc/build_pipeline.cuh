@@ -1884,8 +1884,9 @@ dbg_status build_bucketed_impl(dbg_ctx *ctx, const BucketInput &in, uint64_t bud
   auto nranges = plan_ranges(hist.data(), rec_cap, &sizes);
   *n_node_buckets = (uint32_t)nranges.size();
   const uint64_t etiles = (E + ENDS_TILE - 1) / ENDS_TILE;
-  DevBuf tcount, toff;
+  DevBuf tcount, toff, flags;
   if (E > 0) {
+    DBG_TRY(alloc_tmp(ctx, flags, (E + 31) / 32 * 8));
     DBG_TRY(alloc_tmp(ctx, tcount, etiles * 4));
     DBG_TRY(alloc_tmp(ctx, toff, (etiles + 1) * 8));
   }
@@ -1898,8 +1899,8 @@ dbg_status build_bucketed_impl(dbg_ctx *ctx, const BucketInput &in, uint64_t bud
     uint32_t Rc = 0;
     if (E > 0) {
       DBG_LAUNCH(ctx, ST_ENDPOINTS, (double)E * w,
-                 k_count_ends<K><<<(unsigned)etiles, ENDS_BLOCK, 0, s>>>(g->edge_keys.as<K>(), E, k, lo, hi,
-                                                                         tcount.as<uint32_t>()));
+                 k_count_ends<K><<<(unsigned)etiles, ENDS_BLOCK, 0, s>>>(
+                     g->edge_keys.as<K>(), E, k, lo, hi, flags.as<uint2>(), tcount.as<uint32_t>()));
       DBG_TRY(scan_u32(ctx, tcount.as<uint32_t>(), etiles, toff.as<uint64_t>(), &Rc, ST_ENDPOINTS));
     }
     const uint64_t cap = (uint64_t)Rc + I;
@@ -1916,7 +1917,7 @@ dbg_status build_bucketed_impl(dbg_ctx *ctx, const BucketInput &in, uint64_t bud
     if (Rc > 0)
       DBG_LAUNCH(ctx, ST_ENDPOINTS, (double)E * w + (double)Rc * (w + 4),
                  k_gather_ends<K><<<(unsigned)std::min<uint64_t>(etiles, 152ull * 8), ENDS_BLOCK, 0, s>>>(
-                     g->edge_keys.as<K>(), E, k, lo, hi, toff.as<uint64_t>(), etiles, ra.as<K>(), va.as<uint32_t>(),
+                     g->edge_keys.as<K>(), E, k, flags.as<uint2>(), toff.as<uint64_t>(), etiles, ra.as<K>(), va.as<uint32_t>(),
                      rplan.digits(), d_hist));
     uint64_t R = Rc;
     if (I > 0) {

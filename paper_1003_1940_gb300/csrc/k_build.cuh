@@ -1639,12 +1639,12 @@ __global__ void k_node_prefix_hist(const K *__restrict__ edge_keys, uint64_t E, 
 }
 
 // The edge ends whose node key's prefix is in [lo, hi), ENDS_TILE edges at a
-// time: their number per tile, and, given its scan, the ends as node records
-// in (e, role) order with the node-sort digit histograms.  Deriving an edge's
-// ends twice, from 8 or 16 bytes, costs less than a flag and a 64-bit position
-// per end in memory: 48 and 104 us for
-// a seventh of 13.6 M edges' ends, where flags, their scan and the gather took 50,
-// 190 and 73.
+// time: two flags per edge and their number per tile, and, given its scan, the
+// ends as node records in (e, role) order with the node-sort digit histograms.
+// Deriving an edge's ends is most of the work (two canonical k-mers), so the
+// flags save deriving those of edges out of range again: 55 + 70 us for a
+// seventh of 13.6 M edges' ends (without flags 48 + 104; a 32-bit flag per end
+// scanned into 64-bit positions took 50 + 190 + 73).
 constexpr int ENDS_BLOCK = 256, ENDS_ITEMS = 8, ENDS_TILE = ENDS_BLOCK * ENDS_ITEMS;
 
 template <class K>
@@ -1657,7 +1657,8 @@ __device__ __forceinline__ uint32_t ends_in_range(const K &edge, uint32_t k, uin
 
 template <class K>
 __global__ __launch_bounds__(ENDS_BLOCK) void k_count_ends(const K *__restrict__ edge_keys, uint64_t E, uint32_t k,
-                                                           uint32_t lo, uint32_t hi, uint32_t *__restrict__ tcount) {
+                                                           uint32_t lo, uint32_t hi, uint2 *__restrict__ flags,
+                                                           uint32_t *__restrict__ tcount) {
   __shared__ uint32_t total;
   if (threadIdx.x == 0) total = 0;
   __syncthreads();
@@ -1667,9 +1668,11 @@ __global__ __launch_bounds__(ENDS_BLOCK) void k_count_ends(const K *__restrict__
   for (int i = 0; i < ENDS_ITEMS; i++) {
     const uint64_t e = first + (uint64_t)i * ENDS_BLOCK;
     K s, d;
-    if (e < E) sum += __popc(ends_in_range<K>(edge_keys[e], k, lo, hi, s, d));
+    const uint32_t f = e < E ? ends_in_range<K>(edge_keys[e], k, lo, hi, s, d) : 0u;
+    const unsigned b0 = __ballot_sync(0xffffffffu, f & 1u), b1 = __ballot_sync(0xffffffffu, f & 2u);
+    if ((threadIdx.x & 31) == 0 && e < E) flags[e / 32] = make_uint2(b0, b1);
+    sum += __popc(b0) + __popc(b1);
   }
-  sum = __reduce_add_sync(0xffffffffu, sum);
   if ((threadIdx.x & 31) == 0) atomicAdd(&total, sum);
   __syncthreads();
   if (threadIdx.x == 0) tcount[blockIdx.x] = total;
@@ -1677,7 +1680,7 @@ __global__ __launch_bounds__(ENDS_BLOCK) void k_count_ends(const K *__restrict__
 
 template <class K>
 __global__ __launch_bounds__(ENDS_BLOCK) void k_gather_ends(const K *__restrict__ edge_keys, uint64_t E, uint32_t k,
-                                                            uint32_t lo, uint32_t hi,
+                                                            const uint2 *__restrict__ flags,
                                                             const uint64_t *__restrict__ toff, uint64_t tiles,
                                                             K *__restrict__ rkeys, uint32_t *__restrict__ rvals,
                                                             DigitSpec ds, unsigned long long *__restrict__ hist) {
@@ -1693,11 +1696,9 @@ __global__ __launch_bounds__(ENDS_BLOCK) void k_gather_ends(const K *__restrict_
 #pragma unroll
     for (int i = 0; i < ENDS_ITEMS; i++) {
       const uint64_t e = first + (uint64_t)i * ENDS_BLOCK;
-      K s, d;
-      const uint32_t f = e < E ? ends_in_range<K>(edge_keys[e], k, lo, hi, s, d) : 0u;
-      const unsigned b0 = __ballot_sync(0xffffffffu, f & 1u), b1 = __ballot_sync(0xffffffffu, f & 2u);
-      at[i] = (uint32_t)(__popc(b0 & lt) + __popc(b1 & lt)) << 2 | f;
-      if (lane == 0) s_cnt[i * WARPS + warp] = __popc(b0) + __popc(b1);
+      const uint2 b = e - lane < E ? flags[e / 32] : make_uint2(0u, 0u);
+      at[i] = (uint32_t)(__popc(b.x & lt) + __popc(b.y & lt)) << 2 | (b.x >> lane & 1u) | (b.y >> lane & 1u) << 1;
+      if (lane == 0) s_cnt[i * WARPS + warp] = __popc(b.x) + __popc(b.y);
     }
     __syncthreads();
     if (warp == 0) {
