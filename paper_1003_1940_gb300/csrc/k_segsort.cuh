@@ -168,8 +168,10 @@ __global__ void k_seg_gather(const K *__restrict__ kin, const uint32_t *__restri
 // The tile's range, its base (the first key with its group's low bits
 // cleared: no key of the tile is below it) and, from the last key with its
 // group's low bits set, the bits that key offsets span and the number of
-// local passes over them, into shared memory.  The caller checks that the
-// tile is not oversize.
+// local passes over them, into shared memory.  There is always one pass: a
+// tile of copies of one key, in a group with no bits below it, spans no bits,
+// and the digit passes are also what puts the keys into shared memory.  The
+// caller checks that the tile is not oversize.
 template <class K, class S>
 __device__ __forceinline__ void seg_setup(S &sm, const K *__restrict__ kin, const uint64_t *__restrict__ bound,
                                           uint32_t tile, LowBits lb) {
@@ -182,7 +184,7 @@ __device__ __forceinline__ void seg_setup(S &sm, const K *__restrict__ kin, cons
       sm.base = KeyOps<K>::sub(first, KeyOps<K>::mask_low(first, lb.of(first)));
       const K range = KeyOps<K>::sub(KeyOps<K>::fill_low(last, lb.of(last)), sm.base);
       sm.span_bits = (uint32_t)KeyOps<K>::bitlen(range);
-      sm.passes = (sm.span_bits + RADIX_BITS - 1) / RADIX_BITS;
+      sm.passes = max(1u, (sm.span_bits + RADIX_BITS - 1) / RADIX_BITS);
       sm.range = range;
     }
   }
