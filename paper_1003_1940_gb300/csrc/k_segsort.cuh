@@ -1122,7 +1122,9 @@ __global__ __launch_bounds__(SEG_BLOCK, 4) void k_seg_count(
       const uint32_t j = j0 + (uint32_t)i * SEG_BLOCK + tid;
       d[i] = j < cnt ? KeyOps<K>::sub(kin[s + j], base) : O::empty();
     }
-    if (*reinterpret_cast<volatile uint32_t *>(&sm.overflow)) break;
+    // (the whole warp leaves or none of it: another warp may set the flag while
+    // this one reads it, and the sample below counts with all lanes)
+    if (__any_sync(0xffffffffu, *reinterpret_cast<volatile uint32_t *>(&sm.overflow))) break;
 #pragma unroll
     for (int i = 0; i < S::LOAD; i++) {
       // (128-bit tiles are one batch long; in 64-bit ones, of two, a test here
