@@ -20,6 +20,7 @@
 
 #include "dbg_device.cuh"
 #include "dbg_internal.h"
+#include "window_rows.h"
 
 namespace dbg {
 
@@ -1514,8 +1515,9 @@ __global__ __launch_bounds__(EMIT_BLOCK) void k_emit_prefix_hist(const uint64_t 
     const uint64_t e0 = __ldg(edge_off + r), p = __ldg(base_off + r) + lane;
     const uint32_t cnt = (uint32_t)(__ldg(edge_off + r + 1) - e0);
     const uint64_t *w = packed + (p >> 5);
-    for (uint32_t j0 = 0; j0 < cnt; j0 += 32, w++)
-      if (cnt - j0 > lane)
+    const uint32_t rows = window_rows(cnt);
+    for (uint32_t row = 0; row < rows; row++, w++)
+      if (in_row(cnt, row, lane))
         atomicAdd(&s_hist[key_prefix(canonical_window<K>(w, (uint32_t)p * 2 & 30u, (uint32_t)p & 16u, m), 2 * m)], 1u);
   }
   __syncthreads();
@@ -1565,10 +1567,11 @@ __global__ __launch_bounds__(EMIT_BLOCK) void k_emit_range(const uint64_t *__res
     const uint64_t e0 = __ldg(edge_off + r), p = __ldg(base_off + r) + lane;
     const uint32_t cnt = (uint32_t)(__ldg(edge_off + r + 1) - e0);
     const uint64_t *w = packed + (p >> 5);
-    for (uint32_t j0 = 0; j0 < cnt; j0 += 32, w++) {
+    const uint32_t rows = window_rows(cnt);
+    for (uint32_t row = 0; row < rows; row++, w++) {
       K key = KeyOps<K>::zero();
       bool in = false;
-      if (cnt - j0 > lane) {
+      if (in_row(cnt, row, lane)) {
         key = canonical_window<K>(w, (uint32_t)p * 2 & 30u, (uint32_t)p & 16u, m);
         const uint32_t pf = key_prefix(key, 2 * m);
         in = pf >= lo && pf < hi;
