@@ -602,7 +602,7 @@ dbg_status seg_tiles(dbg_ctx *ctx, const K *kin, uint64_t n, Groups &gr, TileSet
                                                                  (uint32_t)(SEG_BLOCK * Sh::ITEMS),
                                                                  ts.osize.as<uint32_t>(), ts.olist.as<uint32_t>(),
                                                                  ctx->d_counters + CT_GATHERED,
-                                                                 ctx->d_counters + CT_OVERSIZE));
+                                                                 ctx->d_counters + CT_OVERSIZE, ctx->d_err));
   DBG_CUDA_TRY(cudaGetLastError());
   return DBG_OK;
 }

@@ -100,10 +100,22 @@ __global__ void k_seg_bounds(const K *__restrict__ keys, uint64_t n, int low_bit
 }
 
 // osize[t] = the tile's length if it exceeds cap (an oversize tile), else 0;
-// those tiles' numbers in olist, their keys added up in *keys.
-static __global__ void k_seg_oversize(const uint64_t *__restrict__ bound, uint64_t tiles, uint32_t cap,
+// those tiles' numbers in olist, their keys added up in *keys.  If a wait of
+// the global passes ran out (*err), some keys were never written: then every
+// tile is made empty, so that the local kernels, which trust the keys to lie in
+// their groups, read none, and the host finds the error in its next read-back.
+static __global__ void k_seg_oversize(uint64_t *__restrict__ bound, uint64_t tiles, uint32_t cap,
                                       uint32_t *__restrict__ osize, uint32_t *__restrict__ olist,
-                                      uint32_t *__restrict__ keys, uint32_t *__restrict__ count) {
+                                      uint32_t *__restrict__ keys, uint32_t *__restrict__ count,
+                                      const uint32_t *__restrict__ err) {
+  if (*err & (ERR_TIMEOUT | ERR_INTERNAL)) {
+    for (uint64_t t = (uint64_t)blockIdx.x * blockDim.x + threadIdx.x; t < tiles; t += (uint64_t)gridDim.x * blockDim.x) {
+      bound[t] = 0;
+      osize[t] = 0;
+      if (t == tiles - 1) bound[tiles] = 0;
+    }
+    return;
+  }
   for (uint64_t t = (uint64_t)blockIdx.x * blockDim.x + threadIdx.x; t < tiles; t += (uint64_t)gridDim.x * blockDim.x) {
     const uint64_t sz = bound[t + 1] - bound[t];
     osize[t] = sz > cap ? (uint32_t)sz : 0u;
@@ -142,6 +154,7 @@ __global__ void k_permute(const uint64_t *__restrict__ w, uint64_t n, const K *_
                           const uint32_t *__restrict__ vin, K *__restrict__ kout, uint32_t *__restrict__ vout) {
   for (uint64_t i = (uint64_t)blockIdx.x * blockDim.x + threadIdx.x; i < n; i += (uint64_t)gridDim.x * blockDim.x) {
     const uint32_t j = (uint32_t)w[i];
+    if (j >= n) continue;  // (a wait of the words' sort ran out: the host finds the error)
     kout[i] = kin[j];
     vout[i] = vin[j];
   }
