@@ -301,9 +301,10 @@ template <> struct SegShape<Key128> {
 
 // The first global pass of the hybrid sort of n keys of `bits` bits: the
 // largest p >= 2 for which keys sharing their bits from 8p up form groups of
-// at most MAX_MEAN keys on average (for uniform keys); 0 = no hybrid.
+// at most MAX_MEAN keys on average, for keys `density` times as dense as
+// uniform ones; 0 = no hybrid.
 template <class K>
-int hybrid_first_pass(uint64_t n, int bits) {
+int hybrid_first_pass(uint64_t n, int bits, double density = 1.0) {
   const int P = passes_for_bits(bits);
   for (int p = P; p >= 2; p--) {
     const int hi = bits - RADIX_BITS * p;
@@ -311,7 +312,7 @@ int hybrid_first_pass(uint64_t n, int bits) {
       if (n <= (uint64_t)SegShape<K>::TILE) return p;  // one tile holds every key
       continue;
     }
-    if ((double)n <= SegShape<K>::MAX_MEAN * std::ldexp(1.0, hi)) return p;
+    if ((double)n * density <= SegShape<K>::MAX_MEAN * std::ldexp(1.0, hi)) return p;
   }
   return 0;
 }
@@ -329,6 +330,7 @@ template <class K> constexpr uint32_t msd_mean() { return SegShape<K>::TILE / 4;
 template <class K>
 struct SortPlan {
   bool msd = false;
+  uint32_t mean = msd_mean<K>();  // MSD: the groups' size aimed at
   int first_pass = 0, adj = 0;  // least significant first
   int bits = 0;                 // key bits
   int need = 0;                 // MSD: bits that groups of the mean size take,
@@ -353,16 +355,22 @@ struct SortPlan {
 // groups that end above the lowest bits: at most one key value per group in
 // four would be needed, so that the copies of one key alone seldom fill a
 // group.  Up to 2^10 groups in one pass; above, two digits of equal width
-// (the second then varies by bucket).
+// (the second then varies by bucket).  density > 1, for the offsets of one
+// key range: how many times denser than over all values of `bits` bits the keys
+// lie where they are.  Their groups are planned at a quarter of the mean: the
+// range ends anywhere in its last bucket, whose keys may lie in an eighth of
+// it.
 template <class K>
-SortPlan<K> plan_sort(const dbg_ctx *ctx, uint64_t n, int bits, bool unordered) {
+SortPlan<K> plan_sort(const dbg_ctx *ctx, uint64_t n, int bits, bool unordered, double density = 1.0) {
+  const double dense = (double)n * density;
   SortPlan<K> p;
+  if (density > 1.0) p.mean /= 4;
   p.bits = bits;
   if (!ctx->hybrid_sort) return p;
   if (unordered && n <= 0xffffffffull) {
     int need = 0;
     if (n > (uint64_t)SegShape<K>::TILE)
-      while (((uint64_t)msd_mean<K>() << need) < n) need++;
+      while (std::ldexp((double)p.mean, need) < dense) need++;
     if (need + (need ? 2 : 0) <= bits && need <= 24) {
       p.msd = true;
       p.passes = need == 0 ? 0 : need <= 10 ? 1 : 2;
@@ -371,7 +379,7 @@ SortPlan<K> plan_sort(const dbg_ctx *ctx, uint64_t n, int bits, bool unordered) 
       return p;
     }
   }
-  p.first_pass = hybrid_first_pass<K>(n, bits);
+  p.first_pass = hybrid_first_pass<K>(n, bits, density);
   return p;
 }
 
@@ -499,7 +507,7 @@ dbg_status msd_sort(dbg_ctx *ctx, K **keys, K **alt_keys, uint32_t **vals, uint3
   // the second digit of a bucket four times the average size, if it fits
   const int max_w2 = std::min({HAS_VAL ? 11 : MSD_MAX_BITS, p.shift1(), p.need - p.w1 + 2});
   // every bucket has at most max(1, 2 n_b / mean) groups
-  gr.ng_max = two ? (uint32_t)(2 * (n / msd_mean<K>()) + W) : W;
+  gr.ng_max = two ? (uint32_t)(2 * (n / p.mean) + W) : W;
   // [start: W + 1] u64, [cursor: W][gfirst: W + 1][tfirst: W + 1] u32, [tmap] u16, [w2][low] u8
   const size_t bytes = (size_t)(W + 1) * 8 + (size_t)(3 * W + 2) * 4 + (two ? tiles2 * 2 : 0) + 2 * (size_t)W + 16;
   DBG_TRY(alloc_tmp(ctx, gr.tables, bytes));
@@ -512,7 +520,7 @@ dbg_status msd_sort(dbg_ctx *ctx, K **keys, K **alt_keys, uint32_t **vals, uint3
   tb.w2 = reinterpret_cast<uint8_t *>(tb.tmap + (two ? tiles2 : 0));
   tb.low = tb.w2 + W;
   DBG_LAUNCH(ctx, stage, 0.0,
-             k_msd_plan<<<1, 1024, 0, s>>>(d_hist, p.w1, p.shift1(), two ? 1 : 0, msd_mean<K>(), max_w2, tile2, tb,
+             k_msd_plan<<<1, 1024, 0, s>>>(d_hist, p.w1, p.shift1(), two ? 1 : 0, p.mean, max_w2, tile2, tb,
                                            cursor));
   const double bytes_pass = 2.0 * (double)n * (double)(sizeof(K) + (HAS_VAL ? 4 : 0));
   auto swap = [&]() {
@@ -939,6 +947,12 @@ inline int bit_length(uint64_t x) {
   while (x >> b) b++;
   return b;
 }
+// x << shift, as a key
+inline uint64_t key_from(uint64_t x, int shift, uint64_t) { return shift < 64 ? x << shift : 0; }
+inline Key128 key_from(uint64_t x, int shift, Key128) {
+  if (shift >= 64) return Key128{x << (shift - 64), 0};
+  return Key128{shift ? x >> (64 - shift) : 0, x << shift};
+}
 inline ValOrder edge_end_order(uint64_t edges, bool sides, bool isolated) {
   ValOrder vo;
   vo.shift = sides ? 2 : 0;
@@ -956,8 +970,8 @@ inline ValOrder read_order(uint64_t reads) {
 // within groups, the digits are aligned with the top of the key, so that the
 // global passes resolve 8 bits each of it and leave short groups.
 template <class K>
-SortPlan<K> plan_records(const dbg_ctx *ctx, uint64_t R, int bits, bool align) {
-  SortPlan<K> p = plan_sort<K>(ctx, R, bits, ctx->partition_first && ctx->seg_rank);
+SortPlan<K> plan_records(const dbg_ctx *ctx, uint64_t R, int bits, bool align, double density = 1.0) {
+  SortPlan<K> p = plan_sort<K>(ctx, R, bits, ctx->partition_first && ctx->seg_rank, density);
   if (!p.msd && ctx->hybrid_sort && ctx->seg_rank && align) {
     const int adj = (8 - bits % 8) % 8;
     const int q0 = hybrid_first_pass<K>(R, bits + adj);
@@ -1700,6 +1714,23 @@ inline std::vector<std::pair<uint32_t, uint32_t>> plan_ranges(const uint64_t *hi
   return out;
 }
 
+// The keys of prefixes [lo, hi) among keys of key_bits bits: the first of
+// them, the bits of their offsets from it, and how much denser those are than
+// if they filled all values of as many bits.
+template <class K>
+struct KeyRange {
+  K base;
+  int bits;
+  double density;
+};
+template <class K>
+KeyRange<K> key_range(uint32_t lo, uint32_t hi, int key_bits) {
+  hi = std::min(hi, 1u << std::min(PREFIX_BITS, key_bits));  // (short keys have fewer prefixes than there are bins)
+  if (hi <= lo) hi = lo + 1;                                 // (of an empty range)
+  const int low = std::max(0, key_bits - PREFIX_BITS), top = bit_length(hi - lo - 1);
+  return KeyRange<K>{key_from(lo, low, K{}), std::max(1, low + top), std::ldexp(1.0, top) / (hi - lo)};
+}
+
 template <class K>
 dbg_status concat_chunks(dbg_ctx *ctx, std::vector<DevBuf> &chunks, const std::vector<uint64_t> &counts,
                          size_t elem, void *dst) {
@@ -1814,11 +1845,12 @@ dbg_status build_bucketed_impl(dbg_ctx *ctx, const BucketInput &in, uint64_t bud
     DBG_TRY(alloc_tmp(ctx, headpos, (cnt + 1) * 4));
     DBG_CUDA_TRY(cudaMemsetAsync(d_hist, 0, MAX_PASSES * RADIX * 8, s));
     DBG_CUDA_TRY(cudaMemsetAsync(ctx->d_counters + 8, 0, 4, s));
-    const SortPlan<K> plan = plan_sort<K>(ctx, cnt, kbits, ctx->partition_first);
+    const KeyRange<K> kr = key_range<K>(ranges[b].first, ranges[b].second, kbits);
+    const SortPlan<K> plan = plan_sort<K>(ctx, cnt, kr.bits, ctx->partition_first, kr.density);
     DBG_LAUNCH(ctx, ST_EMIT, 8.0 * nwords + 16.0 * n + (double)cnt * w,
                k_emit_range<K><<<emit_grid, EMIT_BLOCK, EMIT_BLOCK / 32 * EMIT_BUF<K> * sizeof(K), s>>>(packed.as<uint64_t>(), base_off.as<uint64_t>(),
                                                                 edge_off.as<uint64_t>(), n, k, ranges[b].first,
-                                                                ranges[b].second, ka.as<K>(), ctx->d_counters + 8,
+                                                                ranges[b].second, kr.base, ka.as<K>(), ctx->d_counters + 8,
                                                                 plan.digits(), d_hist));
     DBG_CUDA_TRY(cudaGetLastError());
     K *kp = ka.as<K>(), *alt = kb.as<K>();
@@ -1830,7 +1862,7 @@ dbg_status build_bucketed_impl(dbg_ctx *ctx, const BucketInput &in, uint64_t bud
       DBG_TRY(sort_count_keys<K>(ctx, &kp, &alt, cnt, plan, d_hist, d_digit_base, &mdense, nullptr, &eb64));
       if (eb64) DBG_CUDA_TRY(cudaMemcpyAsync(headpos.p, mdense.p, eb64 * 4, cudaMemcpyDeviceToDevice, s));
     } else {
-      DBG_TRY((radix_sort<K, false>(ctx, &kp, &alt, &vn, &van, cnt, kbits, d_hist, d_digit_base)));
+      DBG_TRY((radix_sort<K, false>(ctx, &kp, &alt, &vn, &van, cnt, kr.bits, d_hist, d_digit_base)));
       DBG_TRY(run_length_reduce<K>(ctx, kp, cnt, alt, headpos.as<uint32_t>(), &eb64));
     }
     DBG_TRY(check_device_error(ctx));
@@ -1841,7 +1873,7 @@ dbg_status build_bucketed_impl(dbg_ctx *ctx, const BucketInput &in, uint64_t bud
     DBG_TRY(alloc_tmp(ctx, o1, std::max<uint64_t>(1, eb)));
     if (eb)
       DBG_LAUNCH(ctx, ST_ENDPOINTS, (double)eb * (2 * w + 9),
-                 k_edge_finish<K><<<grid_for(eb, 256), 256, 0, s>>>(alt, plan.local() ? nullptr : headpos.as<uint32_t>(),
+                 k_edge_finish<K><<<grid_for(eb, 256), 256, 0, s>>>(alt, kr.base, plan.local() ? nullptr : headpos.as<uint32_t>(),
                                                                    headpos.as<uint32_t>(), eb, k, k1.as<K>(),
                                                                    m1.as<uint32_t>(), o1.as<uint8_t>()));
     ck.push_back(std::move(k1));
@@ -1912,19 +1944,20 @@ dbg_status build_bucketed_impl(dbg_ctx *ctx, const BucketInput &in, uint64_t bud
     DBG_TRY(alloc_tmp(ctx, vb, cap * 4 + MSD_PAD));
     // (planned for every record that the range may hold: isolated reads are
     // counted by the range only)
-    const SortPlan<K> rplan = plan_records<K>(ctx, cap, nbits, false);
+    const KeyRange<K> kr = key_range<K>(lo, hi, nbits);
+    const SortPlan<K> rplan = plan_records<K>(ctx, cap, kr.bits, false, kr.density);
     DBG_CUDA_TRY(cudaMemsetAsync(d_hist, 0, MAX_PASSES * RADIX * 8, s));
     if (Rc > 0)
       DBG_LAUNCH(ctx, ST_ENDPOINTS, (double)E * w + (double)Rc * (w + 4),
                  k_gather_ends<K><<<(unsigned)std::min<uint64_t>(etiles, 152ull * 8), ENDS_BLOCK, 0, s>>>(
-                     g->edge_keys.as<K>(), E, k, flags.as<uint2>(), toff.as<uint64_t>(), etiles, ra.as<K>(), va.as<uint32_t>(),
+                     g->edge_keys.as<K>(), E, k, flags.as<uint2>(), toff.as<uint64_t>(), etiles, kr.base, ra.as<K>(), va.as<uint32_t>(),
                      rplan.digits(), d_hist));
     uint64_t R = Rc;
     if (I > 0) {
       DBG_CUDA_TRY(cudaMemsetAsync(ctx->d_counters + 9, 0, 4, s));
       DBG_LAUNCH(ctx, ST_ENDPOINTS, (double)n * 4,
                  k_isolated_range<K><<<grid_for(n, 256), 256, 0, s>>>(packed.as<uint64_t>(), base_off.as<uint64_t>(),
-                                                                     in.d_lengths, n, k, lo, hi, ra.as<K>() + Rc,
+                                                                     in.d_lengths, n, k, lo, hi, kr.base, ra.as<K>() + Rc,
                                                                      va.as<uint32_t>() + Rc, ctx->d_counters + 9,
                                                                      rplan.digits(), d_hist));
       uint32_t iso = 0;
@@ -1946,7 +1979,8 @@ dbg_status build_bucketed_impl(dbg_ctx *ctx, const BucketInput &in, uint64_t bud
     DBG_TRY(alloc_tmp(ctx, nk, std::max<uint64_t>(1, Vc) * w));
     DBG_TRY(alloc_tmp(ctx, rp, std::max<uint64_t>(1, Vc) * 8));
     if (Vc) {
-      DBG_CUDA_TRY(cudaMemcpyAsync(nk.p, rk_alt, Vc * w, cudaMemcpyDeviceToDevice, s));
+      DBG_LAUNCH(ctx, ST_COPIES, 2.0 * Vc * w,
+                 k_add_base<K><<<grid_for(Vc, 256 * 8), 256, 0, s>>>(rk_alt, Vc, kr.base, nk.as<K>()));
       DBG_CUDA_TRY(cudaMemcpyAsync(rp.p, row_tmp.p, Vc * 8, cudaMemcpyDeviceToDevice, s));
     }
     cnk.push_back(std::move(nk));

@@ -1488,6 +1488,13 @@ namespace dbg {
 // ---------------------------------------------------------------------------
 // Key-range buckets (the bucket path of dbg_build_bucketed).  A key's prefix
 // is its top PREFIX_BITS bits (all its bits when it is shorter).
+//
+// A range's keys are sorted as their offsets from its first key (`base`): the
+// top bits that they share leave the sort, and the digits of its plan are the
+// bits that differ.  (Planned over whole keys, a range of one bin in 9 to 21
+// had groups that many times the size aimed at, and nearly every local tile
+// was too long for shared memory: 7 M instances in 9 edge and 42 node ranges
+// 22.5 ms, with offsets 9.9.)
 // ---------------------------------------------------------------------------
 constexpr int PREFIX_BITS = 12;
 constexpr int PREFIX_BINS = 1 << PREFIX_BITS;
@@ -1539,7 +1546,7 @@ template <class K>
 __global__ __launch_bounds__(EMIT_BLOCK) void k_emit_range(const uint64_t *__restrict__ packed,
                                                            const uint64_t *__restrict__ base_off,
                                                            const uint64_t *__restrict__ edge_off, uint64_t n_reads,
-                                                           uint32_t k, uint32_t lo, uint32_t hi,
+                                                           uint32_t k, uint32_t lo, uint32_t hi, K range_base,
                                                            K *__restrict__ keys, uint32_t *count, DigitSpec ds,
                                                            unsigned long long *__restrict__ hist) {
   extern __shared__ __align__(16) unsigned char emit_buf[];
@@ -1578,7 +1585,7 @@ __global__ __launch_bounds__(EMIT_BLOCK) void k_emit_range(const uint64_t *__res
       }
       const unsigned b = __ballot_sync(0xffffffffu, in);
       if (held + __popc(b) > EMIT_BUF<K>) flush();
-      if (in) buf[held + __popc(b & lt)] = key;
+      if (in) buf[held + __popc(b & lt)] = KeyOps<K>::sub(key, range_base);
       held += __popc(b);
       __syncwarp();
     }
@@ -1607,11 +1614,11 @@ __device__ __forceinline__ void edge_ends(const K &z, int k, K &s, K &d, uint32_
 // Edges of one bucket: key, multiplicity (from the run heads, or directly
 // from mult_in) and orientation.
 template <class K>
-__global__ void k_edge_finish(const K *__restrict__ uniq, const uint32_t *__restrict__ headpos,
+__global__ void k_edge_finish(const K *__restrict__ uniq, K range_base, const uint32_t *__restrict__ headpos,
                               const uint32_t *__restrict__ mult_in, uint64_t E, uint32_t k,
                               K *__restrict__ edge_keys, uint32_t *__restrict__ mult, uint8_t *__restrict__ orient) {
   for (uint64_t e = (uint64_t)blockIdx.x * blockDim.x + threadIdx.x; e < E; e += (uint64_t)gridDim.x * blockDim.x) {
-    const K z = uniq[e];
+    const K z = KeyOps<K>::add(uniq[e], range_base);
     K s, d;
     uint32_t o;
     edge_ends(z, (int)k, s, d, o);
@@ -1685,7 +1692,7 @@ template <class K>
 __global__ __launch_bounds__(ENDS_BLOCK) void k_gather_ends(const K *__restrict__ edge_keys, uint64_t E, uint32_t k,
                                                             const uint2 *__restrict__ flags,
                                                             const uint64_t *__restrict__ toff, uint64_t tiles,
-                                                            K *__restrict__ rkeys, uint32_t *__restrict__ rvals,
+                                                            K range_base, K *__restrict__ rkeys, uint32_t *__restrict__ rvals,
                                                             DigitSpec ds, unsigned long long *__restrict__ hist) {
   constexpr int WARPS = ENDS_BLOCK / 32;
   __shared__ uint32_t s_hist[MAX_PASSES * RADIX];
@@ -1721,11 +1728,13 @@ __global__ __launch_bounds__(ENDS_BLOCK) void k_gather_ends(const K *__restrict_
       edge_ends(edge_keys[e], (int)k, s, d, o);
       uint64_t p = base + s_cnt[i * WARPS + warp] + (at[i] >> 2);
       if (at[i] & 1u) {
+        s = KeyOps<K>::sub(s, range_base);
         rkeys[p] = s;
         rvals[p++] = (uint32_t)(e << 1);
         ds.count(s_hist, s);
       }
       if (at[i] & 2u) {
+        d = KeyOps<K>::sub(d, range_base);
         rkeys[p] = d;
         rvals[p] = (uint32_t)(e << 1) | 1u;
         ds.count(s_hist, d);
@@ -1743,7 +1752,7 @@ __global__ __launch_bounds__(ENDS_BLOCK) void k_gather_ends(const K *__restrict_
 template <class K>
 __global__ void k_isolated_range(const uint64_t *__restrict__ packed, const uint64_t *__restrict__ base_off,
                                  const uint32_t *__restrict__ len, uint64_t n, uint32_t k, uint32_t lo, uint32_t hi,
-                                 K *__restrict__ rkeys, uint32_t *__restrict__ rvals, uint32_t *slot, DigitSpec ds,
+                                 K range_base, K *__restrict__ rkeys, uint32_t *__restrict__ rvals, uint32_t *slot, DigitSpec ds,
                                  unsigned long long *__restrict__ hist) {
   for (uint64_t r = (uint64_t)blockIdx.x * blockDim.x + threadIdx.x; r < n; r += (uint64_t)gridDim.x * blockDim.x) {
     if (len[r] != k) continue;
@@ -1751,11 +1760,19 @@ __global__ void k_isolated_range(const uint64_t *__restrict__ packed, const uint
     const K xh = kmin(x, revcomp(x, (int)k));
     const uint32_t pf = key_prefix(xh, 2 * (int)k);
     if (pf < lo || pf >= hi) continue;
+    const K key = KeyOps<K>::sub(xh, range_base);
     const uint32_t i = atomicAdd(slot, 1u);
-    rkeys[i] = xh;
+    rkeys[i] = key;
     rvals[i] = REC_NONE;
-    ds.count_global(hist, xh);
+    ds.count_global(hist, key);
   }
+}
+
+// A range's node keys from their offsets.
+template <class K>
+__global__ void k_add_base(const K *__restrict__ in, uint64_t n, K range_base, K *__restrict__ out) {
+  for (uint64_t i = (uint64_t)blockIdx.x * blockDim.x + threadIdx.x; i < n; i += (uint64_t)gridDim.x * blockDim.x)
+    out[i] = KeyOps<K>::add(in[i], range_base);
 }
 
 // Copies a chunk of ASCII reads and packs it into the packed array at base
