@@ -443,29 +443,33 @@ struct Groups {
   LowBits lb;
   DevBuf tables, goff;                  // MSD: bucket tables; the groups' places
   DevBuf bound;                         // the local pass's tile bounds, once known
+  DevBuf split;                         // bits by which each group was split since (or none was)
   const uint32_t *ng_dev = nullptr;     // the groups' number (two passes), or
   uint32_t ng = 0;                      // their number (one pass)
-  uint32_t ng_max = 0;                  // at most that many
+  uint32_t ng_max = 0;                  // at most that many (0: no MSD pass)
 };
 
-// The local pass's tile bounds from the places of the groups, which are
-// copied to `cursor` (if given).
+// The local pass's tile bounds from the places of the groups (but those that
+// are split), which are copied to `cursor` (if given).
+inline const uint64_t *group_places(const Groups &gr) {
+  return gr.ng ? gr.tables.as<uint64_t>() : gr.goff.as<uint64_t>();
+}
 template <class K>
 dbg_status msd_bounds(dbg_ctx *ctx, Groups &gr, uint64_t n, uint32_t *cursor, int stage) {
   constexpr uint64_t T = SegShape<K>::TILE;
   const uint64_t tiles = (n + T - 1) / T;
   DBG_TRY(alloc_tmp(ctx, gr.bound, (tiles + 1) * 8));
-  const uint64_t *places = gr.ng ? gr.tables.as<uint64_t>() : gr.goff.as<uint64_t>();
+  const uint64_t *places = group_places(gr);
   DBG_LAUNCH(ctx, stage, 0.0,
              k_msd_bounds<<<std::min(grid_for(gr.ng_max, 256), 152u * 8), 256, 0, ctx->stream>>>(
-                 places, gr.ng_dev, gr.ng, n, T, tiles, gr.bound.as<uint64_t>(), cursor));
+                 places, gr.ng_dev, gr.ng, n, T, tiles, gr.bound.as<uint64_t>(), cursor, gr.split.as<uint8_t>()));
   return DBG_OK;
 }
 
 // One partition pass (k_msd_part) in its shape for digits of up to max_bits.
 template <class K, bool HAS_VAL, bool WIDE>
 dbg_status launch_msd_part(dbg_ctx *ctx, const K *kin, K *kout, const uint32_t *vin, uint32_t *vout, uint64_t n, int shift,
-                     int bits, uint32_t W, const MsdTables &tb, bool two, uint32_t *cursor, int max_bits,
+                     int bits, const MsdTables &tb, bool two, uint32_t *cursor, int max_bits,
                      uint64_t tiles) {
   using Sh = MsdShape<K, HAS_VAL, WIDE>;
   using S = MsdSmem<K, HAS_VAL, Sh::BLOCK, Sh::ITEMS>;
@@ -482,7 +486,7 @@ dbg_status launch_msd_part(dbg_ctx *ctx, const K *kin, K *kout, const uint32_t *
   set_smem_attrs(kern, most);
   const uint64_t slots = (uint64_t)Sh::MINB * (uint64_t)std::max(1, ctx->num_sms);
   kern<<<(unsigned)std::min(tiles, slots), Sh::BLOCK, smem, ctx->stream>>>(
-      kin, kout, vin, vout, n, shift, bits, W, tb, two ? 1 : 0, cursor, 1u << max_bits, ctx->spin_limit, ctx->d_err);
+      kin, kout, vin, vout, n, shift, bits, tb, two ? 1 : 0, cursor, 1u << max_bits, ctx->spin_limit, ctx->d_err);
   return DBG_OK;
 }
 
@@ -508,15 +512,17 @@ dbg_status msd_sort(dbg_ctx *ctx, K **keys, K **alt_keys, uint32_t **vals, uint3
   const int max_w2 = std::min({HAS_VAL ? 11 : MSD_MAX_BITS, p.shift1(), p.need - p.w1 + 2});
   // every bucket has at most max(1, 2 n_b / mean) groups
   gr.ng_max = two ? (uint32_t)(2 * (n / p.mean) + W) : W;
-  // [start: W + 1] u64, [cursor: W][gfirst: W + 1][tfirst: W + 1] u32, [tmap] u16, [w2][low] u8
-  const size_t bytes = (size_t)(W + 1) * 8 + (size_t)(3 * W + 2) * 4 + (two ? tiles2 * 2 : 0) + 2 * (size_t)W + 16;
+  // [start: W + 1] u64, [cursor: W][gfirst: W + 1][tfirst: W + 1] u32, [tmap] u32, [w2][low] u8
+  const size_t bytes = (size_t)(W + 1) * 8 + (size_t)(3 * W + 2) * 4 + (two ? tiles2 * 4 : 0) + 2 * (size_t)W + 16;
   DBG_TRY(alloc_tmp(ctx, gr.tables, bytes));
   MsdTables tb{};
   tb.start = gr.tables.as<uint64_t>();
+  tb.end = tb.start + 1;
   uint32_t *cursor = reinterpret_cast<uint32_t *>(tb.start + W + 1);
   tb.gfirst = cursor + W;
   tb.tfirst = tb.gfirst + W + 1;
-  tb.tmap = reinterpret_cast<uint16_t *>(tb.tfirst + W + 1);
+  tb.ntiles = tb.tfirst + W;
+  tb.tmap = tb.tfirst + W + 1;
   tb.w2 = reinterpret_cast<uint8_t *>(tb.tmap + (two ? tiles2 : 0));
   tb.low = tb.w2 + W;
   DBG_LAUNCH(ctx, stage, 0.0,
@@ -530,10 +536,10 @@ dbg_status msd_sort(dbg_ctx *ctx, K **keys, K **alt_keys, uint32_t **vals, uint3
   const uint32_t *vi = HAS_VAL ? *vals : nullptr;
   uint32_t *vt = HAS_VAL ? *alt_vals : nullptr;
   DBG_LAUNCH(ctx, HAS_VAL ? ST_SORT_NODES : ST_PARTITION_EDGES, bytes_pass,
-             DBG_TRY((wide1 ? launch_msd_part<K, HAS_VAL, true>(ctx, *keys, *alt_keys, vi, vt, n, p.shift1(), p.w1, W,
+             DBG_TRY((wide1 ? launch_msd_part<K, HAS_VAL, true>(ctx, *keys, *alt_keys, vi, vt, n, p.shift1(), p.w1,
                                                                 tb, false, cursor, p.w1, tiles1)
                             : launch_msd_part<K, HAS_VAL, false>(ctx, *keys, *alt_keys, vi, vt, n, p.shift1(), p.w1,
-                                                                 W, tb, false, cursor, p.w1, tiles1))));
+                                                                 tb, false, cursor, p.w1, tiles1))));
   swap();
   if (!two) {
     gr.ng = W;
@@ -548,22 +554,101 @@ dbg_status msd_sort(dbg_ctx *ctx, K **keys, K **alt_keys, uint32_t **vals, uint3
   DBG_CUDA_TRY(cudaMemsetAsync(gcount.p, 0, NG * 4, s));
   DBG_LAUNCH(ctx, stage, (double)n * sizeof(K),
              k_msd_count<K><<<(unsigned)std::min<uint64_t>(tiles2, 4ull * std::max(1, ctx->num_sms)), MSD_BLOCK,
-                              (size_t)4 << max_w2, s>>>(*keys, W, tile2, tb, gcount.as<uint32_t>()));
+                              (size_t)4 << max_w2, s>>>(*keys, tile2, tb, gcount.as<uint32_t>()));
   DBG_TRY(scan_u32_async(ctx, gcount.as<uint32_t>(), NG, gr.goff.as<uint64_t>(), stage));
   gr.lb.low = tb.low;
   gr.lb.shift1 = p.shift1();
+  gr.lb.gfirst = tb.gfirst;
   gr.ng_dev = tb.gfirst + W;
   // the counts' memory now takes the second pass's cursors (the places stay)
   DBG_TRY(msd_bounds<K>(ctx, gr, n, gcount.as<uint32_t>(), stage));
   vi = HAS_VAL ? *vals : nullptr;
   vt = HAS_VAL ? *alt_vals : nullptr;
   DBG_LAUNCH(ctx, stage, bytes_pass,
-             DBG_TRY((wide2 ? launch_msd_part<K, HAS_VAL, true>(ctx, *keys, *alt_keys, vi, vt, n, 0, 0, W, tb, true,
+             DBG_TRY((wide2 ? launch_msd_part<K, HAS_VAL, true>(ctx, *keys, *alt_keys, vi, vt, n, 0, 0, tb, true,
                                                                 gcount.as<uint32_t>(), max_w2, tiles2)
-                            : launch_msd_part<K, HAS_VAL, false>(ctx, *keys, *alt_keys, vi, vt, n, 0, 0, W, tb, true,
+                            : launch_msd_part<K, HAS_VAL, false>(ctx, *keys, *alt_keys, vi, vt, n, 0, 0, tb, true,
                                                                  gcount.as<uint32_t>(), max_w2, tiles2))));
   swap();
   DBG_CUDA_TRY(cudaGetLastError());
+  return DBG_OK;
+}
+
+// Whether the keys in oversize tiles (counters c) are worth a split of the long
+// groups.  Gathering them costs some 30 launches and ten passes over them; a
+// split, 13 launches and the local pass over all keys once more.  So few keys
+// are worth it where launches count, and one in 24 beyond (builds at 31 bases,
+// all gathered against split: 0.64 M instances at 33 % GC 0.69 ms and 0.47, at
+// 20 % 0.78 and 0.48; 27.6 M at 33 %, where one key in 40 is in such tiles,
+// 2.03 and 2.17, at 20 %, one in 3, 4.08 and 2.28; 276 M 15.9 and 16.7, and
+// 37.7 and 17.3).
+inline bool worth_split(const uint32_t *c, uint64_t n) {
+  return c[CT_MIXED] > n / (n <= 1u << 22 ? 256 : 24) && c[CT_MIXED] >= c[CT_GATHERED] / 4;
+}
+
+// Splits the groups that are too long for the local pass, in place: they are
+// partitioned by their next bits into alt_keys / alt_vals and copied back.
+// On return, if *done, gr describes the parts; otherwise (no MSD passes, few
+// keys in oversize tiles, or most of those copies of one key) nothing has
+// changed.  Waits for the stream; the tiles' counts are in the counters.
+template <class K, bool HAS_VAL>
+dbg_status msd_split(dbg_ctx *ctx, K *keys, K *alt_keys, uint32_t *vals, uint32_t *alt_vals, uint64_t n, Groups &gr,
+                     int stage, bool *done) {
+  using Sh = MsdShape<K, HAS_VAL, false>;
+  cudaStream_t s = ctx->stream;
+  *done = false;
+  if (gr.ng_max == 0 || gr.split.p) return DBG_OK;
+  constexpr uint32_t longest = SegShape<K>::TILE / 2, mean = SegShape<K>::TILE / 16;
+  const uint64_t L = n / longest + 1, tiles = n / Sh::TILE + L;
+  if (tiles > 0x7fffffffull) return DBG_OK;
+  DevBuf tables, split;
+  DBG_TRY(alloc_tmp(ctx, split, gr.ng_max));
+  DBG_TRY(alloc_tmp(ctx, tables, L * (8 + 8 + 4 + 4 + 1 + 1) + tiles * 4));
+  MsdTables tb{};
+  tb.start = tables.as<uint64_t>();
+  tb.end = tb.start + L;
+  tb.gfirst = reinterpret_cast<uint32_t *>(tb.end + L);
+  tb.tfirst = tb.gfirst + L;
+  tb.tmap = tb.tfirst + L;
+  tb.w2 = reinterpret_cast<uint8_t *>(tb.tmap + tiles);
+  tb.low = tb.w2 + L;
+  uint32_t *made = ctx->d_counters + CT_SPLIT;
+  tb.ntiles = made + 2;
+  DBG_CUDA_TRY(cudaMemsetAsync(split.p, 0, gr.ng_max, s));
+  DBG_CUDA_TRY(cudaMemsetAsync(made, 0, 4 * sizeof(uint32_t), s));
+  DBG_LAUNCH(ctx, stage, 0.0,
+             k_msd_split<K><<<std::min(grid_for(gr.ng_max, 256), 152u * 8), 256, 0, s>>>(
+                 keys, group_places(gr), gr.ng_dev, gr.ng, gr.lb, longest, mean, Sh::TILE, tb, split.as<uint8_t>(),
+                 made));
+  DBG_CUDA_TRY(cudaGetLastError());
+  uint32_t c[CT_LAST + 1];
+  DBG_TRY(read_counters(ctx, c));
+  const uint32_t listed = c[CT_SPLIT], parts = c[CT_SPLIT + 1], ntiles = c[CT_SPLIT + 2], moved = c[CT_SPLIT + 3];
+  if (!worth_split(c, n) || moved < c[CT_GATHERED] / 4) return DBG_OK;
+  DevBuf pcount, poff;
+  DBG_TRY(alloc_tmp(ctx, pcount, (uint64_t)parts * 4));
+  DBG_TRY(alloc_tmp(ctx, poff, ((uint64_t)parts + 1) * 8));
+  DBG_CUDA_TRY(cudaMemsetAsync(pcount.p, 0, (uint64_t)parts * 4, s));
+  DBG_LAUNCH(ctx, stage, (double)moved * sizeof(K),
+             k_msd_count<K><<<(unsigned)std::min<uint64_t>(ntiles, 4ull * std::max(1, ctx->num_sms)), MSD_BLOCK,
+                              (size_t)4 << MSD_SPLIT_BITS, s>>>(keys, Sh::TILE, tb, pcount.as<uint32_t>()));
+  DBG_TRY(scan_u32_async(ctx, pcount.as<uint32_t>(), parts, poff.as<uint64_t>(), stage));
+  gr.split = std::move(split);
+  DBG_TRY(msd_bounds<K>(ctx, gr, n, nullptr, stage));
+  DBG_LAUNCH(ctx, stage, 0.0,
+             k_split_bounds<<<std::min(listed, 152u * 8), 256, 0, s>>>(tb, listed, poff.as<uint64_t>(),
+                                                                       SegShape<K>::TILE, gr.bound.as<uint64_t>(),
+                                                                       pcount.as<uint32_t>()));
+  const double bytes = 2.0 * (double)moved * (double)(sizeof(K) + (HAS_VAL ? 4 : 0));
+  DBG_LAUNCH(ctx, stage, bytes,
+             DBG_TRY((launch_msd_part<K, HAS_VAL, false>(ctx, keys, alt_keys, vals, alt_vals, n, 0, 0, tb, true,
+                                                         pcount.as<uint32_t>(), MSD_SPLIT_BITS, ntiles))));
+  DBG_LAUNCH(ctx, stage, bytes,
+             (k_split_back<K, HAS_VAL><<<std::min(ntiles, 152u * 8), 512, 0, s>>>(tb, Sh::TILE, alt_keys, keys,
+                                                                                 alt_vals, vals)));
+  DBG_CUDA_TRY(cudaGetLastError());
+  gr.lb.split = gr.split.as<uint8_t>();
+  *done = true;
   return DBG_OK;
 }
 
@@ -595,7 +680,7 @@ dbg_status seg_tiles(dbg_ctx *ctx, const K *kin, uint64_t n, Groups &gr, TileSet
   ts.tiles = tiles;
   DBG_TRY(alloc_tmp(ctx, ts.osize, tiles * 4));
   DBG_TRY(alloc_tmp(ctx, ts.olist, tiles * 4));
-  if (gr.ng) DBG_TRY(msd_bounds<K>(ctx, gr, n, nullptr, stage));
+  if (gr.ng && !gr.bound.p) DBG_TRY(msd_bounds<K>(ctx, gr, n, nullptr, stage));
   if (gr.bound.p) {
     ts.bound = std::move(gr.bound);
   } else {
@@ -604,12 +689,13 @@ dbg_status seg_tiles(dbg_ctx *ctx, const K *kin, uint64_t n, Groups &gr, TileSet
                k_seg_bounds<K><<<grid_for(tiles + 1, 256), 256, 0, s>>>(kin, n, gr.lb.fixed, Sh::TILE, tiles,
                                                                        ts.bound.as<uint64_t>()));
   }
-  DBG_CUDA_TRY(cudaMemsetAsync(ctx->d_counters + CT_GATHERED, 0, (CT_ENDS - CT_GATHERED + 1) * 4, s));
+  DBG_CUDA_TRY(cudaMemsetAsync(ctx->d_counters + CT_GATHERED, 0, (CT_MIXED - CT_GATHERED + 1) * 4, s));
   DBG_LAUNCH(ctx, stage, 0.0,
-             k_seg_oversize<<<grid_for(tiles, 256), 256, 0, s>>>(ts.bound.as<uint64_t>(), tiles,
+             k_seg_oversize<K><<<grid_for(tiles, 256), 256, 0, s>>>(kin, ts.bound.as<uint64_t>(), tiles,
                                                                  (uint32_t)(SEG_BLOCK * Sh::ITEMS),
                                                                  ts.osize.as<uint32_t>(), ts.olist.as<uint32_t>(),
                                                                  ctx->d_counters + CT_GATHERED,
+                                                                 ctx->d_counters + CT_MIXED,
                                                                  ctx->d_counters + CT_OVERSIZE, ctx->d_err));
   DBG_CUDA_TRY(cudaGetLastError());
   return DBG_OK;
@@ -758,6 +844,7 @@ dbg_status seg_sort_records(dbg_ctx *ctx, const K *kin, const uint32_t *vin, K *
 struct EdgeTiles {
   uint64_t tiles = 0;
   DevBuf bound, tcount, toff, mult;
+  bool uneven = false;  // the sort split long groups
   void release() {
     for (DevBuf *b : {&bound, &tcount, &toff, &mult}) b->release();
   }
@@ -776,6 +863,15 @@ dbg_status seg_rle(dbg_ctx *ctx, K *kin, K *kstage, uint64_t n, Groups &gr, int 
   uint64_t H = 0;
   DBG_TRY(seg_tiles<K>(ctx, kin, n, gr, ts, ST_LOCAL_SORT_EDGES));
   const uint64_t tiles = ts.tiles;
+  uint32_t c[CT_LAST + 1];
+  // the tiles again once long groups have been split
+  auto split = [&](bool *done) -> dbg_status {
+    *done = false;
+    if (!worth_split(c, n)) return DBG_OK;
+    DBG_TRY((msd_split<K, false>(ctx, kin, kstage, nullptr, nullptr, n, gr, ST_SORT_EDGES, done)));
+    if (*done) DBG_TRY(seg_tiles<K>(ctx, kin, n, gr, ts, ST_LOCAL_SORT_EDGES));
+    return DBG_OK;
+  };
   DBG_TRY(alloc_tmp(ctx, mstage, n * 4));
   DBG_TRY(alloc_tmp(ctx, tcount, tiles * 4));
   DBG_TRY(alloc_tmp(ctx, toff, (tiles + 1) * 8));
@@ -805,7 +901,6 @@ dbg_status seg_rle(dbg_ctx *ctx, K *kin, K *kstage, uint64_t n, Groups &gr, int 
     DBG_TRY(alloc_tmp(ctx, gheads, ((uint64_t)ts.gathered + 1) * 4));
     return run_length_reduce<K>(ctx, ts.gk.as<K>(), ts.gathered, guniq.as<K>(), gheads.as<uint32_t>(), &H);
   };
-  uint32_t c[CT_LAST + 1];
   bool final = false;  // the scan below covers every tile
   if (ctx->count_first) {
     // count-first; the tiles that overflow their table, or would, are listed
@@ -820,41 +915,52 @@ dbg_status seg_rle(dbg_ctx *ctx, K *kin, K *kstage, uint64_t n, Groups &gr, int 
                                                : sizeof(SegCountSmem<K, RANK_BALLOT>);
     set_smem_attrs(count, csmem);
     DBG_TRY(alloc_tmp(ctx, over, tiles * 4));
-    DBG_LAUNCH(ctx, ST_LOCAL_SORT_EDGES, (double)n * sizeof(K),
-               count<<<(unsigned)tiles, SEG_BLOCK, csmem, s>>>(
-                   kin, ts.bound.as<uint64_t>(), ts.osize.as<uint32_t>(), kstage, mstage.as<uint32_t>(),
-                   tcount.as<uint32_t>(), over.as<uint32_t>(), ctx->d_counters + CT_LISTED, gr.lb, ctx->seg_rank,
-                   ctx->d_counters + CT_LONG));
-    DBG_CUDA_TRY(cudaGetLastError());
-    uint32_t *listed = ctx->d_counters + CT_LISTED;
-    if (ctx->seg_rank) {
-      DBG_TRY(alloc_tmp(ctx, crowded, tiles * 4));
-      set_smem_attrs(k_rank_rle<K>, sizeof(RankRleSmem<K>));
-      DBG_LAUNCH(ctx, ST_LOCAL_SORT_EDGES, 0.0,
-                 k_rank_rle<K><<<(unsigned)std::min<uint64_t>(tiles, 2ull * (uint64_t)std::max(1, ctx->num_sms)),
-                                 RANK_BLOCK, sizeof(RankRleSmem<K>), s>>>(
-                     kin, ts.bound.as<uint64_t>(), kstage, mstage.as<uint32_t>(), tcount.as<uint32_t>(), gr.lb,
-                     over.as<uint32_t>(), listed, crowded.as<uint32_t>(), ctx->d_counters + CT_CROWDED));
+    for (bool again = true; again;) {
+      DBG_LAUNCH(ctx, ST_LOCAL_SORT_EDGES, (double)n * sizeof(K),
+                 count<<<(unsigned)tiles, SEG_BLOCK, csmem, s>>>(
+                     kin, ts.bound.as<uint64_t>(), ts.osize.as<uint32_t>(), kstage, mstage.as<uint32_t>(),
+                     tcount.as<uint32_t>(), over.as<uint32_t>(), ctx->d_counters + CT_LISTED, gr.lb, ctx->seg_rank,
+                     ctx->d_counters + CT_LONG));
       DBG_CUDA_TRY(cudaGetLastError());
-    } else {
-      DBG_TRY(sort_tiles(tiles, over.as<uint32_t>(), listed, 0.0));
-    }
-    DBG_TRY(scan_u32_async(ctx, tcount.as<uint32_t>(), tiles, toff.as<uint64_t>(), ST_LOCAL_SORT_EDGES, CT_TOTAL));
-    DBG_TRY(read_counters(ctx, c));
-    ts.gathered = c[CT_GATHERED];
-    ts.oversize = c[CT_OVERSIZE];
-    ctx->count_overflow_tiles += c[CT_LISTED];
-    ctx->rank_fallback_tiles += c[CT_LONG] + c[CT_CROWDED];
-    final = ts.oversize == 0 && c[CT_CROWDED] == 0;
-    if (!final) {
-      const uint32_t n_crowded = c[CT_CROWDED];
-      DBG_TRY(gather());
-      DBG_TRY(sort_tiles(n_crowded, crowded.as<uint32_t>(), nullptr, 0.0));
-      DBG_TRY(sort_tiles(ts.oversize, ts.olist.as<uint32_t>(), nullptr, 0.0));
+      uint32_t *listed = ctx->d_counters + CT_LISTED;
+      if (ctx->seg_rank) {
+        DBG_TRY(alloc_tmp(ctx, crowded, tiles * 4));
+        set_smem_attrs(k_rank_rle<K>, sizeof(RankRleSmem<K>));
+        DBG_LAUNCH(ctx, ST_LOCAL_SORT_EDGES, 0.0,
+                   k_rank_rle<K><<<(unsigned)std::min<uint64_t>(tiles, 2ull * (uint64_t)std::max(1, ctx->num_sms)),
+                                   RANK_BLOCK, sizeof(RankRleSmem<K>), s>>>(
+                       kin, ts.bound.as<uint64_t>(), kstage, mstage.as<uint32_t>(), tcount.as<uint32_t>(), gr.lb,
+                       over.as<uint32_t>(), listed, crowded.as<uint32_t>(), ctx->d_counters + CT_CROWDED));
+        DBG_CUDA_TRY(cudaGetLastError());
+      } else {
+        DBG_TRY(sort_tiles(tiles, over.as<uint32_t>(), listed, 0.0));
+      }
+      DBG_TRY(scan_u32_async(ctx, tcount.as<uint32_t>(), tiles, toff.as<uint64_t>(), ST_LOCAL_SORT_EDGES, CT_TOTAL));
+      DBG_TRY(read_counters(ctx, c));
+      ts.gathered = c[CT_GATHERED];
+      ts.oversize = c[CT_OVERSIZE];
+      const uint32_t met[3] = {c[CT_LISTED], c[CT_LONG], c[CT_CROWDED]};
+      DBG_TRY(split(&again));
+      if (again) continue;
+      ctx->count_overflow_tiles += met[0];
+      ctx->rank_fallback_tiles += met[1] + met[2];
+      final = ts.oversize == 0 && c[CT_CROWDED] == 0;
+      if (!final) {
+        const uint32_t n_crowded = c[CT_CROWDED];
+        DBG_TRY(gather());
+        DBG_TRY(sort_tiles(n_crowded, crowded.as<uint32_t>(), nullptr, 0.0));
+        DBG_TRY(sort_tiles(ts.oversize, ts.olist.as<uint32_t>(), nullptr, 0.0));
+      }
     }
   } else {
     DBG_TRY(read_counters(ctx, c));
     ts.gathered = c[CT_GATHERED];
+    bool again = false;
+    DBG_TRY(split(&again));
+    if (again) {
+      DBG_TRY(read_counters(ctx, c));
+      ts.gathered = c[CT_GATHERED];
+    }
     DBG_TRY(gather());
     DBG_TRY(sort_tiles(tiles, nullptr, nullptr, (double)n * sizeof(K)));
   }
@@ -871,6 +977,7 @@ dbg_status seg_rle(dbg_ctx *ctx, K *kin, K *kstage, uint64_t n, Groups &gr, int 
     staged->tcount = std::move(tcount);
     staged->toff = std::move(toff);
     staged->mult = std::move(mstage);
+    staged->uneven = gr.split.p != nullptr;
     return DBG_OK;
   }
   DBG_TRY(alloc_buf(ctx, *mult_out, std::max<uint64_t>(1, total) * 4));
@@ -931,6 +1038,14 @@ dbg_status sort_records(dbg_ctx *ctx, K **rk, K **rk_alt, uint32_t **rv, uint32_
   uint32_t c[CT_LAST + 1];
   DBG_TRY(read_counters(ctx, c));
   ts.gathered = c[CT_GATHERED];
+  bool again = false;
+  if (worth_split(c, R))
+    DBG_TRY((msd_split<K, true>(ctx, *rk, *rk_alt, *rv, *rv_alt, R, gr, ST_SORT_NODES, &again)));
+  if (again) {
+    DBG_TRY(seg_tiles<K>(ctx, *rk, R, gr, ts, ST_LOCAL_SORT_NODES));
+    DBG_TRY(read_counters(ctx, c));
+    ts.gathered = c[CT_GATHERED];
+  }
   ts.oversize = c[CT_OVERSIZE];
   DBG_TRY((seg_gather<K, true>(ctx, *rk, *rv, vo, p.bits, ts, ST_LOCAL_SORT_NODES)));
   DBG_TRY(seg_sort_records<K>(ctx, *rk, *rv, *rk_alt, *rv_alt, R, gr, vo, ts));
@@ -1052,9 +1167,9 @@ dbg_status assign_node_ids(dbg_ctx *ctx, const K *rk, const uint32_t *rv, uint64
 // |V| and the number of edge ends; *done = false, with the oversize tiles
 // gathered, where the unfused passes are to do it.
 template <class K>
-dbg_status rank_and_assign(dbg_ctx *ctx, const K *rk, const uint32_t *rv, K *ukeys, uint32_t *vals, uint64_t R,
+dbg_status rank_and_assign(dbg_ctx *ctx, K *rk, uint32_t *rv, K *ukeys, uint32_t *vals, uint64_t R,
                            uint64_t E, uint64_t I, int key_bits, Groups &gr, ValOrder vo, TileSet &ts, dbg_graph *g,
-                           bool sides, bool *done, uint64_t *V, uint64_t *ends) {
+                           bool sides, bool uneven, bool *done, uint64_t *V, uint64_t *ends) {
   cudaStream_t s = ctx->stream;
   const uint64_t tiles = ts.tiles;
   DevBuf heads, tcount, hoff, ecount, eoff, fb;
@@ -1081,14 +1196,26 @@ dbg_status rank_and_assign(dbg_ctx *ctx, const K *rk, const uint32_t *rv, K *uke
   static_assert(SegRankSmem<K>::CAP == SEG_BLOCK * SegShape<K>::ITEMS, "same tile capacity as the digit-pass kernel");
   auto rank = k_seg_rank<K, true>;
   set_smem_attrs(rank, sizeof(SegRankSmem<K>));
-  DBG_LAUNCH(ctx, ST_LOCAL_SORT_NODES, 2.0 * (double)R * (sizeof(K) + 4),
-             rank<<<(unsigned)tiles, RANK_BLOCK, sizeof(SegRankSmem<K>), s>>>(
-                 rk, rv, ts.bound.as<uint64_t>(), ts.osize.as<uint32_t>(), nullptr, nullptr, nullptr, ukeys, vals,
-                 gr.lb, vo, fb.as<uint32_t>(), nlisted, heads.as<uint32_t>(), tcount.as<uint32_t>()));
-  DBG_CUDA_TRY(cudaGetLastError());
-  DBG_TRY(scan_tiles());
-  ts.gathered = c[CT_GATHERED];
-  ts.oversize = c[CT_OVERSIZE];
+  auto split = [&](bool *did) -> dbg_status {
+    DBG_TRY((msd_split<K, true>(ctx, rk, ukeys, rv, vals, R, gr, ST_SORT_NODES, did)));
+    return *did ? seg_tiles<K>(ctx, rk, R, gr, ts, ST_LOCAL_SORT_NODES) : DBG_OK;
+  };
+  // (where the edge keys had long groups, the records have: split before the
+  // first try)
+  bool again = false;
+  if (uneven) DBG_TRY(split(&again));
+  for (again = true; again;) {
+    DBG_LAUNCH(ctx, ST_LOCAL_SORT_NODES, 2.0 * (double)R * (sizeof(K) + 4),
+               rank<<<(unsigned)tiles, RANK_BLOCK, sizeof(SegRankSmem<K>), s>>>(
+                   rk, rv, ts.bound.as<uint64_t>(), ts.osize.as<uint32_t>(), nullptr, nullptr, nullptr, ukeys, vals,
+                   gr.lb, vo, fb.as<uint32_t>(), nlisted, heads.as<uint32_t>(), tcount.as<uint32_t>()));
+    DBG_CUDA_TRY(cudaGetLastError());
+    DBG_TRY(scan_tiles());
+    ts.gathered = c[CT_GATHERED];
+    ts.oversize = c[CT_OVERSIZE];
+    again = false;
+    if (!uneven && worth_split(c, R)) DBG_TRY(split(&again));
+  }
   // many records in oversize tiles, which one CTA each would go through (a
   // million records: about 0.3 ms): the unfused passes
   *done = ts.gathered <= 1u << 20;
@@ -1506,7 +1633,8 @@ dbg_status build_graph_impl(dbg_ctx *ctx, const BuildInput &in, dbg_graph *g) {
     ValOrder fvo = vo;
     uint64_t ends = 0;
     DBG_TRY(sort_records_global<K>(ctx, &rk, &rk_alt, &rv, &rv_alt, R, rplan, fvo, d_hist, d_digit_base, gr, ts));
-    DBG_TRY(rank_and_assign<K>(ctx, rk, rv, rk_alt, rv_alt, R, E, I, nbits, gr, fvo, ts, g, sides, &fused, &V, &ends));
+    DBG_TRY(rank_and_assign<K>(ctx, rk, rv, rk_alt, rv_alt, R, E, I, nbits, gr, fvo, ts, g, sides,
+                               edge_tiles.uneven, &fused, &V, &ends));
     if (!fused) {
       DBG_TRY(seg_sort_records<K>(ctx, rk, rv, rk_alt, rv_alt, R, gr, fvo, ts));
       std::swap(rk, rk_alt);

@@ -262,8 +262,9 @@ dbg_status read_small(dbg_ctx *ctx, const void *d_src, size_t bytes, void *h_dst
 
 // d_counters entries that hold a call's counts until one read_counters brings
 // them all, with the error word: gathered keys and oversize tiles of a local
-// pass, the tiles it listed (and those with long buckets), totals.
-enum Counter { CT_GATHERED = 20, CT_OVERSIZE, CT_LISTED, CT_LONG, CT_CROWDED, CT_TOTAL, CT_ENDS, CT_REMOVED = 28, CT_LAST = 47 };  // (CT_REMOVED: 64 bits)
+// pass, the tiles it listed (and those with long buckets), totals, the gathered
+// keys of tiles that are not one key's copies, the groups that are split.
+enum Counter { CT_GATHERED = 20, CT_OVERSIZE, CT_LISTED, CT_LONG, CT_CROWDED, CT_TOTAL, CT_ENDS, CT_MIXED, CT_REMOVED = 28, CT_SPLIT = 32, CT_LAST = 47 };  // (CT_REMOVED: 64 bits; CT_SPLIT: four)
 // Waits for the stream; counters[0 .. CT_LAST]; a status from the device error
 // word, as check_device_error.
 dbg_status read_counters(dbg_ctx *ctx, uint32_t *counters);

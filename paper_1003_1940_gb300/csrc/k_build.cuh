@@ -85,6 +85,37 @@ struct DigitSpec {
   }
 };
 
+// Where a key's group ends: the number of its bits below the group's shared
+// high bits.  Before any split it is one number for all keys (low == nullptr:
+// fixed), or one by bucket, the key's bits from shift1 up (k_msd.cuh).  split:
+// by how many bits each group has been split since, the groups numbered by key
+// (a bucket's from gfirst[bucket] up).
+struct LowBits {
+  int fixed = 0;
+  const uint8_t *low = nullptr;
+  int shift1 = 0;
+  const uint32_t *gfirst = nullptr;
+  const uint8_t *split = nullptr;
+  template <class K>
+  __device__ __forceinline__ int of(const K &key) const {
+    const uint32_t b = low ? (uint32_t)KeyOps<K>::words_lo(KeyOps<K>::shr(key, shift1)) : 0u;
+    const int bits = low ? low[b] : fixed;
+    if (!split) return bits;
+    const uint32_t above = (uint32_t)KeyOps<K>::words_lo(KeyOps<K>::shr(key, bits));
+    return bits - split[low ? gfirst[b] + (above & ((1u << (shift1 - bits)) - 1u)) : above];
+  }
+};
+
+// Whether most of the c keys from s up are probably one key's copies (seven
+// samples).
+template <class K>
+__device__ __forceinline__ bool copies_of_one(const K *__restrict__ keys, uint64_t s, uint64_t c) {
+  const K mid = keys[s + c / 2];
+  int same = 0;
+  for (int j = 1; j < 8; j++) same += KeyOps<K>::eq(keys[s + c * j / 8], mid) ? 1 : 0;
+  return same >= 5;
+}
+
 // ---------------------------------------------------------------------------
 // read offsets: base_off[r] = sum of L before r, edge_off[r] = sum of
 // max(0, L - k) before r, plus the number of reads of length exactly k.

@@ -16,13 +16,20 @@
 //
 //   plan    W = 2^w1 buckets by the top w1 bits, counted by the producer of
 //           the keys.  A bucket of m keys gets w2 = ceil(log2(m / mean)) more
-//           bits, so that groups hold about `mean` keys whatever the
-//           distribution (canonical keys are twice as dense at the low end as
-//           on average).  One pass is enough when W groups are.
+//           bits (at most two more than the average bucket), so that groups
+//           hold about `mean` keys where the keys lie evenly within buckets
+//           (canonical keys are twice as dense at the low end as on average).
+//           One pass is enough when W groups are.
 //   pass 1  k_msd_part over the keys as they come.
 //   count   k_msd_count: the sizes of each bucket's 2^w2 groups; their scan
 //           gives every group's place.
 //   pass 2  k_msd_part again, tile by tile of each bucket.
+//   split   only when the local pass met many keys in groups too long for it
+//           (an uneven base composition: at 20 % GC a group of AT-rich
+//           prefixes holds ten times the mean): k_msd_split lists those
+//           groups, and they alone are counted and partitioned once more by
+//           as many bits as each takes.  Groups of copies of one key are left
+//           out: no digit divides them.
 #pragma once
 
 #include "k_build.cuh"
@@ -46,14 +53,17 @@ template <class K, bool HAS_VAL, bool WIDE> struct MsdShape {
   static constexpr uint32_t TILE = BLOCK * ITEMS;
 };
 
-// The buckets of pass 1 and, for two passes, their groups and tiles.
+// The buckets of pass 1 and, for two passes, their groups and tiles; or the
+// groups that are split, in no order, as the buckets of that pass.
 struct MsdTables {
   uint64_t *start;         // [W + 1] first key of each bucket
+  uint64_t *end;           // [W] its end (start + 1, unless groups are split)
   uint32_t *gfirst;        // [W + 1] first group of each bucket
   uint32_t *tfirst;        // [W + 1] first tile of each bucket
+  uint32_t *ntiles;        // the tiles' number
   uint8_t *w2;             // [W] bits of the bucket's second digit
   uint8_t *low;            // [W] bits below the bucket's groups
-  uint16_t *tmap;          // [tiles] bucket of each tile
+  uint32_t *tmap;          // [tiles] bucket of each tile
 };
 
 // One block.  Bucket starts from the producer's histogram; with two passes
@@ -112,7 +122,7 @@ static __global__ __launch_bounds__(1024) void k_msd_plan(const unsigned long lo
       tb.tfirst[b] = t;
       g += 1u << tb.w2[b];
       const uint32_t nt = (uint32_t)((c + tile - 1) / tile);
-      for (uint32_t q = 0; q < nt; q++) tb.tmap[t + q] = (uint16_t)b;
+      for (uint32_t q = 0; q < nt; q++) tb.tmap[t + q] = b;
       t += nt;
     }
     if (b == W - 1) {
@@ -132,12 +142,12 @@ static __global__ __launch_bounds__(1024) void k_msd_plan(const unsigned long lo
 constexpr int MSD_BLOCK = 512;
 
 template <class K>
-__global__ __launch_bounds__(MSD_BLOCK) void k_msd_count(const K *__restrict__ keys, uint32_t W, uint32_t TILE,
-                                                         MsdTables tb, uint32_t *__restrict__ gcount) {
+__global__ __launch_bounds__(MSD_BLOCK) void k_msd_count(const K *__restrict__ keys, uint32_t TILE, MsdTables tb,
+                                                         uint32_t *__restrict__ gcount) {
   constexpr int ITEMS = 8;
   extern __shared__ uint32_t s_h[];
   const int tid = threadIdx.x;
-  const uint32_t NT = tb.tfirst[W];
+  const uint32_t NT = *tb.ntiles;
   const uint32_t per = (NT + gridDim.x - 1) / gridDim.x;
   const uint32_t t0 = min(NT, blockIdx.x * per), t1 = min(NT, t0 + per);
   uint32_t cur = 0xffffffffu, ways = 0;
@@ -159,7 +169,7 @@ __global__ __launch_bounds__(MSD_BLOCK) void k_msd_count(const K *__restrict__ k
       __syncthreads();
     }
     const uint64_t base = tb.start[b] + (uint64_t)(t - tb.tfirst[b]) * TILE;
-    const uint64_t end = min(base + TILE, tb.start[b + 1]);
+    const uint64_t end = min(base + TILE, tb.end[b]);
     for (uint64_t p = base + tid; p < end; p += (uint64_t)MSD_BLOCK * ITEMS) {
       K k[ITEMS];
 #pragma unroll
@@ -202,7 +212,7 @@ template <class K, bool HAS_VAL, int BLOCK, int ITEMS, int MINB>
 __global__ __launch_bounds__(BLOCK, MINB) void k_msd_part(const K *__restrict__ kin, K *__restrict__ kout,
                                                           const uint32_t *__restrict__ vin,
                                                           uint32_t *__restrict__ vout, uint64_t n, int shift,
-                                                          int bits, uint32_t W, MsdTables tb, int two,
+                                                          int bits, MsdTables tb, int two,
                                                           uint32_t *__restrict__ cursor, uint32_t max_ways,
                                                           uint32_t spin_limit, uint32_t *__restrict__ err) {
   using S = MsdSmem<K, HAS_VAL, BLOCK, ITEMS>;
@@ -216,13 +226,13 @@ __global__ __launch_bounds__(BLOCK, MINB) void k_msd_part(const K *__restrict__ 
   __shared__ uint32_t s_w[WARPS];
   __shared__ uint64_t s_bar[2];
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
-  const uint32_t NT = two ? tb.tfirst[W] : (uint32_t)((n + TILE - 1) / TILE);
+  const uint32_t NT = two ? *tb.ntiles : (uint32_t)((n + TILE - 1) / TILE);
   const bool bulk = ((reinterpret_cast<uintptr_t>(kin) | (HAS_VAL ? reinterpret_cast<uintptr_t>(vin) : 0)) & 15) == 0;
   auto base_of = [&](uint32_t t, uint32_t b) {
     return two ? tb.start[b] + (uint64_t)(t - tb.tfirst[b]) * TILE : (uint64_t)t * TILE;
   };
   auto count_of = [&](uint64_t base, uint32_t b) {
-    return (uint32_t)min((uint64_t)TILE, (two ? tb.start[b + 1] : n) - base);
+    return (uint32_t)min((uint64_t)TILE, (two ? tb.end[b] : n) - base);
   };
   // (one thread) tile t into buffer q
   auto issue = [&](uint32_t t, int q) {
@@ -353,17 +363,91 @@ __global__ __launch_bounds__(BLOCK, MINB) void k_msd_part(const K *__restrict__ 
 
 // bound[t] = the first key of the group that holds key t * tile_keys, from
 // the groups' places (goff[g] .. goff[g + 1]); bound[tiles] = n.  cursor[g],
-// if given, = goff[g].
+// if given, = goff[g].  Groups that split (their bits, or 0) says to be split
+// are left to k_split_bounds.
+__device__ __forceinline__ void tile_bounds(uint64_t s, uint64_t e, uint64_t tile_keys, uint64_t *bound) {
+  for (uint64_t t = (s + tile_keys - 1) / tile_keys; t * tile_keys < e; t++) bound[t] = s;  // (empty: no tile)
+}
+
 static __global__ void k_msd_bounds(const uint64_t *__restrict__ goff, const uint32_t *__restrict__ groups_of,
                                     uint32_t groups, uint64_t n, uint64_t tile_keys, uint64_t tiles,
-                                    uint64_t *__restrict__ bound, uint32_t *__restrict__ cursor) {
+                                    uint64_t *__restrict__ bound, uint32_t *__restrict__ cursor,
+                                    const uint8_t *__restrict__ split) {
   const uint32_t NG = groups_of ? *groups_of : groups;
   for (uint32_t g = blockIdx.x * blockDim.x + threadIdx.x; g < NG; g += gridDim.x * blockDim.x) {
-    const uint64_t s = goff[g], e = goff[g + 1];  // (empty: no tile)
+    const uint64_t s = goff[g], e = goff[g + 1];
     if (cursor) cursor[g] = (uint32_t)s;
-    for (uint64_t t = (s + tile_keys - 1) / tile_keys; t * tile_keys < e; t++) bound[t] = s;
+    if (!split || !split[g]) tile_bounds(s, e, tile_keys, bound);
   }
   if (blockIdx.x == 0 && threadIdx.x == 0) bound[tiles] = n;
+}
+
+// ---------------------------------------------------------------------------
+// Splitting long groups.  made[0 .. 3]: groups listed, their parts, their
+// tiles, their keys.
+// ---------------------------------------------------------------------------
+constexpr int MSD_SPLIT_BITS = 11;
+
+// Lists the groups of more than `longest` keys as buckets of tb, each with as
+// many bits as bring its parts to `mean` keys; groups of copies of one key are
+// left out.
+template <class K>
+__global__ void k_msd_split(const K *__restrict__ keys, const uint64_t *__restrict__ goff,
+                            const uint32_t *__restrict__ groups_of, uint32_t groups, LowBits lb, uint32_t longest,
+                            uint32_t mean, uint32_t tile, MsdTables tb, uint8_t *__restrict__ split,
+                            uint32_t *__restrict__ made) {
+  const uint32_t NG = groups_of ? *groups_of : groups;
+  for (uint32_t g = blockIdx.x * blockDim.x + threadIdx.x; g < NG; g += gridDim.x * blockDim.x) {
+    const uint64_t s = goff[g], e = goff[g + 1], c = e - s;
+    if (c <= longest) continue;
+    const int low = lb.of(keys[s]);
+    if (low == 0 || copies_of_one(keys, s, c)) continue;
+    int w = 0;
+    while (w < min(MSD_SPLIT_BITS, low) && ((uint64_t)mean << w) < c) w++;
+    const uint32_t nt = (uint32_t)((c + tile - 1) / tile);
+    const uint32_t b = atomicAdd(made, 1u), part = atomicAdd(made + 1, 1u << w), t = atomicAdd(made + 2, nt);
+    atomicAdd(made + 3, (uint32_t)c);
+    split[g] = (uint8_t)w;
+    tb.start[b] = s;
+    tb.end[b] = e;
+    tb.gfirst[b] = part;
+    tb.tfirst[b] = t;
+    tb.w2[b] = (uint8_t)w;
+    tb.low[b] = (uint8_t)(low - w);
+    for (uint32_t q = 0; q < nt; q++) tb.tmap[t + q] = b;
+  }
+}
+
+// From the scan of the parts' sizes (poff): where each part lies, as the
+// partition's cursors, and the tiles' bounds.
+static __global__ void k_split_bounds(MsdTables tb, uint32_t listed, const uint64_t *__restrict__ poff,
+                                      uint64_t tile_keys, uint64_t *__restrict__ bound,
+                                      uint32_t *__restrict__ cursor) {
+  for (uint32_t b = blockIdx.x; b < listed; b += gridDim.x) {
+    const uint32_t p0 = tb.gfirst[b], parts = 1u << tb.w2[b];
+    const uint64_t at = tb.start[b] - poff[p0];  // (modulo 2^64)
+    for (uint32_t j = p0 + threadIdx.x; j < p0 + parts; j += blockDim.x) {
+      const uint64_t s = at + poff[j], e = at + poff[j + 1];
+      cursor[j] = (uint32_t)s;
+      tile_bounds(s, e, tile_keys, bound);
+    }
+  }
+}
+
+// The listed groups' keys (and payloads) back from the partition's output.
+template <class K, bool HAS_VAL>
+__global__ void k_split_back(MsdTables tb, uint32_t tile, const K *__restrict__ kin, K *__restrict__ kout,
+                             const uint32_t *__restrict__ vin, uint32_t *__restrict__ vout) {
+  const uint32_t NT = *tb.ntiles;
+  for (uint32_t t = blockIdx.x; t < NT; t += gridDim.x) {
+    const uint32_t b = tb.tmap[t];
+    const uint64_t base = tb.start[b] + (uint64_t)(t - tb.tfirst[b]) * tile;
+    const uint32_t c = (uint32_t)min((uint64_t)tile, tb.end[b] - base);
+    for (uint32_t j = threadIdx.x; j < c; j += blockDim.x) {
+      kout[base + j] = kin[base + j];
+      if (HAS_VAL) vout[base + j] = vin[base + j];
+    }
+  }
 }
 
 }  // namespace dbg

@@ -44,19 +44,6 @@ struct SegSortSmem {
   uint32_t tile, passes, excl, total, span_bits;
 };
 
-// Where a key's group ends: the number of its bits below the group's shared
-// high bits, one for all keys (low == nullptr: fixed) or by bucket, the
-// key's bits from shift1 up (k_msd.cuh).
-struct LowBits {
-  int fixed = 0;
-  const uint8_t *low = nullptr;
-  int shift1 = 0;
-  template <class K>
-  __device__ __forceinline__ int of(const K &key) const {
-    return low ? low[(uint32_t)KeyOps<K>::words_lo(KeyOps<K>::shr(key, shift1))] : fixed;
-  }
-};
-
 // The order of records with equal keys: ascending payload << shift (the
 // shift drops the side bits that a node record's payload carries on top).
 // sort: they come in no particular order and payload digits take part in the
@@ -100,14 +87,16 @@ __global__ void k_seg_bounds(const K *__restrict__ keys, uint64_t n, int low_bit
 }
 
 // osize[t] = the tile's length if it exceeds cap (an oversize tile), else 0;
-// those tiles' numbers in olist, their keys added up in *keys.  If a wait of
+// those tiles' numbers in olist, their keys added up in *keys, and in *mixed
+// those of tiles that do not look like the copies of one key.  If a wait of
 // the global passes ran out (*err), some keys were never written: then every
 // tile is made empty, so that the local kernels, which trust the keys to lie in
 // their groups, read none, and the host finds the error in its next read-back.
-static __global__ void k_seg_oversize(uint64_t *__restrict__ bound, uint64_t tiles, uint32_t cap,
-                                      uint32_t *__restrict__ osize, uint32_t *__restrict__ olist,
-                                      uint32_t *__restrict__ keys, uint32_t *__restrict__ count,
-                                      const uint32_t *__restrict__ err) {
+template <class K>
+__global__ void k_seg_oversize(const K *__restrict__ kin, uint64_t *__restrict__ bound, uint64_t tiles, uint32_t cap,
+                               uint32_t *__restrict__ osize, uint32_t *__restrict__ olist,
+                               uint32_t *__restrict__ keys, uint32_t *__restrict__ mixed,
+                               uint32_t *__restrict__ count, const uint32_t *__restrict__ err) {
   if (*err & (ERR_TIMEOUT | ERR_INTERNAL)) {
     for (uint64_t t = (uint64_t)blockIdx.x * blockDim.x + threadIdx.x; t < tiles; t += (uint64_t)gridDim.x * blockDim.x) {
       bound[t] = 0;
@@ -117,10 +106,11 @@ static __global__ void k_seg_oversize(uint64_t *__restrict__ bound, uint64_t til
     return;
   }
   for (uint64_t t = (uint64_t)blockIdx.x * blockDim.x + threadIdx.x; t < tiles; t += (uint64_t)gridDim.x * blockDim.x) {
-    const uint64_t sz = bound[t + 1] - bound[t];
+    const uint64_t s = bound[t], sz = bound[t + 1] - s;
     osize[t] = sz > cap ? (uint32_t)sz : 0u;
     if (sz > cap) {
       atomicAdd(keys, (uint32_t)sz);
+      if (!copies_of_one(kin, s, sz)) atomicAdd(mixed, (uint32_t)sz);
       olist[atomicAdd(count, 1u)] = (uint32_t)t;
     }
   }
