@@ -266,6 +266,14 @@ __global__ void k_succ_lone(uint32_t *__restrict__ mk, const uint32_t *__restric
   add_per_block(lists, count);
 }
 
+// The successors from walk words that no walker has changed.
+__global__ void k_words_succ(const uint32_t *__restrict__ mk, uint64_t n, uint32_t *__restrict__ succ) {
+  for (uint64_t x = (uint64_t)blockIdx.x * blockDim.x + threadIdx.x; x < n; x += (uint64_t)gridDim.x * blockDim.x) {
+    const uint32_t w = mk[x];
+    succ[x] = WalkWord<uint32_t>::tail(w) ? NONE32 : WalkWord<uint32_t>::next(w);
+  }
+}
+
 // The predecessor of a strand-node, from the mirror symmetry of the
 // transform: an arc y -> x exists exactly when x^1 -> y^1 does.
 __device__ __forceinline__ uint32_t pred_of(const uint32_t *__restrict__ succ, uint64_t x) {
@@ -368,11 +376,14 @@ __global__ void k_walk_segments(const uint32_t *__restrict__ succ, uint64_t n, u
 }
 
 // word[x] = (list head, rank) from (segment start, offset) and the start's
-// own word, which is final (a start's word resolves to itself).
+// own word, which is final (a start's word resolves to itself).  On a cycle
+// there is no list head: words there end nowhere (k_on_lists tells).
 __global__ void k_resolve_segments(uint64_t n, uint64_t *word) {
   for (uint64_t x = (uint64_t)blockIdx.x * blockDim.x + threadIdx.x; x < n; x += (uint64_t)gridDim.x * blockDim.x) {
-    const uint64_t w = word[x], ws = word[pk_a(w)];
-    if (pk_a(ws) != pk_a(w)) word[x] = pk(pk_a(ws), pk_d(ws) + pk_d(w));
+    const uint64_t w = word[x];
+    if (w == UNSET64) continue;
+    const uint64_t ws = word[pk_a(w)];
+    if (pk_a(ws) != pk_a(w)) word[x] = pk(pk_a(ws), (uint32_t)min((uint64_t)pk_d(ws) + pk_d(w), (uint64_t)0x7fffffffu));
   }
 }
 
@@ -444,6 +455,98 @@ __global__ void k_cycle_break(const uint32_t *__restrict__ cyc_list, uint32_t C,
     const uint32_t m = pk_d(lab[x]);
     cyc[x] = (m & 1u) ? 2 : 1;
     word[x] = m == x ? pk(x, 0) : pk(pred_of(succ, x), 1);
+  }
+}
+
+// ---------------------------------------------------------------------------
+// The cycles of a graph whose other nodes are done (a bitmap over the nodes):
+// they are numbered among themselves, in node order, so that what follows --
+// min labels, opening, ranking -- costs what they hold and not what the graph
+// does.  A strand-node y of theirs is 2 (its node's number) + strand.  20 M nodes
+// in 1.5 M chains and one circle of 5000: 1.94 ms, without the circle 1.56; with
+// the whole graph ranked again for it 8.8.  5 M nodes in one chain and that
+// circle: 1.91, 1.48 and 4.4.
+// ---------------------------------------------------------------------------
+__device__ __forceinline__ uint32_t rest_bits(const uint32_t *__restrict__ done, uint64_t i, uint64_t V) {
+  const uint32_t b = ~done[i];
+  return V - i * 32 >= 32 ? b : b & ((1u << (V - i * 32)) - 1u);
+}
+
+__global__ void k_rest_popc(const uint32_t *__restrict__ done, uint64_t V, uint64_t nw, uint32_t *__restrict__ cnt) {
+  for (uint64_t i = (uint64_t)blockIdx.x * blockDim.x + threadIdx.x; i < nw; i += (uint64_t)gridDim.x * blockDim.x)
+    cnt[i] = __popc(rest_bits(done, i, V));
+}
+
+__global__ void k_rest_list(const uint32_t *__restrict__ done, uint64_t V, uint64_t nw,
+                            const uint64_t *__restrict__ pre, uint32_t *__restrict__ node) {
+  for (uint64_t i = (uint64_t)blockIdx.x * blockDim.x + threadIdx.x; i < nw; i += (uint64_t)gridDim.x * blockDim.x) {
+    uint64_t at = pre[i];
+    for (uint32_t b = rest_bits(done, i, V); b; b &= b - 1u) node[at++] = (uint32_t)(i * 32) + (uint32_t)(__ffs(b) - 1);
+  }
+}
+
+// the graph's arcs, from successors or from walk words
+struct SuccArcs {
+  const uint32_t *succ;
+  __device__ uint32_t next(uint32_t x) const { return succ[x]; }
+};
+template <class W>
+struct WordArcs {
+  const W *mk;
+  __device__ uint32_t next(uint32_t x) const { return WalkWord<W>::next(mk[x]); }
+};
+
+template <class A>
+__global__ void k_cycle_arcs(A arcs, const uint32_t *__restrict__ node, uint32_t C2, uint64_t V,
+                             const uint32_t *__restrict__ done, const uint64_t *__restrict__ pre,
+                             uint32_t *__restrict__ succ, uint32_t *__restrict__ list, uint32_t *err) {
+  for (uint32_t y = blockIdx.x * blockDim.x + threadIdx.x; y < C2; y += gridDim.x * blockDim.x) {
+    const uint32_t nx = arcs.next(2 * node[y >> 1] + (y & 1u)), z = nx >> 1, bit = z & 31u;
+    list[y] = y;
+    if (z >= V || (done[z >> 5] >> bit & 1u)) {  // a cycle's arcs stay on it
+      atomicOr(err, ERR_INTERNAL);
+      succ[y] = y;
+    } else {
+      succ[y] = 2 * (uint32_t)(pre[z >> 5] + __popc(~done[z >> 5] & ((1u << bit) - 1u))) + (nx & 1u);
+    }
+  }
+}
+
+__global__ void k_cycle_seed(const uint32_t *__restrict__ succ, uint32_t C2, uint64_t *__restrict__ lab) {
+  for (uint32_t y = blockIdx.x * blockDim.x + threadIdx.x; y < C2; y += gridDim.x * blockDim.x)
+    lab[y] = pk(pred_of(succ, y), y);
+}
+
+// Nodes whose strand-nodes the segments ranked (their word's start is a list
+// head): their bits in `done`, and their number.
+__global__ void k_on_lists(const uint64_t *__restrict__ word, uint64_t V, uint32_t *__restrict__ done,
+                           uint32_t *count) {
+  uint32_t local = 0;
+  for (uint64_t g = (uint64_t)blockIdx.x * blockDim.x + (threadIdx.x & ~31u); g < V;
+       g += (uint64_t)gridDim.x * blockDim.x) {
+    const uint64_t v = g + (threadIdx.x & 31u);
+    bool on = false;
+    if (v < V) {
+      const uint64_t w = word[2 * v];
+      on = w != UNSET64 && pk_root(word[pk_a(w)], pk_a(w));
+    }
+    const unsigned b = __ballot_sync(0xffffffffu, on);
+    if ((threadIdx.x & 31u) == 0) {
+      done[g / 32] = b;
+      local += __popc(b);
+    }
+  }
+  if ((threadIdx.x & 31u) == 0 && local) atomicAdd(count, local);
+}
+
+// The ranked cycles' words and marks, by the graph's strand-nodes.
+__global__ void k_cycle_back(const uint32_t *__restrict__ node, uint32_t C2, const uint64_t *__restrict__ cword,
+                             const uint8_t *__restrict__ ccyc, uint64_t *__restrict__ word,
+                             uint8_t *__restrict__ cyc) {
+  for (uint32_t y = blockIdx.x * blockDim.x + threadIdx.x; y < C2; y += gridDim.x * blockDim.x) {
+    const uint32_t x = 2 * node[y >> 1] + (y & 1u), h = pk_a(cword[y]);
+    word[x] = pk(2 * node[h >> 1] + (h & 1u), pk_d(cword[y]));
+    cyc[x] = ccyc[y];
   }
 }
 
@@ -785,10 +888,51 @@ __global__ void k_head_popc(const uint32_t *__restrict__ head_bits, uint64_t nw,
     cnt[i] = __popc(head_bits[i]);
 }
 
+// 'A', 'C', 'G', 'T' for 2-bit codes 0..3
+__device__ __forceinline__ char base_char(uint32_t b) { return (char)((0x54474341u >> (8 * (b & 3u))) & 0xffu); }
+
+// Kept cycles beside the walkers' unitigs: the opening node's bit, and in its
+// word CYCLE_WORD | the cycle's length.
+constexpr uint64_t CYCLE_WORD = 1ull << 63;
+
+__global__ void k_cycle_heads(const uint32_t *__restrict__ node, uint32_t C2, const uint32_t *__restrict__ succ,
+                              const uint64_t *__restrict__ word, const uint8_t *__restrict__ cyc,
+                              uint32_t *__restrict__ head_bits, uint64_t *__restrict__ at_head) {
+  for (uint32_t y = blockIdx.x * blockDim.x + threadIdx.x; y < C2; y += gridDim.x * blockDim.x) {
+    const uint32_t h = pk_a(word[y]);
+    if (cyc[y] != 1 || succ[y] != h) continue;  // the last of a kept cycle
+    const uint32_t v = node[h >> 1];
+    atomicOr(head_bits + (v >> 5), 1u << (v & 31u));
+    at_head[v] = CYCLE_WORD | ((uint64_t)pk_d(word[y]) + 1);
+  }
+}
+
+// Nodes and bases of the kept cycles (their tables: k_stage_copy).
+template <class K>
+__global__ void k_cycle_write(const uint32_t *__restrict__ node, uint32_t C2, const uint64_t *__restrict__ word,
+                              const uint8_t *__restrict__ cyc, const uint32_t *__restrict__ head_bits,
+                              const uint64_t *__restrict__ wpre, const uint64_t *__restrict__ uoff,
+                              const uint64_t *__restrict__ node_keys, int k, uint64_t *__restrict__ nodes_out,
+                              char *__restrict__ seq) {
+  for (uint32_t y = blockIdx.x * blockDim.x + threadIdx.x; y < C2; y += gridDim.x * blockDim.x) {
+    if (cyc[y] != 1) continue;
+    const uint32_t x = 2 * node[y >> 1] + (y & 1u), v = node[pk_a(word[y]) >> 1], r = pk_d(word[y]);
+    const uint64_t u = wpre[v >> 5] + __popc(head_bits[v >> 5] & ((1u << (v & 31u)) - 1u));
+    const uint64_t off = uoff[u], so = off + u * (uint64_t)(k - 1);
+    nodes_out[off + r] = x;
+    const K km = strand_kmer<K>(node_keys, x, k);
+    if (r > 0) {
+      seq[so + k - 1 + r] = base_char((uint32_t)KeyOps<K>::low2(km));
+    } else {
+      for (int i = 0; i < k; i++) seq[so + i] = base_char(KeyOps<K>::digit(km, 2 * (k - 1 - i), 2));
+    }
+  }
+}
+
 // The unitigs in the order of their first nodes: unitig u = the u-th set bit
 // of the head bitmap (wpre = the exclusive scan of the words' bit counts),
 // with its length and its walkers' representative << 1 | the other copy is
-// kept (from the head's word).
+// kept (from the head's word), or NONE32 for a cycle.
 __global__ void k_head_list(const uint32_t *__restrict__ head_bits, uint64_t nw, const uint64_t *__restrict__ wpre,
                             const uint64_t *__restrict__ at_head, uint32_t *__restrict__ urec,
                             uint32_t *__restrict__ ulen) {
@@ -797,8 +941,8 @@ __global__ void k_head_list(const uint32_t *__restrict__ head_bits, uint64_t nw,
     uint64_t u = wpre[i];
     while (b) {
       const uint64_t w = at_head[i * 32 + (uint32_t)(__ffs(b) - 1)];
-      urec[u] = (uint32_t)(w >> 31);
-      ulen[u] = (uint32_t)(w & 0x7fffffffu) >> 1;
+      urec[u] = w & CYCLE_WORD ? NONE32 : (uint32_t)(w >> 31);
+      ulen[u] = w & CYCLE_WORD ? (uint32_t)w : (uint32_t)(w & 0x7fffffffu) >> 1;
       u++;
       b &= b - 1u;
     }
@@ -816,9 +960,6 @@ __device__ __forceinline__ uint64_t stage_advance(const uint32_t *__restrict__ p
   }
   return q;
 }
-
-// 'A', 'C', 'G', 'T' for 2-bit codes 0..3
-__device__ __forceinline__ char base_char(uint32_t b) { return (char)((0x54474341u >> (8 * (b & 3u))) & 0xffu); }
 
 // Every kept unitig from its two staged halves.  With the kept walker's
 // head y (the unitig's first strand-node), a nodes taken by it and L in
@@ -860,6 +1001,14 @@ __global__ __launch_bounds__(WALK_BLOCK, 6) void k_stage_copy(
       if (qi >= cnt) break;
       const uint64_t u = u0 + qi;
       const uint32_t ur = urec[u], L = ulen[u];
+      if (ur == NONE32) {  // a cycle: its tables (the rest by k_cycle_write)
+        if (gl == 0) {
+          node_off[u] = uoff[u];
+          seq_off[u] = uoff[u] + u * (uint64_t)(k - 1);
+          circular[u] = 1;
+        }
+        continue;
+      }
       uint4 ra = rec[ur >> 1], rb;
       // the other walker: its record, or its head alone where it took no node
       if (ra.z & WALK_TAIL) rb = make_uint4((ra.z & ~WALK_TAIL) ^ 1u, 0u, 0u, 0u);
@@ -966,6 +1115,59 @@ static dbg_status jump_until_stable(dbg_ctx *ctx, const uint32_t *list, uint32_t
   }
   set_error("list ranking did not converge");
   return DBG_ETIMEOUT;
+}
+
+// The cycles' nodes, their arcs, ranks and marks, numbered among themselves.
+struct Cycles {
+  uint32_t C2 = 0;  // strand-nodes
+  DevBuf node, succ, word, cyc;
+};
+
+// Ranks the C nodes of V that are not in the bitmap `done`, all of them on
+// cycles.
+template <class A>
+static dbg_status rank_cycles(dbg_ctx *ctx, A arcs, const uint32_t *done, uint64_t V, uint64_t C, Cycles &cy) {
+  cudaStream_t s = ctx->stream;
+  const uint64_t nw = (V + 31) / 32;
+  const uint32_t C2 = (uint32_t)(2 * C);
+  cy.C2 = C2;
+  DevBuf cnt, pre, list, lab;
+  DBG_TRY(alloc_tmp(ctx, cnt, nw * 4));
+  DBG_TRY(alloc_tmp(ctx, pre, (nw + 1) * 8));
+  DBG_TRY(alloc_tmp(ctx, cy.node, C * 4));
+  DBG_TRY(alloc_tmp(ctx, cy.succ, (uint64_t)C2 * 4));
+  DBG_TRY(alloc_tmp(ctx, cy.word, (uint64_t)C2 * 8));
+  DBG_TRY(alloc_tmp(ctx, cy.cyc, C2));
+  DBG_TRY(alloc_tmp(ctx, list, (uint64_t)C2 * 4));
+  DBG_TRY(alloc_tmp(ctx, lab, (uint64_t)C2 * 8));
+  DBG_LAUNCH(ctx, ST_COMPACT_CYCLES, 8.0 * nw,
+             k_rest_popc<<<grid_of(nw), 256, 0, s>>>(done, V, nw, cnt.as<uint32_t>()));
+  DBG_TRY(scan_excl_async(ctx, cnt.as<uint32_t>(), nw, pre.as<uint64_t>(), CT_TOTAL));
+  DBG_LAUNCH(ctx, ST_COMPACT_CYCLES, 12.0 * nw + 4.0 * C,
+             k_rest_list<<<grid_of(nw), 256, 0, s>>>(done, V, nw, pre.as<uint64_t>(), cy.node.as<uint32_t>()));
+  DBG_LAUNCH(ctx, ST_COMPACT_CYCLES, 20.0 * C2,
+             k_cycle_arcs<A><<<grid_of(C2), 256, 0, s>>>(arcs, cy.node.as<uint32_t>(), C2, V, done,
+                                                         pre.as<uint64_t>(), cy.succ.as<uint32_t>(),
+                                                         list.as<uint32_t>(), ctx->d_err));
+  DBG_LAUNCH(ctx, ST_COMPACT_CYCLES, 12.0 * C2,
+             k_cycle_seed<<<grid_of(C2), 256, 0, s>>>(cy.succ.as<uint32_t>(), C2, lab.as<uint64_t>()));
+  int R = 2;
+  while ((1ull << (R - 2)) < C2) R++;
+  for (int r = 0; r < R; r++)
+    DBG_LAUNCH(ctx, ST_COMPACT_CYCLES, 20.0 * C2,
+               k_cycle_min<<<grid_of(C2), 256, 0, s>>>(list.as<uint32_t>(), C2, lab.as<uint64_t>()));
+  DBG_LAUNCH(ctx, ST_COMPACT_CYCLES, 25.0 * C2,
+             k_cycle_break<<<grid_of(C2), 256, 0, s>>>(list.as<uint32_t>(), C2, lab.as<uint64_t>(),
+                                                       cy.succ.as<uint32_t>(), cy.cyc.as<uint8_t>(),
+                                                       cy.word.as<uint64_t>()));
+  DBG_CUDA_TRY(cudaGetLastError());
+  uint32_t still = 0;
+  DBG_TRY(jump_until_stable(ctx, list.as<uint32_t>(), C2, cy.word.as<uint64_t>(), &still));
+  if (still != 0) {
+    set_error("%u strand-nodes stayed on cycles after they were opened", still);
+    return DBG_EINTERNAL;
+  }
+  return DBG_OK;
 }
 
 // The general path's ending, from the ranking words (word[x] = (list head,
@@ -1110,7 +1312,8 @@ static dbg_status compact_impl(dbg_ctx *ctx, const dbg_graph *g, dbg_unitigs *u,
       link_node.release();
       link_edge.release();
     }
-    // ---- fast path: short acyclic lists only ----
+    // ---- fast path: short lists, and cycles ----
+    bool words_kept = false;  // the walks left every word as it was
     if (fast) {
       // the heads of the unitigs as a bitmap over the nodes; their words at
       // the head nodes only
@@ -1170,7 +1373,27 @@ static dbg_status compact_impl(dbg_ctx *ctx, const dbg_graph *g, dbg_unitigs *u,
       DBG_TRY(scan_excl_async(ctx, wcnt.as<uint32_t>(), nw, wpre.as<uint64_t>(), CT_TOTAL));
       uint32_t c[CT_LAST + 1];
       DBG_TRY(read_counters(ctx, c));
-      if (c[11] == 0 && c[16] == 0 && ((uint64_t)c[13] << 32 | c[12]) == V) {
+      words_kept = c[17] == 0;
+      if (c[11] == 0 && c[16] == 0) {
+        // nodes that no walker claimed lie on cycles: these are ranked alone,
+        // and their first nodes join the heads
+        Cycles cy;
+        const uint64_t covered = (uint64_t)c[13] << 32 | c[12];
+        if (covered < V) {
+          if (w32)
+            DBG_TRY(rank_cycles(ctx, WordArcs<uint32_t>{mk.as<uint32_t>()}, claimed.as<uint32_t>(), V, V - covered, cy));
+          else
+            DBG_TRY(rank_cycles(ctx, WordArcs<uint64_t>{mk.as<uint64_t>()}, claimed.as<uint32_t>(), V, V - covered, cy));
+          DBG_LAUNCH(ctx, ST_COMPACT_CYCLES, 13.0 * cy.C2,
+                     k_cycle_heads<<<grid_of(cy.C2), 256, 0, s>>>(cy.node.as<uint32_t>(), cy.C2,
+                                                                  cy.succ.as<uint32_t>(), cy.word.as<uint64_t>(),
+                                                                  cy.cyc.as<uint8_t>(), f_bits.as<uint32_t>(),
+                                                                  f_word.as<uint64_t>()));
+          DBG_LAUNCH(ctx, ST_COMPACT_OUTPUT, 8.0 * nw,
+                     k_head_popc<<<grid_of(nw), 256, 0, s>>>(f_bits.as<uint32_t>(), nw, wcnt.as<uint32_t>()));
+          DBG_TRY(scan_excl_async(ctx, wcnt.as<uint32_t>(), nw, wpre.as<uint64_t>(), CT_TOTAL));
+          DBG_TRY(read_counters(ctx, c));
+        }
         mk.release();
         const uint32_t U32 = c[CT_TOTAL];
         const uint64_t Uf = U32;
@@ -1197,6 +1420,12 @@ static dbg_status compact_impl(dbg_ctx *ctx, const dbg_graph *g, dbg_unitigs *u,
                        stage.as<uint32_t>(), page_next.as<uint32_t>(), g->node_keys.as<uint64_t>(), V, Uf, k,
                        u->nodes.as<uint64_t>(), u->seq.as<char>(), u->node_off.as<uint64_t>(),
                        u->seq_off.as<uint64_t>(), u->circular.as<uint8_t>()));
+        if (cy.C2)
+          DBG_LAUNCH(ctx, ST_COMPACT_OUTPUT, (double)cy.C2 / 2 * (8 + 1 + 8 * g->key_words),
+                     k_cycle_write<K><<<grid_of(cy.C2), 256, 0, s>>>(
+                         cy.node.as<uint32_t>(), cy.C2, cy.word.as<uint64_t>(), cy.cyc.as<uint8_t>(),
+                         f_bits.as<uint32_t>(), wpre.as<uint64_t>(), uoff.as<uint64_t>(), g->node_keys.as<uint64_t>(),
+                         k, u->nodes.as<uint64_t>(), u->seq.as<char>()));
         DBG_CUDA_TRY(cudaGetLastError());
         DBG_TRY(read_counters(ctx, c));
         if (c[CT_TOTAL] != V) {
@@ -1206,10 +1435,14 @@ static dbg_status compact_impl(dbg_ctx *ctx, const dbg_graph *g, dbg_unitigs *u,
         return DBG_OK;
       }
     }
-    // ---- general path: long lists or cycles present ----
-    if (w32) {  // (walkers left their numbers in some words: the arcs again)
+    // ---- general path: long lists ----
+    if (w32) {
       DBG_TRY(alloc_tmp(ctx, succ, n1 * 4));
-      DBG_TRY(links_by_bitmap(succ.as<uint32_t>()));
+      if (words_kept)
+        DBG_LAUNCH(ctx, ST_COMPACT_LINKS, 8.0 * n,
+                   k_words_succ<<<grid_of(n), 256, 0, s>>>(mk.as<uint32_t>(), n, succ.as<uint32_t>()));
+      else  // (walkers left their numbers in some words: the arcs again)
+        DBG_TRY(links_by_bitmap(succ.as<uint32_t>()));
     }
     mk.release();
     tails.release();
@@ -1217,21 +1450,46 @@ static dbg_status compact_impl(dbg_ctx *ctx, const dbg_graph *g, dbg_unitigs *u,
     DBG_TRY(alloc_tmp(ctx, active, n1 * 4));
     bool ranked = false;
     if (ctx->compact_mode != 2) {
-      // by segments, unless there are cycles
-      DBG_CUDA_TRY(cudaMemsetAsync(ctx->d_counters + 10, 0, 4 * sizeof(uint32_t), s));
-      DBG_LAUNCH(ctx, ST_COMPACT_RANK, 12.0 * n,
-                 k_walk_segments<<<walk_grid(ctx, n, k_walk_segments, 1024), 256, 0, s>>>(
-                     succ.as<uint32_t>(), n, word.as<uint64_t>(), active.as<uint32_t>(), ctx->d_counters + 10,
-                     reinterpret_cast<unsigned long long *>(ctx->d_counters + 12)));
-      DBG_CUDA_TRY(cudaGetLastError());
+      // by segments; what they do not reach or cannot lead to a head lies on
+      // cycles.  Words that no walk wrote are told apart in a second go, if
+      // the first one's count says that there are some.
       uint32_t got[4] = {0, 0, 0, 0}, left = 0;  // active; total
-      DBG_TRY(read_small(ctx, ctx->d_counters + 10, sizeof(got), got));
-      if (((uint64_t)got[3] << 32 | got[2]) == n) {
-        if (got[0] > 0) DBG_TRY(jump_until_stable(ctx, active.as<uint32_t>(), got[0], word.as<uint64_t>(), &left));
-        ranked = left == 0;
+      auto written = [&]() { return (uint64_t)got[3] << 32 | got[2]; };
+      for (int go = 0; go < 2 && written() < n; go++) {
+        if (go > 0) DBG_CUDA_TRY(cudaMemsetAsync(word.p, 0xff, n * 8, s));
+        DBG_CUDA_TRY(cudaMemsetAsync(ctx->d_counters + 10, 0, 4 * sizeof(uint32_t), s));
+        DBG_LAUNCH(ctx, ST_COMPACT_RANK, 12.0 * n,
+                   k_walk_segments<<<walk_grid(ctx, n, k_walk_segments, 1024), 256, 0, s>>>(
+                       succ.as<uint32_t>(), n, word.as<uint64_t>(), active.as<uint32_t>(), ctx->d_counters + 10,
+                       reinterpret_cast<unsigned long long *>(ctx->d_counters + 12)));
+        DBG_CUDA_TRY(cudaGetLastError());
+        DBG_TRY(read_small(ctx, ctx->d_counters + 10, sizeof(got), got));
       }
-      if (ranked)
-        DBG_LAUNCH(ctx, ST_COMPACT_RANK, 24.0 * n, k_resolve_segments<<<grid_of(n), 256, 0, s>>>(n, word.as<uint64_t>()));
+      if (got[0] > 0) DBG_TRY(jump_until_stable(ctx, active.as<uint32_t>(), got[0], word.as<uint64_t>(), &left));
+      DBG_LAUNCH(ctx, ST_COMPACT_RANK, 24.0 * n, k_resolve_segments<<<grid_of(n), 256, 0, s>>>(n, word.as<uint64_t>()));
+      if (left > 0 || written() < n) {
+        have_cycles = true;
+        DevBuf done;
+        Cycles cy;
+        DBG_TRY(alloc_tmp(ctx, done, (V + 31) / 32 * 4));
+        DBG_CUDA_TRY(cudaMemsetAsync(ctx->d_counters + 10, 0, sizeof(uint32_t), s));
+        DBG_LAUNCH(ctx, ST_COMPACT_CYCLES, 16.0 * V,
+                   k_on_lists<<<grid_of(V), 256, 0, s>>>(word.as<uint64_t>(), V, done.as<uint32_t>(),
+                                                         ctx->d_counters + 10));
+        DBG_CUDA_TRY(cudaGetLastError());
+        uint32_t on = 0;
+        DBG_TRY(read_small(ctx, ctx->d_counters + 10, sizeof(on), &on));
+        active.release();
+        DBG_TRY(rank_cycles(ctx, SuccArcs{succ.as<uint32_t>()}, done.as<uint32_t>(), V, V - on, cy));
+        DBG_TRY(alloc_tmp(ctx, cyc, n1));
+        DBG_CUDA_TRY(cudaMemsetAsync(cyc.p, 0, n, s));
+        DBG_LAUNCH(ctx, ST_COMPACT_CYCLES, 30.0 * cy.C2,
+                   k_cycle_back<<<grid_of(cy.C2), 256, 0, s>>>(cy.node.as<uint32_t>(), cy.C2, cy.word.as<uint64_t>(),
+                                                               cy.cyc.as<uint8_t>(), word.as<uint64_t>(),
+                                                               cyc.as<uint8_t>()));
+        DBG_CUDA_TRY(cudaGetLastError());
+      }
+      ranked = true;
     }
     if (!ranked) {
       DBG_CUDA_TRY(cudaMemsetAsync(word.p, 0xff, n * 8, s));
