@@ -211,12 +211,12 @@ void dbg_graph_free(dbg_graph *g);
 dbg_status dbg_compact(dbg_ctx *ctx, const dbg_graph *g, dbg_unitigs **out);
 
 /* How dbg_compact ranks the lists.  0 (the default): the meeting walks
- * with staged halves when every list is short and acyclic, with 32-bit walk
- * words up to 2^29 - 1 strand-nodes and 64-bit words up to 2^30; few long
- * lists by segments (pointer jumping over about one strand-node in 16); and
- * pointer jumping over all of them with cycle breaking when there are cycles.
+ * with staged halves when every list is short, with 32-bit walk words up to
+ * 2^29 - 1 strand-nodes and 64-bit words up to 2^30; few long lists by
+ * segments (pointer jumping over about one strand-node in 16); the nodes on
+ * cycles, if there are any, apart from the lists by pointer jumping.
  * 1: the same with 64-bit walk words at any size they allow; 2: pointer
- * jumping only.  The unitigs are the same either way.  DBG_EINVAL for another
+ * jumping over all strand-nodes.  The unitigs are the same either way.  DBG_EINVAL for another
  * mode. */
 dbg_status dbg_compact_mode_set(dbg_ctx *ctx, int mode);
 
