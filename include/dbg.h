@@ -88,7 +88,11 @@ typedef struct dbg_options {
 /* Fills *opt with defaults. */
 void dbg_options_init(dbg_options *opt);
 
-/* Creates a context on the device named by opt (NULL = defaults). */
+/* Creates a context on the device named by opt (NULL = defaults).  Between
+ * calls a context keeps one block of 32 MB of device memory for the small
+ * buffers of its calls, from its first build until it is destroyed or an
+ * allocation of it fails: then the block goes back, the call that failed is
+ * made once more without it, and the context holds none from there on. */
 dbg_status dbg_create(dbg_ctx **ctx, const dbg_options *opt);
 void dbg_destroy(dbg_ctx *ctx);
 
@@ -340,7 +344,9 @@ void dbg_server_options_init(dbg_server_options *opt);
  *     a quarter of what it asks, or whatever is free when it runs alone);
  *   - a build that still runs out of device memory (taken outside the
  *     budget) is queued again until another request finishes; alone, it
- *     fails with DBG_ENOMEM.
+ *     fails with DBG_ENOMEM;
+ *   - a worker's block of small buffers is part of its request's footprint,
+ *     and an idle worker holds none.
  * Results are the same graphs dbg_build returns for the same read set. */
 dbg_status dbg_server_create(dbg_server **srv, const dbg_server_options *opt);
 /* Waits for running requests; frees results nobody polled. */
@@ -381,7 +387,10 @@ dbg_status dbg_build_batch(dbg_ctx *ctx, const dbg_readset *sets, uint32_t nsets
  * reduced, so the concatenated results are the sorted edge list.  Nodes are
  * handled the same way over node-key ranges.  The result is bit-identical
  * to dbg_build's.  Packed reads, per-read offsets and the final graph must
- * fit on the device.  mem_budget = 0 uses half the free device memory.
+ * fit on the device.  mem_budget = 0 uses half the free device memory.  The
+ * budget sizes the ranges; tables of a few words per thousand keys and the
+ * context's block, here at most a sixteenth of the budget (and 256 KB at
+ * least), come on top.
  * -------------------------------------------------------------------- */
 dbg_status dbg_build_bucketed(dbg_ctx *ctx, const char *reads, const uint32_t *lengths, uint64_t n, uint32_t k,
                               uint64_t mem_budget, dbg_graph **out);

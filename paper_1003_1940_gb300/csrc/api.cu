@@ -48,7 +48,7 @@ dbg_status alloc_buf(dbg_ctx *ctx, DevBuf &b, size_t bytes) {
   b.al = &ctx->al;
   b.ar = nullptr;
   b.p = ctx->al.get(bytes);
-  if (!b.p && ctx->scratch.drop(ctx->al)) b.p = ctx->al.get(bytes);
+  if (!b.p && ctx->scratch.shortage()) b.p = ctx->al.get(bytes);
   if (!b.p) {
     set_error("device allocation of %zu bytes failed", bytes);
     return DBG_ENOMEM;
@@ -59,12 +59,14 @@ dbg_status alloc_buf(dbg_ctx *ctx, DevBuf &b, size_t bytes) {
 
 void *Scratch::get(Allocator &al, size_t bytes) {
   bytes = (std::max<size_t>(bytes, 1) + 255) & ~(size_t)255;
-  if (bytes > MOST || short_of_memory) return nullptr;
+  if (off || bytes > limit / SHARE) return nullptr;
   if (!base) {
-    base = static_cast<char *>(al.get(CAP));
-    short_of_memory = !base;
+    base = static_cast<char *>(al.get(limit));
+    off = !base;
     if (!base) return nullptr;
-    pieces.assign(1, Piece{0, CAP, false});
+    from = &al;
+    size = limit;
+    pieces.assign(1, Piece{0, size, false});
   }
   for (size_t i = 0; i < pieces.size(); i++) {
     if (pieces[i].used || pieces[i].bytes < bytes) continue;
@@ -78,9 +80,9 @@ void *Scratch::get(Allocator &al, size_t bytes) {
 }
 
 void Scratch::put(void *p) {
-  const size_t off = static_cast<size_t>(static_cast<char *>(p) - base);
+  const size_t off_p = static_cast<size_t>(static_cast<char *>(p) - base);
   size_t i = 0;
-  while (i < pieces.size() && pieces[i].off != off) i++;
+  while (i < pieces.size() && pieces[i].off != off_p) i++;
   if (i == pieces.size()) return;
   pieces[i].used = false;
   if (i + 1 < pieces.size() && !pieces[i + 1].used) {
@@ -91,14 +93,21 @@ void Scratch::put(void *p) {
     pieces[i - 1].bytes += pieces[i].bytes;
     pieces.erase(pieces.begin() + i);
   }
+  if (off) give_back();
 }
 
-bool Scratch::drop(Allocator &al) {
-  short_of_memory = true;
+bool Scratch::give_back() {
   if (!base || pieces.size() != 1 || pieces[0].used) return false;
-  al.put(base, CAP);
+  from->put(base, size);
   base = nullptr;
+  size = 0;
   return true;
+}
+
+bool Scratch::shortage() {
+  off = true;
+  missed = missed || base;
+  return give_back();
 }
 
 dbg_status alloc_tmp(dbg_ctx *ctx, DevBuf &b, size_t bytes) {
@@ -404,7 +413,7 @@ void dbg_destroy(dbg_ctx *ctx) {
   prof_resolve(ctx);
   for (cudaEvent_t e : ctx->ev_pool) cudaEventDestroy(e);
   if (ctx->d_status) cudaFreeAsync(ctx->d_status, ctx->stream);
-  if (ctx->scratch.base) ctx->al.put(ctx->scratch.base, Scratch::CAP);
+  ctx->scratch.give_back();
   if (ctx->stream) cudaStreamSynchronize(ctx->stream);
   if (ctx->d_err) cudaFree(ctx->d_err);
   if (ctx->h_pinned) cudaFreeHost(ctx->h_pinned);
@@ -416,6 +425,11 @@ void dbg_destroy(dbg_ctx *ctx) {
   if (ctx->own_stream && ctx->stream) cudaStreamDestroy(ctx->stream);
   delete ctx;
 }
+
+static dbg_status build_once(dbg_ctx *ctx, const char *reads, const uint32_t *lengths, uint64_t n, uint32_t k,
+                             dbg_graph **out);
+static dbg_status build_bucketed_once(dbg_ctx *ctx, const char *reads, const uint32_t *lengths, uint64_t n,
+                                      uint32_t k, uint64_t mem_budget, dbg_graph **out);
 
 dbg_status dbg_build(dbg_ctx *ctx, const char *reads, const uint32_t *lengths, uint64_t n, uint32_t k,
                      dbg_graph **out) {
@@ -441,6 +455,11 @@ dbg_status dbg_build(dbg_ctx *ctx, const char *reads, const uint32_t *lengths, u
     return DBG_EOVERFLOW;
   }
   DeviceScope scope(ctx->device);
+  return with_scratch(ctx, [&] { return build_once(ctx, reads, lengths, n, k, out); });
+}
+
+static dbg_status build_once(dbg_ctx *ctx, const char *reads, const uint32_t *lengths, uint64_t n, uint32_t k,
+                             dbg_graph **out) {
   cudaStream_t s = ctx->stream;
   dbg_graph *g = new (std::nothrow) dbg_graph();
   if (!g) return DBG_ENOMEM;
@@ -513,12 +532,18 @@ dbg_status dbg_build_bucketed(dbg_ctx *ctx, const char *reads, const uint32_t *l
     return DBG_EOVERFLOW;
   }
   DeviceScope scope(ctx->device);
-  cudaStream_t s = ctx->stream;
   if (mem_budget == 0) {
     size_t free_b = 0, total_b = 0;
     DBG_CUDA_TRY(cudaMemGetInfo(&free_b, &total_b));
     mem_budget = free_b / 2;
   }
+  ScratchLimit block(ctx, mem_budget);
+  return with_scratch(ctx, [&] { return build_bucketed_once(ctx, reads, lengths, n, k, mem_budget, out); });
+}
+
+static dbg_status build_bucketed_once(dbg_ctx *ctx, const char *reads, const uint32_t *lengths, uint64_t n,
+                                      uint32_t k, uint64_t mem_budget, dbg_graph **out) {
+  cudaStream_t s = ctx->stream;
   dbg_graph *g = new (std::nothrow) dbg_graph();
   if (!g) return DBG_ENOMEM;
   g->al = ctx->al;
@@ -856,7 +881,7 @@ dbg_status dbg_roadmap_nodes(dbg_ctx *ctx, const dbg_graph *g, uint32_t min_read
       d_ids = tmp.as<uint32_t>();
     }
   }
-  dbg_status st = roadmap_nodes(ctx, g, min_reads, d_ids, count);
+  dbg_status st = with_scratch(ctx, [&] { return roadmap_nodes(ctx, g, min_reads, d_ids, count); });
   if (st == DBG_OK && ids && d_ids != ids && *count)
     st = copy_plain(ctx->device, ids, d_ids, *count * sizeof(uint32_t));
   cudaStreamSynchronize(ctx->stream);

@@ -1803,6 +1803,28 @@ dbg_status compact_chains(dbg_ctx *ctx, const dbg_graph *g, dbg_unitigs *u, bool
   return g->key_words == 1 ? compact_impl<uint64_t>(ctx, g, u, literal) : compact_impl<Key128>(ctx, g, u, literal);
 }
 
+// *out = the unitigs that `fill` makes.
+template <class F>
+static dbg_status unitigs_of_call(dbg_ctx *ctx, dbg_unitigs **out, F fill) {
+  dbg_unitigs *u = new (std::nothrow) dbg_unitigs();
+  if (!u) return DBG_ENOMEM;
+  u->al = ctx->al;
+  u->device = ctx->device;
+  u->n_copy = ctx->copy_streams;
+  const dbg_status st = fill(u);
+  for (DevBuf *b : {&u->node_off, &u->nodes, &u->seq_off, &u->seq, &u->circular}) b->al = &u->al;
+  cudaStreamSynchronize(ctx->stream);
+  prof_resolve(ctx);
+  if (st != DBG_OK) {
+    cudaGetLastError();
+    cudaMemsetAsync(ctx->d_err, 0, sizeof(uint32_t), ctx->stream);
+    delete u;
+  } else {
+    *out = u;
+  }
+  return st;
+}
+
 }  // namespace dbg
 
 using namespace dbg;
@@ -1823,22 +1845,9 @@ dbg_status dbg_compact(dbg_ctx *ctx, const dbg_graph *g, dbg_unitigs **out) {
   int prev = -1;
   cudaGetDevice(&prev);
   if (prev != ctx->device) cudaSetDevice(ctx->device);
-  dbg_unitigs *u = new (std::nothrow) dbg_unitigs();
-  if (!u) return DBG_ENOMEM;
-  u->al = ctx->al;
-  u->device = ctx->device;
-  u->n_copy = ctx->copy_streams;
-  dbg_status st = compact_chains(ctx, g, u, false);
-  for (DevBuf *b : {&u->node_off, &u->nodes, &u->seq_off, &u->seq, &u->circular}) b->al = &u->al;
-  cudaStreamSynchronize(ctx->stream);
-  prof_resolve(ctx);
-  if (st != DBG_OK) {
-    cudaGetLastError();
-    cudaMemsetAsync(ctx->d_err, 0, sizeof(uint32_t), ctx->stream);
-    delete u;
-  } else {
-    *out = u;
-  }
+  const dbg_status st = with_scratch(ctx, [&] {
+    return unitigs_of_call(ctx, out, [&](dbg_unitigs *u) { return compact_chains(ctx, g, u, false); });
+  });
   if (prev >= 0 && prev != ctx->device) cudaSetDevice(prev);
   return st;
 }
@@ -1863,25 +1872,15 @@ dbg_status dbg_compact_bucketed(dbg_ctx *ctx, const dbg_graph *g, uint64_t mem_b
     cudaMemGetInfo(&free_b, &total_b);
     mem_budget = free_b / 2;
   }
-  dbg_unitigs *u = new (std::nothrow) dbg_unitigs();
-  if (!u) return DBG_ENOMEM;
-  u->al = ctx->al;
-  u->device = ctx->device;
-  u->n_copy = ctx->copy_streams;
   uint32_t launches = 0;
-  dbg_status st = g->key_words == 1 ? compact_bucketed_impl<uint64_t>(ctx, g, mem_budget, u, &launches)
-                                    : compact_bucketed_impl<Key128>(ctx, g, mem_budget, u, &launches);
-  for (DevBuf *b : {&u->node_off, &u->nodes, &u->seq_off, &u->seq, &u->circular}) b->al = &u->al;
-  cudaStreamSynchronize(ctx->stream);
-  prof_resolve(ctx);
+  ScratchLimit block(ctx, mem_budget);
+  const dbg_status st = with_scratch(ctx, [&] {
+    return unitigs_of_call(ctx, out, [&](dbg_unitigs *u) {
+      return g->key_words == 1 ? compact_bucketed_impl<uint64_t>(ctx, g, mem_budget, u, &launches)
+                               : compact_bucketed_impl<Key128>(ctx, g, mem_budget, u, &launches);
+    });
+  });
   if (join_launches) *join_launches = launches;
-  if (st != DBG_OK) {
-    cudaGetLastError();
-    cudaMemsetAsync(ctx->d_err, 0, sizeof(uint32_t), ctx->stream);
-    delete u;
-  } else {
-    *out = u;
-  }
   if (prev >= 0 && prev != ctx->device) cudaSetDevice(prev);
   return st;
 }

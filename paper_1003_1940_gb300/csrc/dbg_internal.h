@@ -36,14 +36,23 @@ struct Allocator {
 // and a small build is made of those.  All work of a context is on its one
 // stream and its calls are not concurrent, so a piece may be reused as soon as
 // it is put back.
+//
+// Once an allocation of the context has failed there is no block any more: it
+// goes back as soon as none of it is in use, and the call that failed is made
+// again without it (with_scratch).  A call within a memory budget holds a block
+// of at most a sixteenth of that (ScratchLimit).
 struct Scratch {
-  static constexpr size_t CAP = (size_t)32 << 20;   // the block
-  static constexpr size_t MOST = (size_t)4 << 20;   // larger buffers go to the allocator
+  static constexpr size_t CAP = (size_t)32 << 20, LEAST = (size_t)256 << 10;  // the block
+  static constexpr size_t SHARE = 8;  // buffers of more than 1 / SHARE of it go to the allocator
   struct Piece { size_t off, bytes; bool used; };
+  Allocator *from = nullptr;
   char *base = nullptr;
+  size_t size = 0, limit = CAP;
   std::vector<Piece> pieces;
-  bool short_of_memory = false;  // an allocation failed: no block from then on
-  bool drop(Allocator &al);      // gives the block back, if none of it is in use
+  bool off = false;     // an allocation failed: no block from then on
+  bool missed = false;  // one failed while the block was held
+  bool give_back();     // if none of it is in use
+  bool shortage();      // an allocation failed; true: the block went back
   void *get(Allocator &al, size_t bytes);  // nullptr: no room
   void put(void *p);
 };
@@ -216,6 +225,31 @@ namespace dbg {
   } while (0)
 
 dbg_status alloc_buf(dbg_ctx *ctx, DevBuf &b, size_t bytes);
+
+// A call of the context, made again if it ran out of memory beside the scratch
+// block.
+template <class F>
+dbg_status with_scratch(dbg_ctx *ctx, F call) {
+  ctx->scratch.missed = false;
+  const dbg_status st = call();
+  return st == DBG_ENOMEM && ctx->scratch.missed ? call() : st;
+}
+
+// The scratch block of a call that may hold `budget` bytes.
+struct ScratchLimit {
+  Scratch &s;
+  const size_t before;
+  ScratchLimit(dbg_ctx *ctx, uint64_t budget) : s(ctx->scratch), before(s.limit) { set(s, budget); }
+  ~ScratchLimit() {
+    s.limit = before;
+    if (s.size < before) s.give_back();
+  }
+  static void set(Scratch &s, uint64_t budget) {
+    s.limit = std::min(s.limit, std::max<size_t>(Scratch::LEAST, (size_t)std::min<uint64_t>(budget / 16, Scratch::CAP)));
+    if (s.size > s.limit) s.give_back();
+  }
+};
+
 // Scratch of a call on the context: from its scratch block if it is small.
 dbg_status alloc_tmp(dbg_ctx *ctx, DevBuf &b, size_t bytes);
 // One allocation for several arrays, which become parts of it.

@@ -145,6 +145,7 @@ static void worker_main(dbg_server *srv, int idx) {
           srv->peak_charged = std::max(srv->peak_charged, bud.in_use);
           break;
         }
+        ctx->scratch.give_back();  // an idle worker holds no device memory
         bud.cv.wait(lk);
       }
     }
@@ -240,6 +241,7 @@ dbg_status dbg_server_create(dbg_server **out, const dbg_server_options *opt) {
       return st;
     }
     for (int kd = 0; kd < 4; kd++) c->sort_variant[kd] = o.sort_variant[kd];
+    ScratchLimit::set(c->scratch, srv->budget / o.workers);  // (a running one's is part of its footprint)
     srv->ctxs.push_back(c);
   }
   for (uint32_t i = 0; i < o.workers; i++) srv->workers.emplace_back(worker_main, srv, (int)i);

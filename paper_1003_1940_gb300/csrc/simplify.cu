@@ -342,20 +342,7 @@ dbg_status copy_items(int device, std::initializer_list<std::pair<void *, std::p
 
 extern "C" {
 
-dbg_status dbg_simplify(dbg_ctx *ctx, const dbg_graph *g, uint32_t min_nodes, dbg_simple **out) {
-  if (!out) return DBG_EINVAL;
-  *out = nullptr;
-  if (!ctx || !g) {
-    set_error("ctx or graph is NULL");
-    return DBG_EINVAL;
-  }
-  if (g->num_nodes >= 0x7fffffffull) {
-    set_error("simplification handles fewer than 2^31 nodes");
-    return DBG_EOVERFLOW;
-  }
-  int prev = -1;
-  cudaGetDevice(&prev);
-  if (prev != ctx->device) cudaSetDevice(ctx->device);
+static dbg_status simplify_once(dbg_ctx *ctx, const dbg_graph *g, uint32_t min_nodes, dbg_simple **out) {
   dbg_simple *sg = new (std::nothrow) dbg_simple();
   if (!sg) return DBG_ENOMEM;
   sg->units.al = ctx->al;
@@ -374,6 +361,24 @@ dbg_status dbg_simplify(dbg_ctx *ctx, const dbg_graph *g, uint32_t min_nodes, db
   } else {
     *out = sg;
   }
+  return st;
+}
+
+dbg_status dbg_simplify(dbg_ctx *ctx, const dbg_graph *g, uint32_t min_nodes, dbg_simple **out) {
+  if (!out) return DBG_EINVAL;
+  *out = nullptr;
+  if (!ctx || !g) {
+    set_error("ctx or graph is NULL");
+    return DBG_EINVAL;
+  }
+  if (g->num_nodes >= 0x7fffffffull) {
+    set_error("simplification handles fewer than 2^31 nodes");
+    return DBG_EOVERFLOW;
+  }
+  int prev = -1;
+  cudaGetDevice(&prev);
+  if (prev != ctx->device) cudaSetDevice(ctx->device);
+  const dbg_status st = with_scratch(ctx, [&] { return simplify_once(ctx, g, min_nodes, out); });
   if (prev >= 0 && prev != ctx->device) cudaSetDevice(prev);
   return st;
 }
