@@ -96,14 +96,17 @@ uint64_t build_footprint(uint64_t n, uint64_t bases, uint64_t N, uint64_t I, uin
   // two key buffers, the local pass's count staging, gathered oversize keys
   // (two buffers, their distinct keys and run heads)
   const uint64_t A = 2 * N * w + 4 * N + 3 * N * w + 4 * N;
-  // the distinct keys' buffer and counts, the graph's edge arrays, two
-  // record buffers (key + payload) and the gathered oversize records
-  const uint64_t B = N * w + 4 * E + E * (w + 5) + 4 * R * (w + 4);
+  // the graph's edge arrays, two record buffers (key + payload), the gathered
+  // oversize records in two more, and two words for each that order them
+  const uint64_t B = E * (w + 5) + 4 * R * (w + 4) + 16 * R;
   // records, row offsets, edge arrays, src / dst, adjacency with its sides,
   // partitioned edge ends, node keys and row_ptr
   const uint64_t C = 2 * R * (w + 4) + 8 * (R + 1) + E * (w + 5) + 8 * E + 20 * E + 16 * E + V * (w + 8);
-  const uint64_t tiles = N / 2048 + 1;  // per-tile bounds, counts and scan words
-  return inputs + std::max({A, B, C}) + 64 * tiles + (64ull << 20);
+  // a bit per record for the nodes' first ones; the groups' and their parts'
+  // counts and places (at most one group per 256 keys, a part per 64), the
+  // tiles' tables
+  const uint64_t tables = R / 8 + 12 * (R / 256) + 12 * (R / 64) + 64 * (R / 2048 + 1);
+  return inputs + std::max({A, B, C}) + tables + (64ull << 20);
 }
 
 // Bytes to charge for request r now (bucketed: what is free, once that is
