@@ -375,7 +375,7 @@ SortPlan<K> plan_sort(const dbg_ctx *ctx, uint64_t n, int bits, bool unordered, 
       p.msd = true;
       p.passes = need == 0 ? 0 : need <= 10 ? 1 : 2;
       p.need = need;
-      p.w1 = p.passes == 2 ? need / 2 : need;
+      p.w1 = p.passes == 2 ? std::min(need / 2, MSD_MAX_BITS - 1) : need;  // (records take one bit less)
       return p;
     }
   }
