@@ -126,7 +126,14 @@ dbg_status alloc_block(dbg_ctx *ctx, DevBuf &block, std::initializer_list<BlockP
   auto padded = [](size_t b) { return (std::max<size_t>(b, 1) + 255) & ~(size_t)255; };
   size_t total = 0;
   for (const BlockPart &x : parts) total += padded(x.bytes);
-  DBG_TRY(alloc_buf(ctx, block, total));
+  if (alloc_buf(ctx, block, total) != DBG_OK) {
+    // the allocator may still have the arrays one by one
+    for (const BlockPart &x : parts) {
+      x.buf->release();
+      if (x.bytes) DBG_TRY(alloc_buf(ctx, *x.buf, x.bytes));
+    }
+    return DBG_OK;
+  }
   char *at = static_cast<char *>(block.p);
   for (const BlockPart &x : parts) {
     x.buf->release();

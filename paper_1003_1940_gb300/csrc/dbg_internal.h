@@ -252,7 +252,8 @@ struct ScratchLimit {
 
 // Scratch of a call on the context: from its scratch block if it is small.
 dbg_status alloc_tmp(dbg_ctx *ctx, DevBuf &b, size_t bytes);
-// One allocation for several arrays, which become parts of it.
+// One allocation for several arrays, which become parts of it; or one for each
+// (those of no bytes: NULL), if the allocator does not have it in one piece.
 struct BlockPart {
   DevBuf *buf;
   size_t bytes;

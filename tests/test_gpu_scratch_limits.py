@@ -22,14 +22,16 @@ class Counted:
     def __init__(self, dbg, limit=1 << 60):
         import torch
         self.limit, self.live, self.peak, self.refused = limit, 0, 0, 0
+        self.largest, self.seen = 1 << 60, set()  # of one allocation: the most allowed; the sizes seen
         self.sizes = {}
 
         def alloc(user, nbytes, stream):
-            if self.live + nbytes > self.limit:
+            if self.live + nbytes > self.limit or nbytes > self.largest:
                 self.refused += 1
                 return None
             p = int(torch.cuda.caching_allocator_alloc(int(nbytes), 0, stream or 0))
             self.sizes[p] = nbytes
+            self.seen.add(nbytes)
             self.live += nbytes
             self.peak = max(self.peak, self.live)
             return p
@@ -120,3 +122,26 @@ def test_budgeted_call(data, budget_mb):
     assert hooks.live == 0
     dbg.dbg_build(hooks.ctx, reads, lengths, 31)
     assert hooks.live == BLOCK  # and the next call has its own again
+
+
+@pytest.mark.parametrize("k", [31, 41])
+def test_arrays_one_by_one(data, k):
+    """Memory that has room for every array but not for several in one piece:
+    the graph's arrays are then allocations of their own."""
+    from paper_1003_1940_gb300 import dbg
+    reads, lengths = data
+    hooks = Counted(dbg)
+    g = dbg.dbg_build(hooks.ctx, reads, lengths, k)
+    want = graph_of(dbg, g)
+    other = Counted(dbg)
+    other.largest = max(n for n in hooks.seen if n != BLOCK) - 1
+    h = dbg.dbg_build(other.ctx, reads, lengths, k)
+    for key, array in graph_of(dbg, h).items():
+        np.testing.assert_array_equal(array, want[key], err_msg=key)
+    assert other.refused > 0
+    other.largest = 1 << 60
+    u, v = dbg.dbg_unitigs_get(dbg.dbg_compact(hooks.ctx, g)), dbg.dbg_unitigs_get(dbg.dbg_compact(other.ctx, h))
+    for key in u:
+        assert np.array_equal(np.asarray(u[key]), np.asarray(v[key])), key
+    del h, v
+    assert other.live in (0, BLOCK)
