@@ -845,6 +845,7 @@ struct EdgeTiles {
   uint64_t tiles = 0;
   DevBuf bound, tcount, toff, mult;
   bool uneven = false;  // the sort split long groups
+  bool dense = false;   // mult holds one per edge, in edge order
   void release() {
     for (DevBuf *b : {&bound, &tcount, &toff, &mult}) b->release();
   }
@@ -1551,6 +1552,19 @@ dbg_status build_graph_impl(dbg_ctx *ctx, const BuildInput &in, dbg_graph *g) {
   // ---- node multiplicities (optional), while the packed reads are here ----
   DevBuf node_counts, read_counts;
   uint64_t Vk = 0, Vr = 0;
+  if ((ctx->node_mult || ctx->node_reads) && E > 0 && !headpos.p) {
+    // the counts' sorts are the fullest point then: 4 bytes per edge beside
+    // them instead of 4 per instance
+    DevBuf dense;
+    DBG_TRY(alloc_tmp(ctx, dense, E * sizeof(uint32_t)));
+    DBG_LAUNCH(ctx, ST_NODE_MULT, 8.0 * E,
+               k_mult_compact<<<(unsigned)std::min<uint64_t>(edge_tiles.tiles, 152ull * 16), 256, 0, s>>>(
+                   edge_tiles.bound.as<uint64_t>(), edge_tiles.tcount.as<uint32_t>(), edge_tiles.toff.as<uint64_t>(),
+                   edge_tiles.tiles, edge_tiles.mult.as<uint32_t>(), dense.as<uint32_t>()));
+    DBG_CUDA_TRY(cudaGetLastError());
+    edge_tiles.mult = std::move(dense);
+    edge_tiles.dense = true;
+  }
   if (ctx->node_mult)
     DBG_TRY(count_node_kmers<K>(ctx, packed, base_off, in.d_lengths, n, N, k, d_hist, d_digit_base, node_counts,
                                 &Vk));
@@ -1587,7 +1601,7 @@ dbg_status build_graph_impl(dbg_ctx *ctx, const BuildInput &in, dbg_graph *g) {
                  k_endpoints_tiles<K><<<(unsigned)((edge_tiles.tiles + per - 1) / per), EMIT_BLOCK, 0, s>>>(
                      edge_tiles.bound.as<uint64_t>(), edge_tiles.tcount.as<uint32_t>(),
                      edge_tiles.toff.as<uint64_t>(), (uint32_t)edge_tiles.tiles, (uint32_t)per, uniq.as<K>(),
-                     edge_tiles.mult.as<uint32_t>(), k, out, nspec, d_hist));
+                     edge_tiles.mult.as<uint32_t>(), edge_tiles.dense, k, out, nspec, d_hist));
     }
   }
   if (I > 0) {

@@ -1408,16 +1408,16 @@ __global__ __launch_bounds__(EMIT_BLOCK) void k_endpoints(const K *__restrict__ 
 }
 
 // The same from the local pass's tiles, where tile t's tcount[t] distinct keys
-// and their multiplicities start at bound[t] and its edges at toff[t]: they
-// need no dense copy in between.  A CTA takes `per` consecutive tiles, so that
+// and their multiplicities start at bound[t] and its edges at toff[t] (so do the
+// multiplicities if they are `dense`): they need no dense copy in between.  A CTA takes `per` consecutive tiles, so that
 // what the chip writes at one time lies together.  Bound by memory: 1.57 ms
 // for 190 M edges (49 bytes each); with a dense copy first 1.57 + 0.96.
 // (per = 24: 1.79; a resident grid that takes every 1216th tile: 2.1.)
 template <class K>
 __global__ __launch_bounds__(EMIT_BLOCK) void k_endpoints_tiles(
     const uint64_t *__restrict__ bound, const uint32_t *__restrict__ tcount, const uint64_t *__restrict__ toff,
-    uint32_t tiles, uint32_t per, const K *__restrict__ ustage, const uint32_t *__restrict__ mstage, uint32_t k, EdgeOut<K> out,
-    DigitSpec ds, unsigned long long *__restrict__ hist) {
+    uint32_t tiles, uint32_t per, const K *__restrict__ ustage, const uint32_t *__restrict__ mstage, bool dense,
+    uint32_t k, EdgeOut<K> out, DigitSpec ds, unsigned long long *__restrict__ hist) {
   __shared__ uint32_t s_hist[MAX_PASSES * RADIX];
   for (int i = threadIdx.x; i < ds.entries(); i += EMIT_BLOCK) s_hist[i] = 0;
   __syncthreads();
@@ -1434,6 +1434,7 @@ __global__ __launch_bounds__(EMIT_BLOCK) void k_endpoints_tiles(
       s_next = bound[next];
       o_next = toff[next];
     }
+    const uint32_t *const mt = mstage + (dense ? o : s);
     for (uint32_t r0 = threadIdx.x; r0 < n; r0 += ROWS * EMIT_BLOCK) {
       K z[ROWS];
       uint32_t c[ROWS];
@@ -1442,7 +1443,7 @@ __global__ __launch_bounds__(EMIT_BLOCK) void k_endpoints_tiles(
         const uint32_t r = r0 + i * EMIT_BLOCK;
         if (r < n) {
           z[i] = ustage[s + r];
-          c[i] = mstage[s + r];
+          c[i] = mt[r];
         }
       }
 #pragma unroll

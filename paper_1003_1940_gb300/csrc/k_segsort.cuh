@@ -1287,6 +1287,16 @@ __global__ void k_seg_compact(const uint64_t *__restrict__ bound, const uint32_t
   }
 }
 
+// The multiplicities alone.
+static __global__ void k_mult_compact(const uint64_t *__restrict__ bound, const uint32_t *__restrict__ tcount,
+                                      const uint64_t *__restrict__ toff, uint64_t tiles,
+                                      const uint32_t *__restrict__ mstage, uint32_t *__restrict__ mult) {
+  for (uint64_t t = blockIdx.x; t < tiles; t += gridDim.x) {
+    const uint64_t s = bound[t], o = toff[t];
+    for (uint32_t r = threadIdx.x; r < tcount[t]; r += blockDim.x) mult[o + r] = mstage[s + r];
+  }
+}
+
 // Edge keys of a tile with few copies each: every copy is ranked, as the
 // records are by k_seg_rank, by a counting sort over buckets of the top bits
 // of the key offsets and comparisons within the bucket; then the runs of equal

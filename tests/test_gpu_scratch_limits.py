@@ -145,3 +145,22 @@ def test_arrays_one_by_one(data, k):
         assert np.array_equal(np.asarray(u[key]), np.asarray(v[key])), key
     del h, v
     assert other.live in (0, BLOCK)
+
+
+@pytest.mark.parametrize("k", [31, 55])
+def test_counts_hold_no_staged_multiplicities(k):
+    """The most device memory of a build with both counts, itemised: the k-mer
+    sort beside the distinct edge keys' buffer and one multiplicity per edge,
+    not per instance."""
+    from paper_1003_1940_gb300 import dbg
+    n, L, w = 200_000, 100, 8 if k <= 31 else 16
+    reads, lengths = readgen.generate(readgen.ReadSetSpec(n * L // 30, n, L, 0.002, k, 8))
+    hooks = Counted(dbg)
+    dbg.dbg_node_mult_set(hooks.ctx, True)
+    dbg.dbg_node_reads_set(hooks.ctx, True)
+    g = dbg.dbg_build(hooks.ctx, reads, lengths, k)
+    N, M, E, V = n * (L - k), n * (L - k + 1), dbg.dbg_graph_num_edges(g), dbg.dbg_graph_num_nodes(g)
+    held = N * w + 4 * E + 4 * V + n * L // 4 + 24 * n
+    sort = M * (2 * w + 8) + 12 * M
+    tables = M // 4 + (2 << 20)
+    assert hooks.peak <= BLOCK + held + sort + tables, (hooks.peak, held, sort)
