@@ -97,12 +97,16 @@ struct LowBits {
   const uint32_t *gfirst = nullptr;
   const uint8_t *split = nullptr;
   template <class K>
-  __device__ __forceinline__ int of(const K &key) const {
-    const uint32_t b = low ? (uint32_t)KeyOps<K>::words_lo(KeyOps<K>::shr(key, shift1)) : 0u;
-    const int bits = low ? low[b] : fixed;
-    if (!split) return bits;
+  __device__ __forceinline__ uint32_t bucket(const K &key) const {
+    return (uint32_t)KeyOps<K>::words_lo(KeyOps<K>::shr(key, shift1));
+  }
+  template <class K>
+  __device__ __forceinline__ int unsplit(const K &key) const { return low ? low[bucket(key)] : fixed; }
+  // ... and of those, the bits that a split took (bits = unsplit(key))
+  template <class K>
+  __device__ __forceinline__ int taken(const K &key, int bits) const {
     const uint32_t above = (uint32_t)KeyOps<K>::words_lo(KeyOps<K>::shr(key, bits));
-    return bits - split[low ? gfirst[b] + (above & ((1u << (shift1 - bits)) - 1u)) : above];
+    return split[low ? gfirst[bucket(key)] + (above & ((1u << (shift1 - bits)) - 1u)) : above];
   }
 };
 

@@ -400,7 +400,7 @@ __global__ void k_msd_split(const K *__restrict__ keys, const uint64_t *__restri
   for (uint32_t g = blockIdx.x * blockDim.x + threadIdx.x; g < NG; g += gridDim.x * blockDim.x) {
     const uint64_t s = goff[g], e = goff[g + 1], c = e - s;
     if (c <= longest) continue;
-    const int low = lb.of(keys[s]);
+    const int low = lb.unsplit(keys[s]);
     if (low == 0 || copies_of_one(keys, s, c)) continue;
     int w = 0;
     while (w < min(MSD_SPLIT_BITS, low) && ((uint64_t)mean << w) < c) w++;

@@ -184,8 +184,13 @@ __device__ __forceinline__ void seg_setup(S &sm, const K *__restrict__ kin, cons
     sm.bound[1] = e;
     if (e > s) {
       const K first = kin[s], last = kin[e - 1];
-      sm.base = KeyOps<K>::sub(first, KeyOps<K>::mask_low(first, lb.of(first)));
-      const K range = KeyOps<K>::sub(KeyOps<K>::fill_low(last, lb.of(last)), sm.base);
+      int low_first = lb.unsplit(first), low_last = lb.unsplit(last);  // (both loads in flight)
+      if (lb.split) {
+        low_first -= lb.taken(first, low_first);
+        low_last -= lb.taken(last, low_last);
+      }
+      sm.base = KeyOps<K>::sub(first, KeyOps<K>::mask_low(first, low_first));
+      const K range = KeyOps<K>::sub(KeyOps<K>::fill_low(last, low_last), sm.base);
       sm.span_bits = (uint32_t)KeyOps<K>::bitlen(range);
       sm.passes = max(1u, (sm.span_bits + RADIX_BITS - 1) / RADIX_BITS);
       sm.range = range;
@@ -1125,9 +1130,9 @@ __global__ __launch_bounds__(SEG_BLOCK, 4) void k_seg_count(
       const uint32_t j = j0 + (uint32_t)i * SEG_BLOCK + tid;
       d[i] = j < cnt ? KeyOps<K>::sub(kin[s + j], base) : O::empty();
     }
-    // (the whole warp leaves or none of it: another warp may set the flag while
-    // this one reads it, and the sample below counts with all lanes)
-    if (__any_sync(0xffffffffu, *reinterpret_cast<volatile uint32_t *>(&sm.overflow))) break;
+    // (not in the first batch: another warp may set the flag between two lanes'
+    // reads of it, and the sample below counts with all lanes of the warp)
+    if (j0 > 0 && *reinterpret_cast<volatile uint32_t *>(&sm.overflow)) break;
 #pragma unroll
     for (int i = 0; i < S::LOAD; i++) {
       // (128-bit tiles are one batch long; in 64-bit ones, of two, a test here
