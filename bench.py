@@ -59,7 +59,7 @@ def parse():
     ap.add_argument("--count-first", type=int, default=1, choices=(0, 1),
                     help="1: the edge keys' local pass counts copies in a hash table before sorting")
     ap.add_argument("--partition-first", type=int, default=1, choices=(0, 1),
-                    help="1: the edge keys' first global pass is an unordered partition")
+                    help="1: the sorts' global passes are unordered partitions, most significant digit first")
     ap.add_argument("--copy-streams", type=int, default=0,
                     help="streams the end-to-end read-back is spread over (0: the library's default)")
     ap.add_argument("--local-rank", type=int, default=1, choices=(0, 1),

@@ -432,10 +432,13 @@ dbg_status dbg_rle_u64_noalloc(const uint64_t *keys, uint64_t n, uint64_t *uniq,
                                uint64_t *count, void *stream);
 
 /* ----------------------------------------------------------------------
- * Radix sort variants and the autotuner.  The onesweep sort of STEP-2/3 is
+ * Radix sort variants and the autotuner.  The stable onesweep passes are
  * compiled in several configurations per key kind (tile shape, TMA or
  * register loads, ballot / atomicOr / match.any ranking); all sort
- * identically.  Kinds: 0 = 64-bit keys, 1 = 64-bit keys + 32-bit payload,
+ * identically.  A build runs them where it does not use the partition passes
+ * (keys of few bits, the gathered keys of oversize tiles, or a switch below
+ * off); the partition passes have no variants, so tuning changes little for
+ * most read sets.  Kinds: 0 = 64-bit keys, 1 = 64-bit keys + 32-bit payload,
  * 2 = 128-bit keys, 3 = 128-bit keys + payload; kinds 4 (64-bit keys) and
  * 5 (128-bit keys) select the ranking method of the hybrid sort's local
  * pass (0 = match.any, 1 = shared-memory atomicOr, 2 = ballots).  A context
@@ -462,8 +465,10 @@ dbg_status dbg_autotune(dbg_ctx *ctx, uint64_t n, const char *cache_path, double
  * memory (for the edge keys fused with STEP-2's duplicate removal).  Runs
  * longer than shared memory holds (6144 keys for k <= 31, 3072 above; e.g.
  * the (k+1)-mers of a tandem repeat) are gathered and sorted over every
- * digit globally instead; the result is the same either way.
- * dbg_sort_fallbacks counts the sorts of the context that had such runs.
+ * digit globally instead, unless they are many and hold many keys each (an
+ * uneven base composition): then the long groups are partitioned once more.
+ * The result is the same either way.  dbg_sort_fallbacks counts the sorts of
+ * the context that gathered such runs.
  * on = 0 sorts every digit globally.
  * -------------------------------------------------------------------- */
 dbg_status dbg_sort_hybrid_set(dbg_ctx *ctx, int on);
@@ -475,7 +480,8 @@ uint64_t dbg_sort_fallbacks(const dbg_ctx *ctx);
  * shared-memory hash table of 2048 slots and sorts only the distinct keys,
  * which at read coverage c are about 1/c of them; a tile whose distinct
  * keys do not fit (about 1500 and up), or whose first keys are nearly all
- * distinct, is sorted copy by copy instead, and dbg_sort_count_overflows counts such tiles over the context's builds.
+ * distinct, is sorted copy by copy instead, and dbg_sort_count_overflows
+ * counts such tiles over the context's builds.
  * Off, every tile is sorted copy by copy.  The edge list is the same
  * either way.
  * -------------------------------------------------------------------- */

@@ -84,3 +84,20 @@ def test_circles_that_share_a_stretch():
     reads += [circle(rng, 1_234, k), bases(rng, 500)]
     u = check(reads, k)
     assert int(u["circular"].sum()) == 1
+
+
+@pytest.mark.parametrize("long_lists", [False, True])
+def test_links_are_made_once(long_lists):
+    """A circle among the chains does not send the graph through the link
+    kernels again (two launches; with long lists one more, which takes the
+    successors from what they made)."""
+    from paper_1003_1940_gb300 import dbg
+    k = 21
+    rng = np.random.default_rng(3)
+    reads = [circle(rng, 500, k)] + [bases(rng, 30_000 if long_lists else 60) for _ in range(2 if long_lists else 3_000)]
+    ctx = dbg.Context()
+    g = dbg.dbg_build(ctx, np.concatenate(reads), np.array([len(r) for r in reads], dtype=np.uint32), k)
+    dbg.dbg_profile_enable(ctx, True)
+    u = dbg.dbg_unitigs_get(dbg.dbg_compact(ctx, g))
+    assert int(u["circular"].sum()) == 1
+    assert dbg.dbg_profile_read(ctx)["compact_links"]["launches"] == (3 if long_lists else 2)
