@@ -177,7 +177,13 @@ class _TorchAllocator:
 
 
 class Context:
-    """dbg_ctx: device, stream, allocator."""
+    """dbg_ctx: device, stream, allocator.
+
+    Graphs and unitigs release their memory on the context's stream, so the
+    dbg_ctx goes after the last of them, in whatever order they are closed or
+    collected (a cycle's finalizers run in no particular order)."""
+
+    _live = _dying = ()  # handles of results not yet freed; dbg_ctx handles that wait for them
 
     def __init__(self, device: int | None = None, stream=None, torch_allocator: bool = True,
                  mem_budget: int = 0, spin_limit: int = 0):
@@ -204,11 +210,23 @@ class Context:
         h = ctypes.c_void_p()
         _check(lib.dbg_create(ctypes.byref(h), ctypes.byref(opt)), "dbg_create")
         self.handle = h
+        self._live, self._dying = set(), []
+
+    def _adopt(self, result):
+        self._live.add(id(result))
+
+    def _release(self, result):
+        self._live.discard(id(result))
+        while self._dying and not self._live and _lib is not None:
+            _lib.dbg_destroy(self._dying.pop())
 
     def close(self):
         if getattr(self, "handle", None) is not None and _lib is not None:
-            _lib.dbg_destroy(self.handle)
-            self.handle = None
+            h, self.handle = self.handle, None
+            if self._live:
+                self._dying.append(h)
+            else:
+                _lib.dbg_destroy(h)
 
     def __del__(self):
         self.close()
@@ -228,34 +246,40 @@ def _ptr(x) -> tuple[int, object]:
     raise TypeError(f"unsupported buffer type {type(x)}")
 
 
-class Graph:
-    """dbg_graph handle; holds its context so the context outlives it."""
+class _Result:
+    """A handle whose memory is released through its context's stream and
+    hooks, so that the context outlives it.  (A server's graphs are not: they
+    may be freed after it.)"""
 
-    def __init__(self, ctx: Context, handle):
+    _free = ""  # the C entry point
+
+    def __init__(self, ctx, handle):
         self.ctx = ctx
         self.handle = handle
+        if isinstance(ctx, Context):
+            ctx._adopt(self)
 
     def free(self):
         if getattr(self, "handle", None) is not None and _lib is not None:
-            _lib.dbg_graph_free(self.handle)
-            self.handle = None
+            h, self.handle = self.handle, None
+            getattr(_lib, self._free)(h)
+            if isinstance(self.ctx, Context):
+                self.ctx._release(self)
 
     def __del__(self):
         self.free()
 
 
-class Unitigs:
-    def __init__(self, ctx: Context, handle):
-        self.ctx = ctx
-        self.handle = handle
+class Graph(_Result):
+    """dbg_graph handle."""
 
-    def free(self):
-        if getattr(self, "handle", None) is not None and _lib is not None:
-            _lib.dbg_unitigs_free(self.handle)
-            self.handle = None
+    _free = "dbg_graph_free"
 
-    def __del__(self):
-        self.free()
+
+class Unitigs(_Result):
+    """dbg_unitigs handle."""
+
+    _free = "dbg_unitigs_free"
 
 
 def dbg_create(**kw) -> Context:
@@ -445,19 +469,10 @@ def dbg_unitigs_get_into(u: Unitigs, node_off: int | None = None, nodes: int | N
     _check(_lib.dbg_unitigs_get(u.handle, *ptrs), "dbg_unitigs_get")
 
 
-class Simple:
+class Simple(_Result):
     """dbg_simple: the simplified graph (units and relabelled edges)."""
 
-    def __init__(self, ctx: Context, handle):
-        self.ctx, self.handle = ctx, handle
-
-    def free(self):
-        if getattr(self, "handle", None) is not None and _lib is not None:
-            _lib.dbg_simple_free(self.handle)
-            self.handle = None
-
-    def __del__(self):
-        self.free()
+    _free = "dbg_simple_free"
 
 
 def dbg_simplify(ctx: Context, g: Graph, min_nodes: int = 3) -> Simple:
