@@ -346,7 +346,7 @@ void dbg_server_options_init(dbg_server_options *opt);
  *     budget) is queued again until another request finishes; alone, it
  *     fails with DBG_ENOMEM;
  *   - a worker's block of small buffers is part of its request's footprint,
- *     and an idle worker holds none.
+ *     and a worker that has been idle for some milliseconds holds none.
  * Results are the same graphs dbg_build returns for the same read set. */
 dbg_status dbg_server_create(dbg_server **srv, const dbg_server_options *opt);
 /* Waits for running requests; frees results nobody polled. */

@@ -449,11 +449,12 @@ struct Groups {
   uint32_t ng_max = 0;                  // at most that many (0: no MSD pass)
 };
 
-// The local pass's tile bounds from the places of the groups (but those that
-// are split), which are copied to `cursor` (if given).
 inline const uint64_t *group_places(const Groups &gr) {
   return gr.ng ? gr.tables.as<uint64_t>() : gr.goff.as<uint64_t>();
 }
+
+// The local pass's tile bounds from the places of the groups (but those that
+// are split), which are copied to `cursor` (if given).
 template <class K>
 dbg_status msd_bounds(dbg_ctx *ctx, Groups &gr, uint64_t n, uint32_t *cursor, int stage) {
   constexpr uint64_t T = SegShape<K>::TILE;
@@ -691,12 +692,10 @@ dbg_status seg_tiles(dbg_ctx *ctx, const K *kin, uint64_t n, Groups &gr, TileSet
   }
   DBG_CUDA_TRY(cudaMemsetAsync(ctx->d_counters + CT_GATHERED, 0, (CT_MIXED - CT_GATHERED + 1) * 4, s));
   DBG_LAUNCH(ctx, stage, 0.0,
-             k_seg_oversize<K><<<grid_for(tiles, 256), 256, 0, s>>>(kin, ts.bound.as<uint64_t>(), tiles,
-                                                                 (uint32_t)(SEG_BLOCK * Sh::ITEMS),
-                                                                 ts.osize.as<uint32_t>(), ts.olist.as<uint32_t>(),
-                                                                 ctx->d_counters + CT_GATHERED,
-                                                                 ctx->d_counters + CT_MIXED,
-                                                                 ctx->d_counters + CT_OVERSIZE, ctx->d_err));
+             k_seg_oversize<K><<<grid_for(tiles, 256), 256, 0, s>>>(
+                 kin, ts.bound.as<uint64_t>(), tiles, (uint32_t)(SEG_BLOCK * Sh::ITEMS), ts.osize.as<uint32_t>(),
+                 ts.olist.as<uint32_t>(), ctx->d_counters + CT_GATHERED, ctx->d_counters + CT_MIXED,
+                 ctx->d_counters + CT_OVERSIZE, ctx->d_err));
   DBG_CUDA_TRY(cudaGetLastError());
   return DBG_OK;
 }

@@ -164,3 +164,33 @@ def test_counts_hold_no_staged_multiplicities(k):
     sort = M * (2 * w + 8) + 12 * M
     tables = M // 4 + (2 << 20)
     assert hooks.peak <= BLOCK + held + sort + tables, (hooks.peak, held, sort)
+
+
+def test_idle_workers_hold_nothing(data):
+    """Device memory after a server has been idle for a while is what it was
+    before its workers built anything (its contexts take cudaMallocAsync memory:
+    the pool's bytes in use are looked at)."""
+    import time
+
+    import torch
+    from paper_1003_1940_gb300 import dbg
+    reads, lengths = data
+
+    def in_use():
+        torch.cuda.synchronize()
+        cudart = ctypes.CDLL(None)
+        pool, used = ctypes.c_void_p(), ctypes.c_uint64()
+        get, attr = cudart.cudaDeviceGetDefaultMemPool, cudart.cudaMemPoolGetAttribute
+        assert get(ctypes.byref(pool), 0) == 0 and attr(pool, 7, ctypes.byref(used)) == 0  # UsedMemCurrent
+        return used.value
+
+    srv = dbg.Server(workers=3)
+    before = in_use()
+    tickets = [dbg.dbg_submit(srv, reads, lengths, 31) for _ in range(6)]
+    for t in tickets:
+        g, _ = dbg.dbg_poll(srv, t)
+        g.free()
+    time.sleep(0.1)
+    held = in_use() - before
+    srv.close()
+    assert held < BLOCK  # (the look-back words of each context stay)
