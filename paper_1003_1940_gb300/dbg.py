@@ -183,7 +183,7 @@ class Context:
     dbg_ctx goes after the last of them, in whatever order they are closed or
     collected (a cycle's finalizers run in no particular order)."""
 
-    _live = _dying = ()  # handles of results not yet freed; dbg_ctx handles that wait for them
+    _live, _dying = frozenset(), ()  # results not yet freed; dbg_ctx handles that wait for them
 
     def __init__(self, device: int | None = None, stream=None, torch_allocator: bool = True,
                  mem_budget: int = 0, spin_limit: int = 0):
@@ -212,11 +212,7 @@ class Context:
         self.handle = h
         self._live, self._dying = set(), []
 
-    def _adopt(self, result):
-        self._live.add(id(result))
-
-    def _release(self, result):
-        self._live.discard(id(result))
+    def _destroy_waiting(self):
         while self._dying and not self._live and _lib is not None:
             _lib.dbg_destroy(self._dying.pop())
 
@@ -251,35 +247,40 @@ class _Result:
     hooks, so that the context outlives it.  (A server's graphs are not: they
     may be freed after it.)"""
 
-    _free = ""  # the C entry point
+    handle = None
 
     def __init__(self, ctx, handle):
         self.ctx = ctx
         self.handle = handle
-        if isinstance(ctx, Context):
-            ctx._adopt(self)
+        ctx._live.add(id(self))
 
     def free(self):
-        if getattr(self, "handle", None) is not None and _lib is not None:
-            h, self.handle = self.handle, None
-            getattr(_lib, self._free)(h)
-            if isinstance(self.ctx, Context):
-                self.ctx._release(self)
+        handle = self.handle
+        if handle is not None and _lib is not None:
+            self.handle = None
+            self._free(handle)
+            ctx = self.ctx
+            ctx._live.discard(id(self))
+            if ctx._dying:
+                ctx._destroy_waiting()
 
-    def __del__(self):
-        self.free()
+    __del__ = free
 
 
 class Graph(_Result):
     """dbg_graph handle."""
 
-    _free = "dbg_graph_free"
+    @staticmethod
+    def _free(handle):
+        _lib.dbg_graph_free(handle)
 
 
 class Unitigs(_Result):
     """dbg_unitigs handle."""
 
-    _free = "dbg_unitigs_free"
+    @staticmethod
+    def _free(handle):
+        _lib.dbg_unitigs_free(handle)
 
 
 def dbg_create(**kw) -> Context:
@@ -472,7 +473,9 @@ def dbg_unitigs_get_into(u: Unitigs, node_off: int | None = None, nodes: int | N
 class Simple(_Result):
     """dbg_simple: the simplified graph (units and relabelled edges)."""
 
-    _free = "dbg_simple_free"
+    @staticmethod
+    def _free(handle):
+        _lib.dbg_simple_free(handle)
 
 
 def dbg_simplify(ctx: Context, g: Graph, min_nodes: int = 3) -> Simple:
@@ -679,6 +682,8 @@ def _readset(reads, lengths, k, flags=0):
 
 class Server:
     """dbg_server: worker threads with one context and stream each."""
+
+    _live, _dying = set(), ()  # (its graphs may be freed after it)
 
     def __init__(self, device=None, workers=4, mem_budget=0, spin_limit=0, sort_variant=(0, 0, 0, 0)):
         import torch
