@@ -97,16 +97,15 @@ __global__ void k_seg_oversize(const K *__restrict__ kin, uint64_t *__restrict__
                                uint32_t *__restrict__ osize, uint32_t *__restrict__ olist,
                                uint32_t *__restrict__ keys, uint32_t *__restrict__ mixed,
                                uint32_t *__restrict__ count, const uint32_t *__restrict__ err) {
-  if (*err & (ERR_TIMEOUT | ERR_INTERNAL)) {
-    for (uint64_t t = (uint64_t)blockIdx.x * blockDim.x + threadIdx.x; t < tiles; t += (uint64_t)gridDim.x * blockDim.x) {
+  for (uint64_t t = (uint64_t)blockIdx.x * blockDim.x + threadIdx.x; t < tiles; t += (uint64_t)gridDim.x * blockDim.x) {
+    const uint32_t gave_up = *err & (ERR_TIMEOUT | ERR_INTERNAL);  // (loaded with the bounds)
+    const uint64_t s = bound[t], sz = bound[t + 1] - s;
+    if (gave_up) {
       bound[t] = 0;
       osize[t] = 0;
       if (t == tiles - 1) bound[tiles] = 0;
+      continue;
     }
-    return;
-  }
-  for (uint64_t t = (uint64_t)blockIdx.x * blockDim.x + threadIdx.x; t < tiles; t += (uint64_t)gridDim.x * blockDim.x) {
-    const uint64_t s = bound[t], sz = bound[t + 1] - s;
     osize[t] = sz > cap ? (uint32_t)sz : 0u;
     if (sz > cap) {
       atomicAdd(keys, (uint32_t)sz);
