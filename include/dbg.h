@@ -220,8 +220,8 @@ dbg_status dbg_compact(dbg_ctx *ctx, const dbg_graph *g, dbg_unitigs **out);
  * segments (pointer jumping over about one strand-node in 16); the nodes on
  * cycles, if there are any, apart from the lists by pointer jumping.
  * 1: the same with 64-bit walk words at any size they allow; 2: pointer
- * jumping over all strand-nodes.  The unitigs are the same either way.  DBG_EINVAL for another
- * mode. */
+ * jumping over all strand-nodes.  The unitigs are the same either way.
+ * DBG_EINVAL for another mode. */
 dbg_status dbg_compact_mode_set(dbg_ctx *ctx, int mode);
 
 /* Streams over which the read-back of a graph (dbg_graph_*_async) or of
